@@ -78,7 +78,7 @@ __device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
 // A wait with a shortened limit: polls with mbarrier.test_wait, so the limit
 // holds even when it is shorter than the interval try_wait may sleep.  Kept
 // out of line: the default path below stays as short as it was.
-__device__ __noinline__ bool mbar_wait_short(uint64_t* bar, uint32_t parity, long long limit) {
+static __device__ __noinline__ bool mbar_wait_short(uint64_t* bar, uint32_t parity, long long limit) {
   const long long t0 = clock64();
   while (!mbar_test(bar, parity)) {
     if (clock64() - t0 > limit) return false;

@@ -413,6 +413,13 @@ void fold_marks(xk_handle* h) {
   h->marks.clear();
 }
 
+// Scratch of the tensor-core form of an M x N product (DGemm::scale) in a
+// buffer of `doubles` doubles that is idle during the call; null when it is too
+// small, which leaves the product to the CUDA cores.
+int* digit_scratch(double* buf, size_t doubles, int M, int N) {
+  return 2 * doubles >= xk::digit_scale_ints(M, N) ? reinterpret_cast<int*>(buf) : nullptr;
+}
+
 // Enqueue one FP64 build on h->stream.  C is in h->C; results land in h->K, h->Ex.
 int enqueue_fp64(xk_handle* h) {
   using xk::DGemm;
@@ -422,6 +429,7 @@ int enqueue_fp64(xk_handle* h) {
   auto G = [&](int M, int Nc, int K, const double* A, long lda, bool ta, const double* B, long ldb,
                bool tb, double* C, long ldc, const double* H, long ldh) {
     DGemm g{M, Nc, K, A, lda, ta, B, ldb, tb, C, ldc, 1.0, H, ldh, 0, h->work};
+    g.scale = digit_scratch(h->MA, (size_t)ga * N, M, Nc);  // M_A: the full K's, idle here
     return xk::dgemm(g, s);
   };
   {  // Eq. rpsEx step 1: orbitals on the grid and at the interpolation points.
@@ -480,6 +488,7 @@ int enqueue_energy(xk_handle* h) {
   auto G = [&](int M, int Nc, int K, const double* A, long lda, bool ta, const double* B, long ldb,
                bool tb, double* C, long ldc) {
     DGemm g{M, Nc, K, A, lda, ta, B, ldb, tb, C, ldc, 1.0, nullptr, 0, 0, h->work};
+    g.scale = digit_scratch(h->MA, (size_t)ga * N, M, Nc);
     return xk::dgemm(g, s);
   };
   {
@@ -514,6 +523,7 @@ int enqueue_full(xk_handle* h) {
   auto G = [&](int M, int Nc, int K, const double* A, long lda, bool ta, const double* B, long ldb,
                bool tb, double* C, long ldc, const double* H, long ldh) {
     DGemm g{M, Nc, K, A, lda, ta, B, ldb, tb, C, ldc, 1.0, H, ldh, 0, h->work};
+    g.scale = digit_scratch(h->M1, (size_t)n * ng, M, Nc);  // M_1: the build's, idle here
     return xk::dgemm(g, s);
   };
   {
@@ -1111,6 +1121,7 @@ int xk_coulomb(xk_handle* h, int32_t grid, double L, const double* C, double* J_
   {
     StepMark m(h, XK_STEP_ORBITALS);
     xk::DGemm g1{(int)ng, n, N, h->phi, N, false, h->Ce, n, false, h->psi, n, 1.0, nullptr, 0, 0, h->work};
+    g1.scale = digit_scratch(h->M1, (size_t)n * ng, (int)ng, n);
     XK_CUDA(xk::dgemm(g1, s));
   }
   {  // density, Poisson solve, J = dV Phi^T (v o Phi), E_J = dV sum rho v
@@ -1118,6 +1129,7 @@ int xk_coulomb(xk_handle* h, int32_t grid, double L, const double* C, double* J_
     XK_CUDA(xk::coulomb_potential_f64(h->psi, (long)ng, n, grid, L, h->Jtw, h->Jrho, h->Jc0, h->Jc1, s));
     XK_CUDA(xk::potential_rows_f64(h->Jc0, h->phi, (long)ng, N, h->Jv, h->Jphiv, s));
     xk::DGemm gj{N, N, (int)ng, h->phi, N, true, h->Jphiv, N, false, h->Jout, N, h->dV, nullptr, 0, 0, h->work};
+    gj.scale = digit_scratch(h->M1, (size_t)n * ng, N, N);
     XK_CUDA(xk::dgemm(gj, s));
     XK_CUDA(xk::dot_f64(h->Jrho, h->Jv, (long)ng, h->dV, h->red, h->Jout + (size_t)N * N, s));
   }

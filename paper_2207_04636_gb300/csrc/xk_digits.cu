@@ -1,0 +1,670 @@
+// FP64 products on the tensor cores by splitting both operands into exact
+// 8-bit digits (the scheme of Ozaki, Ogita, Oishi and Rump, Numer. Algorithms
+// 59 (2012), and its tensor-core form by Ootomo, Ozaki and Yokota, IJHPCA 38
+// (2024)).
+//
+// Every operand row (the K direction) has a power-of-two scale 2^e > max|row|;
+// an element becomes the integer X = round(x 2^(55 - e)), |X| < 127 2^48, and
+// X = sum_i d_i 2^(8 (6 - i)) with seven signed digits |d_i| <= 128, exact in
+// FP16.  A product of two digits is an integer <= 2^14, and tcgen05.mma adds
+// such integers exactly in its FP32 accumulator while the sum stays below
+// 2^24.  The products d_i d'_j of one weight l = i + j share an accumulator;
+// levels 0 to 7 are formed (34 of the 49 products), every 256 terms they are
+// drained into an integer accumulator of 64 + 20 bits (levels 0 to 3 then never
+// exceed 2^24 and are exact; the accumulator's last bit weighs 2^-58 of the
+// largest product).  The result is rounded to FP64 once, so its error is that of the 55-bit
+// operands and the dropped levels: 5e-17 to 3e-16 of the 2-norm on the
+// products of a build, where a chain of FP64 FMAs leaves 1.4e-16 to 9e-15.
+//
+// What bounds it: a 128 x 64 tile takes 34 SS instructions per K = 16 step,
+// each of which reads 6 KB of operands from shared memory at 128 B/clk
+// (48 clk); turning operands into digits (about 20 integer operations an
+// element, at 64 a clock and SM) runs beside them.  FP64 FMAs on the CUDA cores
+// run at 2 a clock and SM.  Measured on random operands (GB300, us; FP64 FMA
+// kernel before): 1755 x 54 x 91125: 970 (14500), 54 x 91125 x 1755: 930
+// (17500), 1755 x 91125 x 54 (stores bound it): 1640 (17700),
+// 351 x 351 x 91125: 910 (26600), 1053 x 1053 x 91125: 8150.  A 27-centre FP64
+// build went from 64.7 to 4.8 ms, its Coulomb matrix from 30.6 to 1.71 ms.
+#include <algorithm>
+#include <cmath>
+#include <type_traits>
+
+#include "tc_common.cuh"
+#include "xk_internal.h"
+
+namespace xk {
+
+namespace {
+
+using namespace tc;
+
+constexpr int kDig = 7;             // digits per operand
+constexpr int kLev = 8;             // accumulator levels (i + j)
+constexpr int DK = 32;              // K per block: 64-byte rows, 64-byte swizzle
+constexpr int DX = 128, DY = 64;    // tile: X rows (MMA M) by Y rows (MMA N)
+constexpr int DX_PLANE = DX * DK * 2, DY_PLANE = DY * DK * 2;
+constexpr int D_STAGE = kDig * (DX_PLANE + DY_PLANE);  // 84 KB
+constexpr int D_STAGES = 2;
+constexpr int D_SMEM = D_STAGES * D_STAGE + 1024;
+constexpr int D_GROUP = 256 / DK;   // K blocks between drains
+// 16 worker warps turn operands into digits and take accumulators out; one
+// more issues the MMAs.  It sits in a warpgroup of its own whose registers go
+// to the workers (setmaxnreg: 640 threads launch with 96; 512 x 112 + 128 x 32 =
+// 640 x 96).
+constexpr int D_WORK = 16;
+constexpr int D_THREADS = 32 * (D_WORK + 4);
+
+// One operand: element (row, k) at p[row ld + k] (kc) or p[k ld + row].
+struct DOperand {
+  const double* p;
+  long ld;
+  int rows;
+  int kc;
+  const int* scale;  // per row: high word of max |row|
+  int pairs;         // kc: rows start on 16-byte boundaries
+};
+
+struct DArgs {
+  DOperand x, y;
+  int K, kchunk, ksplit;
+  int tiles_x, tiles_y;
+  int swapped;       // X rows are the columns of C (else its rows)
+  int M, N;          // C is M x N
+  double* C; long ldc;
+  double alpha, beta;
+  int scaled, added;  // alpha != 1, beta != 0 (an FP64 comparison per result would cost more)
+  const double* H; long ldh;
+  double* work;      // ksplit > 1: partial sums [ksplit][M][N]
+  int* flag;         // set to 1 when a row cannot be split (row_unfit), to 2 when a bounded
+                     // wait gave up: the product is then left to the FP64 FMAs
+};
+
+// Scale exponent e of a row from the high word of its largest |x|:
+// |x| 2^-e <= 1 - 2^-7.  A row of zeros gets 0.
+__device__ __forceinline__ int row_exp(int hi) { return hi ? ((hi + (1 << 14)) >> 20) - 1022 : 0; }
+
+// Rows whose largest |x| is infinite, NaN or below 2^-900 (where an element's
+// subnormals would count) are not split.
+__device__ __forceinline__ bool row_unfit(int hi) {
+  return hi >= 0x7ff00000 || (hi > 0 && hi < ((1023 - 900) << 20));
+}
+
+// The seven digits of x on the grid 2^(e - 55), each plus 128, in the low 7
+// bytes (most significant digit in byte 6).  e20 = (e + 1022) << 20.  Integer
+// operations run at 64 a clock and SM here, so they are what the split costs: x =
+// m 2^(ex - 1078) with m of 56 bits (a subnormal x, taken for a normal one, is
+// below the grid) is shifted by t = e + 1022 - ex >= 0 to one bit below the
+// grid; sign, rounding and the offsets of the digits are then one sum:
+// (y + 1 + 2 sum 128 2^(8 i)) >> 1, or with -y = ~y + 1, whose half rounds the
+// same way without the 1.
+__device__ __forceinline__ uint2 digits_of(double x, int e20) {
+  const uint32_t xh = __double2hiint(x), xl = __double2loint(x);
+  const uint32_t t = (uint32_t)(e20 - (int)(xh & 0x7ff00000u)) >> 20;
+  const uint32_t mh = (xh & 0xfffffu) | 0x100000u;
+  const unsigned long long m =
+      ((unsigned long long)__funnelshift_l(xl, mh, 3) << 32) | (xl << 3);
+  unsigned long long y;
+  asm("shr.u64 %0, %1, %2;" : "=l"(y) : "l"(m), "r"(t));  // t > 63 gives 0
+  const uint32_t sg = (uint32_t)((int)xh >> 31);
+  const unsigned long long z =
+      ((((unsigned long long)((uint32_t)(y >> 32) ^ sg)) << 32) | ((uint32_t)y ^ sg)) +
+      0x0101010101010101ull;
+  return make_uint2((uint32_t)(z >> 1), (uint32_t)(z >> 33));
+}
+
+// FP16 pairs (digit of a, digit of b), most significant first, from the digit
+// words of two elements: byte + 1024 = 0x64xx, less 1024 + 128.
+__device__ __forceinline__ void digit_pairs(const uint2& a, const uint2& b, uint32_t (&o)[kDig]) {
+  const uint32_t c = 0x64646464u;
+  const uint32_t w0 = __byte_perm(a.x, b.x, 0x5410), w1 = __byte_perm(a.x, b.x, 0x7632),
+                 w2 = __byte_perm(a.y, b.y, 0x5410), w3 = __byte_perm(a.y, b.y, 0x6262);
+  o[6] = __byte_perm(w0, c, 0x4240); o[5] = __byte_perm(w0, c, 0x4341);
+  o[4] = __byte_perm(w1, c, 0x4240); o[3] = __byte_perm(w1, c, 0x4341);
+  o[2] = __byte_perm(w2, c, 0x4240); o[1] = __byte_perm(w2, c, 0x4341);
+  o[0] = __byte_perm(w3, c, 0x4140);
+  const __half2 off = __half2half2(__ushort_as_half(0x6480));
+#pragma unroll
+  for (int i = 0; i < kDig; ++i) {
+    const __half2 r = __hsub2(*reinterpret_cast<__half2*>(&o[i]), off);
+    o[i] = *reinterpret_cast<const uint32_t*>(&r);
+  }
+}
+
+// A block of one operand passes through the registers of the 512 workers, n
+// elements each, n = 8 (X, 128 rows) or 4 (Y, 64 rows):
+//  * K contiguous in memory: lane l holds the pairs k = 2 (l % 16), +1 of the
+//    rows n w + l / 16 + 2 i of warp w, so that a load reads 256 B of a row and a
+//    store writes whole 128-byte lines (one 4-byte digit pair per lane);
+//  * rows contiguous: a thread holds n successive k of one row (lanes along the
+//    rows) and stores 2 n bytes of each digit.
+// Rows past the operand's last are read as that one (nothing of them is stored).
+template <int n, bool KC>
+__device__ __forceinline__ void load_block(const DOperand& o, int row0, long k0, long kend, int tid,
+                                           double (&v)[n]) {
+  constexpr int R = 16 * n;  // rows of the block
+  const bool whole = k0 + DK <= kend;
+  if constexpr (KC) {
+    const int r = row0 + (tid >> 5) * n + ((tid >> 4) & 1);
+    const long k = k0 + 2 * (tid & 15);
+    const double* p = o.p + k;
+    if (whole && o.pairs) {
+#pragma unroll
+      for (int i = 0; i < n / 2; ++i) {
+        const double2 t = __ldg(reinterpret_cast<const double2*>(p + (long)min(r + 2 * i, o.rows - 1) * o.ld));
+        v[2 * i] = t.x;
+        v[2 * i + 1] = t.y;
+      }
+    } else if (whole) {
+#pragma unroll
+      for (int i = 0; i < n / 2; ++i) {
+        const double* q = p + (long)min(r + 2 * i, o.rows - 1) * o.ld;
+        v[2 * i] = __ldg(q);
+        v[2 * i + 1] = __ldg(q + 1);
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < n / 2; ++i) {
+        const double* q = p + (long)min(r + 2 * i, o.rows - 1) * o.ld;
+        v[2 * i] = k < kend ? __ldg(q) : 0.0;
+        v[2 * i + 1] = k + 1 < kend ? __ldg(q + 1) : 0.0;
+      }
+    }
+  } else {
+    const long k = k0 + n * (tid / R);
+    const double* p = o.p + k * o.ld + min(row0 + tid % R, o.rows - 1);
+    if (whole) {
+#pragma unroll
+      for (int i = 0; i < n; ++i, p += o.ld) v[i] = __ldg(p);
+    } else {
+#pragma unroll
+      for (int i = 0; i < n; ++i, p += o.ld) v[i] = k + i < kend ? __ldg(p) : 0.0;
+    }
+  }
+}
+
+// Row of the block whose exponent lane l of warp w looks up for its warp.
+template <int n, bool KC>
+__device__ __forceinline__ int block_row(int w, int l) {
+  return KC ? w * n + l % n : (32 * w + l) % (16 * n);
+}
+
+// Digits of the block into the stage; ex: (e + 1022) << 20 of the rows block_row(w, 0..31).
+template <int n, bool KC>
+__device__ __forceinline__ void store_block(uint8_t* st, const int* ex, int tid, const double (&v)[n]) {
+  constexpr int R = 16 * n, PLANE = R * DK * 2;
+  if constexpr (KC) {
+    // rows r0 + 2 i: the swizzle's chunk is that of r0 with bit 1 of r, i.e. bit 0 of i, flipped
+    const int r0 = (tid >> 5) * n + ((tid >> 4) & 1), l = tid & 15;
+#pragma unroll
+    for (int i = 0; i < n / 2; ++i) {
+      const int r = r0 + 2 * i, e = ex[((tid >> 4) & 1) + 2 * i];
+      uint32_t o[kDig];
+      digit_pairs(digits_of(v[2 * i], e), digits_of(v[2 * i + 1], e), o);
+      uint32_t* d = reinterpret_cast<uint32_t*>(st + r * 64 + (((l >> 2) ^ ((r >> 1) & 3)) << 4) + (l & 3) * 4);
+#pragma unroll
+      for (int q = 0; q < kDig; ++q) d[q * (PLANE / 4)] = o[q];
+    }
+  } else {
+    const int r = tid % R, q = tid / R, e = ex[tid & 31];  // q: which n of the 32 k
+    uint32_t o[n / 2][kDig];
+#pragma unroll
+    for (int i = 0; i < n / 2; ++i) digit_pairs(digits_of(v[2 * i], e), digits_of(v[2 * i + 1], e), o[i]);
+    const int byte = q * n * 2;  // within the row's 64 bytes
+    uint8_t* d = st + r * 64 + (((byte >> 4) ^ ((r >> 1) & 3)) << 4) + (byte & 15);
+#pragma unroll
+    for (int b = 0; b < kDig; ++b) {
+      if constexpr (n == 8)
+        *reinterpret_cast<uint4*>(d + b * PLANE) = make_uint4(o[0][b], o[1][b], o[2][b], o[3][b]);
+      else
+        *reinterpret_cast<uint2*>(d + b * PLANE) = make_uint2(o[0][b], o[1][b]);
+    }
+  }
+}
+
+// (hi + lo 2^-20) 2^E rounded to FP64, 0 <= lo < 2^20: the 96-bit number
+// hi : lo is normalised and rounded in 32-bit words (an FP64 operation costs 64
+// times an integer one here).
+__device__ __forceinline__ double pack_f64(long long hi, uint32_t lo, int E) {
+  uint32_t w0 = lo << 12, w1 = (uint32_t)hi, w2 = (uint32_t)((unsigned long long)hi >> 32);
+  const uint32_t sign = w2 & 0x80000000u;
+  if (sign) {
+    w0 = 0u - w0;
+    w1 = ~w1;
+    w2 = ~w2;
+    if (w0 == 0) {
+      w1 += 1;
+      w2 += w1 == 0;
+    }
+  }
+  int ex = 1023 + 63 + E;  // biased exponent when the top bit of w2 is set
+  if (w2 == 0) { w2 = w1; w1 = w0; w0 = 0; ex -= 32; }
+  if (w2 == 0) { w2 = w1; w1 = 0; ex -= 32; }
+  if (w2 == 0) return 0.0;
+  const int z = __clz(w2);
+  ex -= z;
+  const uint32_t h = __funnelshift_l(w1, w2, z), l = __funnelshift_l(w0, w1, z);
+  // 53 bits: h[31:0] l[31:11], rounded by bit 10; the leading one adds to the exponent
+  uint32_t ml = __funnelshift_r(l, h, 11), mh = h >> 11;
+  const uint32_t r = (l >> 10) & 1;
+  ml += r;
+  mh += ml < r;
+  if (ex > 0 && ex < 2046)
+    return __hiloint2double((int)(sign | (((uint32_t)(ex - 1) << 20) + mh)), (int)ml);
+  const double m = (double)(((unsigned long long)mh << 32) | ml);
+  return scalbn(sign ? -m : m, ex - 1075);
+}
+
+// The block after the one being loaded, into L2: one 128-byte line per thread
+// (256 lines of X, 128 of Y; lines that straddle are left to the loads).
+template <bool XK, bool YK>
+__device__ __forceinline__ void prefetch_block(const DArgs& g, long x0, long y0, long k0, long kend, int tid) {
+  const bool isx = tid < 256;
+  const DOperand& o = isx ? g.x : g.y;
+  const int i = isx ? tid : tid - 256;
+  if (i >= 256 - (isx ? 0 : 128)) return;
+  const bool kc = isx ? XK : YK;
+  // K contiguous: two lines a row; rows contiguous: 8 (X) or 4 (Y) lines a k
+  const long r = (isx ? x0 : y0) + (kc ? i >> 1 : (i & (isx ? 7 : 3)) * 16);
+  const long k = k0 + (kc ? (i & 1) * 16 : i >> (isx ? 3 : 2));
+  if (r >= o.rows || k >= kend) return;
+  asm volatile("prefetch.global.L2 [%0];" ::"l"(o.p + (kc ? r * o.ld + k : k * o.ld + r)));
+}
+
+template <bool XK, bool YK>
+__global__ void __launch_bounds__(D_THREADS, 1) digit_gemm_kernel(const __grid_constant__ DArgs g) {
+  extern __shared__ uint8_t d_raw[];
+  uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(d_raw) + 1023) & ~uintptr_t(1023));
+  __shared__ uint64_t full[D_STAGES], empty[D_STAGES], set_ready, free_lo, free_hi, drain;
+  __shared__ uint32_t tslot;
+  __shared__ volatile int abort_flag;
+  __shared__ int skip;
+  // exponents of the rows a warp turns into digits (X, then Y), of two tiles
+  __shared__ int exps[D_WORK][2][64];
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // uniform: the register split needs it
+  // every CTA looks at every row, so that all leave the product out or none
+  if (tid == 0) skip = 0;
+  __syncthreads();
+  {
+    bool bad = false;
+    for (int i = tid; i < g.x.rows; i += D_THREADS) bad |= row_unfit(__ldg(g.x.scale + i));
+    for (int i = tid; i < g.y.rows; i += D_THREADS) bad |= row_unfit(__ldg(g.y.scale + i));
+    if (bad) skip = 1;
+  }
+  __syncthreads();
+  if (skip) {
+    if (tid == 0) *g.flag = 1;
+    return;
+  }
+  if (tid == 0) {
+    for (int s = 0; s < D_STAGES; ++s) {
+      mbar_init(&full[s], D_WORK);
+      mbar_init(&empty[s], 1);
+    }
+    mbar_init(&set_ready, 1);
+    mbar_init(&free_lo, D_WORK);
+    mbar_init(&free_hi, D_WORK);
+    mbar_init(&drain, 1);
+    abort_flag = 0;
+    fence_mbar_init();
+  }
+  if (warp == D_WORK) {
+    tmem_alloc(&tslot, 512);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tbase = tslot;
+  const int ntiles = g.tiles_x * g.tiles_y * g.ksplit;
+  // tile t: X tile fastest, then Y tile, then the K split
+  auto kblocks = [&](int z) {
+    const long k0 = (long)z * g.kchunk, k1 = min((long)g.K, k0 + g.kchunk);
+    return (int)((k1 - k0 + DK - 1) / DK);
+  };
+
+  if (warp >= D_WORK) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 32;");
+    if (warp == D_WORK) {
+      // per block 34 products of two K = 16 steps, the low levels first: their
+      // accumulators are taken out first
+      const uint32_t idesc = idesc_f16(128, DY, false, false, false);
+      const uint64_t d0 = sdesc_sw64(smem_u32(sm), 16, 512);
+      int it = 0, G = 0;
+      bool good = true;
+      auto fail = [&]() {
+        if (lane == 0) { atomicExch(g.flag, 2); abort_flag = 1; }
+        __syncwarp();
+        good = false;
+      };
+      for (int t = blockIdx.x; good && t < ntiles; t += gridDim.x) {
+        const int nkb = kblocks(t / (g.tiles_x * g.tiles_y));
+        for (int kb = 0; kb < nkb; ++kb, ++it) {
+          if (__shfl_sync(0xffffffffu, (int)abort_flag, 0)) { good = false; break; }
+          const int s = it % D_STAGES;
+          const bool first = (kb % D_GROUP) == 0;
+          const bool last = (kb % D_GROUP) == D_GROUP - 1 || kb == nkb - 1;
+          if (!mbar_wait_warp(&full[s], (it / D_STAGES) & 1)) { fail(); break; }
+          if (first && G >= 1 && !mbar_wait_warp(&free_lo, (G - 1) & 1)) { fail(); break; }
+          tc_fence_after();
+          const uint64_t dx = d0 + (uint64_t)((s * D_STAGE) >> 4);
+          const uint64_t dy = dx + (uint64_t)((kDig * DX_PLANE) >> 4);
+#pragma unroll
+          for (int l = kLev - 1; l >= 0; --l) {
+            if (l == 3 && first && G >= 1) {
+              if (!mbar_wait_warp(&free_hi, (G - 1) & 1)) { fail(); break; }
+              tc_fence_after();
+            }
+            const int i0 = l >= kDig ? l - kDig + 1 : 0, i1 = l < kDig ? l : kDig - 1;
+#pragma unroll
+            for (int i = i0; i <= i1; ++i)
+              mma_ss_run2(tbase + 64 * l, dx + (uint64_t)((i * DX_PLANE) >> 4),
+                          dy + (uint64_t)(((l - i) * DY_PLANE) >> 4), 2, 2, idesc,
+                          (first && i == i0) ? 0u : 1u);
+          }
+          if (!good) break;
+          if (elect_one()) {
+            mma_commit(&empty[s]);
+            if (last) mma_commit(&set_ready);
+          }
+          __syncwarp();
+          if (last) ++G;
+        }
+      }
+      if (elect_one()) mma_commit(&drain);
+      __syncwarp();
+      mbar_wait_warp(&drain, 0);
+    }
+  } else {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 112;");
+    // workers
+    const int quad = warp & 3, cg = warp >> 2;  // accumulator rows and columns of this warp
+    const uint32_t tacc = tbase + (static_cast<uint32_t>(quad * 32) << 16) + 16 * cg;
+    bool ok = true;
+    auto lost = [&]() __attribute__((always_inline)) {
+      if (lane == 0) { atomicExch(g.flag, 2); abort_flag = 1; }
+      __syncwarp();
+      ok = false;
+    };
+    long long hi[16];  // levels 0-3, in units of level 3
+    uint32_t lo[16];   // levels 4-7: 20 bits below level 3
+    int G = 0;  // groups taken
+    // the K block being fetched: tile ft, block fkb
+    int ft = blockIdx.x, fkb = 0, fn = 0, fz = 0;
+    int fx0 = 0, fy0 = 0;
+    int fpar = 1;  // which half of exps the tile being fetched uses
+    auto open_tile = [&]() __attribute__((always_inline)) {
+      if (ft >= ntiles) { fn = 0; return; }
+      const int xt = ft % g.tiles_x, r = ft / g.tiles_x;
+      fx0 = xt * DX;
+      fy0 = (r % g.tiles_y) * DY;
+      fz = r / g.tiles_y;
+      fn = kblocks(fz);
+      fpar ^= 1;
+      const long rx = fx0 + block_row<8, XK>(warp, lane), ry = fy0 + block_row<4, YK>(warp, lane);
+      exps[warp][fpar][lane] = (row_exp(__ldg(g.x.scale + min(rx, g.x.rows - 1l))) + 1022) << 20;
+      exps[warp][fpar][32 + lane] = (row_exp(__ldg(g.y.scale + min(ry, g.y.rows - 1l))) + 1022) << 20;
+      __syncwarp();
+    };
+    double vx[8], vy[4];
+    auto fetch = [&]() __attribute__((always_inline)) {
+      const long k0 = (long)fz * g.kchunk + (long)fkb * DK;
+      const long kend = min((long)g.K, (long)(fz + 1) * g.kchunk);
+      load_block<8, XK>(g.x, fx0, k0, kend, tid, vx);
+      load_block<4, YK>(g.y, fy0, k0, kend, tid, vy);
+      prefetch_block<XK, YK>(g, fx0, fy0, k0 + DK, kend, tid);
+      if (++fkb == fn) { fkb = 0; ft += gridDim.x; open_tile(); }
+    };
+    // adds a finished group of accumulators to hi, lo (zeroed at a tile's first
+    // group); levels 5 to 7 are added up in FP32 first (error below 2^-61 of the
+    // largest product)
+    auto take_group = [&](bool fresh) __attribute__((always_inline)) {
+      if (!mbar_wait_warp(&set_ready, G & 1)) { lost(); return; }
+      tc_fence_after();
+      auto level = [](uint32_t a) { return (long long)__float2int_rn(__uint_as_float(a)); };
+#pragma unroll
+      for (int c = 0; c < 16; c += 8) {
+        uint32_t a[8], b[8], d[8];
+        tmem_ld8(tacc + 64 * 5 + c, a);
+        tmem_ld8(tacc + 64 * 6 + c, b);
+        tmem_ld8(tacc + 64 * 7 + c, d);
+        tmem_wait_ld();
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const float f = fmaf(__uint_as_float(d[j]), 0x1p-12f, __uint_as_float(b[j]) * 0x1p-4f);
+          a[j] = (uint32_t)__float2int_rn(fmaf(__uint_as_float(a[j]), 0x1p4f, f));
+        }
+        tmem_ld8(tacc + 64 * 4 + c, b);
+        tmem_wait_ld();
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const long long t = level(b[j]) * (1 << 12) + (int)a[j] + (fresh ? 0 : lo[c + j]);
+          lo[c + j] = (uint32_t)t & 0xfffffu;
+          hi[c + j] = (fresh ? 0 : hi[c + j]) + (t >> 20);
+        }
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&free_lo);
+#pragma unroll
+      for (int c = 0; c < 16; c += 8) {
+        uint32_t a[8], b[8];
+        tmem_ld8(tacc + c, a);
+        tmem_ld8(tacc + 64 + c, b);
+        tmem_wait_ld();
+#pragma unroll
+        for (int j = 0; j < 8; ++j) hi[c + j] += level(a[j]) * (1 << 24) + level(b[j]) * (1 << 16);
+        tmem_ld8(tacc + 64 * 2 + c, a);
+        tmem_ld8(tacc + 64 * 3 + c, b);
+        tmem_wait_ld();
+#pragma unroll
+        for (int j = 0; j < 8; ++j) hi[c + j] += level(a[j]) * (1 << 8) + level(b[j]);
+      }
+      ++G;
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&free_hi);
+    };
+    // writes the 16 results of this thread for tile t
+    auto put_tile = [&](int t) __attribute__((always_inline)) {
+      const int xt = t % g.tiles_x, rr = t / g.tiles_x;
+      const long x = (long)xt * DX + quad * 32 + lane;
+      const long y0 = (long)(rr % g.tiles_y) * DY + 16 * cg;
+      const int left = (int)min(16l, g.y.rows - y0);  // columns of this warp inside C
+      const bool in = x < g.x.rows;
+      const int e = row_exp(in ? __ldg(g.x.scale + x) : 0) - 38;
+      // the 16 rows' exponents: lane j holds that of row j
+      const int ye = row_exp((lane & 15) < left ? __ldg(g.y.scale + y0 + (lane & 15)) : 0);
+      const bool split = g.ksplit > 1;
+      const long ld = split ? g.N : g.ldc;
+      double* c = (split ? g.work + (long)(rr / g.tiles_y) * g.M * g.N : g.C) +
+                  (g.swapped ? y0 * ld + x : x * ld + y0);
+      const long step = g.swapped ? ld : 1;
+      const double* h = g.H + (g.swapped ? y0 * g.ldh + x : x * g.ldh + y0);
+      const long hstep = g.swapped ? g.ldh : 1;
+#pragma unroll
+      for (int j = 0; j < 16; ++j)
+        hi[j] = __double_as_longlong(pack_f64(hi[j], lo[j], e + __shfl_sync(0xffffffffu, ye, j)));
+      if (!in) return;
+      // branches around the FP64 operations: one that is only predicated off
+      // would still take its 16 cycles of the FP64 pipe
+      if (!split && (g.scaled || g.added)) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j)
+          if (j < left) {
+            double v = __longlong_as_double(hi[j]) * g.alpha;
+            if (g.H) v *= h[j * hstep];
+            if (g.added) v += g.beta * c[j * step];
+            c[j * step] = v;
+          }
+      } else if (!split && g.H) {
+        double w[4];
+#pragma unroll
+        for (int j = 0; j < 16; j += 4) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) w[i] = j + i < left ? h[(j + i) * hstep] : 0.0;
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            if (j + i < left) c[(j + i) * step] = __longlong_as_double(hi[j + i]) * w[i];
+        }
+      } else {
+#pragma unroll
+        for (int j = 0; j < 16; ++j)
+          if (j < left) c[j * step] = __longlong_as_double(hi[j]);
+      }
+    };
+
+    open_tile();
+    if (fn) fetch();
+    int it = 0, done = -1;  // done: tile whose results wait in hi, lo
+    int dt = -1;            // tile of the block produced last
+    int dkb = 0, dn = 0;
+    bool due = false;       // the block produced last ended a group
+    int par = 1;
+    for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+      const int nkb = kblocks(t / (g.tiles_x * g.tiles_y));
+      par ^= 1;
+      for (int kb = 0; kb < nkb && ok; ++kb, ++it) {
+        const int s = it % D_STAGES, use = it / D_STAGES;
+        if (__shfl_sync(0xffffffffu, (int)abort_flag, 0) ||
+            (use > 0 && !mbar_wait_warp(&empty[s], (use - 1) & 1))) { lost(); break; }
+        uint8_t* st = sm + s * D_STAGE;
+        store_block<8, XK>(st, exps[warp][par], tid, vx);
+        store_block<4, YK>(st + kDig * DX_PLANE, exps[warp][par] + 32, tid, vy);
+        auto arrive = [&]() {
+          fence_async_smem();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&full[s]);
+        };
+        // the next block's loads fly during the wait above; after a group they
+        // follow its taking (registers)
+        if (due || done >= 0) {
+          arrive();
+          if (done >= 0) { put_tile(done); done = -1; }
+          if (due) {  // the group that ended with the block before this one
+            take_group(dkb < D_GROUP);
+            if (dkb == dn - 1) done = dt;
+          }
+          if (fn) fetch();
+        } else {
+          if (fn) fetch();
+          arrive();
+        }
+        due = (kb % D_GROUP) == D_GROUP - 1 || kb == nkb - 1;
+        dt = t;
+        dkb = kb;
+        dn = nkb;
+      }
+    }
+    if (ok && done >= 0) put_tile(done);
+    if (ok && due) {
+      take_group(dkb < D_GROUP);
+      if (ok && dkb == dn - 1) put_tile(dt);
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == D_WORK) tmem_dealloc(tbase, 512);
+}
+
+// Per row: high word of max |x| (the largest of all for infinities and NaN).
+// K contiguous: one warp per row and K chunk (blockIdx.y).
+__global__ void rowmax_kc_kernel(const double* __restrict__ p, long ld, int rows, int K, int kchunk,
+                                 int* __restrict__ out) {
+  const int lane = threadIdx.x & 31;
+  const long r = (long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (r >= rows) return;
+  const int k0 = blockIdx.y * kchunk, k1 = min(K, k0 + kchunk);
+  const double* row = p + r * ld;
+  int m = 0;
+  for (int k = k0 + lane; k < k1; k += 32) m = max(m, __double2hiint(row[k]) & 0x7fffffff);
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if (lane == 0) atomicMax(out + r, m);
+}
+
+// Rows contiguous (element (r, k) at p[k ld + r]): one thread per row and K chunk.
+__global__ void rowmax_rc_kernel(const double* __restrict__ p, long ld, int rows, int K, int kchunk,
+                                 int* __restrict__ out) {
+  const long r = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (r >= rows) return;
+  const int k0 = blockIdx.y * kchunk, k1 = min(K, k0 + kchunk);
+  int m = 0;
+#pragma unroll 4
+  for (int k = k0; k < k1; ++k) m = max(m, __double2hiint(p[k * ld + r]) & 0x7fffffff);
+  atomicMax(out + r, m);
+}
+
+void launch_rowmax(const DOperand& o, int K, int* out, cudaStream_t s) {
+  // chunks of K so that about 8 blocks per SM read the operand
+  const int rb = o.kc ? (o.rows + 7) / 8 : (o.rows + 255) / 256;
+  const int want = std::max(1, (8 * 152 + rb - 1) / rb);
+  const int kchunk = std::max(o.kc ? 256 : 64, (K + want - 1) / want);
+  const dim3 grid((unsigned)rb, (unsigned)((K + kchunk - 1) / kchunk));
+  if (o.kc)
+    rowmax_kc_kernel<<<grid, 256, 0, s>>>(o.p, o.ld, o.rows, K, kchunk, out);
+  else
+    rowmax_rc_kernel<<<grid, 256, 0, s>>>(o.p, o.ld, o.rows, K, kchunk, out);
+  count_launch();
+}
+
+}  // namespace
+
+size_t digit_scale_ints(int M, int N) { return (size_t)M + N + 8; }
+
+// 2e7 multiply-adds take the FP64 pipe 35 us with every SM at work; the row
+// maxima, the launches and a tile here take about 25 us.
+bool digit_gemm_wanted(const DGemm& g) {
+  return g.scale && !g.upperA && g.K >= 16 && std::min(g.M, g.N) >= 8 &&
+         (double)g.M * g.N * g.K >= 2e7;
+}
+
+// K split (at most cap) of least time: waves of tiles over the SMs times the
+// 256-term groups of a tile, with one group's time for a tile's start and end.
+int digit_ksplit(int M, int N, int K, int cap) {
+  const int X = std::max(M, N), Y = std::min(M, N);
+  const long tiles = (long)((X + DX - 1) / DX) * ((Y + DY - 1) / DY);
+  const int groups = (K + 255) / 256;
+  int best = 1;
+  long cost = 0;
+  for (int ks = 1; ks <= std::min(cap, groups); ++ks) {
+    const long c = ((tiles * ks + 151) / 152) * ((groups + ks - 1) / ks + 1);
+    if (ks == 1 || c < cost) { best = ks; cost = c; }
+  }
+  return best;
+}
+
+cudaError_t digit_gemm(const DGemm& g, int ksplit, int kchunk, cudaStream_t s) {
+  DArgs a{};
+  int* sc = g.scale;  // [flag, 7 unused, M rows of op(A), N columns of op(B)]
+  cudaError_t e = cudaMemsetAsync(sc, 0, ((size_t)g.M + g.N + 8) * 4, s);
+  if (e != cudaSuccess) return e;
+  auto pairs = [](const double* p, long ld) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0 && ld % 2 == 0; };
+  const DOperand A{g.A, g.lda, g.M, g.transA ? 0 : 1, sc + 8, pairs(g.A, g.lda)};
+  const DOperand B{g.B, g.ldb, g.N, g.transB ? 1 : 0, sc + 8 + g.M, pairs(g.B, g.ldb)};
+  launch_rowmax(A, g.K, sc + 8, s);
+  launch_rowmax(B, g.K, sc + 8 + g.M, s);
+  // the longer side of C takes the 128-row side of the tile; as columns of C
+  // it also makes the stores contiguous over the lanes
+  a.swapped = g.N >= g.M ? 1 : 0;
+  a.x = a.swapped ? B : A;
+  a.y = a.swapped ? A : B;
+  a.K = g.K; a.kchunk = kchunk; a.ksplit = ksplit;
+  a.tiles_x = (a.x.rows + DX - 1) / DX;
+  a.tiles_y = (a.y.rows + DY - 1) / DY;
+  a.M = g.M; a.N = g.N; a.C = g.C; a.ldc = g.ldc; a.alpha = g.alpha; a.beta = g.beta;
+  a.scaled = g.alpha != 1.0; a.added = g.beta != 0.0;
+  a.H = g.H; a.ldh = g.ldh; a.work = g.work; a.flag = sc;
+  const long tiles = (long)a.tiles_x * a.tiles_y * ksplit;
+  const unsigned ctas = (unsigned)std::min<long>(tiles, 152);
+  auto launch = [&](auto kernel) {
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, D_SMEM);
+    if (e != cudaSuccess) return e;
+    kernel<<<ctas, D_THREADS, D_SMEM, s>>>(a);
+    count_launch();
+    return cudaGetLastError();
+  };
+  if (a.x.kc) return a.y.kc ? launch(digit_gemm_kernel<true, true>) : launch(digit_gemm_kernel<true, false>);
+  return a.y.kc ? launch(digit_gemm_kernel<false, true>) : launch(digit_gemm_kernel<false, false>);
+}
+
+}  // namespace xk

@@ -4,7 +4,8 @@
 //
 // On GB300 FP64 runs on the CUDA cores at a small fraction of the tensor
 // rate, so every FP64 contraction here is bound by the DFMA pipe; the tiles
-// only need enough register reuse to keep that pipe fed.
+// only need enough register reuse to keep that pipe fed.  Products of 2e7
+// multiply-adds and more go to the tensor cores instead (xk_digits.cu).
 #include "xk_internal.h"
 
 #include <algorithm>
@@ -18,7 +19,10 @@ namespace {
 constexpr int BM = 64, BN = 64, BK = 16, TPB = 256;
 
 template <bool TA, bool TB, bool HAD>
-__global__ void __launch_bounds__(TPB) dgemm_kernel(DGemm g, int kchunk) {
+__global__ void __launch_bounds__(TPB) dgemm_kernel(DGemm g, int kchunk, const int* only_if) {
+  // behind a product on the tensor cores: only when that one was left out
+  const int left_out = only_if ? *only_if : 1;
+  if (!left_out) return;
   __shared__ double As[BK][BM + 1];
   __shared__ double Bs[BK][BN + 1];
   const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
@@ -83,6 +87,8 @@ __global__ void __launch_bounds__(TPB) dgemm_kernel(DGemm g, int kchunk) {
         double v = g.alpha * acc[i][j];
         if (HAD) v *= g.H[m * g.ldh + n];
         if (g.beta != 0.0) v += g.beta * g.C[m * g.ldc + n];
+        // a tensor-core product that gave up half-way has changed C already
+        if (g.beta != 0.0 && only_if && left_out == 2) v = nan("");
         g.C[m * g.ldc + n] = v;
       }
     }
@@ -114,12 +120,12 @@ int choose_ksplit(int M, int N, int K) {
 }
 
 template <bool TA, bool TB>
-cudaError_t launch_tt(const DGemm& g, int kchunk, cudaStream_t s) {
+cudaError_t launch_tt(const DGemm& g, int kchunk, const int* only_if, cudaStream_t s) {
   dim3 grid((g.N + BN - 1) / BN, (g.M + BM - 1) / BM, g.ksplit);
   if (g.H && g.ksplit == 1)
-    dgemm_kernel<TA, TB, true><<<grid, TPB, 0, s>>>(g, kchunk);
+    dgemm_kernel<TA, TB, true><<<grid, TPB, 0, s>>>(g, kchunk, only_if);
   else
-    dgemm_kernel<TA, TB, false><<<grid, TPB, 0, s>>>(g, kchunk);
+    dgemm_kernel<TA, TB, false><<<grid, TPB, 0, s>>>(g, kchunk, only_if);
   count_launch();
   return cudaGetLastError();
 }
@@ -137,17 +143,24 @@ int dgemm_ksplit(int M, int N, int K) {
 cudaError_t dgemm(const DGemm& gin, cudaStream_t s) {
   DGemm g = gin;
   if (g.M <= 0 || g.N <= 0) return cudaSuccess;
+  const bool digits = digit_gemm_wanted(g);
+  if (digits)
+    g.ksplit = digit_ksplit(g.M, g.N, g.K,
+                            !g.work ? 1 : g.ksplit > 0 ? g.ksplit : dgemm_ksplit(g.M, g.N, g.K));
   if (g.ksplit <= 0) g.ksplit = choose_ksplit(g.M, g.N, g.K);
   if (g.ksplit > 1 && !g.work) g.ksplit = 1;
   int kchunk = (g.K + g.ksplit - 1) / g.ksplit;
-  kchunk = ((kchunk + BK - 1) / BK) * BK;
+  const int unit = digits ? 32 : BK;
+  kchunk = ((kchunk + unit - 1) / unit) * unit;
   if (kchunk <= 0) kchunk = BK;
   g.ksplit = std::max(1, (g.K + kchunk - 1) / kchunk);
-  cudaError_t e;
-  if (!g.transA && !g.transB) e = launch_tt<false, false>(g, kchunk, s);
-  else if (g.transA && !g.transB) e = launch_tt<true, false>(g, kchunk, s);
-  else if (!g.transA && g.transB) e = launch_tt<false, true>(g, kchunk, s);
-  else e = launch_tt<true, true>(g, kchunk, s);
+  cudaError_t e = digits ? digit_gemm(g, g.ksplit, kchunk, s) : cudaSuccess;
+  if (e != cudaSuccess) return e;
+  const int* only_if = digits ? g.scale : nullptr;
+  if (!g.transA && !g.transB) e = launch_tt<false, false>(g, kchunk, only_if, s);
+  else if (g.transA && !g.transB) e = launch_tt<true, false>(g, kchunk, only_if, s);
+  else if (!g.transA && g.transB) e = launch_tt<false, true>(g, kchunk, only_if, s);
+  else e = launch_tt<true, true>(g, kchunk, only_if, s);
   if (e != cudaSuccess || g.ksplit == 1) return e;
   const long total = (long)g.M * g.N;
   const int blocks = (int)std::min<long>((total + 255) / 256, 152L * 16);

@@ -40,8 +40,20 @@ struct DGemm {
   double* work;
   bool upperA;  // op(A) is upper triangular: K steps below a row tile are skipped
   double beta;  // C = alpha op(A) op(B) (o H) + beta C (0: C is not read)
+  int* scale;   // nullable: digit_scale_ints(M, N) ints of scratch, with which large
+                // products run on the tensor cores (xk_digits.cu)
 };
 cudaError_t dgemm(const DGemm& g, cudaStream_t s);
+
+// The product of dgemm on the tensor cores, split into exact digits
+// (xk_digits.cu): whether its size calls for it, the K split it wants (at most
+// cap), and the launch (ksplit partial sums of kchunk terms each in g.work
+// when ksplit > 1).  *g.scale is 0 afterwards, or not when the product has to be
+// formed with FP64 FMAs instead (an operand that is not finite).
+size_t digit_scale_ints(int M, int N);
+bool digit_gemm_wanted(const DGemm& g);
+int digit_ksplit(int M, int N, int K, int cap);
+cudaError_t digit_gemm(const DGemm& g, int ksplit, int kchunk, cudaStream_t s);
 // Split count dgemm picks when DGemm::ksplit == 0 (work needs ksplit*M*N).
 int dgemm_ksplit(int M, int N, int K);
 
@@ -102,11 +114,12 @@ cudaError_t isdf_tables_f64(const double* phi, long ng, int N, const double* phi
 cudaError_t select_points_f64(const double* F, int m, int N, int want, double tol_rel,
                               int32_t* piv, int* count, cudaStream_t s);
 // In-place blocked Cholesky (lower) of the n x n matrix A (lda); *status = 1
-// on a non-positive pivot.
-cudaError_t cholesky_blocked_f64(double* A, int n, long lda, int* status, cudaStream_t s);
+// on a non-positive pivot.  scale (here and below): DGemm::scale of the updates.
+cudaError_t cholesky_blocked_f64(double* A, int n, long lda, int* status, int* scale,
+                                 cudaStream_t s);
 // B (n x ncols, ldb) := (L L^T)^{-1} B with the lower factor L (ldl).
 cudaError_t cholesky_solve_f64(const double* L, int n, long ldl, double* B, long ldb, long ncols,
-                               cudaStream_t s);
+                               int* scale, cudaStream_t s);
 
 // *out = -dV (2 sum_t V[t] P[t]^2 - sum_t W[t] Q[t]^2) over lenA and lenC
 // elements, in a fixed order; `work` holds reduce_work_elems() doubles.

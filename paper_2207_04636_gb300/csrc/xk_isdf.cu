@@ -311,7 +311,8 @@ cudaError_t select_points_f64(const double* F, int m, int N, int want, double to
   return e;
 }
 
-cudaError_t cholesky_blocked_f64(double* A, int n, long lda, int* status, cudaStream_t s) {
+cudaError_t cholesky_blocked_f64(double* A, int n, long lda, int* status, int* scale,
+                                 cudaStream_t s) {
   for (int k = 0; k < n; k += NB) {
     const int kb = std::min(NB, n - k);
     potrf_block_kernel<<<1, 256, 0, s>>>(A, lda, k, kb, status);
@@ -323,7 +324,7 @@ cudaError_t cholesky_blocked_f64(double* A, int n, long lda, int* status, cudaSt
       // A22 -= L21 L21^T (the whole square; only its lower triangle is used)
       DGemm g{rest, rest, kb, A + (long)(k + kb) * lda + k, lda, false,
               A + (long)(k + kb) * lda + k, lda, true, A + (long)(k + kb) * lda + k + kb, lda,
-              -1.0, nullptr, 0, 1, nullptr, false, 1.0};
+              -1.0, nullptr, 0, 1, nullptr, false, 1.0, scale};
       cudaError_t e = dgemm(g, s);
       if (e != cudaSuccess) return e;
     }
@@ -332,14 +333,14 @@ cudaError_t cholesky_blocked_f64(double* A, int n, long lda, int* status, cudaSt
 }
 
 cudaError_t cholesky_solve_f64(const double* L, int n, long ldl, double* B, long ldb, long ncols,
-                               cudaStream_t s) {
+                               int* scale, cudaStream_t s) {
   const int cb = nblocks(ncols);
   // forward: L Y = B, block rows in order (left-looking updates)
   for (int k = 0; k < n; k += NB) {
     const int kb = std::min(NB, n - k);
     if (k > 0) {
       DGemm g{kb, (int)ncols, k, L + (long)k * ldl, ldl, false, B, ldb, false, B + (long)k * ldb,
-              ldb, -1.0, nullptr, 0, 1, nullptr, false, 1.0};
+              ldb, -1.0, nullptr, 0, 1, nullptr, false, 1.0, scale};
       cudaError_t e = dgemm(g, s);
       if (e != cudaSuccess) return e;
     }
@@ -354,7 +355,7 @@ cudaError_t cholesky_solve_f64(const double* L, int n, long ldl, double* B, long
       // B_k -= L[k+kb:n, k:k+kb]^T X[k+kb:n]
       DGemm g{kb, (int)ncols, n - k - kb, L + (long)(k + kb) * ldl + k, ldl, true,
               B + (long)(k + kb) * ldb, ldb, false, B + (long)k * ldb, ldb, -1.0, nullptr, 0, 1,
-              nullptr, false, 1.0};
+              nullptr, false, 1.0, scale};
       cudaError_t e = dgemm(g, s);
       if (e != cudaSuccess) return e;
     }
@@ -368,8 +369,12 @@ cudaError_t isdf_tables_f64(const double* phi, long ng, int N, const double* phi
                             int grid, double L, double* Xgg, double* chi, double* V, double* W,
                             double* work, int* status, double* ridge_out, cudaStream_t s) {
   cudaError_t e;
+  // scratch of the tensor-core products: W until W itself is formed, then X_gg
+  const bool digits = 2 * (size_t)na * na >= digit_scale_ints(na, (int)ng);
+  int* scale = digits ? reinterpret_cast<int*>(W) : nullptr;
   auto gram = [&]() {
     DGemm g{na, na, N, phig, N, false, phig, N, true, Xgg, na, 1.0, nullptr, 0, 0, work};
+    g.scale = scale;
     cudaError_t r = dgemm(g, s);
     if (r != cudaSuccess) return r;
     square_kernel<<<nblocks((long)na * na), 256, 0, s>>>(Xgg, na, na, na);
@@ -379,6 +384,7 @@ cudaError_t isdf_tables_f64(const double* phi, long ng, int N, const double* phi
   // X_gR = (Phi_g Phi^T) o (Phi_g Phi^T) into chi
   {
     DGemm g{na, (int)ng, N, phig, N, false, phi, N, true, chi, ng, 1.0, nullptr, 0, 0, work};
+    g.scale = scale;
     e = dgemm(g, s);
     if (e != cudaSuccess) return e;
     square_kernel<<<nblocks((long)na * ng), 256, 0, s>>>(chi, na, ng, ng);
@@ -389,7 +395,7 @@ cudaError_t isdf_tables_f64(const double* phi, long ng, int N, const double* phi
   double ridge = 0.0;
   int st = 0;
   e = cudaMemsetAsync(status, 0, 4, s);
-  if (e == cudaSuccess) e = cholesky_blocked_f64(Xgg, na, na, status, s);
+  if (e == cudaSuccess) e = cholesky_blocked_f64(Xgg, na, na, status, scale, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(&st, status, 4, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return e;
@@ -408,7 +414,7 @@ cudaError_t isdf_tables_f64(const double* phi, long ng, int N, const double* phi
     add_diag_kernel<<<nblocks(na), 256, 0, s>>>(Xgg, na, na, ridge);
     count_launch();
     e = cudaMemsetAsync(status, 0, 4, s);
-    if (e == cudaSuccess) e = cholesky_blocked_f64(Xgg, na, na, status, s);
+    if (e == cudaSuccess) e = cholesky_blocked_f64(Xgg, na, na, status, scale, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&st, status, 4, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return e;
@@ -416,7 +422,7 @@ cudaError_t isdf_tables_f64(const double* phi, long ng, int N, const double* phi
   }
   if (ridge_out) *ridge_out = ridge;
   // chi = X_gg^{-1} X_gR
-  e = cholesky_solve_f64(Xgg, na, na, chi, ng, ng, s);
+  e = cholesky_solve_f64(Xgg, na, na, chi, ng, ng, scale, s);
   if (e != cudaSuccess) return e;
   // V = Pois(chi), two functions per complex transform, in batches
   {
@@ -453,6 +459,7 @@ cudaError_t isdf_tables_f64(const double* phi, long ng, int N, const double* phi
   // W = V chi^T, symmetrised
   {
     DGemm g{na, na, (int)ng, V, ng, false, chi, ng, true, W, na, 1.0, nullptr, 0, 0, work};
+    g.scale = digits ? reinterpret_cast<int*>(Xgg) : nullptr;
     e = dgemm(g, s);
     if (e == cudaSuccess) e = symmetrize_f64(W, na, s);
   }

@@ -1,0 +1,103 @@
+"""FP64 products split into digits on the tensor cores (large products of an
+XK_FP64 handle): exact where FP64 is exact, no further from a wider reference
+than FP64 rounding, and the general path for operands that cannot be split."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def xk():
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2207_04636_gb300 as m
+    return m
+
+
+def _ints(rng, shape, m):
+    return rng.integers(-m, m + 1, size=shape).astype(np.float64)
+
+
+def _case(Ng, N, n, na, seed, m=3):
+    rng = np.random.default_rng(seed)
+    phi, C, V = _ints(rng, (Ng, N), m), _ints(rng, (N, n), m), _ints(rng, (na, Ng), m)
+    W = _ints(rng, (na, na), m)
+    return phi, np.sort(rng.permutation(Ng)[:na]), V, W + W.T, C
+
+
+def _lines(phi, idx, V, W, C):
+    psi = phi @ C
+    psig, phig = psi[idx], phi[idx]
+    V2 = V * (psig @ psi.T)
+    return ((psig.T @ V2) @ phi, (V2 @ psi).T @ phig, ((W * (psig @ psig.T)) @ psig).T @ phig)
+
+
+# Rows, columns and depths on both sides of the 128 x 64 tiles, the 32-deep
+# blocks and the 256-term groups; odd row lengths (unaligned rows) and even.
+SHAPES = [(4992, 24, 16, 400), (4993, 127, 33, 128), (5119, 129, 64, 129), (4097, 66, 65, 255),
+          (6145, 40, 8, 641), (2048, 257, 128, 256), (90001, 33, 31, 65)]
+
+
+@pytest.mark.parametrize("Ng,N,n,na", SHAPES)
+def test_integers_exact(xk, Ng, N, n, na):
+    """Small integers: every sum is an integer below 2^53, so K and the full K
+    equal the host's bit for bit."""
+    phi, idx, V, W, C = _case(Ng, N, n, na, Ng + n, m=1 if Ng > 50000 else 2)
+    h = xk.Handle(phi, idx, V, W, 1.0, n, mode="fp64")
+    K, E = h.build(C)
+    Kf = h.build_full(C)
+    h.release()
+    l1, l2, l3 = _lines(phi, idx, V, W, C)
+    assert max(np.abs(l).max() for l in (l1, l2, l3)) < 2.0 ** 52
+    assert np.array_equal(K, (l1 + l2 - l3).T)
+    psi = phi @ C
+    psig, phig = psi[idx], phi[idx]
+    Y = phig.T @ ((V * (psig @ psi.T)) @ phi)
+    assert np.array_equal(Kf, Y + Y.T - phig.T @ ((W * (psig @ psig.T)) @ phig))
+
+
+@pytest.mark.parametrize("spread", [0, 40])
+def test_against_wider(xk, spread):
+    """Reals (rows scaled by up to 2^spread) against extended precision: eight
+    roundings of 2^-53 in the 2-norm of the three lines."""
+    Ng, N, n, na = 4096, 24, 20, 400
+    rng = np.random.default_rng(5)
+    phi, C = rng.standard_normal((Ng, N)), rng.standard_normal((N, n))
+    phi *= np.exp2(-rng.uniform(0, spread, size=(Ng, 1)))
+    V, W = rng.standard_normal((na, Ng)), rng.standard_normal((na, na))
+    W = W + W.T
+    idx = np.sort(rng.permutation(Ng)[:na])
+    h = xk.Handle(phi, idx, V, W, 1.0, n, mode="fp64")
+    K, _ = h.build(C)
+    h.release()
+    x = _lines(*(a.astype(np.longdouble) if a.dtype.kind == "f" else a for a in (phi, idx, V, W, C)))
+    err = np.linalg.norm((K - (x[0] + x[1] - x[2]).T).astype(np.float64))
+    assert err <= 8 * 2.0 ** -53 * sum(np.linalg.norm(l.astype(np.float64)) for l in x)
+
+
+def test_not_finite(xk):
+    """A NaN or an infinity in C reaches K as FP64 arithmetic has it, and the
+    handle's next build is exact again."""
+    phi, idx, V, W, C = _case(4993, 40, 16, 400, 3)
+    phi[phi == 0] = 1.0
+    h = xk.Handle(phi, idx, V, W, 1.0, 16, mode="fp64")
+    for bad in (np.nan, np.inf):
+        Cb = C.copy()
+        Cb[5, 3] = bad
+        K, E = h.build(Cb)
+        assert np.all(np.isnan(K)) and np.isnan(E)
+    l1, l2, l3 = _lines(phi, idx, V, W, C)
+    assert np.array_equal(h.build(C)[0], (l1 + l2 - l3).T)
+    h.release()
+
+
+def test_tiny_rows(xk):
+    """Rows whose largest entry is below 2^-900 keep the general path: a basis
+    scaled by 2^-950 with C scaled back gives K scaled by 2^-950 exactly."""
+    phi, idx, V, W, C = _case(4993, 40, 16, 400, 4)
+    l1, l2, l3 = _lines(phi, idx, V, W, C)
+    h = xk.Handle(phi * 2.0 ** -950, idx, V, W, 1.0, 16, mode="fp64")
+    K, _ = h.build(C * 2.0 ** 950)
+    h.release()
+    assert np.array_equal(K, (l1 + l2 - l3).T * 2.0 ** -950)
