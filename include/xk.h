@@ -209,8 +209,8 @@ int xk_setup_isdf(int64_t Ng, int32_t N, int32_t n, int32_t Naux,
  * pair matrix.  piv_out (host, want) receives the pivots as indices into
  * rows, in selection order; *count the number taken.  A two-stage selection
  * (Sec. IV.C: per-atom candidates, then a global pivoting over their union)
- * is two levels of calls.  Scratch: about 8 (m^2 + m want + m N) bytes of
- * device memory during the call (admission as xk_setup).
+ * is two levels of calls.  Scratch: about 8 (m want + 2 m N) bytes of device
+ * memory during the call, admitted (as xk_setup) as 8 (m^2 + m want + m N).
  * Errors: XK_EINVAL (null pointers, sizes <= 0, bad tol_rel), XK_ENOMEM,
  * XK_ECUDA.
  */

@@ -109,7 +109,7 @@ cudaError_t isdf_tables_f64(const double* phi, long ng, int N, const double* phi
 // X = (F F^T) o (F F^T) for the m candidate rows F (m x N, device): up to
 // `want` pivots (indices into F, selection order) into piv (host), stopping
 // when the largest remaining diagonal is at most tol_rel times the largest
-// initial one; *count = pivots taken.  Holds m^2 + m want doubles of
+// initial one; *count = pivots taken.  Holds m N + m want doubles of
 // stream-ordered scratch during the call.
 cudaError_t select_points_f64(const double* F, int m, int N, int want, double tol_rel,
                               int32_t* piv, int* count, cudaStream_t s);

@@ -177,85 +177,143 @@ __global__ void unpack_pairs_kernel(const double2* __restrict__ c, long r0, int 
 
 // ---------------------------------------------------------------- point selection
 // Greedy complete-pivoting Cholesky of X = (F F^T) o (F F^T), left-looking:
-// only the diagonal d is kept up to date; each step forms one column.
-// State on the device: d[m] (selected rows set to -1), L[m][want],
-// sel[0] = steps taken, sel[1] = stopped flag, val[t] = pivot value, tol.
+// only the diagonal d is kept up to date; each step forms one column, from
+// the rows themselves, so X is never stored (m^2 doubles, and a product that
+// took half of the time: 10.3 of 21.6 ms for 13824 points).  One launch a step:
+// a block first reduces the previous launch's block maxima to the pivot (every
+// block the same one), then forms the column for its 32 rows and the maximum of
+// their new diagonals.  Its 8 warps take every eighth term of the two dot
+// products (lanes along the rows of the transposed F and of L stored by
+// columns, so loads are contiguous) and are added up in order.
+// State on the device: d[m] (selected rows set to -1), L[want][m], val[t] =
+// pivot value, sel[0] = steps taken, pv / pi = block maxima
+// (two sets, alternating).
 
-__global__ void diag_init_kernel(const double* __restrict__ X, int m, double* __restrict__ d) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x)
-    d[i] = X[(long)i * m + i];
+constexpr int PT_ROWS = 32, PT_WARPS = 8;
+
+// Diagonals are compared as their bit patterns: those of non-negative doubles
+// order like the numbers, a negative sentinel (-1) lies below them all, and an
+// integer comparison takes a sixteenth of an FP64 one here.
+__device__ __forceinline__ long long bits(double x) { return __double_as_longlong(x); }
+
+// Largest value and its row (the lowest on ties) over a warp.
+__device__ __forceinline__ void warp_argmax(long long& v, int& i) {
+  for (int o = 16; o > 0; o >>= 1) {
+    const long long ov = __shfl_xor_sync(0xffffffffu, v, o);
+    const int oi = __shfl_xor_sync(0xffffffffu, i, o);
+    if (ov > v || (ov == v && oi < i)) { v = ov; i = oi; }
+  }
 }
 
-// Pivot of step t: the largest d (the lowest index on ties); stops when it is
-// not above tol (tol = tol_rel * the largest initial diagonal, set at t = 0).
-__global__ void __launch_bounds__(1024) pivot_kernel(double* __restrict__ d, int m, int t,
-                                                     double tol_rel, int* __restrict__ sel,
-                                                     int32_t* __restrict__ piv,
-                                                     double* __restrict__ val,
-                                                     double* __restrict__ tol) {
-  __shared__ double bv[32];
-  __shared__ int bi[32];
-  if (sel[1]) return;
-  double best = -1.0;
-  int bidx = 0x7fffffff;
-  for (int i = threadIdx.x; i < m; i += blockDim.x) {
-    const double v = d[i];
-    if (v > best) { best = v; bidx = i; }  // increasing i: the first maximum is kept
+// d[i] = X(i, i) and the block maxima; FT: the rows transposed, [N][m].
+__global__ void __launch_bounds__(PT_ROWS) diag_init_kernel(const double* __restrict__ FT, int m, int N,
+                                                            double* __restrict__ d,
+                                                            long long* __restrict__ pv,
+                                                            int* __restrict__ pi) {
+  const int i = blockIdx.x * PT_ROWS + threadIdx.x;
+  double s = 0.0;
+  if (i < m)
+    for (int k = 0; k < N; ++k) {
+      const double f = FT[(long)k * m + i];
+      s = fma(f, f, s);
+    }
+  if (i < m) d[i] = s * s;
+  const bool in = i < m && s * s >= 0.0;  // a NaN is never a pivot
+  long long v = in ? bits(s * s) : -1;
+  int idx = in ? i : 0x7fffffff;
+  warp_argmax(v, idx);
+  if (threadIdx.x == 0) { pv[blockIdx.x] = v; pi[blockIdx.x] = idx; }
+}
+
+// Step t: pivot p = the largest d; stops when it is not above tol (tol_rel
+// times the largest initial diagonal).  For every unselected row i,
+// L[i][t] = ((F_i . F_p)^2 - sum_{s<t} L[i][s] L[p][s]) / sqrt(val[t]) and
+// d[i] -= L[i][t]^2; the pivot row gets L[p][t] = sqrt(val[t]).
+__global__ void __launch_bounds__(PT_ROWS * PT_WARPS) point_step_kernel(
+    const double* __restrict__ F, const double* __restrict__ FT, int m, int N, int t, double tol_rel,
+    int* __restrict__ sel, int32_t* __restrict__ piv, double* __restrict__ val,
+    double* __restrict__ tol, double* __restrict__ L, double* __restrict__ d,
+    long long* __restrict__ pv, int* __restrict__ pi) {
+  __shared__ long long bv[PT_WARPS];
+  __shared__ double sf[PT_WARPS][PT_ROWS], sl[PT_WARPS][PT_ROWS];
+  __shared__ int bi[PT_WARPS];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, nb = gridDim.x;
+  long long top = -1;
+  int p = 0x7fffffff;
+  for (int b = tid; b < nb; b += PT_ROWS * PT_WARPS) {
+    const long long x = pv[(t & 1) * nb + b];
+    const int q = pi[(t & 1) * nb + b];
+    if (x > top || (x == top && q < p)) { top = x; p = q; }
   }
-  for (int o = 16; o > 0; o >>= 1) {
-    const double ov = __shfl_xor_sync(0xffffffffu, best, o);
-    const int oi = __shfl_xor_sync(0xffffffffu, bidx, o);
-    if (ov > best || (ov == best && oi < bidx)) { best = ov; bidx = oi; }
-  }
-  if ((threadIdx.x & 31) == 0) { bv[threadIdx.x >> 5] = best; bi[threadIdx.x >> 5] = bidx; }
+  warp_argmax(top, p);
+  if (lane == 0) { bv[w] = top; bi[w] = p; }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    // fold the warps' results in warp order (ties keep the lower index)
-    double b0 = bv[0];
-    int i0 = bi[0];
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w)
-      if (bv[w] > b0 || (bv[w] == b0 && bi[w] < i0)) { b0 = bv[w]; i0 = bi[w]; }
-    if (t == 0) *tol = tol_rel * b0;
-    if (!(b0 > *tol) || i0 >= m) {
-      sel[1] = 1;
-    } else {
-      piv[t] = i0;
-      val[t] = b0;
-      d[i0] = -1.0;
+  top = bv[0];
+  p = bi[0];
+  for (int k = 1; k < PT_WARPS; ++k)
+    if (bv[k] > top || (bv[k] == top && bi[k] < p)) { top = bv[k]; p = bi[k]; }
+  const double v = top >= 0 ? __longlong_as_double(top) : -1.0;
+  const double lim = t == 0 ? tol_rel * v : *tol;
+  const bool stop = !(v > lim) || p >= m;
+  if (blockIdx.x == 0 && tid == 0) {
+    if (t == 0) *tol = lim;
+    if (!stop) {
+      piv[t] = p;
+      val[t] = v;
       sel[0] = t + 1;
     }
   }
-}
-
-// Column t: for every unselected row i (one warp per row),
-// L[i][t] = (X[i][p] - sum_{s<t} L[i][s] L[p][s]) / sqrt(val[t]) and
-// d[i] -= L[i][t]^2; the pivot row gets L[p][t] = sqrt(val[t]).
-__global__ void column_kernel(const double* __restrict__ X, int m, int want, int t,
-                              const int* __restrict__ sel, const int32_t* __restrict__ piv,
-                              const double* __restrict__ val, double* __restrict__ L,
-                              double* __restrict__ d) {
-  if (sel[1] || sel[0] <= t) return;
-  const int p = piv[t];
-  const double sp = sqrt(val[t]);
-  const int lane = threadIdx.x & 31;
-  const long warps = ((long)gridDim.x * blockDim.x) >> 5;
-  const double* lp = L + (long)p * want;
-  for (long i = ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < m; i += warps) {
+  if (stop) {
+    // every block leaves here, in the later launches too
+    if (tid == 0) { pv[((t + 1) & 1) * nb + blockIdx.x] = -1; pi[((t + 1) & 1) * nb + blockIdx.x] = 0x7fffffff; }
+    return;
+  }
+  const int i = blockIdx.x * PT_ROWS + lane;
+  const long ii = i < m ? i : m - 1;
+  double f = 0.0, l = 0.0;
+  const double* fp = F + (long)p * N;
+#pragma unroll 4
+  for (int k = w; k < N; k += PT_WARPS) f = fma(FT[(long)k * m + ii], __ldg(fp + k), f);
+#pragma unroll 8
+  for (int s = w; s < t; s += PT_WARPS) l = fma(L[(long)s * m + ii], L[(long)s * m + p], l);
+  sf[w][lane] = f;
+  sl[w][lane] = l;
+  __syncthreads();
+  if (w != 0) return;
+  for (int k = 1; k < PT_WARPS; ++k) {
+    f += sf[k][lane];
+    l += sl[k][lane];
+  }
+  long long nd = -1;
+  if (i < m) {
+    const double sp = sqrt(v);
+    const double di = d[i];
     if (i == p) {
-      if (lane == 0) L[(long)p * want + t] = sp;
-      continue;
-    }
-    if (d[i] < 0.0) continue;  // selected earlier
-    const double* li = L + i * want;
-    double acc = 0.0;
-    for (int q = lane; q < t; q += 32) acc = fma(li[q], lp[q], acc);
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) {
-      const double l = (X[i * m + p] - acc) / sp;
-      L[i * want + t] = l;
-      d[i] -= l * l;
+      L[(long)t * m + i] = sp;
+      d[i] = -1.0;
+    } else if (di >= 0.0) {
+      const double x = (f * f - l) / sp;
+      L[(long)t * m + i] = x;
+      const double dn = di - x * x;
+      d[i] = dn;
+      // a diagonal that rounding has taken below zero is out, as a selected row is
+      if (dn >= 0.0) nd = bits(dn);
     }
   }
+  int q = nd >= 0 ? i : 0x7fffffff;
+  warp_argmax(nd, q);
+  if (lane == 0) { pv[((t + 1) & 1) * nb + blockIdx.x] = nd; pi[((t + 1) & 1) * nb + blockIdx.x] = q; }
+}
+
+// out[c][r] = in[r][c] for rows x cols.
+__global__ void transpose_kernel(const double* __restrict__ in, int rows, int cols, double* __restrict__ out) {
+  __shared__ double tile[32][33];
+  const long r0 = (long)blockIdx.x * 32, c0 = (long)blockIdx.y * 32;
+  for (int i = threadIdx.y; i < 32; i += 8)
+    if (r0 + i < rows && c0 + threadIdx.x < cols) tile[i][threadIdx.x] = in[(r0 + i) * cols + c0 + threadIdx.x];
+  __syncthreads();
+  for (int i = threadIdx.y; i < 32; i += 8)
+    if (c0 + i < cols && r0 + threadIdx.x < rows) out[(c0 + i) * rows + r0 + threadIdx.x] = tile[threadIdx.x][i];
 }
 
 }  // namespace
@@ -268,34 +326,32 @@ cudaError_t select_points_f64(const double* F, int m, int N, int want, double to
   }
   want = std::min(want, m);
   void* buf = nullptr;
-  const size_t xb = (size_t)m * m * 8, lb = (size_t)m * want * 8;
-  const size_t bytes = xb + lb + (size_t)m * 8 + (size_t)want * 8 + 64 + (size_t)want * 4 + 64;
+  const int nb = (m + PT_ROWS - 1) / PT_ROWS;
+  const size_t fb = (size_t)m * N * 8, lb = (size_t)m * want * 8;
+  const size_t bytes = fb + lb + ((size_t)m + want + 2 + 2 * (size_t)nb) * 8 +
+                       ((size_t)want + 2 * (size_t)nb + 4) * 4;
   cudaError_t e = cudaMallocAsync(&buf, bytes, s);
   if (e != cudaSuccess) return e;
   char* b = static_cast<char*>(buf);
-  double* X = reinterpret_cast<double*>(b);
-  double* L = reinterpret_cast<double*>(b + xb);
-  double* d = reinterpret_cast<double*>(b + xb + lb);
+  double* FT = reinterpret_cast<double*>(b);
+  double* L = reinterpret_cast<double*>(b + fb);
+  double* d = reinterpret_cast<double*>(b + fb + lb);
   double* val = d + m;
   double* tol = val + want;
-  int* sel = reinterpret_cast<int*>(tol + 2);
-  int32_t* dpiv = reinterpret_cast<int32_t*>(sel + 4);
-  {
-    DGemm g{m, m, N, F, N, false, F, N, true, X, m, 1.0, nullptr, 0, 1, nullptr};
-    e = dgemm(g, s);
-  }
+  long long* pv = reinterpret_cast<long long*>(tol + 2);
+  int* sel = reinterpret_cast<int*>(pv + 2 * nb);
+  int* pi = sel + 4;
+  int32_t* dpiv = pi + 2 * nb;
+  e = cudaMemsetAsync(sel, 0, 16, s);
   if (e == cudaSuccess) {
-    square_kernel<<<nblocks((long)m * m), 256, 0, s>>>(X, m, m, m);
-    diag_init_kernel<<<nblocks(m), 256, 0, s>>>(X, m, d);
+    transpose_kernel<<<dim3((unsigned)nb, (unsigned)((N + 31) / 32)), dim3(32, 8), 0, s>>>(F, m, N, FT);
+    diag_init_kernel<<<nb, PT_ROWS, 0, s>>>(FT, m, N, d, pv, pi);
     count_launch(2);
-    e = cudaMemsetAsync(sel, 0, 16, s);
   }
-  if (e == cudaSuccess) e = cudaMemsetAsync(L, 0, lb, s);
-  const int cb = std::max(1, std::min(152 * 8, (m + 7) / 8));  // 8 warps (rows) per block
   for (int t = 0; e == cudaSuccess && t < want; ++t) {
-    pivot_kernel<<<1, 1024, 0, s>>>(d, m, t, tol_rel, sel, dpiv, val, tol);
-    column_kernel<<<cb, 256, 0, s>>>(X, m, want, t, sel, dpiv, val, L, d);
-    count_launch(2);
+    point_step_kernel<<<nb, PT_ROWS * PT_WARPS, 0, s>>>(F, FT, m, N, t, tol_rel, sel, dpiv, val, tol, L,
+                                                       d, pv, pi);
+    count_launch();
     if ((t & 255) == 255) e = cudaGetLastError();
   }
   int got = 0;
