@@ -212,8 +212,9 @@ struct xk_handle {
   size_t full_extra = 0;  // bytes of the tensor path's full-K scratch, admitted on first use
   // xk_coulomb (FP64 handles): allocated and admitted on first use
   double *Jrho = nullptr, *Jv = nullptr, *Jphiv = nullptr, *Jd = nullptr, *Jout = nullptr;
-  double2 *Jc0 = nullptr, *Jc1 = nullptr, *Jtw = nullptr;
+  double *Jtmp = nullptr, *Jtab = nullptr;
   int Jg = 0;
+  double JL = 0.0;  // side length the tables at Jtab belong to
   double *C = nullptr, *psi = nullptr, *psig = nullptr, *V2 = nullptr, *M1 = nullptr,
          *M2 = nullptr, *Q = nullptr, *M3 = nullptr, *L1 = nullptr, *L2 = nullptr,
          *L3 = nullptr, *K = nullptr, *Ex = nullptr, *work = nullptr, *red = nullptr;
@@ -1099,23 +1100,17 @@ int xk_coulomb(xk_handle* h, int32_t grid, double L, const double* C, double* J_
     XK_CUDA(A(&h->Jphiv, ng * N));
     XK_CUDA(A(&h->Jrho, ng));
     XK_CUDA(A(&h->Jv, ng));
-    double* cbuf = nullptr;
-    XK_CUDA(A(&cbuf, 4 * ng));
-    h->Jc0 = reinterpret_cast<double2*>(cbuf);
-    h->Jc1 = h->Jc0 + ng;
+    // the Poisson solve's buffer and tables: 2 ng + 2 grid^2 doubles
+    XK_CUDA(A(&h->Jtmp, 4 * ng + 2 * (size_t)grid));
+    h->Jtab = h->Jtmp + ng;
     XK_CUDA(A(&h->Jout, (size_t)N * N + 1));
-    double* tw = nullptr;
-    XK_CUDA(A(&tw, 2 * (size_t)grid));
-    h->Jtw = reinterpret_cast<double2*>(tw);
-    std::vector<double> t(2 * (size_t)grid);
-    for (int m = 0; m < grid; ++m) {
-      const double a = 2.0 * M_PI * (double)m / (double)grid;
-      t[2 * m] = std::cos(a);
-      t[2 * m + 1] = std::sin(a);
-    }
-    XK_CUDA(cudaMemcpyAsync(tw, t.data(), t.size() * 8, cudaMemcpyHostToDevice, s));
-    XK_CUDA(cudaStreamSynchronize(s));
+    XK_CUDA(xk::poisson_tables_f64(grid, L, h->Jtab, s));
+    h->JL = L;
     h->Jg = grid;
+  }
+  if (h->JL != L) {  // another side length than the last call's
+    XK_CUDA(xk::poisson_tables_f64(grid, L, h->Jtab, s));
+    h->JL = L;
   }
   XK_CUDA(cudaMemcpyAsync(h->Ce, C, (size_t)N * n * 8, cudaMemcpyHostToDevice, s));
   {
@@ -1126,8 +1121,9 @@ int xk_coulomb(xk_handle* h, int32_t grid, double L, const double* C, double* J_
   }
   {  // density, Poisson solve, J = dV Phi^T (v o Phi), E_J = dV sum rho v
     StepMark m(h, XK_STEP_PAIR);
-    XK_CUDA(xk::coulomb_potential_f64(h->psi, (long)ng, n, grid, L, h->Jtw, h->Jrho, h->Jc0, h->Jc1, s));
-    XK_CUDA(xk::potential_rows_f64(h->Jc0, h->phi, (long)ng, N, h->Jv, h->Jphiv, s));
+    XK_CUDA(xk::density_f64(h->psi, (long)ng, n, h->Jrho, s));
+    XK_CUDA(xk::poisson_f64(h->Jrho, h->Jv, h->Jtmp, 1, grid, h->Jtab, nullptr, 0, s));
+    XK_CUDA(xk::potential_rows_f64(h->Jv, h->phi, (long)ng, N, h->Jphiv, s));
     xk::DGemm gj{N, N, (int)ng, h->phi, N, true, h->Jphiv, N, false, h->Jout, N, h->dV, nullptr, 0, 0, h->work};
     gj.scale = digit_scratch(h->M1, (size_t)n * ng, N, N);
     XK_CUDA(xk::dgemm(gj, s));

@@ -75,6 +75,7 @@ struct DArgs {
   int scaled, added;  // alpha != 1, beta != 0 (an FP64 comparison per result would cost more)
   const double* H; long ldh;
   double* work;      // ksplit > 1: partial sums [ksplit][M][N]
+  int nbatch; long cskip;  // swapped only: batches of C's columns (DGemm)
   int* flag;         // set to 1 when a row cannot be split (row_unfit), to 2 when a bounded
                      // wait gave up: the product is then left to the FP64 FMAs
 };
@@ -282,10 +283,11 @@ __global__ void __launch_bounds__(D_THREADS, 1) digit_gemm_kernel(const __grid_c
   __shared__ int exps[D_WORK][2][64];
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // uniform: the register split needs it
-  // every CTA looks at every row, so that all leave the product out or none
+  // A product added to C must not be left out half-way: every CTA looks at every
+  // row first.  Any other is formed again as a whole when a tile meets such a row.
   if (tid == 0) skip = 0;
   __syncthreads();
-  {
+  if (g.added) {
     bool bad = false;
     for (int i = tid; i < g.x.rows; i += D_THREADS) bad |= row_unfit(__ldg(g.x.scale + i));
     for (int i = tid; i < g.y.rows; i += D_THREADS) bad |= row_unfit(__ldg(g.y.scale + i));
@@ -402,8 +404,10 @@ __global__ void __launch_bounds__(D_THREADS, 1) digit_gemm_kernel(const __grid_c
       fn = kblocks(fz);
       fpar ^= 1;
       const long rx = fx0 + block_row<8, XK>(warp, lane), ry = fy0 + block_row<4, YK>(warp, lane);
-      exps[warp][fpar][lane] = (row_exp(__ldg(g.x.scale + min(rx, g.x.rows - 1l))) + 1022) << 20;
-      exps[warp][fpar][32 + lane] = (row_exp(__ldg(g.y.scale + min(ry, g.y.rows - 1l))) + 1022) << 20;
+      const int hx = __ldg(g.x.scale + min(rx, g.x.rows - 1l)), hy = __ldg(g.y.scale + min(ry, g.y.rows - 1l));
+      if (row_unfit(hx) || row_unfit(hy)) *g.flag = 1;
+      exps[warp][fpar][lane] = (row_exp(hx) + 1022) << 20;
+      exps[warp][fpar][32 + lane] = (row_exp(hy) + 1022) << 20;
       __syncwarp();
     };
     double vx[8], vy[4];
@@ -481,6 +485,11 @@ __global__ void __launch_bounds__(D_THREADS, 1) digit_gemm_kernel(const __grid_c
                   (g.swapped ? y0 * ld + x : x * ld + y0);
       const long step = g.swapped ? ld : 1;
       const double* h = g.H + (g.swapped ? y0 * g.ldh + x : x * g.ldh + y0);
+      if (g.nbatch > 0) {
+        const long q = x / g.nbatch;
+        c += q * g.cskip;
+        h -= q * g.nbatch;
+      }
       const long hstep = g.swapped ? g.ldh : 1;
 #pragma unroll
       for (int j = 0; j < 16; ++j)
@@ -645,7 +654,7 @@ cudaError_t digit_gemm(const DGemm& g, int ksplit, int kchunk, cudaStream_t s) {
   launch_rowmax(B, g.K, sc + 8 + g.M, s);
   // the longer side of C takes the 128-row side of the tile; as columns of C
   // it also makes the stores contiguous over the lanes
-  a.swapped = g.N >= g.M ? 1 : 0;
+  a.swapped = g.N >= g.M || g.nbatch > 0 ? 1 : 0;
   a.x = a.swapped ? B : A;
   a.y = a.swapped ? A : B;
   a.K = g.K; a.kchunk = kchunk; a.ksplit = ksplit;
@@ -654,6 +663,7 @@ cudaError_t digit_gemm(const DGemm& g, int ksplit, int kchunk, cudaStream_t s) {
   a.M = g.M; a.N = g.N; a.C = g.C; a.ldc = g.ldc; a.alpha = g.alpha; a.beta = g.beta;
   a.scaled = g.alpha != 1.0; a.added = g.beta != 0.0;
   a.H = g.H; a.ldh = g.ldh; a.work = g.work; a.flag = sc;
+  a.nbatch = g.nbatch; a.cskip = g.cskip;
   const long tiles = (long)a.tiles_x * a.tiles_y * ksplit;
   const unsigned ctas = (unsigned)std::min<long>(tiles, 152);
   auto launch = [&](auto kernel) {

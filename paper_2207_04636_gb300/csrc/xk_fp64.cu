@@ -9,6 +9,8 @@
 #include "xk_internal.h"
 
 #include <algorithm>
+#include <cmath>
+#include <vector>
 
 namespace xk {
 
@@ -84,12 +86,14 @@ __global__ void __launch_bounds__(TPB) dgemm_kernel(DGemm g, int kchunk, const i
       if (g.ksplit > 1) {
         g.work[((long)blockIdx.z * g.M + m) * g.N + n] = acc[i][j];
       } else {
+        const long q = g.nbatch > 0 ? n / g.nbatch : 0;  // batch of the column
+        const long at = m * g.ldc + n + q * g.cskip;
         double v = g.alpha * acc[i][j];
-        if (HAD) v *= g.H[m * g.ldh + n];
-        if (g.beta != 0.0) v += g.beta * g.C[m * g.ldc + n];
+        if (HAD) v *= g.H[m * g.ldh + n - q * g.nbatch];
+        if (g.beta != 0.0) v += g.beta * g.C[at];
         // a tensor-core product that gave up half-way has changed C already
         if (g.beta != 0.0 && only_if && left_out == 2) v = nan("");
-        g.C[m * g.ldc + n] = v;
+        g.C[at] = v;
       }
     }
   }
@@ -143,10 +147,11 @@ int dgemm_ksplit(int M, int N, int K) {
 cudaError_t dgemm(const DGemm& gin, cudaStream_t s) {
   DGemm g = gin;
   if (g.M <= 0 || g.N <= 0) return cudaSuccess;
+  if (g.nbatch > 0) g.ksplit = 1;  // batched columns are stored unsplit
   const bool digits = digit_gemm_wanted(g);
   if (digits)
     g.ksplit = digit_ksplit(g.M, g.N, g.K,
-                            !g.work ? 1 : g.ksplit > 0 ? g.ksplit : dgemm_ksplit(g.M, g.N, g.K));
+                            !g.work || g.nbatch > 0 ? 1 : g.ksplit > 0 ? g.ksplit : dgemm_ksplit(g.M, g.N, g.K));
   if (g.ksplit <= 0) g.ksplit = choose_ksplit(g.M, g.N, g.K);
   if (g.ksplit > 1 && !g.work) g.ksplit = 1;
   int kchunk = (g.K + g.ksplit - 1) / g.ksplit;
@@ -259,83 +264,140 @@ cudaError_t neg_dot_f64(const double* a, const double* b, long len, double* work
 }
 
 // ---------------------------------------------------------------------------
-// Coulomb J on the grid: density, Poisson solve by a 3-D DFT written as three
-// passes of 1-D DFTs (each output an O(g) sum in FP64; the grids here are
-// g <= ~100 per axis, so the O(g^4) total is a few hundred MFLOP), and
-// J = dV Phi^T diag(v) Phi.
+// Coulomb J on the grid: density, Poisson solve, and J = dV Phi^T diag(v) Phi.
 
 namespace {
 int blocks_of(long total) { return (int)std::max<long>(1, std::min<long>((total + 255) / 256, 152L * 16)); }
 }  // namespace
 
-// rho[R] = sum_i psi[R][i]^2, also as a complex grid function (imaginary 0).
-__global__ void density_kernel(const double* __restrict__ psi, long ng, int n,
-                               double* __restrict__ rho, double2* __restrict__ c) {
+// rho[R] = sum_i psi[R][i]^2.
+__global__ void density_kernel(const double* __restrict__ psi, long ng, int n, double* __restrict__ rho) {
   for (long r = blockIdx.x * (long)blockDim.x + threadIdx.x; r < ng;
        r += (long)gridDim.x * blockDim.x) {
     const double* row = psi + r * n;
     double s = 0.0;
     for (int i = 0; i < n; ++i) s = fma(row[i], row[i], s);
     rho[r] = s;
-    c[r] = make_double2(s, 0.0);
   }
 }
 
-// One pass of a length-g DFT along `axis` (0 = slowest index) of `count`
-// values (whole g^3 grids one after another):
-// out[k] = sum_j in[j] exp(sign 2 pi i j k / g), tw[m] = (cos, sin)(2 pi m / g).
-__global__ void dft_axis_kernel(const double2* __restrict__ in, double2* __restrict__ out, int g,
-                                int axis, const double2* __restrict__ tw, double sign, long count) {
-  const long stride = axis == 0 ? (long)g * g : axis == 1 ? g : 1;
-  for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < count;
-       t += (long)gridDim.x * blockDim.x) {
-    const int k = (int)((t / stride) % g);
-    const long base = t - (long)k * stride;
-    double re = 0.0, im = 0.0;
-    int m = 0;  // j k mod g
-    for (int j = 0; j < g; ++j) {
-      const double2 x = in[base + (long)j * stride];
-      const double2 w = tw[m];
-      const double ws = sign * w.y;
-      re = fma(x.x, w.x, fma(-x.y, ws, re));
-      im = fma(x.x, ws, fma(x.y, w.x, im));
-      m += k;
-      if (m >= g) m -= g;
-    }
-    out[t] = make_double2(re, im);
-  }
-}
+// Poisson solves.  On a cubic grid 4 pi / G^2 depends on the squares of the three
+// frequencies only, and the cosine and the sine of one |m| share it: the solve is
+// diagonal in the product of the axes' real Fourier bases (orthonormal columns
+// 1/sqrt(g), sqrt(2/g) cos, sqrt(2/g) sin, and (-1)^j / sqrt(g) for even g), with
+// no complex arithmetic.  Six passes, each a product of the g x g basis with
+// the fastest axis of every function that leaves that axis the slowest:
+//   in [f][p][j], p over the other two axes  ->  out [f][k][p] = sum_j B[k][j] in[f][p][j],
+// three passes into the basis (the third multiplies by 4 pi / G^2), three back,
+// after which the axes are in order again.  Many functions are one large product
+// for the tensor cores (xk_digits.cu); a single one (the Coulomb build) takes
+// axis_kernel.  1053 functions of 45^3: 6 passes of FP64 complex DFTs on two
+// functions each took 112 ms.
+//
+// Tables: [0, g^2) forward B[k][j], [g^2, 2 g^2) its transpose, then 4 pi / G^2
+// as [kx][ky][kz].
 
-// f(G) *= scale * 4 pi / |G|^2 with G = 2 pi m / L, m the signed frequency
-// index of each axis; the G = 0 term is set to zero.
-__global__ void coulomb_multiply_kernel(double2* __restrict__ f, int g, double L, double scale,
-                                        long count) {
+__global__ void poisson_kernel_table(double* __restrict__ lam, int g, double L) {
   const long g3 = (long)g * g * g;
-  const double two_pi_over_L = 6.283185307179586 / L;
-  for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < count;
+  const double w = 6.283185307179586 / L;
+  for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < g3;
        t += (long)gridDim.x * blockDim.x) {
-    const long u = t % g3;
-    const int i0 = (int)(u / ((long)g * g)), i1 = (int)((u / g) % g), i2 = (int)(u % g);
-    const int m0 = i0 <= (g - 1) / 2 ? i0 : i0 - g;
-    const int m1 = i1 <= (g - 1) / 2 ? i1 : i1 - g;
-    const int m2 = i2 <= (g - 1) / 2 ? i2 : i2 - g;
-    const double g2 = two_pi_over_L * two_pi_over_L * ((double)m0 * m0 + (double)m1 * m1 + (double)m2 * m2);
-    const double k = g2 > 0.0 ? scale * 12.566370614359172 / g2 : 0.0;
-    f[t] = make_double2(f[t].x * k, f[t].y * k);
+    // basis function k belongs to the frequency (k + 1) / 2
+    const int m0 = ((int)(t / ((long)g * g)) + 1) / 2, m1 = ((int)((t / g) % g) + 1) / 2,
+              m2 = ((int)(t % g) + 1) / 2;
+    const double g2 = w * w * ((double)m0 * m0 + (double)m1 * m1 + (double)m2 * m2);
+    lam[t] = g2 > 0.0 ? 12.566370614359172 / g2 : 0.0;
   }
 }
 
-// v[R] = Re(c[R]); out[R][nu] = v[R] phi[R][nu].
-__global__ void potential_rows_kernel(const double2* __restrict__ c, const double* __restrict__ phi,
-                                      long ng, int N, double* __restrict__ v, double* __restrict__ out) {
+size_t poisson_table_elems(int g) { return 2 * (size_t)g * g + (size_t)g * g * g; }
+
+cudaError_t poisson_tables_f64(int g, double L, double* tab, cudaStream_t s) {
+  std::vector<double> b(2 * (size_t)g * g), c(g), d(g);
+  const long double tau = 6.283185307179586476925286766559L, rg = sqrtl((long double)g);
+  for (int r = 0; r < g; ++r) {  // sqrt(2/g) cos, sin of 2 pi r / g
+    c[r] = (double)(sqrtl(2.0L) * cosl(tau * r / g) / rg);
+    d[r] = (double)(sqrtl(2.0L) * sinl(tau * r / g) / rg);
+  }
+  for (int k = 0; k < g; ++k)
+    for (int j = 0; j < g; ++j) {
+      const int m = (k + 1) / 2, r = (int)(((long)m * j) % g);
+      double v = (k & 1) ? c[r] : d[r];
+      if (k == 0) v = (double)(1.0L / rg);
+      else if (2 * m == g) v = (double)(((j & 1) ? -1.0L : 1.0L) / rg);
+      b[(size_t)k * g + j] = b[(size_t)g * g + (size_t)j * g + k] = v;
+    }
+  cudaError_t e = cudaMemcpyAsync(tab, b.data(), b.size() * 8, cudaMemcpyHostToDevice, s);
+  if (e != cudaSuccess) return e;
+  poisson_kernel_table<<<blocks_of((long)g * g * g), 256, 0, s>>>(tab + 2 * (size_t)g * g, g, L);
+  count_launch();
+  e = cudaGetLastError();
+  return e == cudaSuccess ? cudaStreamSynchronize(s) : e;
+}
+
+// One pass for few functions: a thread forms four outputs k of one (f, p); the
+// lanes' rows of `in` stay in L1 over the g terms.  Bound by the FP64 pipe.
+__global__ void __launch_bounds__(128) axis_kernel(const double* __restrict__ in, double* __restrict__ out,
+                                                   long rows, int g, const double* __restrict__ B,
+                                                   const double* __restrict__ lam) {
+  const long r = (long)blockIdx.x * 32 + threadIdx.x, g2 = (long)g * g;
+  const int k0 = 4 * (blockIdx.y * blockDim.y + threadIdx.y);
+  if (r >= rows || k0 >= g) return;
+  const double* x = in + r * g;
+  const double* b[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) b[i] = B + (long)min(k0 + i, g - 1) * g;
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 4
+  for (int j = 0; j < g; ++j) {
+    const double v = x[j];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) acc[i] = fma(__ldg(b[i] + j), v, acc[i]);
+  }
+  const long f = r / g2, p = r - f * g2;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    if (k0 + i < g) {
+      const double v = lam ? acc[i] * lam[(k0 + i) * g2 + p] : acc[i];
+      out[f * g2 * g + (k0 + i) * g2 + p] = v;
+    }
+}
+
+cudaError_t poisson_f64(const double* in, double* out, double* tmp, long nf, int g,
+                        const double* tab, int* scale, size_t scale_ints, cudaStream_t s) {
+  const long g2 = (long)g * g;
+  const double* lam = tab + 2 * g2;
+  const double* src = in;
+  for (int pass = 0; pass < 6; ++pass) {
+    double* dst = (pass & 1) ? out : tmp;
+    const double* B = tab + (pass < 3 ? 0 : g2);
+    const double* H = pass == 2 ? lam : nullptr;
+    DGemm q{g, (int)(nf * g2), g, B, g, false, src, g, true, dst, g2, 1.0, H, g2, 1, nullptr};
+    q.nbatch = (int)g2;
+    q.cskip = g2 * (g - 1);
+    q.scale = scale && scale_ints >= digit_scale_ints(q.M, q.N) ? scale : nullptr;
+    cudaError_t e;
+    if (digit_gemm_wanted(q)) {
+      e = dgemm(q, s);
+    } else {
+      axis_kernel<<<dim3((unsigned)((nf * g2 + 31) / 32), (unsigned)((g + 15) / 16)), dim3(32, 4), 0, s>>>(
+          src, dst, nf * g2, g, B, H);
+      count_launch();
+      e = cudaGetLastError();
+    }
+    if (e != cudaSuccess) return e;
+    src = dst;
+  }
+  return cudaSuccess;
+}
+
+// out[R][nu] = v[R] phi[R][nu].
+__global__ void potential_rows_kernel(const double* __restrict__ v, const double* __restrict__ phi,
+                                      long ng, int N, double* __restrict__ out) {
   const long count = ng * N;
   for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < count;
-       t += (long)gridDim.x * blockDim.x) {
-    const long r = t / N;
-    const double vr = c[r].x;
-    out[t] = vr * phi[t];
-    if (t % N == 0) v[r] = vr;
-  }
+       t += (long)gridDim.x * blockDim.x)
+    out[t] = v[t / N] * phi[t];
 }
 
 __global__ void dot_scaled_stage2(const double* __restrict__ part, int np, double scale, double* out) {
@@ -346,32 +408,15 @@ __global__ void dot_scaled_stage2(const double* __restrict__ part, int np, doubl
   if (threadIdx.x == 0) *out = scale * tot;
 }
 
-cudaError_t poisson_c2c_f64(double2* c0, double2* c1, long nb, int g, double L,
-                            const double2* tw, cudaStream_t s) {
-  const long g3 = (long)g * g * g, count = nb * g3;
-  const int b = blocks_of(count);
-  dft_axis_kernel<<<b, 256, 0, s>>>(c0, c1, g, 2, tw, -1.0, count);
-  dft_axis_kernel<<<b, 256, 0, s>>>(c1, c0, g, 1, tw, -1.0, count);
-  dft_axis_kernel<<<b, 256, 0, s>>>(c0, c1, g, 0, tw, -1.0, count);
-  coulomb_multiply_kernel<<<b, 256, 0, s>>>(c1, g, L, 1.0 / (double)g3, count);  // 1/N_g: inverse
-  dft_axis_kernel<<<b, 256, 0, s>>>(c1, c0, g, 2, tw, 1.0, count);
-  dft_axis_kernel<<<b, 256, 0, s>>>(c0, c1, g, 1, tw, 1.0, count);
-  dft_axis_kernel<<<b, 256, 0, s>>>(c1, c0, g, 0, tw, 1.0, count);
-  count_launch(7);
+cudaError_t density_f64(const double* psi, long ng, int n, double* rho, cudaStream_t s) {
+  density_kernel<<<blocks_of(ng), 256, 0, s>>>(psi, ng, n, rho);
+  count_launch();
   return cudaGetLastError();
 }
 
-cudaError_t coulomb_potential_f64(const double* psi, long ng, int n, int g, double L,
-                                  const double2* tw, double* rho, double2* c0, double2* c1,
-                                  cudaStream_t s) {
-  density_kernel<<<blocks_of(ng), 256, 0, s>>>(psi, ng, n, rho, c0);
-  count_launch();
-  return poisson_c2c_f64(c0, c1, 1, g, L, tw, s);
-}
-
-cudaError_t potential_rows_f64(const double2* c, const double* phi, long ng, int N, double* v,
-                               double* out, cudaStream_t s) {
-  potential_rows_kernel<<<blocks_of(ng * N), 256, 0, s>>>(c, phi, ng, N, v, out);
+cudaError_t potential_rows_f64(const double* v, const double* phi, long ng, int N, double* out,
+                               cudaStream_t s) {
+  potential_rows_kernel<<<blocks_of(ng * N), 256, 0, s>>>(v, phi, ng, N, out);
   count_launch();
   return cudaGetLastError();
 }

@@ -42,6 +42,8 @@ struct DGemm {
   double beta;  // C = alpha op(A) op(B) (o H) + beta C (0: C is not read)
   int* scale;   // nullable: digit_scale_ints(M, N) ints of scratch, with which large
                 // products run on the tensor cores (xk_digits.cu)
+  int nbatch;   // > 0: the columns of C come in batches of nbatch: column n is stored
+  long cskip;   // (n / nbatch) cskip elements further on, and H has column n % nbatch
 };
 cudaError_t dgemm(const DGemm& g, cudaStream_t s);
 
@@ -71,22 +73,23 @@ cudaError_t neg_dot_f64(const double* a, const double* b, long len, double* work
                         cudaStream_t s);
 size_t reduce_work_elems();
 
-// Coulomb potential of the density of psi (ng x n) on a cubic g^3 grid of
-// side L: rho[R] = sum_i psi[R][i]^2, then c0 = IDFT[(4 pi / G^2) DFT[rho]]
-// (G = 0 removed; the real part of c0 is the potential).  tw holds
-// (cos, sin)(2 pi m / g) for m < g; c1 is scratch of ng complex values.
-cudaError_t coulomb_potential_f64(const double* psi, long ng, int n, int g, double L,
-                                  const double2* tw, double* rho, double2* c0, double2* c1,
-                                  cudaStream_t s);
-// Pois applied to nb complex g^3 grids in c0 (result in c0; c1 scratch of the
-// same size): 3-D DFT, times 4 pi / G^2 (G = 0 removed), inverse 3-D DFT.
-// The kernel is real and even in G, so real and imaginary parts transform
-// independently (two real functions per complex grid).
-cudaError_t poisson_c2c_f64(double2* c0, double2* c1, long nb, int g, double L,
-                            const double2* tw, cudaStream_t s);
-// v[R] = Re(c[R]) and out[R][nu] = v[R] phi[R][nu].
-cudaError_t potential_rows_f64(const double2* c, const double* phi, long ng, int N, double* v,
-                               double* out, cudaStream_t s);
+// Poisson solves on a cubic g^3 grid in the real product basis of its axes
+// (xk_fp64.cu).  Tables of one (g, L): poisson_table_elems(g) doubles, filled by
+// poisson_tables_f64 (tab stays the caller's; uploads from host memory and
+// waits for it).
+size_t poisson_table_elems(int g);
+cudaError_t poisson_tables_f64(int g, double L, double* tab, cudaStream_t s);
+// out = Pois(in) (Eq. cou-1: 4 pi / G^2 on the grid's reciprocal vectors, G = 0
+// removed) for nf functions of g^3 values each; in is kept, out and tmp (nf g^3
+// each) are not the same memory.  scale: DGemm::scale of the products
+// (scale_ints ints), nullable.
+cudaError_t poisson_f64(const double* in, double* out, double* tmp, long nf, int g,
+                        const double* tab, int* scale, size_t scale_ints, cudaStream_t s);
+// rho[R] = sum_i psi[R][i]^2 for psi (ng x n).
+cudaError_t density_f64(const double* psi, long ng, int n, double* rho, cudaStream_t s);
+// out[R][nu] = v[R] phi[R][nu].
+cudaError_t potential_rows_f64(const double* v, const double* phi, long ng, int N, double* out,
+                               cudaStream_t s);
 // *out = scale * sum_j a[j] b[j] (fixed order); `work` holds reduce_work_elems() doubles.
 cudaError_t dot_f64(const double* a, const double* b, long len, double scale, double* work,
                     double* out, cudaStream_t s);

@@ -3,10 +3,10 @@
 // build consumes,
 //   X_gg = (Phi_g Phi_g^T) o (Phi_g Phi_g^T),  X_gR = (Phi_g Phi^T) o (Phi_g Phi^T)
 //   chi  = X_gg^{-1} X_gR          (Eq. lsqfit; blocked Cholesky, two blocked solves)
-//   V    = Pois(chi_g)              (Eq. rpsPot; DFT-based Poisson, two functions per
-//                                    complex transform)
+//   V    = Pois(chi_g)              (Eq. rpsPot; poisson_f64)
 //   W    = V chi^T, symmetrised     (Eq. thcpot)
-// all in FP64 on the CUDA cores (DFMA-bound on GB300), with a ridge of
+// all in FP64: the large products on the tensor cores (xk_digits.cu), the
+// blocks of the factorisation and the solves on the CUDA cores; with a ridge of
 // 1e-14 tr(X_gg) / N_aux added to the diagonal when the plain factorisation
 // fails.
 #include <algorithm>
@@ -148,30 +148,6 @@ __global__ void trsv_block_kernel(const double* __restrict__ L, long ldl, int k,
 #pragma unroll
     for (int j = 0; j < NB; ++j)
       if (j < kb) B[(long)(k + j) * ldb + c] = y[j];
-  }
-}
-
-// c[q][R] = f[2q][R] + i f[2q+1][R] for the rows [r0, r0 + nf) of f (ld).
-__global__ void pack_pairs_kernel(const double* __restrict__ f, long ld, long r0, int nf, long ng,
-                                  double2* __restrict__ c) {
-  const long np = (nf + 1) / 2, count = np * ng;
-  for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < count;
-       t += (long)gridDim.x * blockDim.x) {
-    const long q = t / ng, R = t % ng;
-    const double re = f[(r0 + 2 * q) * ld + R];
-    const double im = (2 * q + 1 < nf) ? f[(r0 + 2 * q + 1) * ld + R] : 0.0;
-    c[t] = make_double2(re, im);
-  }
-}
-
-__global__ void unpack_pairs_kernel(const double2* __restrict__ c, long r0, int nf, long ng,
-                                    double* __restrict__ out, long ld) {
-  const long np = (nf + 1) / 2, count = np * ng;
-  for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < count;
-       t += (long)gridDim.x * blockDim.x) {
-    const long q = t / ng, R = t % ng;
-    out[(r0 + 2 * q) * ld + R] = c[t].x;
-    if (2 * q + 1 < nf) out[(r0 + 2 * q + 1) * ld + R] = c[t].y;
   }
 }
 
@@ -480,34 +456,23 @@ cudaError_t isdf_tables_f64(const double* phi, long ng, int N, const double* phi
   // chi = X_gg^{-1} X_gR
   e = cholesky_solve_f64(Xgg, na, na, chi, ng, ng, scale, s);
   if (e != cudaSuccess) return e;
-  // V = Pois(chi), two functions per complex transform, in batches
+  // V = Pois(chi) in batches of functions (the scratch holds one)
   {
     const long g3 = (long)grid * grid * grid;
-    std::vector<double> t(2 * (size_t)grid);
-    for (int m = 0; m < grid; ++m) {
-      const double a = 2.0 * M_PI * (double)m / (double)grid;
-      t[2 * m] = std::cos(a);
-      t[2 * m + 1] = std::sin(a);
-    }
-    const int pairs = (int)std::max<long>(1, std::min<long>((na + 1) / 2, (1L << 28) / (g3 * 16)));
+    const size_t ints = 2 * (size_t)na * na;
+    long nf = std::max<long>(1, std::min<long>(na, (1L << 28) / (g3 * 8)));
+    if (scale)  // the row maxima of a batch go into the scratch of the products
+      nf = std::max<long>(1, std::min<long>(nf, ((long)std::min<size_t>(ints, 1u << 30) - grid - 8) /
+                                                    ((long)grid * grid)));
     void* buf = nullptr;
-    e = cudaMallocAsync(&buf, (size_t)(2 * pairs * g3 + grid) * 16, s);
+    e = cudaMallocAsync(&buf, ((size_t)nf * g3 + poisson_table_elems(grid)) * 8, s);
     if (e != cudaSuccess) return e;
-    double2* c0 = static_cast<double2*>(buf);
-    double2* c1 = c0 + pairs * g3;
-    double2* tw = c1 + pairs * g3;
-    e = cudaMemcpyAsync(tw, t.data(), t.size() * 8, cudaMemcpyHostToDevice, s);
-    for (long r0 = 0; e == cudaSuccess && r0 < na; r0 += 2L * pairs) {
-      const int nf = (int)std::min<long>(2L * pairs, na - r0);
-      const long np = (nf + 1) / 2;
-      pack_pairs_kernel<<<nblocks(np * g3), 256, 0, s>>>(chi, ng, r0, nf, g3, c0);
-      count_launch();
-      e = poisson_c2c_f64(c0, c1, np, grid, L, tw, s);
-      if (e != cudaSuccess) break;
-      unpack_pairs_kernel<<<nblocks(np * g3), 256, 0, s>>>(c0, r0, nf, g3, V, ng);
-      count_launch();
-      e = cudaGetLastError();
-    }
+    double* tmp = static_cast<double*>(buf);
+    double* tab = tmp + nf * g3;
+    e = poisson_tables_f64(grid, L, tab, s);
+    for (long r0 = 0; e == cudaSuccess && r0 < na; r0 += nf)
+      e = poisson_f64(chi + r0 * ng, V + r0 * ng, tmp, std::min<long>(nf, na - r0), grid, tab, scale,
+                      ints, s);
     cudaError_t e2 = cudaFreeAsync(buf, s);
     if (e == cudaSuccess) e = e2;
     if (e != cudaSuccess) return e;
