@@ -570,9 +570,7 @@ int enqueue_build(xk_handle* h) {
       xk::StepHook none{nullptr, nullptr};
       cudaError_t e = cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal);
       if (e == cudaSuccess) {
-        e = xk::mixed_enqueue(h->mixed, h->C, h->K, h->Ex, h->stream, none);
-        if (e == cudaSuccess)
-          e = xk::neg_dot_f64(h->K, h->C, (long)h->N * h->n, h->red, h->Ex + 1, h->stream);
+        e = xk::mixed_enqueue(h->mixed, h->C, h->K, h->Ex, h->Ex + 1, h->stream, none);
         cudaGraph_t graph = nullptr;
         const cudaError_t ec = cudaStreamEndCapture(h->stream, &graph);
         if (e == cudaSuccess) e = ec;
@@ -600,9 +598,7 @@ int enqueue_build(xk_handle* h) {
     }
   }
   xk::StepHook hook{h->timing ? &step_hook : nullptr, h};
-  cudaError_t e = xk::mixed_enqueue(h->mixed, h->C, h->K, h->Ex, h->stream, hook);
-  if (e == cudaSuccess)
-    e = xk::neg_dot_f64(h->K, h->C, (long)h->N * h->n, h->red, h->Ex + 1, h->stream);
+  cudaError_t e = xk::mixed_enqueue(h->mixed, h->C, h->K, h->Ex, h->Ex + 1, h->stream, hook);
   if (e != cudaSuccess) return cuda_fail(e, "mixed-precision build");
   return XK_OK;
 }
@@ -1505,7 +1501,8 @@ int xk_batch_build(xk_batch* b, const double* const* C, double* const* K_out, do
     fork(1);
     for (size_t i = 0; i < b->hs.size(); ++i)
       if (e == cudaSuccess)
-        e = xk::mixed_enqueue_post(b->hs[i]->mixed, b->hs[i]->K, b->hs[i]->Ex, b->side[i % ns], none);
+        e = xk::mixed_enqueue_post(b->hs[i]->mixed, b->hs[i]->C, b->hs[i]->K, b->hs[i]->Ex, nullptr,
+                                   b->side[i % ns], none);
     join(1);
     cudaGraph_t graph = nullptr;
     const cudaError_t ec = cudaStreamEndCapture(b->stream, &graph);

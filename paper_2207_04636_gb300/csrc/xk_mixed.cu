@@ -75,6 +75,8 @@ enum {
 };
 enum { AM_PHI = 0, AM_V, AM_W, AM_PHIP, AM_PHIP_RN, AM_C, AM_QCN, AM_PSI, AM_RN2, AM_M1, AM_D23,
        AM_FA, AM_FD, NAM };
+// behind the maxima, cleared with them: blocks of a launch that are done
+enum { CNT_Q = NAM, CNT_K, NAMC };
 
 constexpr float kHalfTarget = 16384.0f;  // 2^14: split inputs are scaled to |x| <= 2^14
 constexpr float kProdTarget = 32768.0f;  // 2^15: V o P is scaled to |x| <= 2^15
@@ -88,40 +90,47 @@ __device__ float pow2_scale(float maxabs, float target) {
   return s;
 }
 
-__device__ __forceinline__ float am_get(const unsigned* am, int i) { return __uint_as_float(am[i]); }
+// (from L2: other blocks of the same launch may have raised it)
+__device__ __forceinline__ float am_get(const unsigned* am, int i) { return __uint_as_float(__ldcg(am + i)); }
 
-// stage 0: C scale; 1: Psi / pair scales; 2: M1, (M2 - M3) scales; 3: full-K scales.
-__global__ void scales_kernel(const unsigned* __restrict__ am, float* __restrict__ sc, int stage) {
+// The scales that follow from the maxima of one stage of a build.  One thread of
+// the first kernel after that stage sets them (a launch of their own cost 3 us
+// each); kernels that need one within that launch derive it from the maximum.
+__device__ void scales_q(const unsigned* am, float* sc) {
+  sc[SC_C] = pow2_scale(am_get(am, AM_C), kHalfTarget);
+  sc[SC_OUT_ORB] = 1.0f / (sc[SC_PHIP] * sc[SC_C]);
+  // |Psi(R,j)| <= |Phi'(R,:)| |Q(:,j)| (Cauchy-Schwarz) bounds the orbital scale
+  sc[SC_PSI] = pow2_scale(sqrtf(am_get(am, AM_PHIP_RN)) * sqrtf(am_get(am, AM_QCN)) * 1.0001f,
+                          kHalfTarget);
+}
+
+__device__ void scales_psi(const unsigned* am, float* sc) {
+  const float sp = sc[SC_PSI];
+  // |P(g,R)| <= max_R sum_i psi_i(R)^2 (Cauchy-Schwarz), so |V o P| <= max|V| rn2
+  const float rn2 = am_get(am, AM_RN2) * sp * sp;
+  const float fab = pow2_scale(am_get(am, AM_V) * rn2, kProdTarget);
+  const float fc = pow2_scale(am_get(am, AM_W) * rn2, kProdTarget);
+  sc[SC_F_AB] = fab;
+  sc[SC_F_C] = fc;
+  sc[SC_OUT_AB] = 1.0f / (fab * sp * sp * sp);
+  sc[SC_OUT_C] = 1.0f / (fc * sp * sp * sp);
+  sc[SC_OUT_FA] = 1.0f / (fab * sp * sp * sc[SC_PHI]);
+  sc[SC_OUT_FC] = 1.0f / (fc * sp * sp * sc[SC_PHI]);
+}
+
+__device__ void scales_lines(const unsigned* am, float* sc) {
+  sc[SC_M1] = pow2_scale(am_get(am, AM_M1), kHalfTarget);
+  sc[SC_D23] = pow2_scale(am_get(am, AM_D23), kHalfTarget);
+  sc[SC_OUT_L1] = 1.0f / (sc[SC_PHI] * sc[SC_M1]);
+  sc[SC_OUT_L23] = 1.0f / (sc[SC_PHI] * sc[SC_D23]);
+}
+
+__global__ void scales_full_kernel(const unsigned* __restrict__ am, float* __restrict__ sc) {
   if (threadIdx.x != 0) return;
-  if (stage == 0) {
-    sc[SC_C] = pow2_scale(am_get(am, AM_C), kHalfTarget);
-    sc[SC_OUT_ORB] = 1.0f / (sc[SC_PHIP] * sc[SC_C]);
-    // |Psi(R,j)| <= |Phi'(R,:)| |Q(:,j)| (Cauchy-Schwarz) bounds the orbital scale
-    sc[SC_PSI] = pow2_scale(sqrtf(am_get(am, AM_PHIP_RN)) * sqrtf(am_get(am, AM_QCN)) * 1.0001f,
-                            kHalfTarget);
-  } else if (stage == 1) {
-    const float sp = sc[SC_PSI];
-    // |P(g,R)| <= max_R sum_i psi_i(R)^2 (Cauchy-Schwarz), so |V o P| <= max|V| rn2
-    const float rn2 = am_get(am, AM_RN2) * sp * sp;
-    const float fab = pow2_scale(am_get(am, AM_V) * rn2, kProdTarget);
-    const float fc = pow2_scale(am_get(am, AM_W) * rn2, kProdTarget);
-    sc[SC_F_AB] = fab;
-    sc[SC_F_C] = fc;
-    sc[SC_OUT_AB] = 1.0f / (fab * sp * sp * sp);
-    sc[SC_OUT_C] = 1.0f / (fc * sp * sp * sp);
-    sc[SC_OUT_FA] = 1.0f / (fab * sp * sp * sc[SC_PHI]);
-    sc[SC_OUT_FC] = 1.0f / (fc * sp * sp * sc[SC_PHI]);
-  } else if (stage == 3) {
-    sc[SC_FA] = pow2_scale(am_get(am, AM_FA), kHalfTarget);
-    sc[SC_FD] = pow2_scale(am_get(am, AM_FD), kHalfTarget);
-    sc[SC_OUT_FY] = 1.0f / (sc[SC_PHI] * sc[SC_FA]);
-    sc[SC_OUT_FZ] = 1.0f / (sc[SC_PHI] * sc[SC_FD]);
-  } else {
-    sc[SC_M1] = pow2_scale(am_get(am, AM_M1), kHalfTarget);
-    sc[SC_D23] = pow2_scale(am_get(am, AM_D23), kHalfTarget);
-    sc[SC_OUT_L1] = 1.0f / (sc[SC_PHI] * sc[SC_M1]);
-    sc[SC_OUT_L23] = 1.0f / (sc[SC_PHI] * sc[SC_D23]);
-  }
+  sc[SC_FA] = pow2_scale(am_get(am, AM_FA), kHalfTarget);
+  sc[SC_FD] = pow2_scale(am_get(am, AM_FD), kHalfTarget);
+  sc[SC_OUT_FY] = 1.0f / (sc[SC_PHI] * sc[SC_FA]);
+  sc[SC_OUT_FZ] = 1.0f / (sc[SC_PHI] * sc[SC_FD]);
 }
 
 __global__ void set_phi_scale_kernel(const unsigned* __restrict__ am, float* __restrict__ sc) {
@@ -169,61 +178,6 @@ __global__ void rownorm2_max_kernel(const T* __restrict__ a, long rows, int cols
   if ((threadIdx.x & 31) == 0) atomicMax(out, __float_as_uint(m * 1.0001f));
 }
 
-// max over columns of sum_r a[r][c]^2 (one block per column).
-__global__ void colnorm2_max_kernel(const double* __restrict__ a, long rows, long ld,
-                                    unsigned* __restrict__ out) {
-  __shared__ float red[8];
-  const long c = blockIdx.x;
-  float s = 0.0f;
-  for (long r = threadIdx.x; r < rows; r += blockDim.x) {
-    const float v = (float)a[r * ld + c];
-    s = fmaf(v, v, s);
-  }
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float t = 0.0f;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-    atomicMax(out, __float_as_uint(t * 1.0001f));
-  }
-}
-
-// rowmax[r] = max_c |a[r][c]| and glob = max over all, for long FP32 rows whose
-// stride is a multiple of 4 (2-D grid: x = column chunks, y = rows; float4 loads).
-__global__ void rowmax2d_kernel(const float* __restrict__ a, long cols, long ld,
-                                unsigned* __restrict__ rowmax, unsigned* __restrict__ glob) {
-  const long r = blockIdx.y;
-  const float4* row = reinterpret_cast<const float4*>(a + r * ld);
-  const long n4 = cols / 4;
-  float m = 0.0f;
-  const long step = (long)gridDim.x * blockDim.x;
-  long c = blockIdx.x * (long)blockDim.x + threadIdx.x;
-  for (; c + 3 * step < n4; c += 4 * step) {
-    float4 v[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) v[u] = row[c + u * step];
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-      m = fmaxf(m, fmaxf(fmaxf(fabsf(v[u].x), fabsf(v[u].y)), fmaxf(fabsf(v[u].z), fabsf(v[u].w))));
-  }
-  for (; c < n4; c += step) {
-    const float4 v = row[c];
-    m = fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
-  }
-  if (blockIdx.x == 0)
-    for (long t = n4 * 4 + threadIdx.x; t < cols; t += blockDim.x) m = fmaxf(m, fabsf(a[r * ld + t]));
-  __shared__ float red[32];
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = fmaxf(m, red[w]);
-    atomicMax(rowmax + r, __float_as_uint(m));
-    atomicMax(glob, __float_as_uint(m));
-  }
-}
-
 // Grid of a row whose largest |value| is mx: q = 2^(ceil(log2 mx) - 8), at
 // least 2^-24 (the FP16 subnormal step), so |x / q| <= 256.
 __device__ __forceinline__ float row_grid(float mx) {
@@ -234,26 +188,27 @@ __device__ __forceinline__ float row_grid(float mx) {
   return ldexpf(1.0f, max(e - 8, -24));
 }
 
-// Row r of dst (one block of 128 threads per row): m, h pieces of
-// src[r][c] * G on the row's grid for c < cols; zero for cols <= c < ld_dst.
+// Largest value of a block of up to 256 threads, in every thread.
+__device__ __forceinline__ float block_max(float v, float* red) {
+  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  v = red[0];
+  for (int w = 1; w < (int)(blockDim.x >> 5); ++w) v = fmaxf(v, red[w]);
+  return v;
+}
+
+// One row by one block: m, h (and l) pieces of row[c] * G on the row's grid for
+// c < cols; zero for cols <= c < ld_dst.  Returns the largest |row[c] G|.
 template <class T>
-__global__ void __launch_bounds__(128) split_mh_rows_kernel(
-    const T* __restrict__ src, long cols, long ld_src, const float* __restrict__ sc, int gidx,
-    __half* __restrict__ mo, __half* __restrict__ ho, __half* __restrict__ lo, long ld_dst) {
-  __shared__ float red[4];
-  const long r = blockIdx.x;
-  const T G = (T)sc[gidx];
-  const T* row = src + r * ld_src;
+__device__ __forceinline__ void split_row(const T* __restrict__ row, long cols, T G, float* red,
+                                          __half* __restrict__ mrow, __half* __restrict__ hrow,
+                                          __half* __restrict__ lrow, long ld_dst) {
   float mx = 0.0f;
   for (long c = threadIdx.x; c < cols; c += blockDim.x) mx = fmaxf(mx, fabsf((float)(row[c] * G)));
-  for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
-  __syncthreads();
-  mx = fmaxf(fmaxf(red[0], red[1]), fmaxf(red[2], red[3]));
+  mx = block_max(mx, red);
   // FP32 from here: rounding x to FP32 (2^-24) is far below the FP16 step of h
   const float q = row_grid(mx), qi = 1.0f / q;  // q a power of two: x * qi == x / q
-  __half* mrow = mo + r * ld_dst;
-  __half* hrow = ho + r * ld_dst;
   for (long c = threadIdx.x; c < ld_dst; c += blockDim.x) {
     __half mh = __float2half(0.0f), hh = __float2half(0.0f), lh = __float2half(0.0f);
     if (c < cols) {
@@ -265,48 +220,102 @@ __global__ void __launch_bounds__(128) split_mh_rows_kernel(
     }
     mrow[c] = mh;
     hrow[c] = hh;
-    if (lo) lo[r * ld_dst + c] = lh;
+    if (lrow) lrow[c] = lh;
   }
 }
 
-// As split_mh_rows_kernel with the row maxima (of |src|, unscaled) given, for
-// FP32 rows (stride a multiple of 4) into pieces of stride a multiple of 8:
-// 2-D grid, x = chunks of 8 columns, y = rows.
-__global__ void split_mh_rows_pre_kernel(const float* __restrict__ src, long cols, long ld_src,
-                                         const unsigned* __restrict__ rowmax,
-                                         const float* __restrict__ sc, int gidx,
-                                         __half* __restrict__ mo, __half* __restrict__ ho,
-                                         long ld_dst) {
-  const long r = blockIdx.y;
-  const float G = sc[gidx];
-  const float q = row_grid(__uint_as_float(rowmax[r]) * G);
-  const float qi = 1.0f / q;  // q is a power of two: x * qi == x / q
-  const float* row = src + r * ld_src;
-  for (long c8 = blockIdx.x * (long)blockDim.x + threadIdx.x; c8 * 8 < ld_dst;
-       c8 += (long)gridDim.x * blockDim.x) {
-    const long c = c8 * 8;
-    float x[8];
-    if (c + 8 <= cols) {
-      const float4 v0 = *reinterpret_cast<const float4*>(row + c);
-      const float4 v1 = *reinterpret_cast<const float4*>(row + c + 4);
-      x[0] = v0.x; x[1] = v0.y; x[2] = v0.z; x[3] = v0.w;
-      x[4] = v1.x; x[5] = v1.y; x[6] = v1.z; x[7] = v1.w;
-    } else {
-#pragma unroll
-      for (int j = 0; j < 8; ++j) x[j] = (c + j < cols) ? row[c + j] : 0.0f;
+// Row r of dst (one block of 128 threads per row): the pieces of src[r][c] * G.
+template <class T>
+__global__ void __launch_bounds__(128) split_mh_rows_kernel(
+    const T* __restrict__ src, long cols, long ld_src, const float* __restrict__ sc, int gidx,
+    __half* __restrict__ mo, __half* __restrict__ ho, __half* __restrict__ lo, long ld_dst) {
+  __shared__ float red[8];
+  const long r = blockIdx.x;
+  split_row<T>(src + r * ld_src, cols, (T)sc[gidx], red, mo + r * ld_dst, ho + r * ld_dst,
+               lo ? lo + r * ld_dst : nullptr, ld_dst);
+}
+
+// Q^T[j][mu] = sum_{k >= mu} L[k][mu] C[k][j] in FP64 (the zero triangle of L is
+// stored), zero for N <= mu < ld; max |Q| -> am_slot.  A block forms 8 x 8 outputs,
+// eight threads to an output's k: bound by the FP64 pipe (2 multiply-adds a clock
+// and SM), so the tile is small enough that the longest ones (mu near 0) do not
+// outlast the rest.  8 us at N = 351, n = 54, where the tiled product, its split sum,
+// the transpose and the two maxima took 38 us.
+constexpr int QT = 8, QS = 8;
+__global__ void __launch_bounds__(QT * QT * QS) q_kernel(const double* __restrict__ L,
+                                                        const double* __restrict__ C, int N, int n,
+                                                        double* __restrict__ QTr, long ld,
+                                                        unsigned* __restrict__ am_slot) {
+  __shared__ double part[QS][QT * QT];
+  const int mu0 = blockIdx.x * QT, j0 = blockIdx.y * QT;
+  const int o = threadIdx.x % (QT * QT), sl = threadIdx.x / (QT * QT);
+  const int mu = mu0 + o / QT, j = j0 + o % QT;
+  double s = 0.0;
+  if (mu < N && j < n) {
+#pragma unroll 8
+    for (int k = mu0 + sl; k < N; k += QS) s = fma(L[(long)k * N + mu], C[(long)k * n + j], s);
+  }
+  part[sl][o] = s;
+  __syncthreads();
+  if (threadIdx.x >= QT * QT) return;
+  // this thread now takes (mu, j) with mu fastest, for the store
+  const int a = threadIdx.x / QT, b = threadIdx.x % QT;
+  s = 0.0;
+  for (int w = 0; w < QS; ++w) s += part[w][b * QT + a];
+  if (j0 + a < n && mu0 + b < ld) QTr[(long)(j0 + a) * ld + mu0 + b] = s;
+  float m = j0 + a < n ? fabsf((float)s) : 0.0f;
+  for (int w = 16; w > 0; w >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, w));
+  if ((threadIdx.x & 31) == 0) atomicMax(am_slot, __float_as_uint(m));
+}
+
+// The pieces of Q^T, a block of 128 threads per row, with max_j sum_mu Q^2; the
+// last block to finish sets the scales of Q and Psi.
+__global__ void __launch_bounds__(128) split_q_kernel(const double* __restrict__ Q, long ld,
+                                                      unsigned* am, float* __restrict__ sc,
+                                                      __half* __restrict__ mo, __half* __restrict__ ho,
+                                                      __half* __restrict__ lo) {
+  __shared__ float red[8];
+  const long r = blockIdx.x;
+  const double* row = Q + r * ld;
+  float s = 0.0f;
+  for (long c = threadIdx.x; c < ld; c += blockDim.x) {
+    const float v = (float)row[c];
+    s = fmaf(v, v, s);
+  }
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0)
+    atomicMax(am + AM_QCN, __float_as_uint(((red[0] + red[1]) + (red[2] + red[3])) * 1.0001f));
+  __syncthreads();
+  split_row<double>(row, ld, (double)pow2_scale(am_get(am, AM_C), kHalfTarget), red, mo + r * ld,
+                    ho + r * ld, lo + r * ld, ld);
+  if (threadIdx.x == 0) {
+    __threadfence();
+    if (atomicAdd(am + CNT_Q, 1u) == gridDim.x - 1) {
+      __threadfence();
+      scales_q(am, sc);
     }
-    uint32_t mw[4], hw[4];
-#pragma unroll
-    for (int j = 0; j < 8; j += 2) {
-      const float x0 = x[j] * G, x1 = x[j + 1] * G;
-      const float m0 = q * rintf(x0 * qi), m1 = q * rintf(x1 * qi);
-      const __half2 hm = __floats2half2_rn(m0, m1);
-      const __half2 hh = __floats2half2_rn(x0 - m0, x1 - m1);
-      mw[j / 2] = *reinterpret_cast<const uint32_t*>(&hm);
-      hw[j / 2] = *reinterpret_cast<const uint32_t*>(&hh);
-    }
-    *reinterpret_cast<uint4*>(mo + r * ld_dst + c) = make_uint4(mw[0], mw[1], mw[2], mw[3]);
-    *reinterpret_cast<uint4*>(ho + r * ld_dst + c) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
+  }
+}
+
+// The orbital pieces at the interpolation points: npc pieces of `rows` rows of
+// v16 16-byte vectors, source and destination pieces sstride / dstride vectors
+// apart.  Block 0 also sets the pair step's scales and clears the row maxima of
+// M1 (n words) for the line step.
+__global__ void __launch_bounds__(256) gather_pieces_kernel(
+    const uint4* __restrict__ src, long sstride, const int32_t* __restrict__ idx, long rows, int v16,
+    int npc, uint4* __restrict__ dst, long dstride, const unsigned* __restrict__ am,
+    float* __restrict__ sc, unsigned* __restrict__ rowmax, int n) {
+  if (blockIdx.x == 0) {
+    if (threadIdx.x == 0) scales_psi(am, sc);
+    for (int i = threadIdx.x; i < n; i += blockDim.x) rowmax[i] = 0;
+  }
+  const long per = rows * v16, total = per * npc;
+  for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < total;
+       t += (long)gridDim.x * blockDim.x) {
+    const long p = t / per, q = t - p * per, r = q / v16;
+    dst[p * dstride + q] = src[p * sstride + (long)idx[r] * v16 + (q - r * v16)];
   }
 }
 
@@ -406,17 +415,6 @@ __global__ void split_rows_f32_kernel(const float* __restrict__ src, long rows, 
   }
 }
 
-__global__ void gather_rows_half_kernel(const __half* __restrict__ src, long ld,
-                                        const int32_t* __restrict__ idx, int rows,
-                                        __half* __restrict__ dst) {
-  const long total = (long)rows * ld;
-  for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < total;
-       t += (long)gridDim.x * blockDim.x) {
-    const long r = t / ld, c = t % ld;
-    dst[t] = src[(long)idx[r] * ld + c];
-  }
-}
-
 // FP64 [rows][cols] -> FP32 [rows][ld_dst], zero padding.
 __global__ void f64_to_f32_kernel(const double* __restrict__ src, long rows, long cols,
                                   float* __restrict__ dst, long ld_dst) {
@@ -464,58 +462,241 @@ __global__ void reduce_parts_kernel(const float* __restrict__ a, int na, const f
   if (am_slot && (threadIdx.x & 31) == 0) atomicMax(am_slot, __float_as_uint(m));
 }
 
-// K[mu][j] = dV * (sum_s L1[s][mu][j] + sum_s L23[s][mu][j]), FP64.
-__global__ void final_k_kernel(const float* __restrict__ L1, int n1, const float* __restrict__ L23,
-                               int n23, long count, double dV, double* __restrict__ K) {
-  for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < count;
-       t += (long)gridDim.x * blockDim.x) {
-    float h1 = 0.0f, l1 = 0.0f, h2 = 0.0f, l2 = 0.0f;
+// Two-sum of the terms p = first, first + step, ... < np of a[p * count], added to hi + lo.
+__device__ __forceinline__ void sum_parts(const float* __restrict__ a, long count, int np, int first,
+                                          int step, float scale, float& hi, float& lo) {
 #pragma unroll 8
-    for (int p = 0; p < n1; ++p) ff_add(h1, l1, L1[(long)p * count + t]);
-#pragma unroll 8
-    for (int p = 0; p < n23; ++p) ff_add(h2, l2, L23[(long)p * count + t]);
-    const double s1 = (double)h1 + (double)l1, s2 = (double)h2 + (double)l2;
-    K[t] = dV * (s1 + s2);
+  for (int p = first; p < np; p += step) ff_add(hi, lo, a[(long)p * count] * scale);
+}
+
+constexpr int RS = 8;          // threads to one sum of partial sums
+constexpr int kFewParts = 32;  // up to so many, one thread
+
+// Adds the RS warps' sums hi + lo of 32 neighbouring outputs; the result is in
+// warp 0.  One thread per output left the loads of 50 to 100 partial sums in one
+// serial chain (21 us at 19000 outputs of 93 partial sums, 4 us this way).
+__device__ __forceinline__ double join_parts(float hi, float lo, float (*sh)[2][32]) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  sh[w][0][lane] = hi;
+  sh[w][1][lane] = lo;
+  __syncthreads();
+  if (w == 0)
+    for (int k = 1; k < RS; ++k) {
+      ff_add(hi, lo, sh[k][0][lane]);
+      lo += sh[k][1][lane];
+    }
+  __syncthreads();
+  return (double)hi + (double)lo;
+}
+
+// First half of the line step.  Blocks below nd: (M2 - M3)^T[j][g] = sum of the
+// M2 partial sums (times the power of two a_scale) less those of M3, FP64, and its
+// largest value.  The others: row maxima of M1 (chunk, row) and its largest value.
+__global__ void __launch_bounds__(32 * RS) lines_sum_kernel(
+    const float* __restrict__ a, int na_, const float* __restrict__ b, int nb_, long rows, int n,
+    const float* __restrict__ a_scale, double* __restrict__ out, long ldo, int nd,
+    const float* __restrict__ M1, long cols, long ld, int chunks, unsigned* __restrict__ rowmax,
+    unsigned* __restrict__ am) {
+  __shared__ float sh[RS][2][32], red[8];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  float m = 0.0f;
+  if ((int)blockIdx.x < nd) {
+    const long count = rows * n;
+    const float as = a_scale ? *a_scale : 1.0f;
+    const bool few = na_ + nb_ <= kFewParts;  // a thread, or a lane of every warp, per output
+    const long t0 = few ? (long)blockIdx.x * (32 * RS) + threadIdx.x : (long)blockIdx.x * 32 + lane;
+    const long t = min(t0, count - 1);
+    float hi = 0.0f, lo = 0.0f;
+    sum_parts(a + t, count, na_, few ? 0 : w, few ? 1 : RS, as, hi, lo);
+    sum_parts(b + t, count, nb_, few ? 0 : w, few ? 1 : RS, -1.0f, hi, lo);
+    const double s = few ? (double)hi + (double)lo : join_parts(hi, lo, sh);
+    if ((few || w == 0) && t0 < count) {
+      const long g = t / n;
+      out[(t - g * n) * ldo + g] = s;
+      m = fabsf((float)s);
+    }
+    m = block_max(m, red);
+    if (threadIdx.x == 0) atomicMax(am + AM_D23, __float_as_uint(m));
+    return;
+  }
+  const int task = (int)blockIdx.x - nd, chunk = task % chunks;
+  const long r = task / chunks;
+  const float4* row = reinterpret_cast<const float4*>(M1 + r * ld);  // ld a multiple of 4
+  const long n4 = cols / 4, step = (long)chunks * blockDim.x;
+  long c = (long)chunk * blockDim.x + threadIdx.x;
+  for (; c + 3 * step < n4; c += 4 * step) {
+    float4 v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) v[u] = row[c + u * step];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      m = fmaxf(m, fmaxf(fmaxf(fabsf(v[u].x), fabsf(v[u].y)), fmaxf(fabsf(v[u].z), fabsf(v[u].w))));
+  }
+  for (; c < n4; c += step) {
+    const float4 v = row[c];
+    m = fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
+  }
+  if (chunk == 0)
+    for (long t = n4 * 4 + threadIdx.x; t < cols; t += blockDim.x) m = fmaxf(m, fabsf(M1[r * ld + t]));
+  m = block_max(m, red);
+  if (threadIdx.x == 0) {
+    atomicMax(rowmax + r, __float_as_uint(m));
+    atomicMax(am + AM_M1, __float_as_uint(m));
   }
 }
 
-// E_x = -dV (2 sum_k ea[k] - sum_k ec[k]) / G^4 with G the orbital scale, in
-// a fixed summation order (one block of 256 threads).
-__global__ void __launch_bounds__(1024) final_ex_kernel(const double* __restrict__ ea, int na_,
-                                                       const double* __restrict__ ec, int nc_,
-                                                       const float* __restrict__ sc, double dV,
-                                                       double* Ex) {
-  // one block of 1024 threads; four independent sums per thread keep several
-  // loads in flight (the n > 128 path has ~10^5 partials per launch); the
-  // order is fixed by the launch shape, so a build repeats bit for bit
-  __shared__ double sa[32], sb[32];
-  double a[4] = {0.0, 0.0, 0.0, 0.0}, b[4] = {0.0, 0.0, 0.0, 0.0};
-  const int T = blockDim.x;
-  int t = threadIdx.x;
-  for (; t + 3 * T < na_; t += 4 * T) {
-    a[0] += ea[t]; a[1] += ea[t + T]; a[2] += ea[t + 2 * T]; a[3] += ea[t + 3 * T];
+// Second half: the pieces of M1 (blocks below n1 * n: chunk, row; the row maxima
+// given) and of (M2 - M3)^T (a block per row), with the scales from the maxima.
+__global__ void __launch_bounds__(256) lines_split_kernel(
+    const float* __restrict__ M1, long cols, long ld_src, const unsigned* __restrict__ rowmax,
+    __half* __restrict__ mo, __half* __restrict__ ho, long ld_dst, int n1, int n,
+    const double* __restrict__ D, long ldd, __half* __restrict__ dm, __half* __restrict__ dh,
+    const unsigned* __restrict__ am, float* __restrict__ sc) {
+  __shared__ float red[8];
+  if (blockIdx.x == 0 && threadIdx.x == 0) scales_lines(am, sc);
+  if ((int)blockIdx.x >= n1 * n) {
+    const long r = (int)blockIdx.x - n1 * n;
+    split_row<double>(D + r * ldd, ldd, (double)pow2_scale(am_get(am, AM_D23), kHalfTarget), red,
+                      dm + r * ldd, dh + r * ldd, nullptr, ldd);
+    return;
   }
-  for (; t < na_; t += T) a[0] += ea[t];
-  t = threadIdx.x;
-  for (; t + 3 * T < nc_; t += 4 * T) {
-    b[0] += ec[t]; b[1] += ec[t + T]; b[2] += ec[t + 2 * T]; b[3] += ec[t + 3 * T];
+  const long r = blockIdx.x / n1;
+  const float G = pow2_scale(am_get(am, AM_M1), kHalfTarget);
+  const float q = row_grid(__uint_as_float(rowmax[r]) * G);
+  const float qi = 1.0f / q;  // q is a power of two: x * qi == x / q
+  const float* row = M1 + r * ld_src;
+  for (long c8 = (blockIdx.x % n1) * (long)blockDim.x + threadIdx.x; c8 * 8 < ld_dst;
+       c8 += (long)n1 * blockDim.x) {
+    const long c = c8 * 8;
+    float x[8];
+    if (c + 8 <= cols) {
+      const float4 v0 = *reinterpret_cast<const float4*>(row + c);
+      const float4 v1 = *reinterpret_cast<const float4*>(row + c + 4);
+      x[0] = v0.x; x[1] = v0.y; x[2] = v0.z; x[3] = v0.w;
+      x[4] = v1.x; x[5] = v1.y; x[6] = v1.z; x[7] = v1.w;
+    } else {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) x[j] = (c + j < cols) ? row[c + j] : 0.0f;
+    }
+    uint32_t mw[4], hw[4];
+#pragma unroll
+    for (int j = 0; j < 8; j += 2) {
+      const float x0 = x[j] * G, x1 = x[j + 1] * G;
+      const float m0 = q * rintf(x0 * qi), m1 = q * rintf(x1 * qi);
+      const __half2 hm = __floats2half2_rn(m0, m1);
+      const __half2 hh = __floats2half2_rn(x0 - m0, x1 - m1);
+      mw[j / 2] = *reinterpret_cast<const uint32_t*>(&hm);
+      hw[j / 2] = *reinterpret_cast<const uint32_t*>(&hh);
+    }
+    *reinterpret_cast<uint4*>(mo + r * ld_dst + c) = make_uint4(mw[0], mw[1], mw[2], mw[3]);
+    *reinterpret_cast<uint4*>(ho + r * ld_dst + c) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
   }
-  for (; t < nc_; t += T) b[0] += ec[t];
-  double x = (a[0] + a[1]) + (a[2] + a[3]), y = (b[0] + b[1]) + (b[2] + b[3]);
-  for (int o = 16; o > 0; o >>= 1) {
-    x += __shfl_xor_sync(0xffffffffu, x, o);
-    y += __shfl_xor_sync(0xffffffffu, y, o);
+}
+
+// E_x = -dV (2 sum ea - sum ec) / G^4 with G the orbital scale.  The partials are
+// summed in kExBlocks chunks per array by as many blocks, the chunks' sums in
+// order by the last block of the launch: a fixed order, so a build repeats bit for
+// bit and xk_energy, which runs the same sums, gives the same E_x.
+constexpr int kExBlocks = 16;
+
+__device__ __forceinline__ double block_sum(double v, double* sh) {
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+  __syncthreads();
+  v = 0.0;
+  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += sh[w];
+  return v;
+}
+
+// Chunk b of 2 kExBlocks (256 threads): b < kExBlocks of ea, else of ec.
+__device__ __forceinline__ void ex_chunk(int b, const double* __restrict__ ea, int na_,
+                                         const double* __restrict__ ec, int nc_, double* sh,
+                                         double* __restrict__ part) {
+  const bool c = b >= kExBlocks;
+  const double* e = c ? ec : ea;
+  const int len = c ? nc_ : na_, per = (len + kExBlocks - 1) / kExBlocks;
+  const int k = c ? b - kExBlocks : b, t1 = min(len, (k + 1) * per);
+  double v = 0.0;
+#pragma unroll 4
+  for (int t = k * per + threadIdx.x; t < t1; t += blockDim.x) v += e[t];
+  v = block_sum(v, sh);
+  if (threadIdx.x == 0) part[b] = v;
+}
+
+__device__ __forceinline__ void ex_total(const double* part, const float* sc, double dV, double* Ex) {
+  double u = 0.0, v = 0.0;
+  for (int k = 0; k < kExBlocks; ++k) {
+    u += __ldcg(part + k);
+    v += __ldcg(part + kExBlocks + k);
   }
-  const int w = threadIdx.x >> 5, nw = T >> 5;
-  if ((threadIdx.x & 31) == 0) { sa[w] = x; sb[w] = y; }
+  const double g = (double)sc[SC_PSI];
+  const double g4 = (g * g) * (g * g);
+  *Ex = -dV * (2.0 * u - v) / g4;
+}
+
+// True in every thread of the launch's last block to arrive.
+__device__ __forceinline__ bool last_block(unsigned* counter, int* flag) {
   __syncthreads();
   if (threadIdx.x == 0) {
-    double u = 0.0, v = 0.0;
-    for (int k = 0; k < nw; ++k) { u += sa[k]; v += sb[k]; }
-    const double g = (double)sc[SC_PSI];
-    const double g4 = (g * g) * (g * g);
-    *Ex = -dV * (2.0 * u - v) / g4;
+    __threadfence();
+    *flag = atomicAdd(counter, 1u) == gridDim.x - 1;
+    __threadfence();
   }
+  __syncthreads();
+  return *flag != 0;
+}
+
+// E_x alone (xk_energy): 2 kExBlocks blocks.
+__global__ void __launch_bounds__(256) final_ex_kernel(const double* __restrict__ ea, int na_,
+                                                      const double* __restrict__ ec, int nc_,
+                                                      const float* __restrict__ sc, double dV,
+                                                      double* part, unsigned* counter, double* Ex) {
+  __shared__ double sh[8];
+  __shared__ int flag;
+  ex_chunk(blockIdx.x, ea, na_, ec, nc_, sh, part);
+  if (last_block(counter, &flag) && threadIdx.x == 0) ex_total(part, sc, dV, Ex);
+}
+
+// K[mu][j] = dV * (sum_s L1[s][mu][j] + sum_s L23[s][mu][j]) in FP64, E_x (the
+// first 2 kExBlocks blocks) and, with EK, the energy of this K, -sum K o C, in a
+// fixed order.
+__global__ void __launch_bounds__(32 * RS) final_kernel(
+    const float* __restrict__ L1, int n1, const float* __restrict__ L23, int n23, long count, double dV,
+    double* __restrict__ K, const double* __restrict__ C, const double* __restrict__ ea, int na_,
+    const double* __restrict__ ec, int nc_, const float* __restrict__ sc, double* part,
+    unsigned* counter, double* Ex, double* EK) {
+  __shared__ float shf[RS][2][32];
+  __shared__ double sh[8];
+  __shared__ int flag;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int nk = (int)gridDim.x - 2 * kExBlocks, kb = (int)blockIdx.x - 2 * kExBlocks;
+  if (kb < 0) {
+    ex_chunk(blockIdx.x, ea, na_, ec, nc_, sh, part);
+  } else {
+    const long t0 = (long)kb * 32 + lane, t = min(t0, count - 1);
+    float h1 = 0.0f, l1 = 0.0f, h2 = 0.0f, l2 = 0.0f;
+    sum_parts(L1 + t, count, n1, w, RS, 1.0f, h1, l1);
+    sum_parts(L23 + t, count, n23, w, RS, 1.0f, h2, l2);
+    const double s1 = join_parts(h1, l1, shf), s2 = join_parts(h2, l2, shf);
+    if (w == 0) {
+      const double k = dV * (s1 + s2);
+      if (t0 < count) K[t] = k;
+      if (EK) {
+        double dot = t0 < count ? k * C[t] : 0.0;
+        for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
+        if (lane == 0) part[2 * kExBlocks + kb] = dot;
+      }
+    }
+  }
+  if (!last_block(counter, &flag)) return;
+  if (EK) {
+    double v = 0.0;
+    for (int b = threadIdx.x; b < nk; b += blockDim.x) v += __ldcg(part + 2 * kExBlocks + b);
+    v = block_sum(v, sh);
+    if (threadIdx.x == 0) *EK = -v;
+  }
+  if (threadIdx.x == 0) ex_total(part, sc, dV, Ex);
 }
 
 // Full K: K[mu][nu] = dV (sum_s Z[s][mu][nu] + sum_s Y[s][nu][mu]), FP64, with
@@ -589,7 +770,7 @@ template <bool kShort>
 __device__ __forceinline__ void gemm_body(const CUtensorMap* pAm, const CUtensorMap* pAh,
                                           const CUtensorMap* pBm, const CUtensorMap* pBh,
                                           const CUtensorMap* pAl, const CUtensorMap* pBl,
-                                          const GemmArgs& g) {
+                                          const GemmArgs& g, int cta, int nctas) {
   extern __shared__ uint8_t g_raw[];
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(g_raw) + 1023) & ~uintptr_t(1023));
   __shared__ uint64_t full[G_STAGES], empty[G_STAGES], set_ready[2], set_free[2], drain;
@@ -639,7 +820,7 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap* pAm, const CUtensor
     prefetch_tmap(pAm); prefetch_tmap(pAh); prefetch_tmap(pBm); prefetch_tmap(pBh);
     int last_parity[G_STAGES] = {-1, -1, -1};
     int it = 0;  // k-blocks issued by this CTA over all its tiles
-    for (int tile = blockIdx.x; tile < ntiles && !abort_flag; tile += gridDim.x) {
+    for (int tile = cta; tile < ntiles && !abort_flag; tile += nctas) {
     int bx, by, bz;
     tile_at(tile, bx, by, bz);
     const int m0 = bx * 128, n0 = by * 128, kbeg = bz * g.kchunk, nkb = kblocks(bz);
@@ -701,7 +882,7 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap* pAm, const CUtensor
     // over all tiles (accumulator sets alternate across tile boundaries too)
     int it = 0, G0 = 0;
     bool good = true;
-    for (int tile = blockIdx.x; good && tile < ntiles; tile += gridDim.x) {
+    for (int tile = cta; good && tile < ntiles; tile += nctas) {
     int bx, by, bz;
     tile_at(tile, bx, by, bz);
     const int nkb = kblocks(bz);
@@ -764,7 +945,7 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap* pAm, const CUtensor
     // Every epilogue warp walks all of the CTA's tiles (after a failed wait
     // without waiting further), so the named barriers below match up.
     int G0 = 0;
-    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    for (int tile = cta; tile < ntiles; tile += nctas) {
     int bx, by, bz;
     tile_at(tile, bx, by, bz);
     const int m0 = bx * 128, n0 = by * 128;
@@ -888,9 +1069,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
                 const __grid_constant__ CUtensorMap mAl, const __grid_constant__ CUtensorMap mBl,
                 GemmArgs g) {
   if (g.wait > 0 && g.wait < kWaitCycles)
-    gemm_body<true>(&mAm, &mAh, &mBm, &mBh, &mAl, &mBl, g);
+    gemm_body<true>(&mAm, &mAh, &mBm, &mBh, &mAl, &mBl, g, blockIdx.x, gridDim.x);
   else
-    gemm_body<false>(&mAm, &mAh, &mBm, &mBh, &mAl, &mBl, g);
+    gemm_body<false>(&mAm, &mAh, &mBm, &mBh, &mAl, &mBl, g, blockIdx.x, gridDim.x);
 }
 
 // SMs of the current device (cached per device).
@@ -945,7 +1126,7 @@ template <bool kShort, bool kP3>
 __device__ __forceinline__ void gemm_wide_body(const CUtensorMap* pAm, const CUtensorMap* pAh,
                                                const CUtensorMap* pBm, const CUtensorMap* pBh,
                                                const CUtensorMap* pAl, const CUtensorMap* pBl,
-                                               const GemmArgs& g) {
+                                               const GemmArgs& g, int cta, int nctas) {
   extern __shared__ uint8_t gw_raw[];
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(gw_raw) + 1023) & ~uintptr_t(1023));
   __shared__ uint64_t full[3], empty[3], set_ready, set_free, drain;
@@ -992,7 +1173,7 @@ __device__ __forceinline__ void gemm_wide_body(const CUtensorMap* pAm, const CUt
     prefetch_tmap(pAm); prefetch_tmap(pAh); prefetch_tmap(pBm); prefetch_tmap(pBh);
     int last_parity[3] = {-1, -1, -1};
     int it = 0;
-    for (int tile = blockIdx.x; tile < ntiles && !abort_flag; tile += gridDim.x) {
+    for (int tile = cta; tile < ntiles && !abort_flag; tile += nctas) {
       int bx, by, bz;
       tile_at(tile, bx, by, bz);
       const int m0 = bx * 128, n0 = by * 256, kbeg = bz * g.kchunk, nkb = kblocks(bz);
@@ -1050,7 +1231,7 @@ __device__ __forceinline__ void gemm_wide_body(const CUtensorMap* pAm, const CUt
     };
     int it = 0, G = 0;  // G: drain groups issued over all tiles
     bool good = true;
-    for (int tile = blockIdx.x; good && tile < ntiles; tile += gridDim.x) {
+    for (int tile = cta; good && tile < ntiles; tile += nctas) {
       int bx, by, bz;
       tile_at(tile, bx, by, bz);
       const int nkb = kblocks(bz);
@@ -1102,7 +1283,7 @@ __device__ __forceinline__ void gemm_wide_body(const CUtensorMap* pAm, const CUt
     const int cb = 64 * qc;
     const uint32_t lane_off = static_cast<uint32_t>(quad * 32) << 16;
     int G = 0;
-    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    for (int tile = cta; tile < ntiles; tile += nctas) {
       int bx, by, bz;
       tile_at(tile, bx, by, bz);
       const int m0 = bx * 128, n0 = by * 256;
@@ -1180,9 +1361,9 @@ __global__ void __launch_bounds__(kWideThreads, 1)
                      const __grid_constant__ CUtensorMap mBm, const __grid_constant__ CUtensorMap mBh,
                      GemmArgs g) {
   if (g.wait > 0 && g.wait < kWaitCycles)
-    gemm_wide_body<true, false>(&mAm, &mAh, &mBm, &mBh, &mAm, &mBm, g);
+    gemm_wide_body<true, false>(&mAm, &mAh, &mBm, &mBh, &mAm, &mBm, g, blockIdx.x, gridDim.x);
   else
-    gemm_wide_body<false, false>(&mAm, &mAh, &mBm, &mBh, &mAm, &mBm, g);
+    gemm_wide_body<false, false>(&mAm, &mAh, &mBm, &mBh, &mAm, &mBm, g, blockIdx.x, gridDim.x);
 }
 
 // Three pieces per operand, K-major, [128][32] / [256][32] boxes with the
@@ -1193,9 +1374,9 @@ __global__ void __launch_bounds__(kWideThreads, 1)
                       const __grid_constant__ CUtensorMap mBh, const __grid_constant__ CUtensorMap mBl,
                       GemmArgs g) {
   if (g.wait > 0 && g.wait < kWaitCycles)
-    gemm_wide_body<true, true>(&mAm, &mAh, &mBm, &mBh, &mAl, &mBl, g);
+    gemm_wide_body<true, true>(&mAm, &mAh, &mBm, &mBh, &mAl, &mBl, g, blockIdx.x, gridDim.x);
   else
-    gemm_wide_body<false, true>(&mAm, &mAh, &mBm, &mBh, &mAl, &mBl, g);
+    gemm_wide_body<false, true>(&mAm, &mAh, &mBm, &mBh, &mAl, &mBl, g, blockIdx.x, gridDim.x);
 }
 
 constexpr int GW3_SMEM = 3 * (3 * 8192 + 3 * 16384) + 1024;
@@ -1224,6 +1405,61 @@ void launch_gemm_wide(const CUtensorMap& mAm, const CUtensorMap& mAh, const CUte
   const long total = (long)tiles.x * tiles.y * tiles.z;
   const unsigned ctas = (unsigned)std::max<long>(1, std::min<long>(total, sm_count()));
   gemm_wide_kernel<<<ctas, kWideThreads, GW_SMEM, s>>>(mAm, mAh, mBm, mBh, g);
+}
+
+// ============================================================ two products, one launch
+// The two line contractions side by side: the first c0 CTAs walk the tiles of
+// product 0, the others those of product 1 (the shorter one, N_aux terms against
+// N_g, filled a fraction of the SMs for a launch of its own: 10 to 15 us).
+struct GemmPair {
+  CUtensorMap am[2], ah[2], bm[2], bh[2];
+  GemmArgs g[2];
+  int c0;
+};
+
+template <bool kWide>
+__global__ void __launch_bounds__(kWide ? kWideThreads : kGemmThreads, 1)
+    gemm_pair_kernel(const __grid_constant__ GemmPair p) {
+  const int k = (int)blockIdx.x < p.c0 ? 0 : 1;
+  const int cta = k ? (int)blockIdx.x - p.c0 : (int)blockIdx.x;
+  const int nctas = k ? (int)gridDim.x - p.c0 : p.c0;
+  const CUtensorMap *am = k ? &p.am[1] : &p.am[0], *ah = k ? &p.ah[1] : &p.ah[0],
+                    *bm = k ? &p.bm[1] : &p.bm[0], *bh = k ? &p.bh[1] : &p.bh[0];
+  const GemmArgs& g = k ? p.g[1] : p.g[0];
+  const bool sh = g.wait > 0 && g.wait < kWaitCycles;
+  if constexpr (kWide) {
+    if (sh) gemm_wide_body<true, false>(am, ah, bm, bh, am, bm, g, cta, nctas);
+    else gemm_wide_body<false, false>(am, ah, bm, bh, am, bm, g, cta, nctas);
+  } else {
+    if (sh) gemm_body<true>(am, ah, bm, bh, am, bm, g, cta, nctas);
+    else gemm_body<false>(am, ah, bm, bh, am, bm, g, cta, nctas);
+  }
+}
+
+// tiles: (M tiles, N tiles, K splits) of each product; the CTAs (at most one per
+// SM and tile) are shared out by K blocks.
+void launch_gemm_pair(GemmPair p, const dim3 (&tiles)[2], bool wide, cudaStream_t s, long long wait) {
+  long total[2], work[2];
+  for (int k = 0; k < 2; ++k) {
+    p.g[k].wait = wait;
+    p.g[k].tiles_x = (int)tiles[k].x;
+    p.g[k].tiles_y = (int)tiles[k].y;
+    p.g[k].tiles_z = (int)tiles[k].z;
+    total[k] = (long)tiles[k].x * tiles[k].y * tiles[k].z;
+    work[k] = total[k] * ((p.g[k].kchunk + 63) / 64 + 4);  // a tile's start and end: about 4 blocks
+  }
+  const long sms = sm_count();
+  long c0 = std::min(total[0], sms), c1 = std::min(total[1], sms);
+  if (c0 + c1 > sms) {
+    c1 = std::max<long>(1, std::min(c1, (sms * work[1] + (work[0] + work[1]) / 2) / (work[0] + work[1])));
+    c0 = std::min(c0, std::max<long>(1, sms - c1));
+  }
+  p.c0 = (int)c0;
+  if (wide)
+    gemm_pair_kernel<true><<<(unsigned)(c0 + c1), kWideThreads, GW_SMEM, s>>>(p);
+  else
+    gemm_pair_kernel<false><<<(unsigned)(c0 + c1), kGemmThreads, G_SMEM, s>>>(p);
+  count_launch();
 }
 
 // ============================================================ T products
@@ -2667,8 +2903,8 @@ struct MixedState {
          *D23T_h = nullptr;
   float *M2p = nullptr, *M3p = nullptr, *M1 = nullptr, *L1p = nullptr, *L23p = nullptr,
         *sc = nullptr;
-  double *D23 = nullptr, *CT64 = nullptr, *D23T64 = nullptr, *red = nullptr, *EpA = nullptr,
-         *EpC = nullptr, *Lf = nullptr, *Q64 = nullptr, *dwork = nullptr;
+  double *D23 = nullptr /* scratch of Q's digit product */, *CT64 = nullptr, *D23T64 = nullptr, *part = nullptr, *EpA = nullptr,
+         *EpC = nullptr, *Lf = nullptr, *dwork = nullptr;
   unsigned* am = nullptr;
   unsigned* rowmax = nullptr;
   int* status = nullptr;
@@ -3015,6 +3251,10 @@ cudaError_t mixed_create(int64_t Ng, int N, int n, int NaT, int g0, int g1, cons
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, G_SMEM);
   if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(gemm_pair_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, G_SMEM);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(gemm_pair_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, GW_SMEM);
+  if (e == cudaSuccess)
     e = cudaFuncSetAttribute(tprod_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TP_SMEM);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(gemm_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, GW_SMEM);
@@ -3080,9 +3320,9 @@ cudaError_t mixed_create(int64_t Ng, int N, int n, int NaT, int g0, int g1, cons
   MX(m->D23T_m, (size_t)n * p.Na8); MX(m->D23T_h, (size_t)n * p.Na8);
   MX(m->L1p, (size_t)p.splitsL1 * N * n); MX(m->L23p, (size_t)p.splitsL23 * N * n);
   MX(m->EpA, (size_t)p.epA); MX(m->EpC, (size_t)p.epC);
-  MX(m->sc, NSC); MX(m->am, NAM); MX(m->status, 4); MX(m->rowmax, (size_t)n);
-  MX(m->red, reduce_work_elems());
-  MX(m->Lf, (size_t)N * N); MX(m->Q64, (size_t)N * n);
+  MX(m->sc, NSC); MX(m->am, NAMC); MX(m->status, 4); MX(m->rowmax, (size_t)n);
+  MX(m->Lf, (size_t)N * N);
+  MX(m->part, std::max((size_t)N * n, (size_t)512));  // sums of the final kernel's blocks
   MX(m->dwork, dwork_elems(Ng, N, n));
 #undef MX
   double *stage = nullptr, *stage2 = nullptr;
@@ -3101,7 +3341,10 @@ cudaError_t mixed_create(int64_t Ng, int N, int n, int NaT, int g0, int g1, cons
     cudaFree(stage2);
     return err == cudaSuccess ? cudaSuccess : bail(err);
   };
-  e = cudaMemsetAsync(m->am, 0, NAM * 4, s);
+  e = cudaMemsetAsync(m->am, 0, NAMC * 4, s);
+  // the padding columns of these two are read but never written
+  if (e == cudaSuccess) e = cudaMemsetAsync(m->CT64, 0, (size_t)n * p.Np * 8, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(m->D23T64, 0, (size_t)n * p.Na8 * 8, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(m->sc, 0, NSC * 4, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(m->status, 0, 16, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(m->idx, idx, nat * 4, cudaMemcpyHostToDevice, s);
@@ -3303,23 +3546,27 @@ cudaError_t mixed_enqueue_pre(MixedState* m, const double* C, cudaStream_t s, co
   cudaError_t e;
   // ---- step 1: Psi = Phi C
   hook(0, 1);
-  e = cudaMemsetAsync(m->am + AM_C, 0, (NAM - AM_C) * 4, s);
+  e = cudaMemsetAsync(m->am + AM_C, 0, (NAMC - AM_C) * 4, s);
   if (e != cudaSuccess) return e;
-  {
-    // L^T is upper triangular: each row tile of Q only needs K >= its first row
-    DGemm g{N, n, N, m->Lf, N, true, C, n, false, m->Q64, n, 1.0, nullptr, 0, q_ksplit(N), m->dwork,
-            true};
-    e = dgemm(g, s);
+  {  // Q^T = C^T L.  From 6e7 multiply-adds (of which the triangle needs half) the
+     // FP64 pipe takes longer than the digit products on the tensor cores (73 against
+     // 40 us at N = 832, n = 128)
+    DGemm g{n, N, N, C, n, true, m->Lf, N, false, m->CT64, m->Np, 1.0, nullptr, 0, q_ksplit(N), m->dwork};
+    if (2 * (size_t)m->Naux * n >= digit_scale_ints(n, N))
+      g.scale = reinterpret_cast<int*>(m->D23);
+    if ((double)N * N * n >= 6e7 && digit_gemm_wanted(g)) {
+      e = dgemm(g, s);
+      if (e != cudaSuccess) return e;
+      absmax_kernel<double><<<blocks_for((long)N * n), 256, 0, s>>>(m->CT64, n, N, m->Np, m->am + AM_C);
+    } else {
+      q_kernel<<<dim3((unsigned)((m->Np + QT - 1) / QT), (unsigned)((n + QT - 1) / QT)), QT * QT * QS, 0,
+                 s>>>(m->Lf, C, N, n, m->CT64, m->Np, m->am + AM_C);
+    }
+    split_q_kernel<<<(unsigned)n, 128, 0, s>>>(m->CT64, m->Np, m->am, m->sc, m->CT_m, m->CT_h, m->CT_l);
+    count_launch(2);
+    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
-  absmax_kernel<double><<<blocks_for((long)N * n), 256, 0, s>>>(m->Q64, N, n, n, m->am + AM_C);
-  colnorm2_max_kernel<<<n, 256, 0, s>>>(m->Q64, N, n, m->am + AM_QCN);
-  scales_kernel<<<1, 32, 0, s>>>(m->am, m->sc, 0);
-  count_launch(3);
-  e = transpose<double>(m->Q64, N, n, n, m->CT64, m->Np, s);  // Q^T [j][mu], zero for mu >= N
-  if (e == cudaSuccess)
-    e = split_rows<double>(m->CT64, n, m->Np, m->Np, m->sc, SC_C, m->CT_m, m->CT_h, m->Np, s, m->CT_l);
-  if (e != cudaSuccess) return e;
   if (!m->large) {  // Psi = Phi' Q (three pieces each), written directly as per-row pieces
     GemmArgs g{(int)ng, n, N, (int)m->Np, nullptr, 0, 0, m->sc, SC_OUT_ORB, m->status,
                m->psi_m, m->psi_h, np, SC_PSI, m->am + AM_RN2};
@@ -3339,14 +3586,13 @@ cudaError_t mixed_enqueue_pre(MixedState* m, const double* C, cudaStream_t s, co
                                                   m->psi_h, m->psi_l, np, m->am + AM_RN2);
     count_launch();
   }
-  scales_kernel<<<1, 32, 0, s>>>(m->am, m->sc, 1);
-  const long nat = m->NaT;  // the orbitals at every interpolation point (psig is the slice's view)
-  gather_rows_half_kernel<<<blocks_for(nat * np), 256, 0, s>>>(m->psi_m, np, m->idx, (int)nat, m->psigA_m);
-  gather_rows_half_kernel<<<blocks_for(nat * np), 256, 0, s>>>(m->psi_h, np, m->idx, (int)nat, m->psigA_h);
-  count_launch(4);
-  if (m->psi_l) {
-    gather_rows_half_kernel<<<blocks_for(nat * np), 256, 0, s>>>(m->psi_l, np, m->idx, (int)nat, m->psigA_l);
-    count_launch();
+  {  // the orbitals at every interpolation point (psig is the slice's view)
+    const long nat = m->NaT;
+    const int npc = m->large ? 3 : 2, v16 = np / 8;
+    gather_pieces_kernel<<<blocks_for(npc * nat * v16), 256, 0, s>>>(
+        reinterpret_cast<const uint4*>(m->psi_m), ng * v16, m->idx, nat, v16, npc,
+        reinterpret_cast<uint4*>(m->psigA_m), nat * v16, m->am, m->sc, m->rowmax, n);
+    count_launch(2);  // and the orbital product
   }
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
@@ -3483,7 +3729,7 @@ cudaError_t mixed_enqueue_full(MixedState* m, const double* C, double* Kf, cudaS
                                                       m->am + AM_FA);
   reduce_parts_kernel<<<blocks_for(cnt), 256, 0, s>>>(m->MpA, m->splitsF, m->MpC, m->splitsFC, cnt,
                                                       m->DD, m->am + AM_FD);
-  scales_kernel<<<1, 32, 0, s>>>(m->am, m->sc, 3);
+  scales_full_kernel<<<1, 32, 0, s>>>(m->am, m->sc);
   count_launch(3);
   e = transpose<double>(m->DA, na, N, N, m->DAT64, m->Na8, s);
   if (e == cudaSuccess) e = transpose<double>(m->DD, na, N, N, m->DDT64, m->Na8, s);
@@ -3525,7 +3771,8 @@ cudaError_t mixed_enqueue_energy(MixedState* m, const double* C, double* Ex, cud
   if (e != cudaSuccess) return e;
   hook(1, 0);
   hook(7, 1);
-  final_ex_kernel<<<1, 1024, 0, s>>>(m->EpA, (int)m->epA, m->EpC, (int)m->epC, m->sc, m->dV, Ex);
+  final_ex_kernel<<<2 * kExBlocks, 256, 0, s>>>(m->EpA, (int)m->epA, m->EpC, (int)m->epC, m->sc, m->dV,
+                                                m->part, m->am + CNT_K, Ex);
   count_launch();
   e = cudaGetLastError();
   hook(7, 0);
@@ -3650,75 +3897,63 @@ cudaError_t mixed_enqueue_pair(MixedState* m, cudaStream_t s, const StepHook& ho
   return cudaSuccess;
 }
 
-cudaError_t mixed_enqueue_post(MixedState* m, double* K, double* Ex, cudaStream_t s,
-                               const StepHook& hook) {
+cudaError_t mixed_enqueue_post(MixedState* m, const double* C, double* K, double* Ex, double* EK,
+                               cudaStream_t s, const StepHook& hook) {
   const long ng = m->Ng, na = m->Naux;
   const int N = m->N, n = m->n;
   cudaError_t e;
   // ---- step 4: line1^T = Phi^T M1^T and (line2 - line3)^T = Phi_g^T (M2 - M3)
   hook(4, 1);
-  // the fused role's M2 copies hold accumulator units: scaled here (exact, 2^k)
-  reduce_parts_kernel<<<blocks_for(na * n), 256, 0, s>>>(m->M2p, m->partsA, m->M3p, m->partsC,
-                                                         na * n, m->D23, m->am + AM_D23,
-                                                         m->fused ? m->sc + SC_OUT_AB : nullptr);
-  e = cudaMemsetAsync(m->rowmax, 0, (size_t)n * 4, s);
-  if (e != cudaSuccess) return e;
   {
-    const unsigned chunks = (unsigned)std::min<long>(16, (ng + 1023) / 1024);
-    rowmax2d_kernel<<<dim3(chunks, n), 256, 0, s>>>(m->M1, ng, m->Ng4, m->rowmax, m->am + AM_M1);
-    scales_kernel<<<1, 32, 0, s>>>(m->am, m->sc, 2);
-    const unsigned schunks = (unsigned)std::min<long>(64, (m->Ng8 / 8 + 255) / 256);
-    split_mh_rows_pre_kernel<<<dim3(schunks, n), 256, 0, s>>>(
-        m->M1, ng, m->Ng4, m->rowmax, m->sc, SC_M1, m->M1_m, m->M1_h, m->Ng8);
-  }
-  count_launch(4);
-  e = transpose<double>(m->D23, na, n, n, m->D23T64, m->Na8, s);
-  if (e == cudaSuccess) e = split_rows<double>(m->D23T64, n, m->Na8, m->Na8, m->sc, SC_D23, m->D23T_m, m->D23T_h, m->Na8, s);
-  if (e != cudaSuccess) return e;
-  {
-    GemmArgs g{N, n, (int)ng, m->kchunkL1, m->L1p, n, (long)N * n, m->sc, SC_OUT_L1, m->status,
-               nullptr, nullptr, 0, 0, nullptr};
-    if (m->large)
-      launch_gemm_wide(m->m_phiT_m, m->m_phiT_h, m->m_M1_m, m->m_M1_h, g,
-                       dim3((unsigned)((N + 127) / 128), (unsigned)((n + 255) / 256), (unsigned)m->splitsL1),
-                       s, m->wait_cycles);
-    else
-      launch_gemm(m->m_phiT_m, m->m_phiT_h, m->m_M1_m, m->m_M1_h, m->m_phiT_m, m->m_M1_m, g,
-                  dim3((unsigned)((N + 127) / 128), (unsigned)((n + 127) / 128), (unsigned)m->splitsL1), s, m->wait_cycles);
+    // the fused role's M2 copies hold accumulator units: scaled here (exact, 2^k)
+    const int per = m->partsA + m->partsC <= kFewParts ? 32 * RS : 32;
+    const int nd = (int)((na * n + per - 1) / per);
+    const int chunks = (int)std::min<long>(16, (ng + 1023) / 1024);
+    lines_sum_kernel<<<(unsigned)(nd + chunks * n), 32 * RS, 0, s>>>(
+        m->M2p, m->partsA, m->M3p, m->partsC, na, n, m->fused ? m->sc + SC_OUT_AB : nullptr, m->D23T64,
+        m->Na8, nd, m->M1, ng, m->Ng4, chunks, m->rowmax, m->am);
+    const int n1 = (int)std::min<long>(64, (m->Ng8 / 8 + 255) / 256);
+    lines_split_kernel<<<(unsigned)((n1 + 1) * n), 256, 0, s>>>(
+        m->M1, ng, m->Ng4, m->rowmax, m->M1_m, m->M1_h, m->Ng8, n1, n, m->D23T64, m->Na8, m->D23T_m,
+        m->D23T_h, m->am, m->sc);
+    count_launch(2);
   }
   {
-    GemmArgs g{N, n, (int)na, m->kchunkL23, m->L23p, n, (long)N * n, m->sc, SC_OUT_L23, m->status,
-               nullptr, nullptr, 0, 0, nullptr};
-    if (m->large)
-      launch_gemm_wide(m->m_phigT_m, m->m_phigT_h, m->m_D23T_m, m->m_D23T_h, g,
-                       dim3((unsigned)((N + 127) / 128), (unsigned)((n + 255) / 256), (unsigned)m->splitsL23),
-                       s, m->wait_cycles);
-    else
-      launch_gemm(m->m_phigT_m, m->m_phigT_h, m->m_D23T_m, m->m_D23T_h, m->m_phigT_m, m->m_D23T_m, g,
-                  dim3((unsigned)((N + 127) / 128), (unsigned)((n + 127) / 128), (unsigned)m->splitsL23), s, m->wait_cycles);
+    GemmPair p{};
+    p.g[0] = GemmArgs{N, n, (int)ng, m->kchunkL1, m->L1p, n, (long)N * n, m->sc, SC_OUT_L1, m->status,
+                      nullptr, nullptr, 0, 0, nullptr};
+    p.g[1] = GemmArgs{N, n, (int)na, m->kchunkL23, m->L23p, n, (long)N * n, m->sc, SC_OUT_L23, m->status,
+                      nullptr, nullptr, 0, 0, nullptr};
+    p.am[0] = m->m_phiT_m; p.ah[0] = m->m_phiT_h; p.bm[0] = m->m_M1_m; p.bh[0] = m->m_M1_h;
+    p.am[1] = m->m_phigT_m; p.ah[1] = m->m_phigT_h; p.bm[1] = m->m_D23T_m; p.bh[1] = m->m_D23T_h;
+    const unsigned tx = (unsigned)((N + 127) / 128),
+                   ty = (unsigned)(m->large ? (n + 255) / 256 : (n + 127) / 128);
+    const dim3 tiles[2] = {dim3(tx, ty, (unsigned)m->splitsL1), dim3(tx, ty, (unsigned)m->splitsL23)};
+    launch_gemm_pair(p, tiles, m->large, s, m->wait_cycles);
   }
-  count_launch(2);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   hook(4, 0);
 
   // ---- step 5: K_{mu i} and E_x in FP64
   hook(7, 1);
-  final_k_kernel<<<blocks_for((long)N * n), 256, 0, s>>>(m->L1p, m->splitsL1, m->L23p,
-                                                         m->splitsL23, (long)N * n, m->dV, K);
-  final_ex_kernel<<<1, 1024, 0, s>>>(m->EpA, (int)m->epA, m->EpC, (int)m->epC, m->sc, m->dV, Ex);
-  count_launch(2);
+  const long count = (long)N * n;
+  const unsigned nk = (unsigned)((count + 31) / 32);  // each leaves a sum behind the 2 kExBlocks
+  final_kernel<<<2 * kExBlocks + nk, 32 * RS, 0, s>>>(
+      m->L1p, m->splitsL1, m->L23p, m->splitsL23, count, m->dV, K, C, m->EpA, (int)m->epA, m->EpC,
+      (int)m->epC, m->sc, m->part, m->am + CNT_K, Ex, EK);
+  count_launch();
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   hook(7, 0);
   return cudaSuccess;
 }
 
-cudaError_t mixed_enqueue(MixedState* m, const double* C, double* K, double* Ex, cudaStream_t s,
-                          const StepHook& hook) {
+cudaError_t mixed_enqueue(MixedState* m, const double* C, double* K, double* Ex, double* EK,
+                          cudaStream_t s, const StepHook& hook) {
   cudaError_t e = mixed_enqueue_pre(m, C, s, hook);
   if (e == cudaSuccess) e = mixed_enqueue_pair(m, s, hook);
-  if (e == cudaSuccess) e = mixed_enqueue_post(m, K, Ex, s, hook);
+  if (e == cudaSuccess) e = mixed_enqueue_post(m, C, K, Ex, EK, s, hook);
   return e;
 }
 

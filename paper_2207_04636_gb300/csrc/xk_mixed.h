@@ -35,17 +35,18 @@ cudaError_t mixed_create(int64_t Ng, int N, int n, int NaT, int g0, int g1, cons
                          cudaStream_t s, MixedState** out);
 void mixed_destroy(MixedState* m);
 
-// Enqueue one build: C_dev (N x n FP64) -> K_dev (N x n FP64), Ex_dev.
+// Enqueue one build: C_dev (N x n FP64) -> K_dev (N x n FP64), Ex_dev and, when
+// EK_dev is given, the energy of that K, -sum K o C.
 cudaError_t mixed_enqueue(MixedState* m, const double* C_dev, double* K_dev, double* Ex_dev,
-                          cudaStream_t s, const StepHook& hook);
+                          double* EK_dev, cudaStream_t s, const StepHook& hook);
 
 // The same build in three parts: orbitals (step 1), the pair contractions
 // (steps 2-3), and the line contractions with K and E_x (steps 4-5).
 cudaError_t mixed_enqueue_pre(MixedState* m, const double* C_dev, cudaStream_t s,
                               const StepHook& hook);
 cudaError_t mixed_enqueue_pair(MixedState* m, cudaStream_t s, const StepHook& hook);
-cudaError_t mixed_enqueue_post(MixedState* m, double* K_dev, double* Ex_dev, cudaStream_t s,
-                               const StepHook& hook);
+cudaError_t mixed_enqueue_post(MixedState* m, const double* C_dev, double* K_dev, double* Ex_dev,
+                               double* EK_dev, cudaStream_t s, const StepHook& hook);
 
 // E_x alone (no K): the orbitals, then the pair products S with the sums
 // sum V' o S^2 and sum W' o S^2 only (no second product, no line
