@@ -1180,19 +1180,28 @@ int xk_ace(xk_handle* h, double* Kij_out, double* xi_out, double* sign_out, int*
   DeviceGuard g(h->device);
   cudaStream_t s = h->stream;
   const int N = h->N, n = h->n;
-  xk::DGemm kij{n, n, N, h->C, n, true, h->K, n, false, h->Kij, n, 1.0, nullptr, 0, 0, h->work};
-  XK_CUDA(xk::dgemm(kij, s));
-  XK_CUDA(xk::symmetrize_f64(h->Kij, n, s));
-  XK_CUDA(cudaMemcpyAsync(h->Lf, h->Kij, (size_t)n * n * 8, cudaMemcpyDeviceToDevice, s));
-  XK_CUDA(xk::cholesky_f64(h->Lf, n, h->status, s));
-  int st = 0;
-  XK_CUDA(cudaMemcpyAsync(&st, h->status, 4, cudaMemcpyDeviceToHost, s));
-  XK_CUDA(cudaStreamSynchronize(s));
-  int br = 0;
+  int st = 0, br = 0;
   std::vector<double> sg(n, 1.0);
-  if (st == 0) {
-    XK_CUDA(xk::trsm_right_lt_f64(h->Lf, n, h->K, N, h->xi, s));
+  // K_ij: from 2e7 multiply-adds the digit product (then symmetrised), below the
+  // kernel that spreads it over the SMs
+  xk::DGemm kij{n, n, N, h->C, n, true, h->K, n, false, h->Kij, n, 1.0, nullptr, 0, 0, h->work};
+  kij.scale = digit_scratch(h->xi, (size_t)N * n, n, n);
+  if (xk::digit_gemm_wanted(kij)) {
+    XK_CUDA(xk::dgemm(kij, s));
+    XK_CUDA(xk::symmetrize_f64(h->Kij, n, s));
   } else {
+    XK_CUDA(xk::kij_f64(h->C, h->K, N, n, h->Kij, s));
+  }
+  XK_CUDA(cudaMemcpyAsync(h->Lf, h->Kij, (size_t)n * n * 8, cudaMemcpyDeviceToDevice, s));
+  XK_CUDA(xk::cholesky_tiled_f64(h->Lf, n, h->status, s));
+  // the Cholesky branch's vectors are formed and copied before the host has seen
+  // whether it holds: one wait instead of two
+  XK_CUDA(xk::trsm_right_lt_f64(h->Lf, n, h->K, N, h->xi, s, h->U));
+  XK_CUDA(cudaMemcpyAsync(&st, h->status, 4, cudaMemcpyDeviceToHost, s));
+  XK_CUDA(cudaMemcpyAsync(Kij_out, h->Kij, (size_t)n * n * 8, cudaMemcpyDeviceToHost, s));
+  XK_CUDA(cudaMemcpyAsync(xi_out, h->xi, (size_t)N * n * 8, cudaMemcpyDeviceToHost, s));
+  XK_CUDA(cudaStreamSynchronize(s));
+  if (st != 0) {
     br = 1;
     XK_CUDA(cudaMemcpyAsync(h->Lf, h->Kij, (size_t)n * n * 8, cudaMemcpyDeviceToDevice, s));
     XK_CUDA(xk::jacobi_eig_f64(h->Lf, h->U, n, 60, h->status + 1, s));
@@ -1200,10 +1209,9 @@ int xk_ace(xk_handle* h, double* Kij_out, double* xi_out, double* sign_out, int*
     XK_CUDA(xk::dgemm(ku, s));
     XK_CUDA(xk::scale_eigcols_f64(h->Lf, n, h->Y, N, 1e-12, h->xi, h->sgn, s));
     XK_CUDA(cudaMemcpyAsync(sg.data(), h->sgn, (size_t)n * 8, cudaMemcpyDeviceToHost, s));
+    XK_CUDA(cudaMemcpyAsync(xi_out, h->xi, (size_t)N * n * 8, cudaMemcpyDeviceToHost, s));
+    XK_CUDA(cudaStreamSynchronize(s));
   }
-  XK_CUDA(cudaMemcpyAsync(Kij_out, h->Kij, (size_t)n * n * 8, cudaMemcpyDeviceToHost, s));
-  XK_CUDA(cudaMemcpyAsync(xi_out, h->xi, (size_t)N * n * 8, cudaMemcpyDeviceToHost, s));
-  XK_CUDA(cudaStreamSynchronize(s));
   if (sign_out) std::memcpy(sign_out, sg.data(), (size_t)n * 8);
   if (branch) *branch = br;
   return XK_OK;

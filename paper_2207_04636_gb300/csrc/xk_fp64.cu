@@ -522,6 +522,212 @@ cudaError_t symmetrize_f64(double* A, int n, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+// Small products and factorisations (the occ-RI K_ij, the blocks of the ISDF
+// Cholesky).  One SM forms 2 FP64 multiply-adds a clock, so even these want many
+// SMs: tiles are kept at a few thousand multiply-adds.
+
+// Kij[i][j] = sum_mu (C[mu][i] K[mu][j] + C[mu][j] K[mu][i]) / 2.  A block forms the
+// 4 x 4 outputs of one tile pair on or above the diagonal, 16 threads to an output's mu
+// (8 x 8 tiles put the whole product on 28 SMs at n = 54: 27 us).  The tiled product (five
+// blocks of 64 x 64), its split sum and the symmetrisation took 97 us.
+constexpr int KT = 4, KS = 16;
+__global__ void __launch_bounds__(KT * KT * KS) kij_kernel(const double* __restrict__ C,
+                                                          const double* __restrict__ K, int N, int n,
+                                                          double* __restrict__ Kij) {
+  __shared__ double part[KS][KT * KT];
+  if (blockIdx.x > blockIdx.y) return;
+  const int o = threadIdx.x % (KT * KT), sl = threadIdx.x / (KT * KT);
+  const int i = blockIdx.x * KT + o / KT, j = blockIdx.y * KT + o % KT;
+  double u = 0.0, v = 0.0;
+  if (i < n && j < n) {
+#pragma unroll 4
+    for (long mu = sl; mu < N; mu += KS) {
+      const double *c = C + mu * n, *k = K + mu * n;
+      u = fma(c[i], k[j], u);
+      v = fma(c[j], k[i], v);
+    }
+  }
+  part[sl][o] = u + v;
+  __syncthreads();
+  if (sl != 0 || i >= n || j >= n) return;
+  double s = part[0][o];
+  for (int w = 1; w < KS; ++w) s += part[w][o];
+  Kij[(long)i * n + j] = Kij[(long)j * n + i] = 0.5 * s;
+}
+
+cudaError_t kij_f64(const double* C, const double* K, int N, int n, double* Kij, cudaStream_t s) {
+  const unsigned t = (unsigned)((n + KT - 1) / KT);
+  kij_kernel<<<dim3(t, t), KT * KT * KS, 0, s>>>(C, K, N, n, Kij);
+  count_launch();
+  return cudaGetLastError();
+}
+
+// 1 / d by Newton's iteration from the hardware's approximation (about 20 bits): every
+// FP64 instruction of a warp takes the SM's FP64 pipe for 16 cycles, a division some 30.
+__device__ __forceinline__ double fast_recip(double d) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
+  r = fma(r, fma(-d, r, 1.0), r);
+  r = fma(r, fma(-d, r, 1.0), r);
+  return fma(r, fma(-d, r, 1.0), r);
+}
+
+// In-place Cholesky factor L (lower) of the kb x kb block at (k, k) of A by one block of
+// 256 threads, the triangle in registers: thread t owns the elements e = t, t + 256, ... of
+// an enumeration in which the trailing triangles of all columns are prefixes, so no lane
+// idles.  Column c: its owners publish it (unscaled), two warps divide it by the pivot, then
+// a[i][j] -= a[i][c] (a[j][c] / a[c][c]); the scaling follows at the end.  *status gets the column (from 1) of the first pivot that is not positive; that pivot
+// counts as 1.  The matrix in global memory, two barriers, a square root and a division in
+// sequence took 87 us at kb = 54, this 65 us: the chain of dependent FP64 instructions per
+// column (about 10) bounds it now.
+constexpr int CB = 64;
+constexpr int CE = (CB * (CB + 1) / 2 + 255) / 256;  // elements a thread
+__global__ void __launch_bounds__(256) chol_block_kernel(double* __restrict__ A, long lda, int k, int kb,
+                                                        int* __restrict__ status) {
+  __shared__ double col[CB], fcol[CB], rs[CB];
+  __shared__ int bad;
+  const int tid = threadIdx.x;
+  double* D = A + (long)k * lda + k;
+  const int total = kb * (kb + 1) / 2;
+  double v[CE];
+  int ei[CE], ej[CE];
+#pragma unroll
+  for (int q = 0; q < CE; ++q) {
+    // e = j'(j'+1)/2 + i', 0 <= i' <= j', counted from the last row and column
+    const int e = tid + 256 * q;
+    int jp = (int)((sqrtf(8.0f * e + 1.0f) - 1.0f) * 0.5f);
+    while (jp * (jp + 1) / 2 > e) --jp;
+    while ((jp + 1) * (jp + 2) / 2 <= e) ++jp;
+    ej[q] = kb - 1 - jp;
+    ei[q] = kb - 1 - (e - jp * (jp + 1) / 2);
+    v[q] = e < total ? D[(long)ei[q] * lda + ej[q]] : 0.0;
+  }
+  if (tid == 0) bad = 0;
+  __syncthreads();
+  for (int c = 0; c < kb; ++c) {
+    const int m = kb - c, live = m * (m + 1) / 2, next = (m - 1) * m / 2;  // e in [next, live): column c
+#pragma unroll
+    for (int q = 0; q < CE; ++q) {
+      const int e = tid + 256 * q;
+      if (e < live && e >= next) col[ei[q]] = v[q];
+    }
+    __syncthreads();
+    if (tid < CB && tid >= c && tid < kb) {
+      double d = col[c];
+      const long long bits = __double_as_longlong(d);  // d > 0, by integers
+      if (bits <= 0 || bits > 0x7ff0000000000000LL) {
+        d = 1.0;
+        if (tid == c && !bad) bad = c + 1;
+      }
+      if (tid == c) rs[c] = d;
+      double f = col[tid];
+      if (__double2hiint(d) < ((1023 - 1000) << 20)) {  // a reciprocal that would overflow
+        d *= 0x1p200;
+        f *= 0x1p200;
+      }
+      fcol[tid] = f * fast_recip(d);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < CE; ++q)
+      if (tid + 256 * q < next) v[q] = fma(-col[ei[q]], fcol[ej[q]], v[q]);
+    __syncthreads();
+  }
+  __syncthreads();
+  if (tid < kb) rs[tid] = 1.0 / sqrt(rs[tid]);
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < CE; ++q)
+    if (tid + 256 * q < total) D[(long)ei[q] * lda + ej[q]] = v[q] * rs[ej[q]];
+  if (tid == 0 && bad) atomicCAS(status, 0, k + bad);
+}
+
+// Panel below a factored diagonal block: rows r >= k + kb of A[:, k:k+kb] := row
+// L11^{-T}, one warp per row: the row in registers (two columns a lane), L11's
+// columns from shared memory; each step broadcasts one finished entry.
+__global__ void __launch_bounds__(256) chol_panel_kernel(double* __restrict__ A, long lda, int k, int kb,
+                                                        int n) {
+  __shared__ double lt[CB][CB];  // lt[c][j] = L11[j][c]
+  __shared__ double inv[CB];
+  const double* D = A + (long)k * lda + k;
+  for (int t = threadIdx.x; t < kb * CB; t += 256) {
+    const int c = t / CB, j = t % CB;
+    lt[c][j] = j < kb && j >= c ? D[(long)j * lda + c] : 0.0;
+    if (j == 0) inv[c] = 1.0 / D[(long)c * lda + c];
+  }
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  const long r = k + kb + (long)blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (r >= n) return;
+  double* row = A + r * lda + k;
+  double x0 = lane < kb ? row[lane] : 0.0, x1 = lane + 32 < kb ? row[lane + 32] : 0.0;
+  for (int c = 0; c < kb; ++c) {
+    const double b = __shfl_sync(0xffffffffu, c < 32 ? x0 : x1, c & 31) * inv[c];
+    const double* l = lt[c];
+    if (lane == (c & 31)) {
+      if (c < 32) x0 = b; else x1 = b;
+    }
+    if (lane > c) x0 = fma(-b, l[lane], x0);
+    if (lane + 32 > c) x1 = fma(-b, l[lane + 32], x1);
+  }
+  if (lane < kb) row[lane] = x0;
+  if (lane + 32 < kb) row[lane + 32] = x1;
+}
+
+// A[i][j] -= sum_c P[i][c] P[j][c] for i >= j >= k + kb, P the panel A[:, k:k+kb]: 16 x 16 tiles.
+__global__ void __launch_bounds__(256) chol_update_kernel(double* __restrict__ A, long lda, int k, int kb,
+                                                         int n) {
+  __shared__ double pi[16][CB + 1], pj[16][CB + 1];
+  if (blockIdx.x > blockIdx.y) return;
+  const long i0 = k + kb + (long)blockIdx.y * 16, j0 = k + kb + (long)blockIdx.x * 16;
+  for (int t = threadIdx.x; t < 16 * kb; t += 256) {
+    const int r = t / kb, c = t % kb;
+    pi[r][c] = i0 + r < n ? A[(i0 + r) * lda + k + c] : 0.0;
+    pj[r][c] = j0 + r < n ? A[(j0 + r) * lda + k + c] : 0.0;
+  }
+  __syncthreads();
+  const int ti = threadIdx.x >> 4, tj = threadIdx.x & 15;
+  double s = 0.0;
+  for (int c = 0; c < kb; ++c) s = fma(pi[ti][c], pj[tj][c], s);
+  const long i = i0 + ti, j = j0 + tj;
+  if (i < n && j <= i) A[i * lda + j] -= s;
+}
+
+cudaError_t cholesky_step_f64(double* A, long lda, int k, int kb, int n, int* status, cudaStream_t s) {
+  const int rest = n - k - kb;
+  chol_block_kernel<<<1, 256, 0, s>>>(A, lda, k, kb, status);
+  if (rest > 0) chol_panel_kernel<<<(unsigned)((rest + 7) / 8), 256, 0, s>>>(A, lda, k, kb, n);
+  count_launch(rest > 0 ? 2 : 1);
+  return cudaGetLastError();
+}
+
+// Zeroes the upper triangle.
+__global__ void lower_kernel(double* A, int n) {
+  for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < (long)n * n;
+       t += (long)gridDim.x * blockDim.x)
+    if (t % n > t / n) A[t] = 0.0;
+}
+
+cudaError_t cholesky_tiled_f64(double* A, int n, int* status, cudaStream_t s) {
+  cudaError_t e = cudaMemsetAsync(status, 0, 4, s);
+  if (e != cudaSuccess) return e;
+  for (int k = 0; k < n; k += CB) {
+    const int kb = std::min(CB, n - k), rest = n - k - kb;
+    e = cholesky_step_f64(A, n, k, kb, n, status, s);
+    if (e != cudaSuccess) return e;
+    if (rest <= 0) break;
+    const unsigned t = (unsigned)((rest + 15) / 16);
+    chol_update_kernel<<<dim3(t, t), 256, 0, s>>>(A, n, k, kb, n);
+    count_launch();
+  }
+  lower_kernel<<<blocks_of((long)n * n), 256, 0, s>>>(A, n);
+  count_launch();
+  return cudaGetLastError();
+}
+
+// Cholesky in one block, for the tensor path's set-up only: its Phi' = Phi L^{-T} is
+// rounded to FP16 pieces, whose last bits follow those of L and would move the K of a
+// geometry by about 1e-9 (relative), so its order of operations is kept.
 __global__ void cholesky_kernel(double* A, int n, int* status) {
   __shared__ int fail;
   if (threadIdx.x == 0) fail = 0;
@@ -571,10 +777,71 @@ __global__ void trsm_kernel(const double* __restrict__ L, int n, const double* _
   }
 }
 
+// X L^T = B, one warp per row for n <= 32 Q: the row in registers (Q columns a
+// lane); step c broadcasts x[c] = b[c] / L[c][c] and subtracts its multiple of column c of
+// L (lanes along the column: LT is L transposed, with the reciprocals of its diagonal: a
+// division a step would be most of the FP64 work) from the entries that follow.
+template <int Q>
+__global__ void __launch_bounds__(64) trsm_warp_kernel(const double* __restrict__ LT, int n,
+                                                       const double* __restrict__ B, int rows,
+                                                       double* __restrict__ X) {
+  const int lane = threadIdx.x & 31;
+  const long r = (long)blockIdx.x * 2 + (threadIdx.x >> 5);
+  if (r >= rows) return;
+  double x[Q];
+#pragma unroll
+  for (int q = 0; q < Q; ++q) x[q] = 32 * q + lane < n ? B[r * n + 32 * q + lane] : 0.0;
+#pragma unroll
+  for (int p = 0; p < Q; ++p) {
+    const int c1 = min(32, n - 32 * p);
+#pragma unroll 4
+    for (int c = 0; c < c1; ++c) {
+      const double* l = LT + (long)(32 * p + c) * n + lane;
+      double f[Q];
+#pragma unroll
+      for (int q = p; q < Q; ++q) f[q] = 32 * q + lane < n ? __ldg(l + 32 * q) : 0.0;
+      const double b = __shfl_sync(0xffffffffu, x[p], c) * __shfl_sync(0xffffffffu, f[p], c);
+      // row 32 p + c of LT is zero before its diagonal
+      x[p] = lane == c ? b : lane > c ? fma(-b, f[p], x[p]) : x[p];
+#pragma unroll
+      for (int q = p + 1; q < Q; ++q) x[q] = fma(-b, f[q], x[q]);
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < Q; ++q)
+    if (32 * q + lane < n) X[r * n + 32 * q + lane] = x[q];
+}
+
+// T = A^T with the reciprocals of the diagonal.
+__global__ void transpose_recip_kernel(const double* __restrict__ A, int n, double* __restrict__ T) {
+  __shared__ double tile[32][33];
+  const int r0 = blockIdx.x * 32, c0 = blockIdx.y * 32;
+  for (int i = threadIdx.y; i < 32; i += 8)
+    if (r0 + i < n && c0 + (int)threadIdx.x < n) tile[i][threadIdx.x] = A[(long)(r0 + i) * n + c0 + threadIdx.x];
+  __syncthreads();
+  for (int i = threadIdx.y; i < 32; i += 8)
+    if (c0 + i < n && r0 + (int)threadIdx.x < n) {
+      double v = tile[threadIdx.x][i];
+      if (c0 + i == r0 + (int)threadIdx.x) v = 1.0 / v;
+      T[(long)(c0 + i) * n + r0 + threadIdx.x] = v;
+    }
+}
+
 cudaError_t trsm_right_lt_f64(const double* L, int n, const double* B, int rows, double* X,
-                              cudaStream_t s) {
-  trsm_kernel<<<(rows + 127) / 128, 128, 0, s>>>(L, n, B, rows, X);
-  count_launch();
+                              cudaStream_t s, double* LT) {
+  if (!LT || n > 512) {
+    trsm_kernel<<<(rows + 127) / 128, 128, 0, s>>>(L, n, B, rows, X);
+    count_launch();
+    return cudaGetLastError();
+  }
+  const unsigned t = (unsigned)((n + 31) / 32);
+  transpose_recip_kernel<<<dim3(t, t), dim3(32, 8), 0, s>>>(L, n, LT);
+  const unsigned blocks = (unsigned)((rows + 1) / 2);
+  if (n <= 64) trsm_warp_kernel<2><<<blocks, 64, 0, s>>>(LT, n, B, rows, X);
+  else if (n <= 128) trsm_warp_kernel<4><<<blocks, 64, 0, s>>>(LT, n, B, rows, X);
+  else if (n <= 256) trsm_warp_kernel<8><<<blocks, 64, 0, s>>>(LT, n, B, rows, X);
+  else trsm_warp_kernel<16><<<blocks, 64, 0, s>>>(LT, n, B, rows, X);
+  count_launch(2);
   return cudaGetLastError();
 }
 

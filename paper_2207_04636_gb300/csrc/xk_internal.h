@@ -133,14 +133,22 @@ cudaError_t closed_form_ex_f64(const double* V, const double* P, long lenA, cons
 // A <- (A + A^T) / 2 for an n x n matrix.
 cudaError_t symmetrize_f64(double* A, int n, cudaStream_t s);
 
-// In-place Cholesky A = L L^T (lower, n x n, one block).  *status = 0 on
-// success, k + 1 if the k-th pivot is not positive.
+// Kij = (C^T K + K^T C) / 2 for C, K of N x n.
+cudaError_t kij_f64(const double* C, const double* K, int N, int n, double* Kij, cudaStream_t s);
+
+// In-place Cholesky A = L L^T (lower, n x n, zeros above).  *status = 0 on
+// success, k + 1 if the k-th pivot is not positive (A then holds no factor).
+// cholesky_f64: one block (the tensor path's set-up).
+cudaError_t cholesky_tiled_f64(double* A, int n, int* status, cudaStream_t s);
 cudaError_t cholesky_f64(double* A, int n, int* status, cudaStream_t s);
+// One step of it, for a blocked factorisation: the kb x kb block at (k, k), kb <= 64,
+// and the panel below it (*status as above, set only on failure).
+cudaError_t cholesky_step_f64(double* A, long lda, int k, int kb, int n, int* status, cudaStream_t s);
 
 // X <- B L^{-T} for L lower n x n and B rows x n (row-major): solves
-// X L^T = B row by row.
+// X L^T = B row by row.  LT: n x n scratch (nullable: the slow general kernel).
 cudaError_t trsm_right_lt_f64(const double* L, int n, const double* B, int rows, double* X,
-                              cudaStream_t s);
+                              cudaStream_t s, double* LT = nullptr);
 
 // Cyclic Jacobi eigendecomposition of the symmetric n x n matrix A (one
 // block): on return A holds the eigenvalues on its diagonal and U the

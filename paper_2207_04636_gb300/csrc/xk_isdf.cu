@@ -43,84 +43,18 @@ __global__ void copy_diag_kernel(const double* __restrict__ a, int n, long ld, d
     out[i] = a[(long)i * ld + i];
 }
 
-// In-place Cholesky (lower) of the kb x kb diagonal block at (k, k); one
-// block of 256 threads, the block held in shared memory.  A non-positive
-// pivot sets *status = 1 (the pivot is replaced by 1 so the loop ends).
-__global__ void potrf_block_kernel(double* __restrict__ A, long lda, int k, int kb,
-                                   int* __restrict__ status) {
-  __shared__ double a[NB][NB + 1];
-  for (int t = threadIdx.x; t < kb * kb; t += blockDim.x) {
-    const int i = t / kb, j = t % kb;
-    a[i][j] = A[(long)(k + i) * lda + k + j];
-  }
-  __syncthreads();
-  for (int j = 0; j < kb; ++j) {
-    if (threadIdx.x == 0) {
-      double d = a[j][j];
-      if (!(d > 0.0)) {
-        atomicExch(status, 1);
-        d = 1.0;
-      }
-      a[j][j] = sqrt(d);
-    }
-    __syncthreads();
-    const double piv = a[j][j];
-    for (int i = j + 1 + threadIdx.x; i < kb; i += blockDim.x) a[i][j] /= piv;
-    __syncthreads();
-    // trailing update of the lower triangle: a[i][l] -= a[i][j] a[l][j], j < l <= i
-    const int m = kb - j - 1;
-    for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
-      const int i = j + 1 + t / m, l = j + 1 + t % m;
-      if (l <= i) a[i][l] -= a[i][j] * a[l][j];
-    }
-    __syncthreads();
-  }
-  for (int t = threadIdx.x; t < kb * kb; t += blockDim.x) {
-    const int i = t / kb, j = t % kb;
-    if (j <= i) A[(long)(k + i) * lda + k + j] = a[i][j];
-  }
-}
-
-// Panel below the diagonal block: row r of A[k+kb:n, k:k+kb] := x with
-// x L11^T = row (forward substitution; one thread per row).
-__global__ void trsm_panel_kernel(double* __restrict__ A, long lda, int k, int kb, int n) {
-  __shared__ double l[NB][NB + 1];
-  for (int t = threadIdx.x; t < kb * kb; t += blockDim.x) {
-    const int i = t / kb, j = t % kb;
-    l[i][j] = j <= i ? A[(long)(k + i) * lda + k + j] : 0.0;
-  }
-  __syncthreads();
-  for (long r = k + kb + blockIdx.x * (long)blockDim.x + threadIdx.x; r < n;
-       r += (long)gridDim.x * blockDim.x) {
-    double* row = A + r * lda + k;
-    double x[NB];
-#pragma unroll
-    for (int j = 0; j < NB; ++j) {
-      if (j < kb) {
-        double v = row[j];
-#pragma unroll
-        for (int p = 0; p < j; ++p) v -= x[p] * l[j][p];
-        x[j] = v / l[j][j];
-        row[j] = x[j];
-      } else {
-        x[j] = 0.0;
-      }
-    }
-  }
-}
-
 // Column c of B[k:k+kb, :] := L_kk^{-1} column (forward, lower = true) or
 // L_kk^{-T} column (backward, lower = false); one thread per column, the
 // block of L in shared memory (identity past kb), the column in registers.
 template <bool LOWER>
 __global__ void trsv_block_kernel(const double* __restrict__ L, long ldl, int k, int kb,
                                   double* __restrict__ B, long ldb, long ncols) {
-  __shared__ double l[NB][NB + 1];
+  __shared__ double l[NB][NB + 1];  // with the diagonal's reciprocals: a division costs 30 FMAs
   for (int t = threadIdx.x; t < NB * NB; t += blockDim.x) {
     const int i = t / NB, j = t % NB;
     double v = (i == j) ? 1.0 : 0.0;
     if (i < kb && j < kb && j <= i) v = L[(long)(k + i) * ldl + k + j];
-    l[i][j] = v;
+    l[i][j] = i == j ? 1.0 / v : v;
   }
   __syncthreads();
   for (long c = blockIdx.x * (long)blockDim.x + threadIdx.x; c < ncols;
@@ -134,7 +68,7 @@ __global__ void trsv_block_kernel(const double* __restrict__ L, long ldl, int k,
         double v = y[j];
 #pragma unroll
         for (int p = 0; p < j; ++p) v -= l[j][p] * y[p];
-        y[j] = v / l[j][j];
+        y[j] = v * l[j][j];
       }
     } else {
 #pragma unroll
@@ -142,7 +76,7 @@ __global__ void trsv_block_kernel(const double* __restrict__ L, long ldl, int k,
         double v = y[j];
 #pragma unroll
         for (int p = j + 1; p < NB; ++p) v -= l[p][j] * y[p];
-        y[j] = v / l[j][j];
+        y[j] = v * l[j][j];
       }
     }
 #pragma unroll
@@ -347,17 +281,15 @@ cudaError_t cholesky_blocked_f64(double* A, int n, long lda, int* status, int* s
                                  cudaStream_t s) {
   for (int k = 0; k < n; k += NB) {
     const int kb = std::min(NB, n - k);
-    potrf_block_kernel<<<1, 256, 0, s>>>(A, lda, k, kb, status);
-    count_launch();
+    cudaError_t e = cholesky_step_f64(A, lda, k, kb, n, status, s);
+    if (e != cudaSuccess) return e;
     if (k + kb < n) {
       const int rest = n - k - kb;
-      trsm_panel_kernel<<<std::max(1, std::min(152 * 4, (rest + 127) / 128)), 128, 0, s>>>(A, lda, k, kb, n);
-      count_launch();
       // A22 -= L21 L21^T (the whole square; only its lower triangle is used)
       DGemm g{rest, rest, kb, A + (long)(k + kb) * lda + k, lda, false,
               A + (long)(k + kb) * lda + k, lda, true, A + (long)(k + kb) * lda + k + kb, lda,
               -1.0, nullptr, 0, 1, nullptr, false, 1.0, scale};
-      cudaError_t e = dgemm(g, s);
+      e = dgemm(g, s);
       if (e != cudaSuccess) return e;
     }
   }

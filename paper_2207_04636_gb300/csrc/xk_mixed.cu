@@ -236,20 +236,20 @@ __global__ void __launch_bounds__(128) split_mh_rows_kernel(
 }
 
 // Q^T[j][mu] = sum_{k >= mu} L[k][mu] C[k][j] in FP64 (the zero triangle of L is
-// stored), zero for N <= mu < ld; max |Q| -> am_slot.  A block forms 8 x 8 outputs,
-// eight threads to an output's k: bound by the FP64 pipe (2 multiply-adds a clock
-// and SM), so the tile is small enough that the longest ones (mu near 0) do not
-// outlast the rest.  8 us at N = 351, n = 54, where the tiled product, its split sum,
-// the transpose and the two maxima took 38 us.
-constexpr int QT = 8, QS = 8;
-__global__ void __launch_bounds__(QT * QT * QS) q_kernel(const double* __restrict__ L,
+// stored), zero for N <= mu < ld; max |Q| -> am_slot.  A block forms 4 x 8 outputs,
+// eight threads to an output's k: bound by the FP64 pipe (2 multiply-adds a clock and
+// SM), so the tile is small enough that the longest ones (mu near 0) do not outlast
+// the rest.  The tiled product, its split sum, the transpose and the two maxima took
+// 38 us at N = 351, n = 54.
+constexpr int QM = 4, QJ = 8, QS = 8;
+__global__ void __launch_bounds__(QM * QJ * QS) q_kernel(const double* __restrict__ L,
                                                         const double* __restrict__ C, int N, int n,
                                                         double* __restrict__ QTr, long ld,
                                                         unsigned* __restrict__ am_slot) {
-  __shared__ double part[QS][QT * QT];
-  const int mu0 = blockIdx.x * QT, j0 = blockIdx.y * QT;
-  const int o = threadIdx.x % (QT * QT), sl = threadIdx.x / (QT * QT);
-  const int mu = mu0 + o / QT, j = j0 + o % QT;
+  __shared__ double part[QS][QM * QJ];
+  const int mu0 = blockIdx.x * QM, j0 = blockIdx.y * QJ;
+  const int o = threadIdx.x % (QM * QJ), sl = threadIdx.x / (QM * QJ);
+  const int mu = mu0 + o / QJ, j = j0 + o % QJ;
   double s = 0.0;
   if (mu < N && j < n) {
 #pragma unroll 8
@@ -257,15 +257,15 @@ __global__ void __launch_bounds__(QT * QT * QS) q_kernel(const double* __restric
   }
   part[sl][o] = s;
   __syncthreads();
-  if (threadIdx.x >= QT * QT) return;
+  if (threadIdx.x >= QM * QJ) return;
   // this thread now takes (mu, j) with mu fastest, for the store
-  const int a = threadIdx.x / QT, b = threadIdx.x % QT;
+  const int a = threadIdx.x / QM, b = threadIdx.x % QM;
   s = 0.0;
-  for (int w = 0; w < QS; ++w) s += part[w][b * QT + a];
+  for (int w = 0; w < QS; ++w) s += part[w][b * QJ + a];
   if (j0 + a < n && mu0 + b < ld) QTr[(long)(j0 + a) * ld + mu0 + b] = s;
   float m = j0 + a < n ? fabsf((float)s) : 0.0f;
   for (int w = 16; w > 0; w >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, w));
-  if ((threadIdx.x & 31) == 0) atomicMax(am_slot, __float_as_uint(m));
+  if (threadIdx.x == 0) atomicMax(am_slot, __float_as_uint(m));
 }
 
 // The pieces of Q^T, a block of 128 threads per row, with max_j sum_mu Q^2; the
@@ -3559,7 +3559,7 @@ cudaError_t mixed_enqueue_pre(MixedState* m, const double* C, cudaStream_t s, co
       if (e != cudaSuccess) return e;
       absmax_kernel<double><<<blocks_for((long)N * n), 256, 0, s>>>(m->CT64, n, N, m->Np, m->am + AM_C);
     } else {
-      q_kernel<<<dim3((unsigned)((m->Np + QT - 1) / QT), (unsigned)((n + QT - 1) / QT)), QT * QT * QS, 0,
+      q_kernel<<<dim3((unsigned)((m->Np + QM - 1) / QM), (unsigned)((n + QJ - 1) / QJ)), QM * QJ * QS, 0,
                  s>>>(m->Lf, C, N, n, m->CT64, m->Np, m->am + AM_C);
     }
     split_q_kernel<<<(unsigned)n, 128, 0, s>>>(m->CT64, m->Np, m->am, m->sc, m->CT_m, m->CT_h, m->CT_l);

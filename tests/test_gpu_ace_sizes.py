@@ -1,0 +1,34 @@
+"""xk_ace's K_ij, Cholesky and vectors over its block sizes (64-column blocks,
+32-wide row registers, the 512-column limit), against NumPy on the same K and C."""
+import numpy as np
+import pytest
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n", [1, 31, 33, 64, 65, 128, 130, 257, 513])
+def test_sizes(n):
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2207_04636_gb300 as xk
+    N, Ng = n + 5, 1200
+    rng = np.random.default_rng(n)
+    phi = rng.standard_normal((Ng, N)) / np.sqrt(Ng)
+    C = np.linalg.qr(rng.standard_normal((N, n)))[0]
+    # every grid point an interpolation point, a positive diagonal V and no W: K_ij is
+    # 2 sum_R V(R, R) rho(R) psi_i(R) psi_j(R), positive definite
+    idx = np.arange(Ng)
+    V, W = np.diag(rng.uniform(5.0, 15.0, Ng)), np.zeros((Ng, Ng))
+    h = xk.Handle(phi, idx, V, W, 1.0, n, mode="fp64")
+    K, _ = h.build(C)
+    Kij, xi, sg, br = h.ace()
+    h.release()
+    Kij0, xi0, s0, br0 = oracle.ace_factor(K, C)
+    assert br == br0 == "cholesky" and np.array_equal(sg, np.ones(n))
+    # N-term FP64 sums
+    assert np.abs(Kij - Kij0).max() <= 4 * N * 2.0 ** -53 * (np.abs(C).T @ np.abs(K)).max()
+    # xi xi^T gives K back on the occupied space: n-term sums, times K_ij's conditioning
+    err = np.abs((xi @ xi.T) @ C - K).max()
+    assert err <= 16 * n * 2.0 ** -53 * np.linalg.cond(Kij0) * np.abs(K).max()
