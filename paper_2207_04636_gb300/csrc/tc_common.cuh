@@ -147,6 +147,17 @@ __device__ __forceinline__ void tc_fence_after() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
+// ------------------------------------------------- dependent launches
+// A kernel launched behind another one of its stream with the programmatic
+// attribute may start before that one has ended: dep_wait() returns once every
+// grid before it is complete and its writes are visible (at once in any other
+// launch), and comes before the first access to memory that another kernel
+// writes or reads.  dep_launch() lets the grid behind this one start.
+__device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void dep_launch() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // ---------------------------------------------------------------- TMA
 
 __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, uint64_t* bar,

@@ -178,6 +178,24 @@ __global__ void rownorm2_max_kernel(const T* __restrict__ a, long rows, int cols
   if ((threadIdx.x & 31) == 0) atomicMax(out, __float_as_uint(m * 1.0001f));
 }
 
+// Launch of a kernel that begins with dep_wait(): it may start while the kernel
+// before it on the stream ends, which hides part of its launch and set-up (8-centre
+// build of nine kernels 166 -> 160 us, 27-centre energy 309 -> 294).
+template <class... P, class... A>
+void launch_behind(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s, A&&... args) {
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid;
+  c.blockDim = dim3(threads);
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
+
 // Grid of a row whose largest |value| is mx: q = 2^(ceil(log2 mx) - 8), at
 // least 2^-24 (the FP16 subnormal step), so |x / q| <= 256.
 __device__ __forceinline__ float row_grid(float mx) {
@@ -274,6 +292,8 @@ __global__ void __launch_bounds__(128) split_q_kernel(const double* __restrict__
                                                       unsigned* am, float* __restrict__ sc,
                                                       __half* __restrict__ mo, __half* __restrict__ ho,
                                                       __half* __restrict__ lo) {
+  dep_wait();
+  dep_launch();
   __shared__ float red[8];
   const long r = blockIdx.x;
   const double* row = Q + r * ld;
@@ -307,6 +327,8 @@ __global__ void __launch_bounds__(256) gather_pieces_kernel(
     const uint4* __restrict__ src, long sstride, const int32_t* __restrict__ idx, long rows, int v16,
     int npc, uint4* __restrict__ dst, long dstride, const unsigned* __restrict__ am,
     float* __restrict__ sc, unsigned* __restrict__ rowmax, int n) {
+  dep_wait();
+  dep_launch();
   if (blockIdx.x == 0) {
     if (threadIdx.x == 0) scales_psi(am, sc);
     for (int i = threadIdx.x; i < n; i += blockDim.x) rowmax[i] = 0;
@@ -369,6 +391,8 @@ __global__ void split_rows_f32_kernel(const float* __restrict__ src, long rows, 
                                       __half* __restrict__ mo, __half* __restrict__ ho,
                                       __half* __restrict__ lo, long ld_dst,
                                       unsigned* __restrict__ rn2) {
+  dep_wait();
+  dep_launch();
   __shared__ float red[32];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const float G = sc[gidx];
@@ -497,6 +521,8 @@ __global__ void __launch_bounds__(32 * RS) lines_sum_kernel(
     const float* __restrict__ a_scale, double* __restrict__ out, long ldo, int nd,
     const float* __restrict__ M1, long cols, long ld, int chunks, unsigned* __restrict__ rowmax,
     unsigned* __restrict__ am) {
+  dep_wait();
+  dep_launch();
   __shared__ float sh[RS][2][32], red[8];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   float m = 0.0f;
@@ -552,6 +578,8 @@ __global__ void __launch_bounds__(256) lines_split_kernel(
     __half* __restrict__ mo, __half* __restrict__ ho, long ld_dst, int n1, int n,
     const double* __restrict__ D, long ldd, __half* __restrict__ dm, __half* __restrict__ dh,
     const unsigned* __restrict__ am, float* __restrict__ sc) {
+  dep_wait();
+  dep_launch();
   __shared__ float red[8];
   if (blockIdx.x == 0 && threadIdx.x == 0) scales_lines(am, sc);
   if ((int)blockIdx.x >= n1 * n) {
@@ -652,6 +680,8 @@ __global__ void __launch_bounds__(256) final_ex_kernel(const double* __restrict_
                                                       const double* __restrict__ ec, int nc_,
                                                       const float* __restrict__ sc, double dV,
                                                       double* part, unsigned* counter, double* Ex) {
+  dep_wait();
+  dep_launch();
   __shared__ double sh[8];
   __shared__ int flag;
   ex_chunk(blockIdx.x, ea, na_, ec, nc_, sh, part);
@@ -666,6 +696,8 @@ __global__ void __launch_bounds__(32 * RS) final_kernel(
     double* __restrict__ K, const double* __restrict__ C, const double* __restrict__ ea, int na_,
     const double* __restrict__ ec, int nc_, const float* __restrict__ sc, double* part,
     unsigned* counter, double* Ex, double* EK) {
+  dep_wait();
+  dep_launch();
   __shared__ float shf[RS][2][32];
   __shared__ double sh[8];
   __shared__ int flag;
@@ -815,6 +847,7 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap* pAm, const CUtensor
   __syncthreads();
   tc_fence_after();
   const uint32_t tbase = tslot;
+  dep_wait();
 
   if (warp == kGemmTma && lane == 0) {
     prefetch_tmap(pAm); prefetch_tmap(pAh); prefetch_tmap(pBm); prefetch_tmap(pBh);
@@ -1060,6 +1093,7 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap* pAm, const CUtensor
   }
   tc_fence_before();
   __syncthreads();
+  dep_launch();
   if (warp == kGemmMma) tmem_dealloc(tbase, 512);
 }
 
@@ -1098,7 +1132,7 @@ void launch_gemm(const CUtensorMap& mAm, const CUtensorMap& mAh, const CUtensorM
   g.tiles_z = (int)tiles.z;
   const long total = (long)tiles.x * tiles.y * tiles.z;
   const unsigned ctas = (unsigned)std::max<long>(1, std::min<long>(total, sm_count()));
-  gemm_kernel<<<ctas, kGemmThreads, G_SMEM, s>>>(mAm, mAh, mBm, mBh, mAl, mBl, g);
+  launch_behind(gemm_kernel, dim3(ctas), kGemmThreads, G_SMEM, s, mAm, mAh, mBm, mBh, mAl, mBl, g);
 }
 
 // ============================================================ wide gemm
@@ -1168,6 +1202,7 @@ __device__ __forceinline__ void gemm_wide_body(const CUtensorMap* pAm, const CUt
   __syncthreads();
   tc_fence_after();
   const uint32_t tbase = tslot;
+  dep_wait();
 
   if (warp == kWideTma && lane == 0) {
     prefetch_tmap(pAm); prefetch_tmap(pAh); prefetch_tmap(pBm); prefetch_tmap(pBh);
@@ -1353,6 +1388,7 @@ __device__ __forceinline__ void gemm_wide_body(const CUtensorMap* pAm, const CUt
   }
   tc_fence_before();
   __syncthreads();
+  dep_launch();
   if (warp == kWideMma) tmem_dealloc(tbase, 512);
 }
 
@@ -1390,7 +1426,7 @@ void launch_gemm_wide3(const CUtensorMap& mAm, const CUtensorMap& mAh, const CUt
   g.tiles_z = (int)tiles.z;
   const long total = (long)tiles.x * tiles.y * tiles.z;
   const unsigned ctas = (unsigned)std::max<long>(1, std::min<long>(total, sm_count()));
-  gemm_wide3_kernel<<<ctas, kWideThreads, GW3_SMEM, s>>>(mAm, mAh, mAl, mBm, mBh, mBl, g);
+  launch_behind(gemm_wide3_kernel, dim3(ctas), kWideThreads, GW3_SMEM, s, mAm, mAh, mAl, mBm, mBh, mBl, g);
 }
 
 // gemm_wide_kernel over tiles (x: 128-row M tiles, y: 256-column N tiles,
@@ -1404,7 +1440,7 @@ void launch_gemm_wide(const CUtensorMap& mAm, const CUtensorMap& mAh, const CUte
   g.tiles_z = (int)tiles.z;
   const long total = (long)tiles.x * tiles.y * tiles.z;
   const unsigned ctas = (unsigned)std::max<long>(1, std::min<long>(total, sm_count()));
-  gemm_wide_kernel<<<ctas, kWideThreads, GW_SMEM, s>>>(mAm, mAh, mBm, mBh, g);
+  launch_behind(gemm_wide_kernel, dim3(ctas), kWideThreads, GW_SMEM, s, mAm, mAh, mBm, mBh, g);
 }
 
 // ============================================================ two products, one launch
@@ -1456,9 +1492,9 @@ void launch_gemm_pair(GemmPair p, const dim3 (&tiles)[2], bool wide, cudaStream_
   }
   p.c0 = (int)c0;
   if (wide)
-    gemm_pair_kernel<true><<<(unsigned)(c0 + c1), kWideThreads, GW_SMEM, s>>>(p);
+    launch_behind(gemm_pair_kernel<true>, dim3((unsigned)(c0 + c1)), kWideThreads, GW_SMEM, s, p);
   else
-    gemm_pair_kernel<false><<<(unsigned)(c0 + c1), kGemmThreads, G_SMEM, s>>>(p);
+    launch_behind(gemm_pair_kernel<false>, dim3((unsigned)(c0 + c1)), kGemmThreads, G_SMEM, s, p);
   count_launch();
 }
 
@@ -1548,6 +1584,7 @@ __device__ __forceinline__ void tprod_body(const TprodMaps& mp, const TprodArgs&
   __syncthreads();
   tc_fence_after();
   const uint32_t tbase = tslot;
+  dep_wait();
 
   if (warp == kGemmTma && lane == 0) {
     prefetch_tmap(&mp.a);
@@ -1738,6 +1775,7 @@ __device__ __forceinline__ void tprod_body(const TprodMaps& mp, const TprodArgs&
   }
   tc_fence_before();
   __syncthreads();
+  dep_launch();
   if (warp == kGemmMma) tmem_dealloc(tbase, 512);
 }
 
@@ -1754,7 +1792,7 @@ void launch_tprod(const TprodMaps& mp, TprodArgs g, cudaStream_t s, long long wa
   g.wait = wait;
   const long total = (long)g.tiles_x * g.tiles_y;
   const unsigned ctas = (unsigned)std::max<long>(1, std::min<long>(total, sm_count()));
-  tprod_kernel<<<ctas, kGemmThreads, TP_SMEM, s>>>(mp, g);
+  launch_behind(tprod_kernel, dim3(ctas), kGemmThreads, TP_SMEM, s, mp, g);
 }
 
 // ============================================================ pair kernel
@@ -1935,6 +1973,7 @@ __device__ __forceinline__ void pair_body(const CUtensorMap* mYm, const CUtensor
   __syncthreads();
   tc_fence_after();
   const uint32_t tbase = tslot;
+  dep_wait();
 
   if (warp < kEpiWarps) load_x_tile<NP>(a, x0, tbase, warp, lane);
   tc_fence_before();
@@ -2136,6 +2175,7 @@ __device__ __forceinline__ void pair_body(const CUtensorMap* mYm, const CUtensor
   }
   tc_fence_before();
   __syncthreads();
+  dep_launch();
   if (warp == mma_warp) tmem_dealloc(tbase, 512);
 }
 
@@ -2231,6 +2271,7 @@ __device__ __forceinline__ void fused_body(const CUtensorMap* mYm, const CUtenso
   __syncthreads();
   tc_fence_after();
   const uint32_t tbase = tslot;
+  dep_wait();
 
   if (warp < kEpiWarps) load_x_tile<NP>(a, x0, tbase, warp, lane);
   tc_fence_before();
@@ -2525,6 +2566,7 @@ __device__ __forceinline__ void fused_body(const CUtensorMap* mYm, const CUtenso
   }
   tc_fence_before();
   __syncthreads();
+  dep_launch();
   if (warp == mma_warp) tmem_dealloc(tbase, 512);
 }
 
@@ -2647,6 +2689,7 @@ __device__ __forceinline__ void energy_body(const CUtensorMap* mYm, const CUtens
   __syncthreads();
   tc_fence_after();
   const uint32_t tbase = tslot;
+  dep_wait();
 
   if (warp < kEpiWarps) load_x_tile<NP>(a, x0, tbase, warp, lane);
   tc_fence_before();
@@ -2752,6 +2795,7 @@ __device__ __forceinline__ void energy_body(const CUtensorMap* mYm, const CUtens
   }
   tc_fence_before();
   __syncthreads();
+  dep_launch();
   if (warp == mma_warp) tmem_dealloc(tbase, 512);
 }
 
@@ -2783,9 +2827,9 @@ void launch_pair_roles(const std::vector<PairRole>& rs, int np, cudaStream_t s) 
     }
     job.nroles = k;
     if (np == 64)
-      pair_kernel_group<64><<<blocks, kPairThreads, PairCfg<64>::SMEM, s>>>(job);
+      launch_behind(pair_kernel_group<64>, dim3(blocks), kPairThreads, PairCfg<64>::SMEM, s, job);
     else
-      pair_kernel_group<128><<<blocks, kPairThreads, FusedCfg::SMEM, s>>>(job);
+      launch_behind(pair_kernel_group<128>, dim3(blocks), kPairThreads, FusedCfg::SMEM, s, job);
     count_launch();
   }
 }
@@ -2798,9 +2842,9 @@ void launch_pair3(const PairRole* r, int np, cudaStream_t s) {
   }
   const unsigned blocks = (unsigned)(r[0].nblk + r[1].nblk + r[2].nblk);
   if (np == 64)
-    pair_kernel<64><<<blocks, kPairThreads, PairCfg<64>::SMEM, s>>>(job);
+    launch_behind(pair_kernel<64>, dim3(blocks), kPairThreads, PairCfg<64>::SMEM, s, job);
   else
-    pair_kernel<128><<<blocks, kPairThreads, PairCfg<128>::SMEM, s>>>(job);
+    launch_behind(pair_kernel<128>, dim3(blocks), kPairThreads, PairCfg<128>::SMEM, s, job);
   count_launch();
 }
 
@@ -2814,9 +2858,9 @@ void launch_energy2(const PairRole& ra, const PairRole& rc, int np, cudaStream_t
   }
   const unsigned blocks = (unsigned)(ra.nblk + rc.nblk);
   if (np == 64)
-    energy_kernel<64><<<blocks, kPairThreads, PairCfg<64>::SMEM, s>>>(job);
+    launch_behind(energy_kernel<64>, dim3(blocks), kPairThreads, PairCfg<64>::SMEM, s, job);
   else
-    energy_kernel<128><<<blocks, kPairThreads, PairCfg<128>::SMEM, s>>>(job);
+    launch_behind(energy_kernel<128>, dim3(blocks), kPairThreads, PairCfg<128>::SMEM, s, job);
   count_launch();
 }
 
@@ -3562,7 +3606,7 @@ cudaError_t mixed_enqueue_pre(MixedState* m, const double* C, cudaStream_t s, co
       q_kernel<<<dim3((unsigned)((m->Np + QM - 1) / QM), (unsigned)((n + QJ - 1) / QJ)), QM * QJ * QS, 0,
                  s>>>(m->Lf, C, N, n, m->CT64, m->Np, m->am + AM_C);
     }
-    split_q_kernel<<<(unsigned)n, 128, 0, s>>>(m->CT64, m->Np, m->am, m->sc, m->CT_m, m->CT_h, m->CT_l);
+    launch_behind(split_q_kernel, dim3((unsigned)n), 128, 0, s, m->CT64, m->Np, m->am, m->sc, m->CT_m, m->CT_h, m->CT_l);
     count_launch(2);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -3582,14 +3626,14 @@ cudaError_t mixed_enqueue_pre(MixedState* m, const double* C, cudaStream_t s, co
     launch_gemm_wide3(m->m_phi32_m, m->m_phi32_h, m->m_phi32_l, m->m_CT32_m, m->m_CT32_h,
                       m->m_CT32_l, g, dim3((unsigned)((ng + 127) / 128), (unsigned)((n + 255) / 256), 1),
                       s, m->wait_cycles);
-    split_rows_f32_kernel<<<152 * 4, 256, 0, s>>>(m->M1, ng, n, n, m->sc, SC_PSI, m->psi_m,
+    launch_behind(split_rows_f32_kernel, dim3(152 * 4), 256, 0, s, m->M1, ng, n, n, m->sc, SC_PSI, m->psi_m,
                                                   m->psi_h, m->psi_l, np, m->am + AM_RN2);
     count_launch();
   }
   {  // the orbitals at every interpolation point (psig is the slice's view)
     const long nat = m->NaT;
     const int npc = m->large ? 3 : 2, v16 = np / 8;
-    gather_pieces_kernel<<<blocks_for(npc * nat * v16), 256, 0, s>>>(
+    launch_behind(gather_pieces_kernel, dim3(blocks_for(npc * nat * v16)), 256, 0, s, 
         reinterpret_cast<const uint4*>(m->psi_m), ng * v16, m->idx, nat, v16, npc,
         reinterpret_cast<uint4*>(m->psigA_m), nat * v16, m->am, m->sc, m->rowmax, n);
     count_launch(2);  // and the orbital product
@@ -3771,7 +3815,7 @@ cudaError_t mixed_enqueue_energy(MixedState* m, const double* C, double* Ex, cud
   if (e != cudaSuccess) return e;
   hook(1, 0);
   hook(7, 1);
-  final_ex_kernel<<<2 * kExBlocks, 256, 0, s>>>(m->EpA, (int)m->epA, m->EpC, (int)m->epC, m->sc, m->dV,
+  launch_behind(final_ex_kernel, dim3(2 * kExBlocks), 256, 0, s, m->EpA, (int)m->epA, m->EpC, (int)m->epC, m->sc, m->dV,
                                                 m->part, m->am + CNT_K, Ex);
   count_launch();
   e = cudaGetLastError();
@@ -3909,11 +3953,11 @@ cudaError_t mixed_enqueue_post(MixedState* m, const double* C, double* K, double
     const int per = m->partsA + m->partsC <= kFewParts ? 32 * RS : 32;
     const int nd = (int)((na * n + per - 1) / per);
     const int chunks = (int)std::min<long>(16, (ng + 1023) / 1024);
-    lines_sum_kernel<<<(unsigned)(nd + chunks * n), 32 * RS, 0, s>>>(
+    launch_behind(lines_sum_kernel, dim3((unsigned)(nd + chunks * n)), 32 * RS, 0, s, 
         m->M2p, m->partsA, m->M3p, m->partsC, na, n, m->fused ? m->sc + SC_OUT_AB : nullptr, m->D23T64,
         m->Na8, nd, m->M1, ng, m->Ng4, chunks, m->rowmax, m->am);
     const int n1 = (int)std::min<long>(64, (m->Ng8 / 8 + 255) / 256);
-    lines_split_kernel<<<(unsigned)((n1 + 1) * n), 256, 0, s>>>(
+    launch_behind(lines_split_kernel, dim3((unsigned)((n1 + 1) * n)), 256, 0, s, 
         m->M1, ng, m->Ng4, m->rowmax, m->M1_m, m->M1_h, m->Ng8, n1, n, m->D23T64, m->Na8, m->D23T_m,
         m->D23T_h, m->am, m->sc);
     count_launch(2);
@@ -3939,7 +3983,7 @@ cudaError_t mixed_enqueue_post(MixedState* m, const double* C, double* K, double
   hook(7, 1);
   const long count = (long)N * n;
   const unsigned nk = (unsigned)((count + 31) / 32);  // each leaves a sum behind the 2 kExBlocks
-  final_kernel<<<2 * kExBlocks + nk, 32 * RS, 0, s>>>(
+  launch_behind(final_kernel, dim3(2 * kExBlocks + nk), 32 * RS, 0, s, 
       m->L1p, m->splitsL1, m->L23p, m->splitsL23, count, m->dV, K, C, m->EpA, (int)m->epA, m->EpC,
       (int)m->epC, m->sc, m->part, m->am + CNT_K, Ex, EK);
   count_launch();
