@@ -1122,6 +1122,7 @@ int xk_coulomb(xk_handle* h, int32_t grid, double L, const double* C, double* J_
     XK_CUDA(xk::potential_rows_f64(h->Jv, h->phi, (long)ng, N, h->Jphiv, s));
     xk::DGemm gj{N, N, (int)ng, h->phi, N, true, h->Jphiv, N, false, h->Jout, N, h->dV, nullptr, 0, 0, h->work};
     gj.scale = digit_scratch(h->M1, (size_t)n * ng, N, N);
+    gj.sym = true;
     XK_CUDA(xk::dgemm(gj, s));
     XK_CUDA(xk::dot_f64(h->Jrho, h->Jv, (long)ng, h->dV, h->red, h->Jout + (size_t)N * N, s));
   }

@@ -54,6 +54,10 @@ constexpr int D_GROUP = 256 / DK;   // K blocks between drains
 constexpr int D_WORK = 16;
 constexpr int D_THREADS = 32 * (D_WORK + 4);
 
+// Tiles of a symmetric product that reach y <= x: 2 (i + 1) of X tile i, the last
+// X tile's all.
+int sym_tiles(int tiles_x, int tiles_y) { return (tiles_x - 1) * tiles_x + tiles_y; }
+
 // One operand: element (row, k) at p[row ld + k] (kc) or p[k ld + row].
 struct DOperand {
   const double* p;
@@ -68,6 +72,8 @@ struct DArgs {
   DOperand x, y;
   int K, kchunk, ksplit;
   int tiles_x, tiles_y;
+  int tiles;         // of one K split: tiles_x * tiles_y, or those that reach y <= x (sym)
+  int sym;
   int swapped;       // X rows are the columns of C (else its rows)
   int M, N;          // C is M x N
   double* C; long ldc;
@@ -318,8 +324,21 @@ __global__ void __launch_bounds__(D_THREADS, 1) digit_gemm_kernel(const __grid_c
   __syncthreads();
   tc_fence_after();
   const uint32_t tbase = tslot;
-  const int ntiles = g.tiles_x * g.tiles_y * g.ksplit;
-  // tile t: X tile fastest, then Y tile, then the K split
+  const int ntiles = g.tiles * g.ksplit;
+  // tile t: X tile fastest, then Y tile, then the K split (symmetric: Y fastest)
+  auto place = [&](int t, int& xt, int& yt, int& z) __attribute__((always_inline)) {
+    z = t / g.tiles;
+    const int r = t - z * g.tiles;
+    if (g.sym) {
+      xt = min((int)((sqrtf(4.0f * r + 1.0f) - 1.0f) * 0.5f), g.tiles_x - 1);
+      while (xt > 0 && xt * (xt + 1) > r) --xt;
+      while (xt < g.tiles_x - 1 && (xt + 1) * (xt + 2) <= r) ++xt;
+      yt = r - xt * (xt + 1);
+    } else {
+      xt = r % g.tiles_x;
+      yt = r / g.tiles_x;
+    }
+  };
   auto kblocks = [&](int z) {
     const long k0 = (long)z * g.kchunk, k1 = min((long)g.K, k0 + g.kchunk);
     return (int)((k1 - k0 + DK - 1) / DK);
@@ -340,7 +359,7 @@ __global__ void __launch_bounds__(D_THREADS, 1) digit_gemm_kernel(const __grid_c
         good = false;
       };
       for (int t = blockIdx.x; good && t < ntiles; t += gridDim.x) {
-        const int nkb = kblocks(t / (g.tiles_x * g.tiles_y));
+        const int nkb = kblocks(t / g.tiles);
         for (int kb = 0; kb < nkb; ++kb, ++it) {
           if (__shfl_sync(0xffffffffu, (int)abort_flag, 0)) { good = false; break; }
           const int s = it % D_STAGES;
@@ -397,10 +416,10 @@ __global__ void __launch_bounds__(D_THREADS, 1) digit_gemm_kernel(const __grid_c
     int fpar = 1;  // which half of exps the tile being fetched uses
     auto open_tile = [&]() __attribute__((always_inline)) {
       if (ft >= ntiles) { fn = 0; return; }
-      const int xt = ft % g.tiles_x, r = ft / g.tiles_x;
+      int xt, yt;
+      place(ft, xt, yt, fz);
       fx0 = xt * DX;
-      fy0 = (r % g.tiles_y) * DY;
-      fz = r / g.tiles_y;
+      fy0 = yt * DY;
       fn = kblocks(fz);
       fpar ^= 1;
       const long rx = fx0 + block_row<8, XK>(warp, lane), ry = fy0 + block_row<4, YK>(warp, lane);
@@ -471,17 +490,19 @@ __global__ void __launch_bounds__(D_THREADS, 1) digit_gemm_kernel(const __grid_c
     };
     // writes the 16 results of this thread for tile t
     auto put_tile = [&](int t) __attribute__((always_inline)) {
-      const int xt = t % g.tiles_x, rr = t / g.tiles_x;
+      int xt, yt, z;
+      place(t, xt, yt, z);
       const long x = (long)xt * DX + quad * 32 + lane;
-      const long y0 = (long)(rr % g.tiles_y) * DY + 16 * cg;
-      const int left = (int)min(16l, g.y.rows - y0);  // columns of this warp inside C
+      const long y0 = (long)yt * DY + 16 * cg;
+      // columns of this warp inside C (symmetric: those up to x)
+      const int left = (int)min(16l, (g.sym ? min((long)g.y.rows, x + 1) : (long)g.y.rows) - y0);
       const bool in = x < g.x.rows;
       const int e = row_exp(in ? __ldg(g.x.scale + x) : 0) - 38;
       // the 16 rows' exponents: lane j holds that of row j
-      const int ye = row_exp((lane & 15) < left ? __ldg(g.y.scale + y0 + (lane & 15)) : 0);
+      const int ye = row_exp(y0 + (lane & 15) < g.y.rows ? __ldg(g.y.scale + y0 + (lane & 15)) : 0);
       const bool split = g.ksplit > 1;
       const long ld = split ? g.N : g.ldc;
-      double* c = (split ? g.work + (long)(rr / g.tiles_y) * g.M * g.N : g.C) +
+      double* c = (split ? g.work + (long)z * g.M * g.N : g.C) +
                   (g.swapped ? y0 * ld + x : x * ld + y0);
       const long step = g.swapped ? ld : 1;
       const double* h = g.H + (g.swapped ? y0 * g.ldh + x : x * g.ldh + y0);
@@ -497,7 +518,17 @@ __global__ void __launch_bounds__(D_THREADS, 1) digit_gemm_kernel(const __grid_c
       if (!in) return;
       // branches around the FP64 operations: one that is only predicated off
       // would still take its 16 cycles of the FP64 pipe
-      if (!split && (g.scaled || g.added)) {
+      if (!split && g.sym) {  // and its mirror image
+        double* cm = g.C + x * ld + y0;
+#pragma unroll
+        for (int j = 0; j < 16; ++j)
+          if (j < left) {
+            double v = __longlong_as_double(hi[j]);
+            if (g.scaled) v *= g.alpha;
+            c[j * step] = v;
+            cm[j] = v;
+          }
+      } else if (!split && (g.scaled || g.added)) {
 #pragma unroll
         for (int j = 0; j < 16; ++j)
           if (j < left) {
@@ -531,7 +562,7 @@ __global__ void __launch_bounds__(D_THREADS, 1) digit_gemm_kernel(const __grid_c
     bool due = false;       // the block produced last ended a group
     int par = 1;
     for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-      const int nkb = kblocks(t / (g.tiles_x * g.tiles_y));
+      const int nkb = kblocks(t / g.tiles);
       par ^= 1;
       for (int kb = 0; kb < nkb && ok; ++kb, ++it) {
         const int s = it % D_STAGES, use = it / D_STAGES;
@@ -629,9 +660,9 @@ bool digit_gemm_wanted(const DGemm& g) {
 
 // K split (at most cap) of least time: waves of tiles over the SMs times the
 // 256-term groups of a tile, with one group's time for a tile's start and end.
-int digit_ksplit(int M, int N, int K, int cap) {
-  const int X = std::max(M, N), Y = std::min(M, N);
-  const long tiles = (long)((X + DX - 1) / DX) * ((Y + DY - 1) / DY);
+int digit_ksplit(int M, int N, int K, bool sym, int cap) {
+  const int X = std::max(M, N), Y = std::min(M, N), tx = (X + DX - 1) / DX, ty = (Y + DY - 1) / DY;
+  const long tiles = sym ? sym_tiles(tx, ty) : (long)tx * ty;
   const int groups = (K + 255) / 256;
   int best = 1;
   long cost = 0;
@@ -664,7 +695,9 @@ cudaError_t digit_gemm(const DGemm& g, int ksplit, int kchunk, cudaStream_t s) {
   a.scaled = g.alpha != 1.0; a.added = g.beta != 0.0;
   a.H = g.H; a.ldh = g.ldh; a.work = g.work; a.flag = sc;
   a.nbatch = g.nbatch; a.cskip = g.cskip;
-  const long tiles = (long)a.tiles_x * a.tiles_y * ksplit;
+  a.sym = g.sym;
+  a.tiles = g.sym ? sym_tiles(a.tiles_x, a.tiles_y) : a.tiles_x * a.tiles_y;
+  const long tiles = (long)a.tiles * ksplit;
   const unsigned ctas = (unsigned)std::min<long>(tiles, 152);
   auto launch = [&](auto kernel) {
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, D_SMEM);

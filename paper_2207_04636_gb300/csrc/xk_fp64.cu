@@ -104,13 +104,15 @@ __global__ void splitk_reduce_kernel(DGemm g) {
   const long total = (long)g.M * g.N;
   for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < total;
        t += (long)gridDim.x * blockDim.x) {
+    const long m = t / g.N, n = t % g.N;
+    if (g.sym && n < m) continue;
     double s = 0.0;
     for (int z = 0; z < g.ksplit; ++z) s += g.work[(long)z * total + t];
-    const long m = t / g.N, n = t % g.N;
     double v = g.alpha * s;
     if (g.H) v *= g.H[m * g.ldh + n];
     if (g.beta != 0.0) v += g.beta * g.C[m * g.ldc + n];
     g.C[m * g.ldc + n] = v;
+    if (g.sym) g.C[n * g.ldc + m] = v;
   }
 }
 
@@ -150,7 +152,7 @@ cudaError_t dgemm(const DGemm& gin, cudaStream_t s) {
   if (g.nbatch > 0) g.ksplit = 1;  // batched columns are stored unsplit
   const bool digits = digit_gemm_wanted(g);
   if (digits)
-    g.ksplit = digit_ksplit(g.M, g.N, g.K,
+    g.ksplit = digit_ksplit(g.M, g.N, g.K, g.sym,
                             !g.work || g.nbatch > 0 ? 1 : g.ksplit > 0 ? g.ksplit : dgemm_ksplit(g.M, g.N, g.K));
   if (g.ksplit <= 0) g.ksplit = choose_ksplit(g.M, g.N, g.K);
   if (g.ksplit > 1 && !g.work) g.ksplit = 1;
@@ -335,28 +337,29 @@ cudaError_t poisson_tables_f64(int g, double L, double* tab, cudaStream_t s) {
   return e == cudaSuccess ? cudaStreamSynchronize(s) : e;
 }
 
-// One pass for few functions: a thread forms four outputs k of one (f, p); the
+// One pass for few functions: a thread forms two outputs k of one (f, p) (four left a
+// third of the SMs with twice the others' work: 22 us at 45^3 against 15); the
 // lanes' rows of `in` stay in L1 over the g terms.  Bound by the FP64 pipe.
 __global__ void __launch_bounds__(128) axis_kernel(const double* __restrict__ in, double* __restrict__ out,
                                                    long rows, int g, const double* __restrict__ B,
                                                    const double* __restrict__ lam) {
   const long r = (long)blockIdx.x * 32 + threadIdx.x, g2 = (long)g * g;
-  const int k0 = 4 * (blockIdx.y * blockDim.y + threadIdx.y);
+  const int k0 = 2 * (blockIdx.y * blockDim.y + threadIdx.y);
   if (r >= rows || k0 >= g) return;
   const double* x = in + r * g;
-  const double* b[4];
+  const double* b[2];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) b[i] = B + (long)min(k0 + i, g - 1) * g;
-  double acc[4] = {0.0, 0.0, 0.0, 0.0};
-#pragma unroll 4
+  for (int i = 0; i < 2; ++i) b[i] = B + (long)min(k0 + i, g - 1) * g;
+  double acc[2] = {0.0, 0.0};
+#pragma unroll 8
   for (int j = 0; j < g; ++j) {
     const double v = x[j];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) acc[i] = fma(__ldg(b[i] + j), v, acc[i]);
+    for (int i = 0; i < 2; ++i) acc[i] = fma(__ldg(b[i] + j), v, acc[i]);
   }
   const long f = r / g2, p = r - f * g2;
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < 2; ++i)
     if (k0 + i < g) {
       const double v = lam ? acc[i] * lam[(k0 + i) * g2 + p] : acc[i];
       out[f * g2 * g + (k0 + i) * g2 + p] = v;
@@ -380,7 +383,7 @@ cudaError_t poisson_f64(const double* in, double* out, double* tmp, long nf, int
     if (digit_gemm_wanted(q)) {
       e = dgemm(q, s);
     } else {
-      axis_kernel<<<dim3((unsigned)((nf * g2 + 31) / 32), (unsigned)((g + 15) / 16)), dim3(32, 4), 0, s>>>(
+      axis_kernel<<<dim3((unsigned)((nf * g2 + 31) / 32), (unsigned)((g + 7) / 8)), dim3(32, 4), 0, s>>>(
           src, dst, nf * g2, g, B, H);
       count_launch();
       e = cudaGetLastError();

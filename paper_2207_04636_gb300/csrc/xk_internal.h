@@ -44,6 +44,7 @@ struct DGemm {
                 // products run on the tensor cores (xk_digits.cu)
   int nbatch;   // > 0: the columns of C come in batches of nbatch: column n is stored
   long cskip;   // (n / nbatch) cskip elements further on, and H has column n % nbatch
+  bool sym;     // C is symmetric (M = N, no H, beta = 0): one half may be formed and mirrored
 };
 cudaError_t dgemm(const DGemm& g, cudaStream_t s);
 
@@ -54,7 +55,7 @@ cudaError_t dgemm(const DGemm& g, cudaStream_t s);
 // formed with FP64 FMAs instead (an operand that is not finite).
 size_t digit_scale_ints(int M, int N);
 bool digit_gemm_wanted(const DGemm& g);
-int digit_ksplit(int M, int N, int K, int cap);
+int digit_ksplit(int M, int N, int K, bool sym, int cap);
 cudaError_t digit_gemm(const DGemm& g, int ksplit, int kchunk, cudaStream_t s);
 // Split count dgemm picks when DGemm::ksplit == 0 (work needs ksplit*M*N).
 int dgemm_ksplit(int M, int N, int K);

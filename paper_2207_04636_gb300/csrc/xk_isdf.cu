@@ -339,6 +339,7 @@ cudaError_t isdf_tables_f64(const double* phi, long ng, int N, const double* phi
   auto gram = [&]() {
     DGemm g{na, na, N, phig, N, false, phig, N, true, Xgg, na, 1.0, nullptr, 0, 0, work};
     g.scale = scale;
+    g.sym = true;
     cudaError_t r = dgemm(g, s);
     if (r != cudaSuccess) return r;
     square_kernel<<<nblocks((long)na * na), 256, 0, s>>>(Xgg, na, na, na);

@@ -101,3 +101,25 @@ def test_tiny_rows(xk):
     K, _ = h.build(C * 2.0 ** 950)
     h.release()
     assert np.array_equal(K, (l1 + l2 - l3).T * 2.0 ** -950)
+
+
+@pytest.mark.parametrize("N", [64, 65, 129, 200, 257])
+def test_symmetric_product(xk, N):
+    """J forms one half of a symmetric product: every tile on or below the diagonal,
+    mirrored; the Poisson solve's even and odd grids."""
+    import oracle
+
+    grid = 24 if N % 2 else 21
+    rng = np.random.default_rng(N)
+    phi, C = rng.standard_normal((grid ** 3, N)), rng.standard_normal((N, 5)) / N
+    idx, V, W = np.arange(8), np.zeros((8, grid ** 3)), np.zeros((8, 8))
+    dV = 6.0 ** 3 / grid ** 3
+    h = xk.Handle(phi, idx, V, W, dV, 5, mode="fp64")
+    J, EJ = h.coulomb(C, grid, 6.0)
+    h.release()
+    J0, EJ0 = oracle.coulomb_j(phi, C, 6.0, grid, dV)
+    assert np.array_equal(J, J.T)
+    # sums of grid^3 products in FP64 on the host, the potential's rounding alike
+    tol = 2.0 ** -53 * np.sqrt(grid ** 3) * 16
+    assert np.linalg.norm(J - J0) <= tol * np.linalg.norm(J0)
+    assert abs(EJ - EJ0) <= tol * abs(EJ0)
