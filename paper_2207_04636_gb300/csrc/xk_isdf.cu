@@ -13,6 +13,7 @@
 #include <cmath>
 #include <vector>
 
+#include "tc_common.cuh"
 #include "xk_internal.h"
 
 namespace xk {
@@ -145,8 +146,10 @@ __global__ void __launch_bounds__(PT_ROWS * PT_WARPS) point_step_kernel(
     double* __restrict__ tol, double* __restrict__ L, double* __restrict__ d,
     long long* __restrict__ pv, int* __restrict__ pi) {
   __shared__ long long bv[PT_WARPS];
-  __shared__ double sf[PT_WARPS][PT_ROWS], sl[PT_WARPS][PT_ROWS];
+  __shared__ double rsp, sf[PT_WARPS][PT_ROWS], sl[PT_WARPS][PT_ROWS];
   __shared__ int bi[PT_WARPS];
+  tc::dep_wait();
+  tc::dep_launch();
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, nb = gridDim.x;
   long long top = -1;
   int p = 0x7fffffff;
@@ -180,6 +183,9 @@ __global__ void __launch_bounds__(PT_ROWS * PT_WARPS) point_step_kernel(
   }
   const int i = blockIdx.x * PT_ROWS + lane;
   const long ii = i < m ? i : m - 1;
+  // 1 / sqrt(val): some 60 dependent FP64 instructions, beside the other warps' sums
+  if (tid == PT_ROWS * PT_WARPS - 1) rsp = 1.0 / sqrt(v);
+  const double di = w == 0 && i < m ? d[i] : -1.0;
   double f = 0.0, l = 0.0;
   const double* fp = F + (long)p * N;
 #pragma unroll 4
@@ -196,13 +202,11 @@ __global__ void __launch_bounds__(PT_ROWS * PT_WARPS) point_step_kernel(
   }
   long long nd = -1;
   if (i < m) {
-    const double sp = sqrt(v);
-    const double di = d[i];
     if (i == p) {
-      L[(long)t * m + i] = sp;
+      L[(long)t * m + i] = v * rsp;
       d[i] = -1.0;
     } else if (di >= 0.0) {
-      const double x = (f * f - l) / sp;
+      const double x = (f * f - l) * rsp;
       L[(long)t * m + i] = x;
       const double dn = di - x * x;
       d[i] = dn;
@@ -258,11 +262,20 @@ cudaError_t select_points_f64(const double* F, int m, int N, int want, double to
     diag_init_kernel<<<nb, PT_ROWS, 0, s>>>(FT, m, N, d, pv, pi);
     count_launch(2);
   }
+  // each step may be launched while the one before it ends (tc::dep_wait)
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3((unsigned)nb);
+  c.blockDim = dim3(PT_ROWS * PT_WARPS);
+  c.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = &at;
+  c.numAttrs = 1;
   for (int t = 0; e == cudaSuccess && t < want; ++t) {
-    point_step_kernel<<<nb, PT_ROWS * PT_WARPS, 0, s>>>(F, FT, m, N, t, tol_rel, sel, dpiv, val, tol, L,
-                                                       d, pv, pi);
+    e = cudaLaunchKernelEx(&c, point_step_kernel, F, (const double*)FT, m, N, t, tol_rel, sel, dpiv, val,
+                           tol, L, d, pv, pi);
     count_launch();
-    if ((t & 255) == 255) e = cudaGetLastError();
   }
   int got = 0;
   if (e == cudaSuccess) e = cudaMemcpyAsync(&got, sel, 4, cudaMemcpyDeviceToHost, s);
