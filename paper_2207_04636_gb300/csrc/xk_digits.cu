@@ -78,6 +78,7 @@ struct DArgs {
   int M, N;          // C is M x N
   double* C; long ldc;
   double alpha, beta;
+  int careful;        // added to C, or in place
   int scaled, added;  // alpha != 1, beta != 0 (an FP64 comparison per result would cost more)
   const double* H; long ldh;
   double* work;      // ksplit > 1: partial sums [ksplit][M][N]
@@ -289,11 +290,12 @@ __global__ void __launch_bounds__(D_THREADS, 1) digit_gemm_kernel(const __grid_c
   __shared__ int exps[D_WORK][2][64];
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // uniform: the register split needs it
-  // A product added to C must not be left out half-way: every CTA looks at every
-  // row first.  Any other is formed again as a whole when a tile meets such a row.
+  // A product that is added to C, or overwrites an operand, must not be left out half-way:
+  // every CTA looks at every row first.  Any other is formed again as a whole when a
+  // tile meets such a row.
   if (tid == 0) skip = 0;
   __syncthreads();
-  if (g.added) {
+  if (g.careful) {
     bool bad = false;
     for (int i = tid; i < g.x.rows; i += D_THREADS) bad |= row_unfit(__ldg(g.x.scale + i));
     for (int i = tid; i < g.y.rows; i += D_THREADS) bad |= row_unfit(__ldg(g.y.scale + i));
@@ -654,7 +656,7 @@ size_t digit_scale_ints(int M, int N) { return (size_t)M + N + 8; }
 // 2e7 multiply-adds take the FP64 pipe 35 us with every SM at work; the row
 // maxima, the launches and a tile here take about 25 us.
 bool digit_gemm_wanted(const DGemm& g) {
-  return g.scale && !g.upperA && g.K >= 16 && std::min(g.M, g.N) >= 8 &&
+  return g.scale && g.K >= 16 && std::min(g.M, g.N) >= 8 &&
          (double)g.M * g.N * g.K >= 2e7;
 }
 
@@ -692,7 +694,7 @@ cudaError_t digit_gemm(const DGemm& g, int ksplit, int kchunk, cudaStream_t s) {
   a.tiles_x = (a.x.rows + DX - 1) / DX;
   a.tiles_y = (a.y.rows + DY - 1) / DY;
   a.M = g.M; a.N = g.N; a.C = g.C; a.ldc = g.ldc; a.alpha = g.alpha; a.beta = g.beta;
-  a.scaled = g.alpha != 1.0; a.added = g.beta != 0.0;
+  a.scaled = g.alpha != 1.0; a.added = g.beta != 0.0; a.careful = a.added || in_place(g);
   a.H = g.H; a.ldh = g.ldh; a.work = g.work; a.flag = sc;
   a.nbatch = g.nbatch; a.cskip = g.cskip;
   a.sym = g.sym;

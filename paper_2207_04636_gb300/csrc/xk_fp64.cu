@@ -22,16 +22,18 @@ constexpr int BM = 64, BN = 64, BK = 16, TPB = 256;
 
 template <bool TA, bool TB, bool HAD>
 __global__ void __launch_bounds__(TPB) dgemm_kernel(DGemm g, int kchunk, const int* only_if) {
-  // behind a product on the tensor cores: only when that one was left out
+  // behind a product on the tensor cores: only when that one was left out (a few
+  // blocks then walk the tiles; a grid of all of them took 25 us to start and end)
   const int left_out = only_if ? *only_if : 1;
   if (!left_out) return;
+  const long gx = (g.N + BN - 1) / BN, gy = (g.M + BM - 1) / BM, ntiles = gx * gy * g.ksplit;
   __shared__ double As[BK][BM + 1];
   __shared__ double Bs[BK][BN + 1];
   const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-  const long m0 = (long)blockIdx.y * BM, n0 = (long)blockIdx.x * BN;
-  const long kend = min((long)g.K, (long)blockIdx.z * kchunk + kchunk);
-  // rows m0.. of an upper-triangular op(A) vanish for k < m0
-  const long kbeg = g.upperA ? max((long)blockIdx.z * kchunk, m0) : (long)blockIdx.z * kchunk;
+  for (long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+  const long bz = tile / (gx * gy);
+  const long m0 = (tile / gx % gy) * BM, n0 = (tile % gx) * BN;
+  const long kbeg = bz * kchunk, kend = min((long)g.K, kbeg + kchunk);
   double acc[4][4];
 #pragma unroll
   for (int i = 0; i < 4; ++i)
@@ -84,7 +86,7 @@ __global__ void __launch_bounds__(TPB) dgemm_kernel(DGemm g, int kchunk, const i
       const long n = n0 + tx + 16 * j;
       if (n >= g.N) continue;
       if (g.ksplit > 1) {
-        g.work[((long)blockIdx.z * g.M + m) * g.N + n] = acc[i][j];
+        g.work[(bz * g.M + m) * g.N + n] = acc[i][j];
       } else {
         const long q = g.nbatch > 0 ? n / g.nbatch : 0;  // batch of the column
         const long at = m * g.ldc + n + q * g.cskip;
@@ -92,10 +94,11 @@ __global__ void __launch_bounds__(TPB) dgemm_kernel(DGemm g, int kchunk, const i
         if (HAD) v *= g.H[m * g.ldh + n - q * g.nbatch];
         if (g.beta != 0.0) v += g.beta * g.C[at];
         // a tensor-core product that gave up half-way has changed C already
-        if (g.beta != 0.0 && only_if && left_out == 2) v = nan("");
+        if ((g.beta != 0.0 || in_place(g)) && only_if && left_out == 2) v = nan("");
         g.C[at] = v;
       }
     }
+  }
   }
 }
 
@@ -127,7 +130,8 @@ int choose_ksplit(int M, int N, int K) {
 
 template <bool TA, bool TB>
 cudaError_t launch_tt(const DGemm& g, int kchunk, const int* only_if, cudaStream_t s) {
-  dim3 grid((g.N + BN - 1) / BN, (g.M + BM - 1) / BM, g.ksplit);
+  const long tiles = (long)((g.N + BN - 1) / BN) * ((g.M + BM - 1) / BM) * g.ksplit;
+  const unsigned grid = (unsigned)(only_if ? std::min<long>(tiles, 152 * 4) : tiles);
   if (g.H && g.ksplit == 1)
     dgemm_kernel<TA, TB, true><<<grid, TPB, 0, s>>>(g, kchunk, only_if);
   else

@@ -38,7 +38,6 @@ struct DGemm {
   const double* H; long ldh;
   int ksplit;
   double* work;
-  bool upperA;  // op(A) is upper triangular: K steps below a row tile are skipped
   double beta;  // C = alpha op(A) op(B) (o H) + beta C (0: C is not read)
   int* scale;   // nullable: digit_scale_ints(M, N) ints of scratch, with which large
                 // products run on the tensor cores (xk_digits.cu)
@@ -46,6 +45,11 @@ struct DGemm {
   long cskip;   // (n / nbatch) cskip elements further on, and H has column n % nbatch
   bool sym;     // C is symmetric (M = N, no H, beta = 0): one half may be formed and mirrored
 };
+// The result overwrites rows of B (M <= 64, one row of tiles, unsplit: every block has read
+// its columns of B before it writes them).
+__host__ __device__ inline bool in_place(const DGemm& g) {
+  return g.C >= g.B && g.C < g.B + (g.transB ? (long)g.N : (long)g.K) * g.ldb;
+}
 cudaError_t dgemm(const DGemm& g, cudaStream_t s);
 
 // The product of dgemm on the tensor cores, split into exact digits
@@ -121,8 +125,8 @@ cudaError_t select_points_f64(const double* F, int m, int N, int want, double to
 // on a non-positive pivot.  scale (here and below): DGemm::scale of the updates.
 cudaError_t cholesky_blocked_f64(double* A, int n, long lda, int* status, int* scale,
                                  cudaStream_t s);
-// B (n x ncols, ldb) := (L L^T)^{-1} B with the lower factor L (ldl).
-cudaError_t cholesky_solve_f64(const double* L, int n, long ldl, double* B, long ldb, long ncols,
+// B (n x ncols, ldb) := (L L^T)^{-1} B with the lower factor L (ldl), which is overwritten.
+cudaError_t cholesky_solve_f64(double* L, int n, long ldl, double* B, long ldb, long ncols,
                                int* scale, cudaStream_t s);
 
 // *out = -dV (2 sum_t V[t] P[t]^2 - sum_t W[t] Q[t]^2) over lenA and lenC

@@ -44,45 +44,84 @@ __global__ void copy_diag_kernel(const double* __restrict__ a, int n, long ld, d
     out[i] = a[(long)i * ld + i];
 }
 
-// Column c of B[k:k+kb, :] := L_kk^{-1} column (forward, lower = true) or
-// L_kk^{-T} column (backward, lower = false); one thread per column, the
-// block of L in shared memory (identity past kb), the column in registers.
-template <bool LOWER>
-__global__ void trsv_block_kernel(const double* __restrict__ L, long ldl, int k, int kb,
-                                  double* __restrict__ B, long ldb, long ncols) {
-  __shared__ double l[NB][NB + 1];  // with the diagonal's reciprocals: a division costs 30 FMAs
-  for (int t = threadIdx.x; t < NB * NB; t += blockDim.x) {
-    const int i = t / NB, j = t % NB;
-    double v = (i == j) ? 1.0 : 0.0;
-    if (i < kb && j < kb && j <= i) v = L[(long)(k + i) * ldl + k + j];
-    l[i][j] = i == j ? 1.0 / v : v;
+// The triangular solves chi = L^{-T} L^{-1} X_gR run as two sweeps of one product per
+// block row (64 rows of chi against every earlier or later one), with the 64 x 64
+// diagonal blocks inverted beforehand:
+//   forward   Y_k = D_k (B_k - sum_{j<k} L_kj Y_j)        D_k = L_kk^{-1}
+//   backward  X_k = D_k^T (Y_k - sum_{j>k} L_jk^T X_j)
+// The lower triangle of the factor takes F_kj = -D_k L_kj and D_k, the upper one
+// G_kj = -(L_jk D_k)^T, so that each is one product [F_k0 .. D_k] [Y_0 .. B_k] or
+// [D_k^T G_k,k+1 ..] [Y_k X_k+1 ..], in place.  Substitution inside the blocks ran at the
+// FP64 FMA rate: 17.6 of 62 ms at 1053 functions of 45^3 points, 3.5 ms this way.
+
+// D_k into the diagonal blocks (zeros above), one block of 64 threads per k: thread c
+// forms column c by forward substitution.
+__global__ void __launch_bounds__(NB) invert_diag_kernel(double* __restrict__ A, int n, long lda) {
+  __shared__ double l[NB][NB + 1], rd[NB];
+  const int k = blockIdx.x * NB, kb = min(NB, n - k), c = threadIdx.x;
+  double* D = A + (long)k * lda + k;
+  for (int i = 0; i < kb; ++i) l[i][c] = c <= i && c < kb ? D[(long)i * lda + c] : 0.0;
+  __syncthreads();
+  if (c < kb) rd[c] = 1.0 / l[c][c];
+  __syncthreads();
+  if (c >= kb) return;
+  double x[NB];
+#pragma unroll
+  for (int i = 0; i < NB; ++i) {
+    if (i < kb) {
+      double v = i == c ? 1.0 : 0.0;
+#pragma unroll
+      for (int j = 0; j < i; ++j) v = fma(-l[i][j], x[j], v);
+      x[i] = v * rd[i];
+      D[(long)i * lda + c] = i >= c ? x[i] : 0.0;
+    } else {
+      x[i] = 0.0;
+    }
+  }
+}
+
+// For block rows j > k (blockIdx.x: the pair, blockIdx.y: 16 of the 64 columns or rows):
+// upper: G_kj = -(L_jk D_k)^T into block (k, j); else F_jk = -D_j L_jk in place.
+__global__ void __launch_bounds__(256) scale_blocks_kernel(double* __restrict__ A, int n, long lda, int upper) {
+  __shared__ double l[NB][NB + 1], d[NB][NB + 1];
+  int j = (int)((sqrtf(8.0f * blockIdx.x + 1.0f) + 1.0f) * 0.5f);  // pair = j (j - 1) / 2 + k
+  while (j * (j - 1) / 2 > (int)blockIdx.x) --j;
+  while ((j + 1) * j / 2 <= (int)blockIdx.x) ++j;
+  const int k = (int)blockIdx.x - j * (j - 1) / 2;
+  const int jr = j * NB, kr = k * NB, jb = min(NB, n - jr);  // block row k < j is whole
+  const int q0 = blockIdx.y * 16, dr = upper ? kr : jr, db = upper ? NB : jb;
+  // in place: a block reads the 16 columns of L_jk it rewrites (F), or rows for G
+  for (int t = threadIdx.x; t < NB * NB; t += 256) {
+    const int r = t / NB, c = t % NB;
+    d[r][c] = r < db && c <= r ? A[(long)(dr + r) * lda + dr + c] : 0.0;
+    const bool mine = upper ? r >= q0 && r < q0 + 16 : c >= q0 && c < q0 + 16;
+    l[r][c] = mine && r < jb ? A[(long)(jr + r) * lda + kr + c] : 0.0;
   }
   __syncthreads();
-  for (long c = blockIdx.x * (long)blockDim.x + threadIdx.x; c < ncols;
-       c += (long)gridDim.x * blockDim.x) {
-    double y[NB];
-#pragma unroll
-    for (int j = 0; j < NB; ++j) y[j] = j < kb ? B[(long)(k + j) * ldb + c] : 0.0;
-    if (LOWER) {
-#pragma unroll
-      for (int j = 0; j < NB; ++j) {
-        double v = y[j];
-#pragma unroll
-        for (int p = 0; p < j; ++p) v -= l[j][p] * y[p];
-        y[j] = v * l[j][j];
-      }
+  for (int t = threadIdx.x; t < 16 * NB; t += 256) {
+    double s = 0.0;
+    if (upper) {
+      const int r = q0 + t / NB, c = t % NB;  // (L_jk D_k)[r][c]
+      for (int p = c; p < NB; ++p) s = fma(l[r][p], d[p][c], s);
+      if (r < jb) A[(long)(kr + c) * lda + jr + r] = -s;
     } else {
-#pragma unroll
-      for (int j = NB - 1; j >= 0; --j) {
-        double v = y[j];
-#pragma unroll
-        for (int p = j + 1; p < NB; ++p) v -= l[p][j] * y[p];
-        y[j] = v * l[j][j];
-      }
+      const int r = t / 16, c = q0 + t % 16;  // (D_j L_jk)[r][c]
+      for (int p = 0; p <= r; ++p) s = fma(d[r][p], l[p][c], s);
+      if (r < jb) A[(long)(jr + r) * lda + kr + c] = -s;
     }
-#pragma unroll
-    for (int j = 0; j < NB; ++j)
-      if (j < kb) B[(long)(k + j) * ldb + c] = y[j];
+  }
+}
+
+// The diagonal blocks transposed in place.
+__global__ void __launch_bounds__(256) transpose_diag_kernel(double* __restrict__ A, int n, long lda) {
+  const int k = blockIdx.x * NB, kb = min(NB, n - k);
+  double* D = A + (long)k * lda + k;
+  for (int t = threadIdx.x; t < kb * kb; t += 256) {
+    const int i = t / kb, j = t % kb;
+    if (j >= i) continue;
+    const double v = D[(long)i * lda + j];
+    D[(long)i * lda + j] = D[(long)j * lda + i];
+    D[(long)j * lda + i] = v;
   }
 }
 
@@ -301,7 +340,7 @@ cudaError_t cholesky_blocked_f64(double* A, int n, long lda, int* status, int* s
       // A22 -= L21 L21^T (the whole square; only its lower triangle is used)
       DGemm g{rest, rest, kb, A + (long)(k + kb) * lda + k, lda, false,
               A + (long)(k + kb) * lda + k, lda, true, A + (long)(k + kb) * lda + k + kb, lda,
-              -1.0, nullptr, 0, 1, nullptr, false, 1.0, scale};
+              -1.0, nullptr, 0, 1, nullptr, 1.0, scale};
       e = dgemm(g, s);
       if (e != cudaSuccess) return e;
     }
@@ -309,35 +348,33 @@ cudaError_t cholesky_blocked_f64(double* A, int n, long lda, int* status, int* s
   return cudaGetLastError();
 }
 
-cudaError_t cholesky_solve_f64(const double* L, int n, long ldl, double* B, long ldb, long ncols,
+// B := (L L^T)^{-1} B; L (lower) is overwritten.
+cudaError_t cholesky_solve_f64(double* L, int n, long ldl, double* B, long ldb, long ncols,
                                int* scale, cudaStream_t s) {
-  const int cb = nblocks(ncols);
-  // forward: L Y = B, block rows in order (left-looking updates)
-  for (int k = 0; k < n; k += NB) {
-    const int kb = std::min(NB, n - k);
-    if (k > 0) {
-      DGemm g{kb, (int)ncols, k, L + (long)k * ldl, ldl, false, B, ldb, false, B + (long)k * ldb,
-              ldb, -1.0, nullptr, 0, 1, nullptr, false, 1.0, scale};
-      cudaError_t e = dgemm(g, s);
-      if (e != cudaSuccess) return e;
-    }
-    trsv_block_kernel<true><<<cb, 256, 0, s>>>(L, ldl, k, kb, B, ldb, ncols);
-    count_launch();
+  const int nb = (n + NB - 1) / NB;
+  const unsigned pairs = (unsigned)(nb * (nb - 1) / 2);
+  invert_diag_kernel<<<(unsigned)nb, NB, 0, s>>>(L, n, ldl);
+  count_launch();
+  if (pairs > 0) {
+    scale_blocks_kernel<<<dim3(pairs, NB / 16), 256, 0, s>>>(L, n, ldl, 1);
+    scale_blocks_kernel<<<dim3(pairs, NB / 16), 256, 0, s>>>(L, n, ldl, 0);
+    count_launch(2);
   }
-  // backward: L^T X = Y, block rows in reverse order
-  const int last = ((n - 1) / NB) * NB;
-  for (int k = last; k >= 0; k -= NB) {
-    const int kb = std::min(NB, n - k);
-    if (k + kb < n) {
-      // B_k -= L[k+kb:n, k:k+kb]^T X[k+kb:n]
-      DGemm g{kb, (int)ncols, n - k - kb, L + (long)(k + kb) * ldl + k, ldl, true,
-              B + (long)(k + kb) * ldb, ldb, false, B + (long)k * ldb, ldb, -1.0, nullptr, 0, 1,
-              nullptr, false, 1.0, scale};
-      cudaError_t e = dgemm(g, s);
-      if (e != cudaSuccess) return e;
-    }
-    trsv_block_kernel<false><<<cb, 256, 0, s>>>(L, ldl, k, kb, B, ldb, ncols);
-    count_launch();
+  auto row = [&](int k, int k0, int k1) {  // B_k := L[k rows, k0:k1] B[k0:k1]
+    DGemm g{std::min(NB, n - k), (int)ncols, k1 - k0, L + (long)k * ldl + k0, ldl, false,
+            B + (long)k0 * ldb, ldb, false, B + (long)k * ldb, ldb, 1.0, nullptr, 0, 1, nullptr, 0.0,
+            scale};
+    return dgemm(g, s);
+  };
+  for (int k = 0; k < n; k += NB) {
+    cudaError_t e = row(k, 0, std::min(n, k + NB));
+    if (e != cudaSuccess) return e;
+  }
+  transpose_diag_kernel<<<(unsigned)nb, 256, 0, s>>>(L, n, ldl);
+  count_launch();
+  for (int k = (nb - 1) * NB; k >= 0; k -= NB) {
+    cudaError_t e = row(k, k, n);
+    if (e != cudaSuccess) return e;
   }
   return cudaGetLastError();
 }
