@@ -226,6 +226,16 @@ struct xk_handle {
 
   xk::MixedState* mixed = nullptr;
   Slot slots[kSlots];
+  // One pinned block for the slots and for the small results of the blocking calls
+  // (res: E_x, E_K or E_J; res_st: the status word, or that of a factorisation): a block
+  // each cost 0.2 ms to allocate and as much to free.
+  char* pinned = nullptr;
+  double* res = nullptr;
+  int* res_st = nullptr;
+  // One device block that dalloc carves the tables and scratch from (a cudaMalloc and
+  // cudaFree each took 0.2 to 0.4 ms); later buffers get their own.
+  char* arena = nullptr;
+  size_t arena_left = 0;
 
   // one tensor-path build captured as a CUDA graph on first use (C in h->C,
   // K and E_x in h->K, h->Ex), replayed while step timing is off; dropped
@@ -312,6 +322,13 @@ bool valid_sizes(int64_t Ng, int32_t N, int32_t n, int32_t Naux) {
 
 template <class T>
 cudaError_t dalloc(xk_handle* h, T** p, size_t elems) {
+  const size_t bytes = (std::max<size_t>(elems, 1) * sizeof(T) + 255) / 256 * 256;
+  if (bytes <= h->arena_left) {
+    *p = reinterpret_cast<T*>(h->arena);
+    h->arena += bytes;
+    h->arena_left -= bytes;
+    return cudaSuccess;
+  }
   void* q = nullptr;
   cudaError_t e = cudaMalloc(&q, std::max<size_t>(elems, 1) * sizeof(T));
   if (e != cudaSuccess) return e;
@@ -338,11 +355,8 @@ void free_handle(xk_handle* h) {
   if (h->stream) cudaStreamSynchronize(h->stream);
   for (Slot& s : h->slots) {
     if (s.done) cudaEventDestroy(s.done);
-    if (s.C) cudaFreeHost(s.C);
-    if (s.K) cudaFreeHost(s.K);
-    if (s.Ex) cudaFreeHost(s.Ex);
-    if (s.st) cudaFreeHost(s.st);
   }
+  if (h->pinned) cudaFreeHost(h->pinned);
   drop_graph(h);
   if (h->mixed) xk::mixed_destroy(h->mixed);
   fold_marks(h);
@@ -352,19 +366,15 @@ void free_handle(xk_handle* h) {
   delete h;
 }
 
-// Status word of the tensor-path kernels of the builds enqueued so far on
-// `s`: read and cleared in stream order (so a later build on the stream
-// starts from zero), then waited for.  0 when none gave up.
-int take_status(xk_handle* h, cudaStream_t s, cudaError_t* err) {
-  *err = cudaSuccess;
-  if (!h->mixed) return 0;
-  int st[4] = {0, 0, 0, 0};
+// Status word of the tensor-path kernels of the builds enqueued so far on `s`: copied to
+// h->res_st and cleared in stream order (so a later build on the stream starts from
+// zero); 0 once the stream has been waited for when none gave up.
+cudaError_t enqueue_status(xk_handle* h, cudaStream_t s) {
+  h->res_st[0] = 0;
+  if (!h->mixed) return cudaSuccess;
   int* dev = xk::mixed_status_ptr(h->mixed);
-  cudaError_t e = cudaMemcpyAsync(st, dev, 16, cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(dev, 0, 16, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  *err = e;
-  return st[0];
+  cudaError_t e = cudaMemcpyAsync(h->res_st, dev, 16, cudaMemcpyDeviceToHost, s);
+  return e == cudaSuccess ? cudaMemsetAsync(dev, 0, 16, s) : e;
 }
 
 // Records the start or the end of `step` when timing is on.
@@ -707,6 +717,17 @@ static int setup_impl(int64_t Ng, int32_t N, int32_t n, int32_t Naux, const doub
   if (e != cudaSuccess) return bail(cuda_fail(e, "cudaStreamCreate"));
 
   const size_t ng = (size_t)Ng, na = (size_t)Naux;
+  {  // everything below but the tensor path's own tables, in one block when there is one
+    const size_t bytes = mode == XK_FP64 ? need : need - xk::mixed_footprint(Ng, N, n, ga, Naux);
+    void* q = nullptr;
+    if (cudaMalloc(&q, bytes) == cudaSuccess) {
+      h->allocs.push_back(q);
+      h->arena = static_cast<char*>(q);
+      h->arena_left = bytes;
+    } else {
+      (void)cudaGetLastError();
+    }
+  }
 #define XK_ALLOC(ptr, elems)                                  \
   do {                                                        \
     cudaError_t e_ = dalloc(h, &(ptr), (elems));              \
@@ -812,13 +833,24 @@ static int setup_impl(int64_t Ng, int32_t N, int32_t n, int32_t Naux, const doub
     if (e != cudaSuccess) return bail(cuda_fail(e, "xk_setup mixed tables"));
   }
 #undef XK_ALLOC
-  for (Slot& s : h->slots) {
-    e = cudaHostAlloc((void**)&s.C, (size_t)N * n * 8, cudaHostAllocDefault);
-    if (e == cudaSuccess) e = cudaHostAlloc((void**)&s.K, (size_t)N * n * 8, cudaHostAllocDefault);
-    if (e == cudaSuccess) e = cudaHostAlloc((void**)&s.Ex, 16, cudaHostAllocDefault);
-    if (e == cudaSuccess) e = cudaHostAlloc((void**)&s.st, 16, cudaHostAllocDefault);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s.done, cudaEventDisableTiming);
+  h->arena_left = 0;  // later buffers are admitted and allocated by themselves
+  {
+    const size_t kb = ((size_t)N * n * 8 + 255) / 256 * 256, per = 2 * kb + 512;
+    e = cudaHostAlloc((void**)&h->pinned, kSlots * per + 512, cudaHostAllocDefault);
     if (e != cudaSuccess) return bail(cuda_fail(e, "xk_setup slots"));
+    char* p = h->pinned;
+    h->res = reinterpret_cast<double*>(p);
+    h->res_st = reinterpret_cast<int*>(p + 256);
+    p += 512;
+    for (Slot& s : h->slots) {
+      s.C = reinterpret_cast<double*>(p);
+      s.K = reinterpret_cast<double*>(p + kb);
+      s.Ex = reinterpret_cast<double*>(p + 2 * kb);
+      s.st = reinterpret_cast<int*>(p + 2 * kb + 256);
+      p += per;
+      e = cudaEventCreateWithFlags(&s.done, cudaEventDisableTiming);
+      if (e != cudaSuccess) return bail(cuda_fail(e, "xk_setup slots"));
+    }
   }
   if (isdf_tmp) {  // the ISDF set-up's temporaries are freed: return their bytes
     h->footprint = need;
@@ -1002,18 +1034,16 @@ int xk_build(xk_handle* h, const double* C, double* K_out, double* Ex) {
   XK_CUDA(cudaMemcpyAsync(h->C, C, kb, cudaMemcpyHostToDevice, h->stream));
   int rc = enqueue_build(h);
   if (rc != XK_OK) return rc;
+  // the small results go ahead of K into pinned memory: one wait for all
+  XK_CUDA(cudaMemcpyAsync(h->res, h->Ex, 8, cudaMemcpyDeviceToHost, h->stream));
+  XK_CUDA(enqueue_status(h, h->stream));
   XK_CUDA(cudaMemcpyAsync(K_out, h->K, kb, cudaMemcpyDeviceToHost, h->stream));
-  XK_CUDA(cudaMemcpyAsync(Ex, h->Ex, 8, cudaMemcpyDeviceToHost, h->stream));
   XK_CUDA(cudaStreamSynchronize(h->stream));
+  *Ex = h->res[0];
   h->has_build = true;
-  {
-    cudaError_t e = cudaSuccess;
-    const int st = take_status(h, h->stream, &e);
-    if (e != cudaSuccess) return cuda_fail(e, "xk_build status");
-    if (st != 0)
-      return fail(XK_ETIMEDOUT, "xk_build: a bounded wait inside a kernel gave up (code " +
-                                    std::to_string(st) + ")");
-  }
+  if (h->res_st[0] != 0)
+    return fail(XK_ETIMEDOUT, "xk_build: a bounded wait inside a kernel gave up (code " +
+                                  std::to_string(h->res_st[0]) + ")");
   return XK_OK;
 }
 
@@ -1048,16 +1078,12 @@ int xk_build_full(xk_handle* h, const double* C, double* K_out) {
   XK_CUDA(cudaMemcpyAsync(h->Ce, C, (size_t)h->N * h->n * 8, cudaMemcpyHostToDevice, h->stream));
   int rc = enqueue_full(h);
   if (rc != XK_OK) return rc;
+  XK_CUDA(enqueue_status(h, h->stream));
   XK_CUDA(cudaMemcpyAsync(K_out, h->Kf, (size_t)h->N * h->N * 8, cudaMemcpyDeviceToHost, h->stream));
   XK_CUDA(cudaStreamSynchronize(h->stream));
-  {
-    cudaError_t e = cudaSuccess;
-    const int st = take_status(h, h->stream, &e);
-    if (e != cudaSuccess) return cuda_fail(e, "xk_build_full status");
-    if (st != 0)
-      return fail(XK_ETIMEDOUT, "xk_build_full: a bounded wait inside a kernel gave up (code " +
-                                    std::to_string(st) + ")");
-  }
+  if (h->res_st[0] != 0)
+    return fail(XK_ETIMEDOUT, "xk_build_full: a bounded wait inside a kernel gave up (code " +
+                                  std::to_string(h->res_st[0]) + ")");
   return XK_OK;
 }
 
@@ -1126,9 +1152,10 @@ int xk_coulomb(xk_handle* h, int32_t grid, double L, const double* C, double* J_
     XK_CUDA(xk::dgemm(gj, s));
     XK_CUDA(xk::dot_f64(h->Jrho, h->Jv, (long)ng, h->dV, h->red, h->Jout + (size_t)N * N, s));
   }
+  XK_CUDA(cudaMemcpyAsync(h->res, h->Jout + (size_t)N * N, 8, cudaMemcpyDeviceToHost, s));
   XK_CUDA(cudaMemcpyAsync(J_out, h->Jout, (size_t)N * N * 8, cudaMemcpyDeviceToHost, s));
-  XK_CUDA(cudaMemcpyAsync(E_J, h->Jout + (size_t)N * N, 8, cudaMemcpyDeviceToHost, s));
   XK_CUDA(cudaStreamSynchronize(s));
+  *E_J = h->res[0];
   return XK_OK;
 }
 
@@ -1140,16 +1167,13 @@ int xk_energy(xk_handle* h, const double* C, double* Ex) {
   XK_CUDA(cudaMemcpyAsync(h->Ce, C, cb, cudaMemcpyHostToDevice, h->stream));
   int rc = enqueue_energy(h);
   if (rc != XK_OK) return rc;
-  XK_CUDA(cudaMemcpyAsync(Ex, h->Ce + (size_t)h->N * h->n, 8, cudaMemcpyDeviceToHost, h->stream));
+  XK_CUDA(cudaMemcpyAsync(h->res, h->Ce + (size_t)h->N * h->n, 8, cudaMemcpyDeviceToHost, h->stream));
+  XK_CUDA(enqueue_status(h, h->stream));
   XK_CUDA(cudaStreamSynchronize(h->stream));
-  {
-    cudaError_t e = cudaSuccess;
-    const int st = take_status(h, h->stream, &e);
-    if (e != cudaSuccess) return cuda_fail(e, "xk_energy status");
-    if (st != 0)
-      return fail(XK_ETIMEDOUT, "xk_energy: a bounded wait inside a kernel gave up (code " +
-                                    std::to_string(st) + ")");
-  }
+  *Ex = h->res[0];
+  if (h->res_st[0] != 0)
+    return fail(XK_ETIMEDOUT, "xk_energy: a bounded wait inside a kernel gave up (code " +
+                                  std::to_string(h->res_st[0]) + ")");
   return XK_OK;
 }
 
@@ -1181,7 +1205,7 @@ int xk_ace(xk_handle* h, double* Kij_out, double* xi_out, double* sign_out, int*
   DeviceGuard g(h->device);
   cudaStream_t s = h->stream;
   const int N = h->N, n = h->n;
-  int st = 0, br = 0;
+  int br = 0;
   std::vector<double> sg(n, 1.0);
   // K_ij: from 2e7 multiply-adds the digit product (then symmetrised), below the
   // kernel that spreads it over the SMs
@@ -1198,11 +1222,11 @@ int xk_ace(xk_handle* h, double* Kij_out, double* xi_out, double* sign_out, int*
   // the Cholesky branch's vectors are formed and copied before the host has seen
   // whether it holds: one wait instead of two
   XK_CUDA(xk::trsm_right_lt_f64(h->Lf, n, h->K, N, h->xi, s, h->U));
-  XK_CUDA(cudaMemcpyAsync(&st, h->status, 4, cudaMemcpyDeviceToHost, s));
+  XK_CUDA(cudaMemcpyAsync(h->res_st, h->status, 4, cudaMemcpyDeviceToHost, s));
   XK_CUDA(cudaMemcpyAsync(Kij_out, h->Kij, (size_t)n * n * 8, cudaMemcpyDeviceToHost, s));
   XK_CUDA(cudaMemcpyAsync(xi_out, h->xi, (size_t)N * n * 8, cudaMemcpyDeviceToHost, s));
   XK_CUDA(cudaStreamSynchronize(s));
-  if (st != 0) {
+  if (h->res_st[0] != 0) {
     br = 1;
     XK_CUDA(cudaMemcpyAsync(h->Lf, h->Kij, (size_t)n * n * 8, cudaMemcpyDeviceToDevice, s));
     XK_CUDA(xk::jacobi_eig_f64(h->Lf, h->U, n, 60, h->status + 1, s));
@@ -1530,18 +1554,19 @@ int xk_batch_build(xk_batch* b, const double* const* C, double* const* K_out, do
   xk::g_launches.fetch_add(b->launches);
   for (size_t i = 0; i < count; ++i) {
     xk_handle* h = b->hs[i];
-    XK_CUDA(cudaMemcpyAsync(K_out[i], h->K, (size_t)h->N * h->n * 8, cudaMemcpyDeviceToHost, b->stream));
-    XK_CUDA(cudaMemcpyAsync(Ex_out + i, h->Ex, 8, cudaMemcpyDeviceToHost, b->stream));
+    XK_CUDA(cudaMemcpyAsync(h->res, h->Ex, 8, cudaMemcpyDeviceToHost, b->stream));
+    XK_CUDA(enqueue_status(h, b->stream));  // each read and cleared before returning
   }
+  for (size_t i = 0; i < count; ++i)
+    XK_CUDA(cudaMemcpyAsync(K_out[i], b->hs[i]->K, (size_t)b->hs[i]->N * b->hs[i]->n * 8,
+                            cudaMemcpyDeviceToHost, b->stream));
   XK_CUDA(cudaStreamSynchronize(b->stream));
-  // every member's status word, each read and cleared before returning
   int first = 0;
-  for (xk_handle* h : b->hs) {
+  for (size_t i = 0; i < count; ++i) {
+    xk_handle* h = b->hs[i];
     h->has_build = true;
-    cudaError_t e = cudaSuccess;
-    const int st = take_status(h, b->stream, &e);
-    if (e != cudaSuccess) return cuda_fail(e, "xk_batch_build status");
-    if (st != 0 && first == 0) first = st;
+    Ex_out[i] = h->res[0];
+    if (first == 0) first = h->res_st[0];
   }
   if (first != 0)
     return fail(XK_ETIMEDOUT, "xk_batch_build: a bounded wait inside a kernel gave up (code " +
