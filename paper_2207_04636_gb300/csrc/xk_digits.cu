@@ -16,15 +16,21 @@
 // operands and the dropped levels: 5e-17 to 3e-16 of the 2-norm on the
 // products of a build, where a chain of FP64 FMAs leaves 1.4e-16 to 9e-15.
 //
-// What bounds it: a 128 x 64 tile takes 34 SS instructions per K = 16 step,
-// each of which reads 6 KB of operands from shared memory at 128 B/clk
-// (48 clk); turning operands into digits (about 20 integer operations an
-// element, at 64 a clock and SM) runs beside them.  FP64 FMAs on the CUDA cores
-// run at 2 a clock and SM.  Measured on random operands (GB300, us; FP64 FMA
-// kernel before): 1755 x 54 x 91125: 970 (14500), 54 x 91125 x 1755: 930
-// (17500), 1755 x 91125 x 54 (stores bound it): 1640 (17700),
-// 351 x 351 x 91125: 910 (26600), 1053 x 1053 x 91125: 8150.  A 27-centre FP64
-// build went from 64.7 to 4.8 ms, its Coulomb matrix from 30.6 to 1.71 ms.
+// What bounds it: a 128 x 64 tile takes 34 digit products per K = 16 step, 1088
+// clocks of the tensor cores.  One instruction forms up to four of them: the digits of Y
+// lie one after another in shared memory and the levels in TMEM, so N = 256 rows of
+// Y's digits j .. j + 3 against one digit of X give levels i + j .. i + j + 3, and the
+// operands are read 112 KB at a time instead of 204 (875 clocks instead of 1600).  Beside
+// them run the workers: about 13 integer operations an element (64 a clock and SM),
+// their loads, and the drains.  Measured with parts left out (1053 x 1053 x 91125,
+// 6.6 ms): matrix instructions and drains 4.5, workers alone 5.4, workers without loads
+// 4.2 ms; refilling a register pair as soon as its digits are formed, to have loads in
+// flight longer, made it 7.0.
+// FP64 FMAs on the CUDA cores run at 2 a clock and SM.  Measured on random operands
+// (GB300, us; FP64 FMA kernel before): 1755 x 54 x 91125: 814 (14500), 54 x 91125 x
+// 1755: 821 (17500), 1755 x 91125 x 54 (taking and storing the results bounds it): 1270
+// (17700), 351 x 351 x 91125: 816 (26600), 1053 x 1053 x 91125: 6630.  A 27-centre
+// FP64 build went from 64.7 to 4.06 ms, its Coulomb matrix from 30.6 to 1.12 ms.
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
@@ -65,7 +71,6 @@ struct DOperand {
   int rows;
   int kc;
   const int* scale;  // per row: high word of max |row|
-  int pairs;         // kc: rows start on 16-byte boundaries
 };
 
 struct DArgs {
@@ -91,60 +96,67 @@ struct DArgs {
 // |x| 2^-e <= 1 - 2^-7.  A row of zeros gets 0.
 __device__ __forceinline__ int row_exp(int hi) { return hi ? ((hi + (1 << 14)) >> 20) - 1022 : 0; }
 
+__device__ __forceinline__ uint32_t row_e21(int hi) {
+  return ((uint32_t)(row_exp(hi) + 1022) << 21) | 0x1fffffu;
+}
+
 // Rows whose largest |x| is infinite, NaN or below 2^-900 (where an element's
 // subnormals would count) are not split.
 __device__ __forceinline__ bool row_unfit(int hi) {
   return hi >= 0x7ff00000 || (hi > 0 && hi < ((1023 - 900) << 20));
 }
 
-// The seven digits of x on the grid 2^(e - 55), each plus 128, in the low 7
-// bytes (most significant digit in byte 6).  e20 = (e + 1022) << 20.  Integer
-// operations run at 64 a clock and SM here, so they are what the split costs: x =
-// m 2^(ex - 1078) with m of 56 bits (a subnormal x, taken for a normal one, is
-// below the grid) is shifted by t = e + 1022 - ex >= 0 to one bit below the
-// grid; sign, rounding and the offsets of the digits are then one sum:
-// (y + 1 + 2 sum 128 2^(8 i)) >> 1, or with -y = ~y + 1, whose half rounds the
-// same way without the 1.
-__device__ __forceinline__ uint2 digits_of(double x, int e20) {
+// The seven digits of |x| on the grid 2^(e - 55), each plus 128, in the upper 7
+// bytes (most significant digit in byte 7).  e21 = (e + 1022) 2^21 + 2^21 - 1.  Integer
+// operations run at 64 a clock and SM here, so they are what the split costs: |x| =
+// m 2^(ex - 1085) with m of 63 bits (a subnormal x, taken for a normal one, is
+// below the grid) is shifted by t = e + 1022 - ex >= 0 to eight bits below the
+// grid, t being what is left of e21 - 2 high word (one multiply-add, on the other pipe;
+// the doubling drops the sign) above its mantissa bits; one sum then adds the offsets
+// 128 2^(8 i) of the digits and half a grid step.
+__device__ __forceinline__ uint2 digits_of(double x, uint32_t e21) {
   const uint32_t xh = __double2hiint(x), xl = __double2loint(x);
-  const uint32_t t = (uint32_t)(e20 - (int)(xh & 0x7ff00000u)) >> 20;
+  const uint32_t t = (e21 - 2u * xh) >> 21;
   const uint32_t mh = (xh & 0xfffffu) | 0x100000u;
   const unsigned long long m =
-      ((unsigned long long)__funnelshift_l(xl, mh, 3) << 32) | (xl << 3);
+      ((unsigned long long)__funnelshift_l(xl, mh, 10) << 32) | (xl << 10);
   unsigned long long y;
   asm("shr.u64 %0, %1, %2;" : "=l"(y) : "l"(m), "r"(t));  // t > 63 gives 0
-  const uint32_t sg = (uint32_t)((int)xh >> 31);
-  const unsigned long long z =
-      ((((unsigned long long)((uint32_t)(y >> 32) ^ sg)) << 32) | ((uint32_t)y ^ sg)) +
-      0x0101010101010101ull;
-  return make_uint2((uint32_t)(z >> 1), (uint32_t)(z >> 33));
+  y += 0x8080808080808080ull;
+  return make_uint2((uint32_t)y, (uint32_t)(y >> 32));
 }
 
-// FP16 pairs (digit of a, digit of b), most significant first, from the digit
-// words of two elements: byte + 1024 = 0x64xx, less 1024 + 128.
-__device__ __forceinline__ void digit_pairs(const uint2& a, const uint2& b, uint32_t (&o)[kDig]) {
+// FP16 pairs (digit of x, digit of y), most significant first: byte + 1024 = 0x64xx,
+// less 1024 + 128, times the element's sign (+-1 from the high words' sign bits).
+__device__ __forceinline__ void digit_pairs(double x, double y, uint32_t e21, uint32_t (&o)[kDig]) {
+  const uint2 a = digits_of(x, e21), b = digits_of(y, e21);
   const uint32_t c = 0x64646464u;
-  const uint32_t w0 = __byte_perm(a.x, b.x, 0x5410), w1 = __byte_perm(a.x, b.x, 0x7632),
-                 w2 = __byte_perm(a.y, b.y, 0x5410), w3 = __byte_perm(a.y, b.y, 0x6262);
-  o[6] = __byte_perm(w0, c, 0x4240); o[5] = __byte_perm(w0, c, 0x4341);
-  o[4] = __byte_perm(w1, c, 0x4240); o[3] = __byte_perm(w1, c, 0x4341);
-  o[2] = __byte_perm(w2, c, 0x4240); o[1] = __byte_perm(w2, c, 0x4341);
-  o[0] = __byte_perm(w3, c, 0x4140);
-  const __half2 off = __half2half2(__ushort_as_half(0x6480));
+  const uint32_t w0 = __byte_perm(a.y, b.y, 0x7632), w1 = __byte_perm(a.y, b.y, 0x5410),
+                 w2 = __byte_perm(a.x, b.x, 0x7632), w3 = __byte_perm(a.x, b.x, 0x5151);
+  o[0] = __byte_perm(w0, c, 0x4341); o[1] = __byte_perm(w0, c, 0x4240);
+  o[2] = __byte_perm(w1, c, 0x4341); o[3] = __byte_perm(w1, c, 0x4240);
+  o[4] = __byte_perm(w2, c, 0x4341); o[5] = __byte_perm(w2, c, 0x4240);
+  o[6] = __byte_perm(w3, c, 0x4140);
+  const uint32_t sg =
+      (__byte_perm(__double2hiint(x), __double2hiint(y), 0x7632) & 0x80008000u) | 0x3c003c00u;
+  const __half2 s = *reinterpret_cast<const __half2*>(&sg);
+  const __half2 off = __hmul2(s, __half2half2(__ushort_as_half(0xe480)));  // -1152
 #pragma unroll
   for (int i = 0; i < kDig; ++i) {
-    const __half2 r = __hsub2(*reinterpret_cast<__half2*>(&o[i]), off);
+    const __half2 r = __hfma2(*reinterpret_cast<__half2*>(&o[i]), s, off);
     o[i] = *reinterpret_cast<const uint32_t*>(&r);
   }
 }
 
 // A block of one operand passes through the registers of the 512 workers, n
-// elements each, n = 8 (X, 128 rows) or 4 (Y, 64 rows):
-//  * K contiguous in memory: lane l holds the pairs k = 2 (l % 16), +1 of the
-//    rows n w + l / 16 + 2 i of warp w, so that a load reads 256 B of a row and a
-//    store writes whole 128-byte lines (one 4-byte digit pair per lane);
-//  * rows contiguous: a thread holds n successive k of one row (lanes along the
-//    rows) and stores 2 n bytes of each digit.
+// elements each, n = 8 (X, 128 rows) or 4 (Y, 64 rows).  Position 2 j of the
+// block's K order holds term j and position 2 j + 1 term j + 16, in both operands:
+//  * K contiguous in memory: lane l holds the pairs k = l % 16, + 16 of the rows
+//    n w + l / 16 + 2 i of warp w, so that a load reads whole 128-byte pieces of two rows
+//    (on any alignment) and a store writes whole 128-byte lines (one 4-byte digit
+//    pair per lane);
+//  * rows contiguous: a thread holds n successive positions of one row (lanes along
+//    the rows) and stores 2 n bytes of each digit.
 // Rows past the operand's last are read as that one (nothing of them is stored).
 template <int n, bool KC>
 __device__ __forceinline__ void load_block(const DOperand& o, int row0, long k0, long kend, int tid,
@@ -153,39 +165,39 @@ __device__ __forceinline__ void load_block(const DOperand& o, int row0, long k0,
   const bool whole = k0 + DK <= kend;
   if constexpr (KC) {
     const int r = row0 + (tid >> 5) * n + ((tid >> 4) & 1);
-    const long k = k0 + 2 * (tid & 15);
+    const long k = k0 + (tid & 15);
     const double* p = o.p + k;
-    if (whole && o.pairs) {
-#pragma unroll
-      for (int i = 0; i < n / 2; ++i) {
-        const double2 t = __ldg(reinterpret_cast<const double2*>(p + (long)min(r + 2 * i, o.rows - 1) * o.ld));
-        v[2 * i] = t.x;
-        v[2 * i + 1] = t.y;
-      }
-    } else if (whole) {
+    if (whole) {
 #pragma unroll
       for (int i = 0; i < n / 2; ++i) {
         const double* q = p + (long)min(r + 2 * i, o.rows - 1) * o.ld;
         v[2 * i] = __ldg(q);
-        v[2 * i + 1] = __ldg(q + 1);
+        v[2 * i + 1] = __ldg(q + 16);
       }
     } else {
 #pragma unroll
       for (int i = 0; i < n / 2; ++i) {
         const double* q = p + (long)min(r + 2 * i, o.rows - 1) * o.ld;
         v[2 * i] = k < kend ? __ldg(q) : 0.0;
-        v[2 * i + 1] = k + 1 < kend ? __ldg(q + 1) : 0.0;
+        v[2 * i + 1] = k + 16 < kend ? __ldg(q + 16) : 0.0;
       }
     }
   } else {
-    const long k = k0 + n * (tid / R);
+    const long k = k0 + n / 2 * (tid / R);
     const double* p = o.p + k * o.ld + min(row0 + tid % R, o.rows - 1);
+    const long half = 16 * o.ld;
     if (whole) {
 #pragma unroll
-      for (int i = 0; i < n; ++i, p += o.ld) v[i] = __ldg(p);
+      for (int i = 0; i < n / 2; ++i, p += o.ld) {
+        v[2 * i] = __ldg(p);
+        v[2 * i + 1] = __ldg(p + half);
+      }
     } else {
 #pragma unroll
-      for (int i = 0; i < n; ++i, p += o.ld) v[i] = k + i < kend ? __ldg(p) : 0.0;
+      for (int i = 0; i < n / 2; ++i, p += o.ld) {
+        v[2 * i] = k + i < kend ? __ldg(p) : 0.0;
+        v[2 * i + 1] = k + i + 16 < kend ? __ldg(p + half) : 0.0;
+      }
     }
   }
 }
@@ -196,27 +208,29 @@ __device__ __forceinline__ int block_row(int w, int l) {
   return KC ? w * n + l % n : (32 * w + l) % (16 * n);
 }
 
-// Digits of the block into the stage; ex: (e + 1022) << 20 of the rows block_row(w, 0..31).
+// Digits of the block into the stage; ex: e21 (digits_of) of the rows block_row(w, 0..31).
 template <int n, bool KC>
-__device__ __forceinline__ void store_block(uint8_t* st, const int* ex, int tid, const double (&v)[n]) {
+__device__ __forceinline__ void store_block(uint8_t* st, const uint32_t* ex, int tid, const double (&v)[n]) {
   constexpr int R = 16 * n, PLANE = R * DK * 2;
   if constexpr (KC) {
     // rows r0 + 2 i: the swizzle's chunk is that of r0 with bit 1 of r, i.e. bit 0 of i, flipped
     const int r0 = (tid >> 5) * n + ((tid >> 4) & 1), l = tid & 15;
 #pragma unroll
     for (int i = 0; i < n / 2; ++i) {
-      const int r = r0 + 2 * i, e = ex[((tid >> 4) & 1) + 2 * i];
+      const int r = r0 + 2 * i;
+      const uint32_t e = ex[((tid >> 4) & 1) + 2 * i];
       uint32_t o[kDig];
-      digit_pairs(digits_of(v[2 * i], e), digits_of(v[2 * i + 1], e), o);
+      digit_pairs(v[2 * i], v[2 * i + 1], e, o);
       uint32_t* d = reinterpret_cast<uint32_t*>(st + r * 64 + (((l >> 2) ^ ((r >> 1) & 3)) << 4) + (l & 3) * 4);
 #pragma unroll
       for (int q = 0; q < kDig; ++q) d[q * (PLANE / 4)] = o[q];
     }
   } else {
-    const int r = tid % R, q = tid / R, e = ex[tid & 31];  // q: which n of the 32 k
+    const int r = tid % R, q = tid / R;  // q: which n of the 32 k
+    const uint32_t e = ex[tid & 31];
     uint32_t o[n / 2][kDig];
 #pragma unroll
-    for (int i = 0; i < n / 2; ++i) digit_pairs(digits_of(v[2 * i], e), digits_of(v[2 * i + 1], e), o[i]);
+    for (int i = 0; i < n / 2; ++i) digit_pairs(v[2 * i], v[2 * i + 1], e, o[i]);
     const int byte = q * n * 2;  // within the row's 64 bytes
     uint8_t* d = st + r * 64 + (((byte >> 4) ^ ((r >> 1) & 3)) << 4) + (byte & 15);
 #pragma unroll
@@ -237,29 +251,27 @@ __device__ __forceinline__ double pack_f64(long long hi, uint32_t lo, int E) {
   const uint32_t sign = w2 & 0x80000000u;
   if (sign) {
     w0 = 0u - w0;
-    w1 = ~w1;
-    w2 = ~w2;
-    if (w0 == 0) {
-      w1 += 1;
-      w2 += w1 == 0;
-    }
+    const unsigned long long m = ~(unsigned long long)hi + (w0 == 0);
+    w1 = (uint32_t)m;
+    w2 = (uint32_t)(m >> 32);
   }
   int ex = 1023 + 63 + E;  // biased exponent when the top bit of w2 is set
-  if (w2 == 0) { w2 = w1; w1 = w0; w0 = 0; ex -= 32; }
-  if (w2 == 0) { w2 = w1; w1 = 0; ex -= 32; }
-  if (w2 == 0) return 0.0;
+  if (w2 == 0) {
+    w2 = w1; w1 = w0; w0 = 0; ex -= 32;
+    if (w2 == 0) { w2 = w1; w1 = 0; ex -= 32; }
+    if (w2 == 0) return 0.0;
+  }
   const int z = __clz(w2);
   ex -= z;
   const uint32_t h = __funnelshift_l(w1, w2, z), l = __funnelshift_l(w0, w1, z);
   // 53 bits: h[31:0] l[31:11], rounded by bit 10; the leading one adds to the exponent
-  uint32_t ml = __funnelshift_r(l, h, 11), mh = h >> 11;
-  const uint32_t r = (l >> 10) & 1;
-  ml += r;
-  mh += ml < r;
-  if (ex > 0 && ex < 2046)
-    return __hiloint2double((int)(sign | (((uint32_t)(ex - 1) << 20) + mh)), (int)ml);
-  const double m = (double)(((unsigned long long)mh << 32) | ml);
-  return scalbn(sign ? -m : m, ex - 1075);
+  const unsigned long long m =
+      (((unsigned long long)(h >> 11) << 32) | __funnelshift_r(l, h, 11)) + ((l >> 10) & 1);
+  if ((uint32_t)(ex - 1) < 2045u)
+    return __longlong_as_double(
+        (long long)(m + ((unsigned long long)(sign | ((uint32_t)(ex - 1) << 20)) << 32)));
+  const double d = (double)m;
+  return scalbn(sign ? -d : d, ex - 1075);
 }
 
 // The block after the one being loaded, into L2: one 128-byte line per thread
@@ -287,7 +299,7 @@ __global__ void __launch_bounds__(D_THREADS, 1) digit_gemm_kernel(const __grid_c
   __shared__ volatile int abort_flag;
   __shared__ int skip;
   // exponents of the rows a warp turns into digits (X, then Y), of two tiles
-  __shared__ int exps[D_WORK][2][64];
+  __shared__ uint32_t exps[D_WORK][2][64];
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // uniform: the register split needs it
   // A product that is added to C, or overwrites an operand, must not be left out half-way:
@@ -351,7 +363,6 @@ __global__ void __launch_bounds__(D_THREADS, 1) digit_gemm_kernel(const __grid_c
     if (warp == D_WORK) {
       // per block 34 products of two K = 16 steps, the low levels first: their
       // accumulators are taken out first
-      const uint32_t idesc = idesc_f16(128, DY, false, false, false);
       const uint64_t d0 = sdesc_sw64(smem_u32(sm), 16, 512);
       int it = 0, G = 0;
       bool good = true;
@@ -372,20 +383,30 @@ __global__ void __launch_bounds__(D_THREADS, 1) digit_gemm_kernel(const __grid_c
           tc_fence_after();
           const uint64_t dx = d0 + (uint64_t)((s * D_STAGE) >> 4);
           const uint64_t dy = dx + (uint64_t)((kDig * DX_PLANE) >> 4);
-#pragma unroll
-          for (int l = kLev - 1; l >= 0; --l) {
-            if (l == 3 && first && G >= 1) {
-              if (!mbar_wait_warp(&free_hi, (G - 1) & 1)) { fail(); break; }
-              tc_fence_after();
-            }
-            const int i0 = l >= kDig ? l - kDig + 1 : 0, i1 = l < kDig ? l : kDig - 1;
-#pragma unroll
-            for (int i = i0; i <= i1; ++i)
-              mma_ss_run2(tbase + 64 * l, dx + (uint64_t)((i * DX_PLANE) >> 4),
-                          dy + (uint64_t)(((l - i) * DY_PLANE) >> 4), 2, 2, idesc,
-                          (first && i == i0) ? 0u : 1u);
+          // digit i of X by digits j0 .. j0 + c - 1 of Y, whose planes follow one another, gives
+          // levels i + j0 onward, whose columns do
+          auto run = [&](int i, int j0, int c, bool acc) __attribute__((always_inline)) {
+            mma_ss_run2(tbase + 64 * (i + j0), dx + (uint64_t)((i * DX_PLANE) >> 4),
+                        dy + (uint64_t)((j0 * DY_PLANE) >> 4), 2, 2,
+                        idesc_f16(128, DY * c, false, false, false), acc ? 1u : 0u);
+          };
+          // levels 4 to 7; digit 1 reaches all four
+          run(1, 3, 4, !first);
+          run(0, 4, 3, true);
+          run(2, 2, 4, true);
+          run(3, 1, 4, true);
+          run(4, 0, 4, true);
+          run(5, 0, 3, true);
+          run(6, 0, 2, true);
+          if (first && G >= 1) {
+            if (!mbar_wait_warp(&free_hi, (G - 1) & 1)) { fail(); break; }
+            tc_fence_after();
           }
-          if (!good) break;
+          // levels 0 to 3
+          run(0, 0, 4, !first);
+          run(1, 0, 3, true);
+          run(2, 0, 2, true);
+          run(3, 0, 1, true);
           if (elect_one()) {
             mma_commit(&empty[s]);
             if (last) mma_commit(&set_ready);
@@ -416,19 +437,26 @@ __global__ void __launch_bounds__(D_THREADS, 1) digit_gemm_kernel(const __grid_c
     int ft = blockIdx.x, fkb = 0, fn = 0, fz = 0;
     int fx0 = 0, fy0 = 0;
     int fpar = 1;  // which half of exps the tile being fetched uses
+    // A tile of as many blocks as there are stages finds block kb in stage kb; when
+    // this CTA's tile before it had the same Y rows, their digits are there already (the
+    // products of 33 to 64 terms, a third of their conversions: 1755 x 91125 x 54 1440 ->
+    // 1270 us)
+    bool fkeep = false, vkeep = false;  // tile being fetched; block in vx, vy
     auto open_tile = [&]() __attribute__((always_inline)) {
       if (ft >= ntiles) { fn = 0; return; }
       int xt, yt;
       place(ft, xt, yt, fz);
+      const int pn = fn, py = fy0;
       fx0 = xt * DX;
       fy0 = yt * DY;
       fn = kblocks(fz);
+      fkeep = g.ksplit == 1 && fn == D_STAGES && pn == fn && py == fy0;
       fpar ^= 1;
       const long rx = fx0 + block_row<8, XK>(warp, lane), ry = fy0 + block_row<4, YK>(warp, lane);
       const int hx = __ldg(g.x.scale + min(rx, g.x.rows - 1l)), hy = __ldg(g.y.scale + min(ry, g.y.rows - 1l));
       if (row_unfit(hx) || row_unfit(hy)) *g.flag = 1;
-      exps[warp][fpar][lane] = (row_exp(hx) + 1022) << 20;
-      exps[warp][fpar][32 + lane] = (row_exp(hy) + 1022) << 20;
+      exps[warp][fpar][lane] = row_e21(hx);
+      exps[warp][fpar][32 + lane] = row_e21(hy);
       __syncwarp();
     };
     double vx[8], vy[4];
@@ -436,7 +464,8 @@ __global__ void __launch_bounds__(D_THREADS, 1) digit_gemm_kernel(const __grid_c
       const long k0 = (long)fz * g.kchunk + (long)fkb * DK;
       const long kend = min((long)g.K, (long)(fz + 1) * g.kchunk);
       load_block<8, XK>(g.x, fx0, k0, kend, tid, vx);
-      load_block<4, YK>(g.y, fy0, k0, kend, tid, vy);
+      vkeep = fkeep;
+      if (!fkeep) load_block<4, YK>(g.y, fy0, k0, kend, tid, vy);
       prefetch_block<XK, YK>(g, fx0, fy0, k0 + DK, kend, tid);
       if (++fkb == fn) { fkb = 0; ft += gridDim.x; open_tile(); }
     };
@@ -446,7 +475,12 @@ __global__ void __launch_bounds__(D_THREADS, 1) digit_gemm_kernel(const __grid_c
     auto take_group = [&](bool fresh) __attribute__((always_inline)) {
       if (!mbar_wait_warp(&set_ready, G & 1)) { lost(); return; }
       tc_fence_after();
-      auto level = [](uint32_t a) { return (long long)__float2int_rn(__uint_as_float(a)); };
+      auto level = [](uint32_t a) { return __float2int_rn(__uint_as_float(a)); };
+      auto mad = [](int a, int b, long long c) {  // one instruction, off the busy pipe
+        long long r;
+        asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+        return r;
+      };
 #pragma unroll
       for (int c = 0; c < 16; c += 8) {
         uint32_t a[8], b[8], d[8];
@@ -463,7 +497,8 @@ __global__ void __launch_bounds__(D_THREADS, 1) digit_gemm_kernel(const __grid_c
         tmem_wait_ld();
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-          const long long t = level(b[j]) * (1 << 12) + (int)a[j] + (fresh ? 0 : lo[c + j]);
+          // (int)a < 2^29
+          const long long t = mad(level(b[j]), 1 << 12, (int)a[j] + (fresh ? 0 : (int)lo[c + j]));
           lo[c + j] = (uint32_t)t & 0xfffffu;
           hi[c + j] = (fresh ? 0 : hi[c + j]) + (t >> 20);
         }
@@ -478,12 +513,12 @@ __global__ void __launch_bounds__(D_THREADS, 1) digit_gemm_kernel(const __grid_c
         tmem_ld8(tacc + 64 + c, b);
         tmem_wait_ld();
 #pragma unroll
-        for (int j = 0; j < 8; ++j) hi[c + j] += level(a[j]) * (1 << 24) + level(b[j]) * (1 << 16);
+        for (int j = 0; j < 8; ++j) hi[c + j] = mad(level(b[j]), 1 << 16, mad(level(a[j]), 1 << 24, hi[c + j]));
         tmem_ld8(tacc + 64 * 2 + c, a);
         tmem_ld8(tacc + 64 * 3 + c, b);
         tmem_wait_ld();
 #pragma unroll
-        for (int j = 0; j < 8; ++j) hi[c + j] += level(a[j]) * (1 << 8) + level(b[j]);
+        for (int j = 0; j < 8; ++j) hi[c + j] = mad(level(b[j]), 1, mad(level(a[j]), 1 << 8, hi[c + j]));
       }
       ++G;
       tc_fence_before();
@@ -572,7 +607,7 @@ __global__ void __launch_bounds__(D_THREADS, 1) digit_gemm_kernel(const __grid_c
             (use > 0 && !mbar_wait_warp(&empty[s], (use - 1) & 1))) { lost(); break; }
         uint8_t* st = sm + s * D_STAGE;
         store_block<8, XK>(st, exps[warp][par], tid, vx);
-        store_block<4, YK>(st + kDig * DX_PLANE, exps[warp][par] + 32, tid, vy);
+        if (!vkeep) store_block<4, YK>(st + kDig * DX_PLANE, exps[warp][par] + 32, tid, vy);
         auto arrive = [&]() {
           fence_async_smem();
           __syncwarp();
@@ -680,9 +715,8 @@ cudaError_t digit_gemm(const DGemm& g, int ksplit, int kchunk, cudaStream_t s) {
   int* sc = g.scale;  // [flag, 7 unused, M rows of op(A), N columns of op(B)]
   cudaError_t e = cudaMemsetAsync(sc, 0, ((size_t)g.M + g.N + 8) * 4, s);
   if (e != cudaSuccess) return e;
-  auto pairs = [](const double* p, long ld) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0 && ld % 2 == 0; };
-  const DOperand A{g.A, g.lda, g.M, g.transA ? 0 : 1, sc + 8, pairs(g.A, g.lda)};
-  const DOperand B{g.B, g.ldb, g.N, g.transB ? 1 : 0, sc + 8 + g.M, pairs(g.B, g.ldb)};
+  const DOperand A{g.A, g.lda, g.M, g.transA ? 0 : 1, sc + 8};
+  const DOperand B{g.B, g.ldb, g.N, g.transB ? 1 : 0, sc + 8 + g.M};
   launch_rowmax(A, g.K, sc + 8, s);
   launch_rowmax(B, g.K, sc + 8 + g.M, s);
   // the longer side of C takes the 128-row side of the tile; as columns of C

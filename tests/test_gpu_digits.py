@@ -123,3 +123,17 @@ def test_symmetric_product(xk, N):
     tol = 2.0 ** -53 * np.sqrt(grid ** 3) * 16
     assert np.linalg.norm(J - J0) <= tol * np.linalg.norm(J0)
     assert abs(EJ - EJ0) <= tol * abs(EJ0)
+
+
+@pytest.mark.parametrize("n", [32, 33, 48, 64, 65])
+def test_kept_rows(xk, n):
+    """Products of 33 to 64 terms keep the digits of Y rows that successive tiles
+    share: more than 152 tiles along X (tiles t and t + 152 share them or not), three
+    along Y, and the depths beside the two that fit."""
+    phi, idx, V, W, C = _case(25001, 72, n, 130, n, m=1)
+    h = xk.Handle(phi, idx, V, W, 1.0, n, mode="fp64")
+    K, _ = h.build(C)
+    h.release()
+    l1, l2, l3 = _lines(phi, idx, V, W, C)
+    assert max(np.abs(l).max() for l in (l1, l2, l3)) < 2.0 ** 52
+    assert np.array_equal(K, (l1 + l2 - l3).T)
