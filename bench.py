@@ -46,11 +46,10 @@ PAIR_DRAM_BYTES_PER_PAIR = 1496e6 / (2.0 * 1755 * 91125 + 1755.0 * 1755)
 # capture on the 27-centre cell with n = 128, 827 MB over 1.630e8 pairs
 # (profiles/pair_kernel_fused_cubic27_n128.md).
 FUSED_DRAM_BYTES_PER_PAIR = 827e6 / (1755.0 * 91125 + 1755.0 * 1755)
-# FP64 on the CUDA cores of GB300: 2 DFMA (4 flops) per clock per SM, measured
-# 3.81 flops/clock/SM with an FMA-chain probe; x 152 SMs x 2070 MHz.
-FP64_FLOPS_PER_CLK_SM = 4.0
-SM_COUNT = 152
-SM_MAX_MHZ = 2070.0
+# Large FP64 products run on the tensor cores as this many exact products of
+# digits (xk_digits.cu), so the FP64 ceiling is the FP16 tensor rate over it.  (The
+# CUDA cores' own FP64 rate: 4 flops per clock per SM x 152 x 2070 MHz = 1.26 TFLOP/s.)
+DIGIT_PRODUCTS = 34
 
 
 def parse():
@@ -875,8 +874,9 @@ def main():
             fl_j = 2.0 * N * N * Ng + 2.0 * Ng * N * n
             coul = {"ms_per_build": ms_j, "E_J": EJ,
                     "fp64_tflops_per_s": fl_j / (ms_j * 1e-3) / 1e12,
-                    "fp64_peak_tflops": FP64_FLOPS_PER_CLK_SM * SM_COUNT * SM_MAX_MHZ * 1e6 / 1e12,
-                    "note": "xk_coulomb on the FP64 handle: density, DFT Poisson solve, "
+                    "fp64_peak_tflops": peaks()[0].get(
+                        "bf16_tflops", FALLBACK_PEAKS["bf16_tflops"]) / DIGIT_PRODUCTS,
+                    "note": "xk_coulomb on the FP64 handle: density, Poisson solve, "
                             "J = dV Phi^T diag(v) Phi, host buffers in and out"}
         if full is not None:
             t0 = time.perf_counter()
@@ -895,11 +895,12 @@ def main():
         if mode == "fp64":
             dom = max((k for k in st if st[k][1] > 0), key=lambda k: st[k][0])
             dom_ms = st[dom][0] / max(1, st[dom][1])
-            peak = FP64_FLOPS_PER_CLK_SM * SM_COUNT * SM_MAX_MHZ * 1e6 / 1e12
-            roof = {"bound": "alu", "kernel": f"step '{dom}' (FP64 DFMA GEMM)",
+            peak = pk.get("bf16_tflops", FALLBACK_PEAKS["bf16_tflops"]) / DIGIT_PRODUCTS
+            roof = {"bound": "tensor", "kernel": f"step '{dom}' (FP64 product of 8-bit digits)",
                     "achieved": fl[dom] / (dom_ms * 1e-3) / 1e12, "peak": peak,
                     "unit": "TFLOP/s",
-                    "peak_source": "FP64 DFMA rate: 4 flop/clk/SM x 152 SMs x 2070 MHz",
+                    "peak_source": f"dense bf16/fp16 tensor rate ({pk_src}) / {DIGIT_PRODUCTS} "
+                                   "digit products",
                     "traffic": None}
         else:
             dom = "pair"

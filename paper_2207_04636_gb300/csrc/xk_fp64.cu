@@ -3,9 +3,9 @@
 // reduction, and the small dense FP64 factorisations of the occ-RI K_ij.
 //
 // On GB300 FP64 runs on the CUDA cores at a small fraction of the tensor
-// rate, so every FP64 contraction here is bound by the DFMA pipe; the tiles
-// only need enough register reuse to keep that pipe fed.  Products of 2e7
-// multiply-adds and more go to the tensor cores instead (xk_digits.cu).
+// rate, so a contraction here is bound by the DFMA pipe; the tiles only need
+// enough register reuse to keep that pipe fed.  Products of 2e7 multiply-adds and
+// more, nearly all of the work, go to the tensor cores instead (xk_digits.cu).
 #include "xk_internal.h"
 
 #include <algorithm>
