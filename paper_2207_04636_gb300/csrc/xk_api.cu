@@ -437,12 +437,21 @@ int enqueue_fp64(xk_handle* h) {
   cudaStream_t s = h->stream;
   const int ng = (int)h->Ng, N = h->N, n = h->n, na = h->Naux, ga = h->ga;
   const double* psl = h->psig + (size_t)h->g0 * n;  // Psi_g of the held slice
-  auto G = [&](int M, int Nc, int K, const double* A, long lda, bool ta, const double* B, long ldb,
-               bool tb, double* C, long ldc, const double* H, long ldh) {
+  auto make = [&](int M, int Nc, int K, const double* A, long lda, bool ta, const double* B, long ldb,
+                  bool tb, double* C, long ldc, const double* H, long ldh) {
     DGemm g{M, Nc, K, A, lda, ta, B, ldb, tb, C, ldc, 1.0, H, ldh, 0, h->work};
     g.scale = digit_scratch(h->MA, (size_t)ga * N, M, Nc);  // M_A: the full K's, idle here
-    return xk::dgemm(g, s);
+    return g;
   };
+  auto G = [&](auto... a) { return xk::dgemm(make(a...), s); };
+  // V2's largest entries per row and column come with it, at the end of M_A: reading V2
+  // twice more for them took 0.4 of 4.06 ms on the 27-centre cell
+  DGemm gp = make(ga, ng, n, psl, n, false, h->psi, n, true, h->V2, ng, h->V, ng);
+  const size_t ints = 2 * (size_t)ga * N, maxima = (size_t)ga + ng;
+  if (xk::digit_maxima(gp) && ints >= maxima + xk::digit_scale_ints(std::max(ga, ng), std::max(n, ng))) {
+    gp.rmax = reinterpret_cast<int*>(h->MA) + (ints - maxima);
+    gp.cmax = gp.rmax + ga;
+  }
   {  // Eq. rpsEx step 1: orbitals on the grid and at the interpolation points.
     StepMark m(h, XK_STEP_ORBITALS);
     XK_CUDA(G(ng, n, N, h->phi, N, false, h->C, n, false, h->psi, n, nullptr, 0));
@@ -450,15 +459,19 @@ int enqueue_fp64(xk_handle* h) {
   }
   {  // Steps 2-3: pair kernel at (R_g, R) and the Hadamard with V, fused.
     StepMark m(h, XK_STEP_PAIR);
-    XK_CUDA(G(ga, ng, n, psl, n, false, h->psi, n, true, h->V2, ng, h->V, ng));
+    XK_CUDA(xk::dgemm(gp, s));
   }
   {  // Line 2, first contraction (order (a)): M2 = V2 Psi.
     StepMark m(h, XK_STEP_M2);
-    XK_CUDA(G(ga, n, ng, h->V2, ng, false, h->psi, n, false, h->M2, n, nullptr, 0));
+    DGemm g = make(ga, n, ng, h->V2, ng, false, h->psi, n, false, h->M2, n, nullptr, 0);
+    g.amax = gp.rmax;
+    XK_CUDA(xk::dgemm(g, s));
   }
   {  // Line 1, first contraction: M1 = Psi_g^T V2.
     StepMark m(h, XK_STEP_M1);
-    XK_CUDA(G(n, ng, ga, psl, n, true, h->V2, ng, false, h->M1, ng, nullptr, 0));
+    DGemm g = make(n, ng, ga, psl, n, true, h->V2, ng, false, h->M1, ng, nullptr, 0);
+    g.bmax = gp.cmax;
+    XK_CUDA(xk::dgemm(g, s));
   }
   {  // Line 1, contraction with the basis on the grid.
     StepMark m(h, XK_STEP_LINE1);

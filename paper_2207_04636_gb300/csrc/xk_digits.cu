@@ -30,7 +30,7 @@
 // (GB300, us; FP64 FMA kernel before): 1755 x 54 x 91125: 814 (14500), 54 x 91125 x
 // 1755: 821 (17500), 1755 x 91125 x 54 (taking and storing the results bounds it): 1270
 // (17700), 351 x 351 x 91125: 816 (26600), 1053 x 1053 x 91125: 6630.  A 27-centre
-// FP64 build went from 64.7 to 4.06 ms, its Coulomb matrix from 30.6 to 1.12 ms.
+// FP64 build went from 64.7 to 3.65 ms, its Coulomb matrix from 30.6 to 1.12 ms.
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
@@ -86,6 +86,7 @@ struct DArgs {
   int careful;        // added to C, or in place
   int scaled, added;  // alpha != 1, beta != 0 (an FP64 comparison per result would cost more)
   const double* H; long ldh;
+  int *xmax, *ymax;  // digit_maxima: largest |C| per X and Y row (nullable)
   double* work;      // ksplit > 1: partial sums [ksplit][M][N]
   int nbatch; long cskip;  // swapped only: batches of C's columns (DGemm)
   int* flag;         // set to 1 when a row cannot be split (row_unfit), to 2 when a bounded
@@ -552,6 +553,33 @@ __global__ void __launch_bounds__(D_THREADS, 1) digit_gemm_kernel(const __grid_c
 #pragma unroll
       for (int j = 0; j < 16; ++j)
         hi[j] = __double_as_longlong(pack_f64(hi[j], lo[j], e + __shfl_sync(0xffffffffu, ye, j)));
+      // with H; the maxima are what rowmax_*_kernel would find in C (in this form of the
+      // kernel alone: the others' registers, and 2 % of their time, are spared)
+      if (XK && YK && g.xmax) {
+        const int mine = in ? left : 0;
+        uint32_t mx = 0, my = 0;
+        double w[4];
+#pragma unroll
+        for (int j = 0; j < 16; j += 4) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) w[i] = j + i < mine ? h[(j + i) * hstep] : 0.0;
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            uint32_t b = 0;
+            if (j + i < mine) {
+              const double v = __longlong_as_double(hi[j + i]) * w[i];
+              c[(j + i) * step] = v;
+              b = (uint32_t)__double2hiint(v) & 0x7fffffffu;
+            }
+            mx = max(mx, b);
+            b = __reduce_max_sync(0xffffffffu, b);
+            if (lane == j + i) my = b;
+          }
+        }
+        if (in) atomicMax(g.xmax + x, (int)mx);
+        if (lane < left) atomicMax(g.ymax + y0 + lane, (int)my);
+        return;
+      }
       if (!in) return;
       // branches around the FP64 operations: one that is only predicated off
       // would still take its 16 cycles of the FP64 pipe
@@ -695,6 +723,12 @@ bool digit_gemm_wanted(const DGemm& g) {
          (double)g.M * g.N * g.K >= 2e7;
 }
 
+// One K group: the product is not split, so its epilogue has every final result.
+bool digit_maxima(const DGemm& g) {
+  return digit_gemm_wanted(g) && !g.transA && g.transB && g.H && g.K <= 256 && g.alpha == 1.0 && g.beta == 0.0 && !g.sym &&
+         g.nbatch == 0 && !in_place(g);
+}
+
 // K split (at most cap) of least time: waves of tiles over the SMs times the
 // 256-term groups of a tile, with one group's time for a tile's start and end.
 int digit_ksplit(int M, int N, int K, bool sym, int cap) {
@@ -715,10 +749,10 @@ cudaError_t digit_gemm(const DGemm& g, int ksplit, int kchunk, cudaStream_t s) {
   int* sc = g.scale;  // [flag, 7 unused, M rows of op(A), N columns of op(B)]
   cudaError_t e = cudaMemsetAsync(sc, 0, ((size_t)g.M + g.N + 8) * 4, s);
   if (e != cudaSuccess) return e;
-  const DOperand A{g.A, g.lda, g.M, g.transA ? 0 : 1, sc + 8};
-  const DOperand B{g.B, g.ldb, g.N, g.transB ? 1 : 0, sc + 8 + g.M};
-  launch_rowmax(A, g.K, sc + 8, s);
-  launch_rowmax(B, g.K, sc + 8 + g.M, s);
+  const DOperand A{g.A, g.lda, g.M, g.transA ? 0 : 1, g.amax ? g.amax : sc + 8};
+  const DOperand B{g.B, g.ldb, g.N, g.transB ? 1 : 0, g.bmax ? g.bmax : sc + 8 + g.M};
+  if (!g.amax) launch_rowmax(A, g.K, sc + 8, s);
+  if (!g.bmax) launch_rowmax(B, g.K, sc + 8 + g.M, s);
   // the longer side of C takes the 128-row side of the tile; as columns of C
   // it also makes the stores contiguous over the lanes
   a.swapped = g.N >= g.M || g.nbatch > 0 ? 1 : 0;
@@ -729,6 +763,13 @@ cudaError_t digit_gemm(const DGemm& g, int ksplit, int kchunk, cudaStream_t s) {
   a.tiles_y = (a.y.rows + DY - 1) / DY;
   a.M = g.M; a.N = g.N; a.C = g.C; a.ldc = g.ldc; a.alpha = g.alpha; a.beta = g.beta;
   a.scaled = g.alpha != 1.0; a.added = g.beta != 0.0; a.careful = a.added || in_place(g);
+  if (g.rmax) {
+    e = cudaMemsetAsync(g.rmax, 0, (size_t)g.M * 4, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(g.cmax, 0, (size_t)g.N * 4, s);
+    if (e != cudaSuccess) return e;
+    a.xmax = a.swapped ? g.cmax : g.rmax;
+    a.ymax = a.swapped ? g.rmax : g.cmax;
+  }
   a.H = g.H; a.ldh = g.ldh; a.work = g.work; a.flag = sc;
   a.nbatch = g.nbatch; a.cskip = g.cskip;
   a.sym = g.sym;

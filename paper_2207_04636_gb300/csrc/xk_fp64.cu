@@ -26,6 +26,12 @@ __global__ void __launch_bounds__(TPB) dgemm_kernel(DGemm g, int kchunk, const i
   // blocks then walk the tiles; a grid of all of them took 25 us to start and end)
   const int left_out = only_if ? *only_if : 1;
   if (!left_out) return;
+  // the maxima it left are not C's: rows that are not split, so that products of C
+  // take this kernel too
+  if (only_if && g.rmax) {
+    for (long i = blockIdx.x * (long)TPB + threadIdx.x; i < g.M; i += (long)gridDim.x * TPB) g.rmax[i] = 0x7ff00000;
+    for (long i = blockIdx.x * (long)TPB + threadIdx.x; i < g.N; i += (long)gridDim.x * TPB) g.cmax[i] = 0x7ff00000;
+  }
   const long gx = (g.N + BN - 1) / BN, gy = (g.M + BM - 1) / BM, ntiles = gx * gy * g.ksplit;
   __shared__ double As[BK][BM + 1];
   __shared__ double Bs[BK][BN + 1];

@@ -44,6 +44,9 @@ struct DGemm {
   int nbatch;   // > 0: the columns of C come in batches of nbatch: column n is stored
   long cskip;   // (n / nbatch) cskip elements further on, and H has column n % nbatch
   bool sym;     // C is symmetric (M = N, no H, beta = 0): one half may be formed and mirrored
+  int *rmax, *cmax;          // digit_maxima(g): high words of the largest |C| per row and
+                             // column, for products that take C as an operand
+  const int *amax, *bmax;    // those of op(A)'s rows / op(B)'s columns, when they are known
 };
 // The result overwrites rows of B (M <= 64, one row of tiles, unsplit: every block has read
 // its columns of B before it writes them).
@@ -58,6 +61,7 @@ cudaError_t dgemm(const DGemm& g, cudaStream_t s);
 // when ksplit > 1).  *g.scale is 0 afterwards, or not when the product has to be
 // formed with FP64 FMAs instead (an operand that is not finite).
 size_t digit_scale_ints(int M, int N);
+bool digit_maxima(const DGemm& g);  // whether the product can leave rmax and cmax
 bool digit_gemm_wanted(const DGemm& g);
 int digit_ksplit(int M, int N, int K, bool sym, int cap);
 cudaError_t digit_gemm(const DGemm& g, int ksplit, int kchunk, cudaStream_t s);

@@ -137,3 +137,24 @@ def test_kept_rows(xk, n):
     l1, l2, l3 = _lines(phi, idx, V, W, C)
     assert max(np.abs(l).max() for l in (l1, l2, l3)) < 2.0 ** 52
     assert np.array_equal(K, (l1 + l2 - l3).T)
+
+
+@pytest.mark.parametrize("Ng,N,n,na", [(6145, 40, 32, 130), (5000, 70, 64, 641), (4100, 300, 257, 129)])
+@pytest.mark.parametrize("bad", [None, np.nan])
+def test_maxima_of_a_product(xk, Ng, N, n, na, bad):
+    """The largest entries of V2 come with it (up to 256 terms; 257 are read again):
+    exact results from rows of different size, and after a NaN, whose products go the
+    general way."""
+    phi, idx, V, W, C = _case(Ng, N, n, na, n, m=1)
+    V = V * 2.0 ** np.random.default_rng(1).integers(-3, 4, size=na)[:, None]
+    bound = _lines(*(np.abs(a) if a is not idx else a for a in (phi, idx, V, W, C)))
+    assert 8 * sum(l.max() for l in bound) < 2.0 ** 53
+    h = xk.Handle(phi, idx, V, W, 1.0, n, mode="fp64")
+    if bad is not None:
+        Cb = C.copy()
+        Cb[0, 0] = bad
+        assert np.isnan(h.build(Cb)[1])
+    K, _ = h.build(C)
+    h.release()
+    l1, l2, l3 = _lines(phi, idx, V, W, C)
+    assert np.array_equal(K, (l1 + l2 - l3).T)
