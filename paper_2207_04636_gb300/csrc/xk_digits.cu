@@ -456,6 +456,9 @@ __global__ void __launch_bounds__(D_THREADS, 1) digit_gemm_kernel(const __grid_c
       const long rx = fx0 + block_row<8, XK>(warp, lane), ry = fy0 + block_row<4, YK>(warp, lane);
       const int hx = __ldg(g.x.scale + min(rx, g.x.rows - 1l)), hy = __ldg(g.y.scale + min(ry, g.y.rows - 1l));
       if (row_unfit(hx) || row_unfit(hy)) *g.flag = 1;
+      // with one block a tile this half held the exponents of the block stored just now:
+      // every lane has read its own
+      __syncwarp();
       exps[warp][fpar][lane] = row_e21(hx);
       exps[warp][fpar][32 + lane] = row_e21(hy);
       __syncwarp();

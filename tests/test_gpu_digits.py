@@ -158,3 +158,19 @@ def test_maxima_of_a_product(xk, Ng, N, n, na, bad):
     h.release()
     l1, l2, l3 = _lines(phi, idx, V, W, C)
     assert np.array_equal(K, (l1 + l2 - l3).T)
+
+
+@pytest.mark.parametrize("n", [16, 31, 32])
+def test_one_block_tiles(xk, n):
+    """Products of up to 32 terms: one block a tile and several tiles a CTA, so the
+    exponents of a tile's rows are replaced as soon as its block is stored; rows of
+    different size, so that a wrong exponent shows."""
+    phi, idx, V, W, C = _case(6145, 40, n, 641, n, m=1)
+    phi *= np.exp2(np.random.default_rng(2).integers(0, 4, size=phi.shape[0]))[:, None]
+    bound = _lines(*(np.abs(a) if a is not idx else a for a in (phi, idx, V, W, C)))
+    assert sum(l.max() for l in bound) < 2.0 ** 53
+    h = xk.Handle(phi, idx, V, W, 1.0, n, mode="fp64")
+    K, _ = h.build(C)
+    h.release()
+    l1, l2, l3 = _lines(phi, idx, V, W, C)
+    assert np.array_equal(K, (l1 + l2 - l3).T)
