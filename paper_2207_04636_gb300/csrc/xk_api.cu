@@ -206,7 +206,16 @@ struct xk_handle {
   // FP64 tables and scratch
   double *phi = nullptr, *phig = nullptr, *V = nullptr, *W = nullptr;
   int32_t* idx = nullptr;
-  double* Ce = nullptr;  // xk_energy: C (N x n) and E_x (one more double), apart from the build's
+  // The FP64 tables are held in units of powers of two, so that the digit products
+  // (xk_digits.cu), which keep a row of an operand on one grid, lose nothing when basis
+  // functions or interpolation points are of unlike size (functions scaled by up to 2^(+-15)
+  // and C by the inverse left Psi an error of 5e-9 of its norm, an FMA chain 3.4e-16):
+  //   phi[R][mu] = Phi 2^-be[mu] (columns of largest element in [1/2, 1)), C taken times 2^be,
+  //   phig[g][mu] = phi[R_g][mu] 2^-ge[g], psig likewise, V[g] = V_g 2^(2 ge[g]), W likewise on
+  //   both sides; V2, M1, M2, Q, M3 and the lines follow, K leaves times 2^be.
+  int *be = nullptr, *ge = nullptr;  // N, N_aux
+  double* Ce = nullptr;  // C (N x n) times 2^be, of every FP64 call, and E_x of xk_energy (one more
+                         // double); tensor path: C of all calls but a build
   // xk_build_full: K_{mu nu} (N x N); FP64 path also M_A, M_C (N_aux x N), Y, Z (N x N)
   double *Kf = nullptr, *MA = nullptr, *MC = nullptr, *Yf = nullptr, *Zf = nullptr;
   size_t full_extra = 0;  // bytes of the tensor path's full-K scratch, admitted on first use
@@ -309,7 +318,7 @@ Plan plan_fp64(int64_t Ng, int N, int n, int Naux, int ga = -1) {
           + 3 * (size_t)n * n + 2 * (size_t)N * n + n;   // K_ij, L, U, Y, xi, sign
   p.work = max_work(Ng, N, n, Naux, false, ga);
   p.f64 += p.work;
-  p.i32 = na + 2;
+  p.i32 = 2 * na + N + 2;
   return p;
 }
 
@@ -431,6 +440,11 @@ int* digit_scratch(double* buf, size_t doubles, int M, int N) {
   return 2 * doubles >= xk::digit_scale_ints(M, N) ? reinterpret_cast<int*>(buf) : nullptr;
 }
 
+// Ce = C times 2^be.
+cudaError_t take_c(xk_handle* h, const double* C) {
+  return xk::scale_f64(C, h->Ce, h->N, h->n, h->be, 1, nullptr, 0, h->stream);
+}
+
 // Enqueue one FP64 build on h->stream.  C is in h->C; results land in h->K, h->Ex.
 int enqueue_fp64(xk_handle* h) {
   using xk::DGemm;
@@ -454,8 +468,9 @@ int enqueue_fp64(xk_handle* h) {
   }
   {  // Eq. rpsEx step 1: orbitals on the grid and at the interpolation points.
     StepMark m(h, XK_STEP_ORBITALS);
-    XK_CUDA(G(ng, n, N, h->phi, N, false, h->C, n, false, h->psi, n, nullptr, 0));
-    XK_CUDA(xk::gather_rows_f64(h->psi, n, h->idx, na, n, h->psig, n, s));
+    XK_CUDA(take_c(h, h->C));
+    XK_CUDA(G(ng, n, N, h->phi, N, false, h->Ce, n, false, h->psi, n, nullptr, 0));
+    XK_CUDA(xk::gather_rows_f64(h->psi, n, h->idx, na, n, h->psig, n, s, h->ge));
   }
   {  // Steps 2-3: pair kernel at (R_g, R) and the Hadamard with V, fused.
     StepMark m(h, XK_STEP_PAIR);
@@ -489,7 +504,7 @@ int enqueue_fp64(xk_handle* h) {
   }
   {  // K_{mu i} = dV (line1 + line2 - line3)^T and E_x = -sum K o C.
     StepMark m(h, XK_STEP_ASSEMBLE);
-    XK_CUDA(xk::assemble_k_f64(h->L1, h->L2, h->L3, n, N, h->dV, h->K, s));
+    XK_CUDA(xk::assemble_k_f64(h->L1, h->L2, h->L3, n, N, h->dV, h->be, h->K, s));
     XK_CUDA(xk::neg_dot_f64(h->K, h->C, (long)N * n, h->red, h->Ex, s));
   }
   return XK_OK;
@@ -517,8 +532,9 @@ int enqueue_energy(xk_handle* h) {
   };
   {
     StepMark m(h, XK_STEP_ORBITALS);
+    XK_CUDA(take_c(h, h->Ce));
     XK_CUDA(G(ng, n, N, h->phi, N, false, h->Ce, n, false, h->psi, n));
-    XK_CUDA(xk::gather_rows_f64(h->psi, n, h->idx, na, n, h->psig, n, s));
+    XK_CUDA(xk::gather_rows_f64(h->psi, n, h->idx, na, n, h->psig, n, s, h->ge));
   }
   {  // P = Psi_g Psi^T and Q = Psi_g Psi_g^T
     StepMark m(h, XK_STEP_PAIR);
@@ -552,8 +568,9 @@ int enqueue_full(xk_handle* h) {
   };
   {
     StepMark m(h, XK_STEP_ORBITALS);
+    XK_CUDA(take_c(h, h->Ce));
     XK_CUDA(G(ng, n, N, h->phi, N, false, h->Ce, n, false, h->psi, n, nullptr, 0));
-    XK_CUDA(xk::gather_rows_f64(h->psi, n, h->idx, na, n, h->psig, n, s));
+    XK_CUDA(xk::gather_rows_f64(h->psi, n, h->idx, na, n, h->psig, n, s, h->ge));
   }
   {  // V2 = V o (Psi_g Psi^T), M_A = V2 Phi
     StepMark m(h, XK_STEP_PAIR);
@@ -569,7 +586,7 @@ int enqueue_full(xk_handle* h) {
     StepMark m(h, XK_STEP_ASSEMBLE);
     XK_CUDA(G(N, N, na, h->phig, N, true, h->MA, N, false, h->Yf, N, nullptr, 0));
     XK_CUDA(G(N, N, na, h->phig, N, true, h->MC, N, false, h->Zf, N, nullptr, 0));
-    XK_CUDA(xk::assemble_full_f64(h->Yf, h->Zf, N, h->dV, h->Kf, s));
+    XK_CUDA(xk::assemble_full_f64(h->Yf, h->Zf, N, h->dV, h->be, h->Kf, s));
   }
   return XK_OK;
 }
@@ -768,6 +785,8 @@ static int setup_impl(int64_t Ng, int32_t N, int32_t n, int32_t Naux, const doub
     XK_ALLOC(h->V, gs * ng);
     XK_ALLOC(h->W, gs * na);
     XK_ALLOC(h->idx, na);
+    XK_ALLOC(h->be, (size_t)N);
+    XK_ALLOC(h->ge, na);
     XK_ALLOC(h->psi, ng * n);
     XK_ALLOC(h->psig, na * n);
     XK_ALLOC(h->V2, gs * ng);
@@ -788,11 +807,19 @@ static int setup_impl(int64_t Ng, int32_t N, int32_t n, int32_t Naux, const doub
     if (e == cudaSuccess && !isdf)
       e = cudaMemcpyAsync(h->W, W, gs * na * 8, cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(h->idx, idx, na * 4, cudaMemcpyHostToDevice, h->stream);
-    if (e == cudaSuccess)  // the basis at the slice's points
-      e = xk::gather_rows_f64(h->phi, N, h->idx + g0, ga, N, h->phig, N, h->stream);
+    if (e == cudaSuccess && isdf)
+      e = xk::gather_rows_f64(h->phi, N, h->idx, Naux, N, h->phig, N, h->stream);
     if (e == cudaSuccess && isdf)  // X_gg in Q, chi in V2 (both scratch of the build)
       e = xk::isdf_tables_f64(h->phi, (long)ng, N, h->phig, Naux, grid, L, h->Q, h->V2, h->V, h->W,
                               h->work, h->status, &h->ridge, h->stream);
+    // the units of the tables; |ge| <= 64 keeps V and W far from the ends of the range
+    if (e == cudaSuccess) e = xk::col_exponents_f64(h->phi, N, Ng, N, 1022, h->be, h->stream);
+    if (e == cudaSuccess) e = xk::scale_f64(h->phi, h->phi, Ng, N, nullptr, 0, h->be, -1, h->stream);
+    if (e == cudaSuccess) e = xk::row_exponents_f64(h->phi, N, h->idx, Naux, N, 64, h->ge, h->stream);
+    if (e == cudaSuccess)
+      e = xk::gather_rows_f64(h->phi, N, h->idx + g0, ga, N, h->phig, N, h->stream, h->ge + g0);
+    if (e == cudaSuccess) e = xk::scale_f64(h->V, h->V, gs, ng, h->ge + g0, 2, nullptr, 0, h->stream);
+    if (e == cudaSuccess) e = xk::scale_f64(h->W, h->W, gs, na, h->ge + g0, 2, h->ge, 2, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e == cudaErrorInvalidValue && isdf)
       return bail(fail(XK_EINVAL, "xk_setup_isdf: X_gg is not positive definite even with the ridge"));
@@ -1006,10 +1033,16 @@ int xk_tables(xk_handle* h, double* W_out, const int32_t* rows, int32_t nrows, d
   std::lock_guard<std::mutex> lk(h->mu);
   DeviceGuard g(h->device);
   const size_t na = (size_t)h->Naux, ng = (size_t)h->Ng;
-  if (W_out) XK_CUDA(cudaMemcpyAsync(W_out, h->W, na * na * 8, cudaMemcpyDeviceToHost, h->stream));
-  for (int32_t i = 0; i < nrows; ++i)
-    XK_CUDA(cudaMemcpyAsync(V_rows_out + (size_t)i * ng, h->V + (size_t)rows[i] * ng, ng * 8,
-                            cudaMemcpyDeviceToHost, h->stream));
+  // out of the handle's units by way of the build's scratch (Q, Psi)
+  if (W_out) {
+    XK_CUDA(xk::scale_f64(h->W, h->Q, h->Naux, h->Naux, h->ge, -2, h->ge, -2, h->stream));
+    XK_CUDA(cudaMemcpyAsync(W_out, h->Q, na * na * 8, cudaMemcpyDeviceToHost, h->stream));
+  }
+  for (int32_t i = 0; i < nrows; ++i) {
+    XK_CUDA(xk::scale_f64(h->V + (size_t)rows[i] * ng, h->psi, 1, h->Ng, h->ge + rows[i], -2, nullptr, 0,
+                          h->stream));
+    XK_CUDA(cudaMemcpyAsync(V_rows_out + (size_t)i * ng, h->psi, ng * 8, cudaMemcpyDeviceToHost, h->stream));
+  }
   XK_CUDA(cudaStreamSynchronize(h->stream));
   if (ridge) *ridge = h->ridge;
   return XK_OK;
@@ -1150,6 +1183,7 @@ int xk_coulomb(xk_handle* h, int32_t grid, double L, const double* C, double* J_
   XK_CUDA(cudaMemcpyAsync(h->Ce, C, (size_t)N * n * 8, cudaMemcpyHostToDevice, s));
   {
     StepMark m(h, XK_STEP_ORBITALS);
+    XK_CUDA(take_c(h, h->Ce));
     xk::DGemm g1{(int)ng, n, N, h->phi, N, false, h->Ce, n, false, h->psi, n, 1.0, nullptr, 0, 0, h->work};
     g1.scale = digit_scratch(h->M1, (size_t)n * ng, (int)ng, n);
     XK_CUDA(xk::dgemm(g1, s));
@@ -1163,6 +1197,7 @@ int xk_coulomb(xk_handle* h, int32_t grid, double L, const double* C, double* J_
     gj.scale = digit_scratch(h->M1, (size_t)n * ng, N, N);
     gj.sym = true;
     XK_CUDA(xk::dgemm(gj, s));
+    XK_CUDA(xk::scale_f64(h->Jout, h->Jout, N, N, h->be, 1, h->be, 1, s));
     XK_CUDA(xk::dot_f64(h->Jrho, h->Jv, (long)ng, h->dV, h->red, h->Jout + (size_t)N * N, s));
   }
   XK_CUDA(cudaMemcpyAsync(h->res, h->Jout + (size_t)N * N, 8, cudaMemcpyDeviceToHost, s));

@@ -14,7 +14,9 @@
 // exceed 2^24 and are exact; the accumulator's last bit weighs 2^-58 of the
 // largest product).  The result is rounded to FP64 once, so its error is that of the 55-bit
 // operands and the dropped levels: 5e-17 to 3e-16 of the 2-norm on the
-// products of a build, where a chain of FP64 FMAs leaves 1.4e-16 to 9e-15.
+// products of a build, where a chain of FP64 FMAs leaves 1.4e-16 to 9e-15.  The 55 bits
+// count from the largest element of the row, so the callers see to it that the two operands
+// are not graded in opposite directions along K (units of powers of two: xk_api.cu).
 //
 // What bounds it: a 128 x 64 tile takes 34 digit products per K = 16 step, 1088
 // clocks of the tensor cores.  One instruction forms up to four of them: the digits of Y

@@ -190,42 +190,119 @@ cudaError_t dgemm(const DGemm& gin, cudaStream_t s) {
 
 __global__ void gather_rows_kernel(const double* __restrict__ in, long ld_in,
                                    const int32_t* __restrict__ idx, int rows, int cols,
-                                   double* __restrict__ out, long ld_out) {
+                                   double* __restrict__ out, long ld_out, const int* __restrict__ re) {
   const long total = (long)rows * cols;
   for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < total;
        t += (long)gridDim.x * blockDim.x) {
     const long r = t / cols, c = t % cols;
-    out[r * ld_out + c] = in[(long)idx[r] * ld_in + c];
+    const double v = in[(long)idx[r] * ld_in + c];
+    out[r * ld_out + c] = re ? scalbn(v, -re[r]) : v;
   }
 }
 
 cudaError_t gather_rows_f64(const double* in, long ld_in, const int32_t* idx, int rows, int cols,
-                            double* out, long ld_out, cudaStream_t s) {
+                            double* out, long ld_out, cudaStream_t s, const int* re) {
   const long total = (long)rows * cols;
   if (total == 0) return cudaSuccess;
   const int blocks = (int)std::min<long>((total + 255) / 256, 152L * 16);
-  gather_rows_kernel<<<blocks, 256, 0, s>>>(in, ld_in, idx, rows, cols, out, ld_out);
+  gather_rows_kernel<<<blocks, 256, 0, s>>>(in, ld_in, idx, rows, cols, out, ld_out, re);
+  count_launch();
+  return cudaGetLastError();
+}
+
+__device__ __forceinline__ int exponent_of(int hi, int limit) {  // hi: high word of |x|
+  return hi <= 0 || hi >= 0x7ff00000 ? 0 : max(-limit, min(limit, (hi >> 20) - 1022));
+}
+
+// One warp per row.
+__global__ void row_exponents_kernel(const double* __restrict__ p, long ld, const int32_t* __restrict__ idx,
+                                     int rows, int cols, int limit, int* __restrict__ out) {
+  const int lane = threadIdx.x & 31;
+  const long r = (long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (r >= rows) return;
+  const double* row = p + (idx ? (long)idx[r] : r) * ld;
+  int m = 0;
+  for (int c = lane; c < cols; c += 32) m = max(m, __double2hiint(row[c]) & 0x7fffffff);
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if (lane == 0) out[r] = exponent_of(m, limit);
+}
+
+cudaError_t row_exponents_f64(const double* p, long ld, const int32_t* idx, int rows, int cols, int limit,
+                              int* out, cudaStream_t s) {
+  row_exponents_kernel<<<(unsigned)((rows + 7) / 8), 256, 0, s>>>(p, ld, idx, rows, cols, limit, out);
+  count_launch();
+  return cudaGetLastError();
+}
+
+// One thread per column and chunk of rows (blockIdx.y).
+__global__ void col_max_kernel(const double* __restrict__ p, long ld, long rows, int cols, long chunk,
+                               int* __restrict__ out) {
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= cols) return;
+  const long r0 = blockIdx.y * chunk, r1 = min(rows, r0 + chunk);
+  int m = 0;
+  for (long r = r0; r < r1; ++r) m = max(m, __double2hiint(p[r * ld + c]) & 0x7fffffff);
+  atomicMax(out + c, m);
+}
+
+__global__ void exponents_kernel(int* __restrict__ x, int n, int limit) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) x[i] = exponent_of(x[i], limit);
+}
+
+cudaError_t col_exponents_f64(const double* p, long ld, long rows, int cols, int limit, int* out,
+                              cudaStream_t s) {
+  cudaError_t e = cudaMemsetAsync(out, 0, (size_t)cols * 4, s);
+  if (e != cudaSuccess) return e;
+  const long chunk = std::max(64L, (rows + 1023) / 1024);
+  col_max_kernel<<<dim3((unsigned)((cols + 127) / 128), (unsigned)((rows + chunk - 1) / chunk)), 128, 0, s>>>(
+      p, ld, rows, cols, chunk, out);
+  exponents_kernel<<<(unsigned)((cols + 255) / 256), 256, 0, s>>>(out, cols, limit);
+  count_launch(2);
+  return cudaGetLastError();
+}
+
+__global__ void scale_kernel(const double* src, double* dst, long rows, long cols, const int* __restrict__ re,
+                             int rm, const int* __restrict__ ce, int cm) {
+  const long total = rows * cols;
+  for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < total;
+       t += (long)gridDim.x * blockDim.x) {
+    const long r = t / cols, c = t - r * cols;
+    const int e = (re ? rm * re[r] : 0) + (ce ? cm * ce[c] : 0);
+    if (e != 0)
+      dst[t] = scalbn(src[t], e);
+    else if (src != dst)
+      dst[t] = src[t];
+  }
+}
+
+cudaError_t scale_f64(const double* src, double* dst, long rows, long cols, const int* re, int rm,
+                      const int* ce, int cm, cudaStream_t s) {
+  const long total = rows * cols;
+  if (total == 0) return cudaSuccess;
+  scale_kernel<<<(unsigned)std::min<long>((total + 255) / 256, 152L * 16), 256, 0, s>>>(src, dst, rows, cols, re,
+                                                                                       rm, ce, cm);
   count_launch();
   return cudaGetLastError();
 }
 
 __global__ void assemble_k_kernel(const double* __restrict__ L1, const double* __restrict__ L2,
                                   const double* __restrict__ L3, int n, int N, double dV,
-                                  double* __restrict__ K) {
+                                  const int* __restrict__ ce, double* __restrict__ K) {
   const long total = (long)n * N;
   for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < total;
        t += (long)gridDim.x * blockDim.x) {
     const long mu = t / n, i = t % n;
     const long src = i * N + mu;
-    K[t] = dV * ((L1[src] + L2[src]) - L3[src]);
+    K[t] = scalbn(dV * ((L1[src] + L2[src]) - L3[src]), ce[mu]);
   }
 }
 
 cudaError_t assemble_k_f64(const double* L1, const double* L2, const double* L3, int n, int N,
-                           double dV, double* K, cudaStream_t s) {
+                           double dV, const int* ce, double* K, cudaStream_t s) {
   const long total = (long)n * N;
   const int blocks = (int)std::min<long>((total + 255) / 256, 152L * 8);
-  assemble_k_kernel<<<blocks, 256, 0, s>>>(L1, L2, L3, n, N, dV, K);
+  assemble_k_kernel<<<blocks, 256, 0, s>>>(L1, L2, L3, n, N, dV, ce, K);
   count_launch();
   return cudaGetLastError();
 }
@@ -442,22 +519,23 @@ cudaError_t dot_f64(const double* a, const double* b, long len, double scale, do
   return cudaGetLastError();
 }
 
-// Full K: K[mu][nu] = dV (Y[mu][nu] + Y[nu][mu] - Z[mu][nu]) (N x N).
+// Full K: K[mu][nu] = dV (Y[mu][nu] + Y[nu][mu] - Z[mu][nu]) 2^(ce[mu] + ce[nu]) (N x N).
 __global__ void assemble_full_kernel(const double* __restrict__ Y, const double* __restrict__ Z,
-                                     int N, double dV, double* __restrict__ K) {
+                                     int N, double dV, const int* __restrict__ ce,
+                                     double* __restrict__ K) {
   const long count = (long)N * N;
   for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < count;
        t += (long)gridDim.x * blockDim.x) {
     const long mu = t / N, nu = t % N;
-    K[t] = dV * ((Y[t] + Y[nu * N + mu]) - Z[t]);
+    K[t] = scalbn(dV * ((Y[t] + Y[nu * N + mu]) - Z[t]), ce[mu] + ce[nu]);
   }
 }
 
-cudaError_t assemble_full_f64(const double* Y, const double* Z, int N, double dV, double* K,
-                              cudaStream_t s) {
+cudaError_t assemble_full_f64(const double* Y, const double* Z, int N, double dV, const int* ce,
+                              double* K, cudaStream_t s) {
   const long count = (long)N * N;
   const int blocks = (int)std::min<long>((count + 255) / 256, 152L * 16);
-  assemble_full_kernel<<<std::max(blocks, 1), 256, 0, s>>>(Y, Z, N, dV, K);
+  assemble_full_kernel<<<std::max(blocks, 1), 256, 0, s>>>(Y, Z, N, dV, ce, K);
   count_launch();
   return cudaGetLastError();
 }

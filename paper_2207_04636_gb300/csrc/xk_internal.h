@@ -55,6 +55,20 @@ __host__ __device__ inline bool in_place(const DGemm& g) {
 }
 cudaError_t dgemm(const DGemm& g, cudaStream_t s);
 
+// Powers of two.  The digit products (xk_digits.cu) hold an operand's row on one grid, so
+// terms of a product lose bits when its two operands are graded in opposite directions
+// along K; scaling by powers of two, exact, puts them on one footing.
+// The exponents e of the largest |x| of every row (of rows idx[0..rows) of p, idx nullable) or
+// column of a matrix, 2^(e-1) <= |x| < 2^e, at most `limit` in size; 0 for rows of zeros or
+// with infinities or NaN.
+cudaError_t row_exponents_f64(const double* p, long ld, const int32_t* idx, int rows, int cols, int limit,
+                              int* out, cudaStream_t s);
+cudaError_t col_exponents_f64(const double* p, long ld, long rows, int cols, int limit, int* out,
+                              cudaStream_t s);
+// dst[r][c] = src[r][c] 2^(rm re[r] + cm ce[c]) (re, ce nullable; dst may be src).
+cudaError_t scale_f64(const double* src, double* dst, long rows, long cols, const int* re, int rm,
+                      const int* ce, int cm, cudaStream_t s);
+
 // The product of dgemm on the tensor cores, split into exact digits
 // (xk_digits.cu): whether its size calls for it, the K split it wants (at most
 // cap), and the launch (ksplit partial sums of kchunk terms each in g.work
@@ -68,13 +82,13 @@ cudaError_t digit_gemm(const DGemm& g, int ksplit, int kchunk, cudaStream_t s);
 // Split count dgemm picks when DGemm::ksplit == 0 (work needs ksplit*M*N).
 int dgemm_ksplit(int M, int N, int K);
 
-// out[r, c] = in[idx[r] * ld_in + c] for r < rows, c < cols (row gather).
+// out[r, c] = in[idx[r] * ld_in + c] 2^-re[r] for r < rows, c < cols (row gather; re nullable).
 cudaError_t gather_rows_f64(const double* in, long ld_in, const int32_t* idx, int rows, int cols,
-                            double* out, long ld_out, cudaStream_t s);
+                            double* out, long ld_out, cudaStream_t s, const int* re = nullptr);
 
-// K[mu, i] = dV * (L1[i, mu] + L2[i, mu] - L3[i, mu]); L* are n x N.
+// K[mu, i] = dV * (L1[i, mu] + L2[i, mu] - L3[i, mu]) 2^ce[mu]; L* are n x N.
 cudaError_t assemble_k_f64(const double* L1, const double* L2, const double* L3, int n, int N,
-                           double dV, double* K, cudaStream_t s);
+                           double dV, const int* ce, double* K, cudaStream_t s);
 
 // *out = -sum_j a[j] * b[j] over `len` doubles, fixed summation order.
 // `work` holds at least reduce_work_elems() doubles.
@@ -103,9 +117,9 @@ cudaError_t potential_rows_f64(const double* v, const double* phi, long ng, int 
 cudaError_t dot_f64(const double* a, const double* b, long len, double scale, double* work,
                     double* out, cudaStream_t s);
 
-// K[mu][nu] = dV (Y[mu][nu] + Y[nu][mu] - Z[mu][nu]) for N x N matrices.
-cudaError_t assemble_full_f64(const double* Y, const double* Z, int N, double dV, double* K,
-                              cudaStream_t s);
+// K[mu][nu] = dV (Y[mu][nu] + Y[nu][mu] - Z[mu][nu]) 2^(ce[mu] + ce[nu]) for N x N matrices.
+cudaError_t assemble_full_f64(const double* Y, const double* Z, int N, double dV, const int* ce,
+                              double* K, cudaStream_t s);
 
 // GPU ISDF set-up (xk_isdf.cu), all FP64: from Phi (ng x N) and Phi_g
 // (na x N), X_gg into Xgg (na x na, overwritten by its Cholesky factor),

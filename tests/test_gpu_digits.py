@@ -174,3 +174,52 @@ def test_one_block_tiles(xk, n):
     h.release()
     l1, l2, l3 = _lines(phi, idx, V, W, C)
     assert np.array_equal(K, (l1 + l2 - l3).T)
+
+
+def test_graded_basis(xk):
+    """Basis functions scaled by 2^k and the rows of C by 2^-k are the same calculation:
+    every result of an FP64 handle follows to the last bit."""
+    grid, N, n, na = 17, 129, 64, 129
+    rng = np.random.default_rng(8)
+    Ng = grid ** 3
+    phi, C = rng.standard_normal((Ng, N)), rng.standard_normal((N, n)) / N
+    V, W = rng.standard_normal((na, Ng)), rng.standard_normal((na, na))
+    idx = np.sort(rng.permutation(Ng)[:na])
+
+    def run(k):
+        s = np.exp2(k)
+        h = xk.Handle(phi * s, idx, V, W + W.T, 0.25, n, mode="fp64")
+        c = C / s[:, None]
+        K, E = h.build(c)
+        Kij, xi, _, _ = h.ace()
+        J, EJ = h.coulomb(c, grid, 6.0)
+        out = (K / s[:, None], E, Kij, xi / s[:, None], h.energy(c), J / s[:, None] / s, EJ,
+               h.build_full(c) / s[:, None] / s)
+        h.release()
+        return out
+
+    for a, b in zip(run(np.zeros(N)), run(rng.integers(-40, 41, size=N).astype(np.float64))):
+        assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("r", [0, 10, 30])
+def test_small_points(xk, r):
+    """Interpolation points where the basis is 2^-r of its usual size, with potentials that
+    make up for it, against extended precision: eight roundings of 2^-53 in the 2-norm of
+    the three lines, as for points of one size.  V and W are returned as they came."""
+    Ng, N, n, na = 4096, 24, 20, 400
+    rng = np.random.default_rng(9)
+    phi, C = rng.standard_normal((Ng, N)), rng.standard_normal((N, n))
+    idx = np.sort(rng.permutation(Ng)[:na])
+    s = np.exp2(-rng.integers(0, r + 1, size=na).astype(np.float64))
+    phi[idx] *= s[:, None]
+    V, W = rng.standard_normal((na, Ng)) / s[:, None] ** 2, rng.standard_normal((na, na))
+    W = (W + W.T) / s[:, None] ** 2 / s ** 2
+    h = xk.Handle(phi, idx, V, W, 1.0, n, mode="fp64")
+    K, _ = h.build(C)
+    W1, V1, _ = h.tables([0, na - 1])
+    h.release()
+    assert np.array_equal(W1, W) and np.array_equal(V1, V[[0, na - 1]])
+    x = _lines(*(a.astype(np.longdouble) if a.dtype.kind == "f" else a for a in (phi, idx, V, W, C)))
+    err = np.linalg.norm((K - (x[0] + x[1] - x[2]).T).astype(np.float64))
+    assert err <= 8 * 2.0 ** -53 * sum(np.linalg.norm(l.astype(np.float64)) for l in x)
