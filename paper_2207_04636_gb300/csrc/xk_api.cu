@@ -1256,10 +1256,12 @@ int xk_ace(xk_handle* h, double* Kij_out, double* xi_out, double* sign_out, int*
   int br = 0;
   std::vector<double> sg(n, 1.0);
   // K_ij: from 2e7 multiply-adds the digit product (then symmetrised), below the
-  // kernel that spreads it over the SMs
-  xk::DGemm kij{n, n, N, h->C, n, true, h->K, n, false, h->Kij, n, 1.0, nullptr, 0, 0, h->work};
+  // kernel that spreads it over the SMs.  C's and K's rows are graded oppositely, by the
+  // size of their basis function: the digits are taken of rows brought to one size (in Ce, Y).
+  xk::DGemm kij{n, n, N, h->Ce, n, true, h->Y, n, false, h->Kij, n, 1.0, nullptr, 0, 0, h->work};
   kij.scale = digit_scratch(h->xi, (size_t)N * n, n, n);
   if (xk::digit_gemm_wanted(kij)) {
+    XK_CUDA(xk::balance_rows_f64(h->C, h->K, N, n, h->Ce, h->Y, s));
     XK_CUDA(xk::dgemm(kij, s));
     XK_CUDA(xk::symmetrize_f64(h->Kij, n, s));
   } else {

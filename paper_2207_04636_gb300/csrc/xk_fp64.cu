@@ -214,22 +214,49 @@ __device__ __forceinline__ int exponent_of(int hi, int limit) {  // hi: high wor
   return hi <= 0 || hi >= 0x7ff00000 ? 0 : max(-limit, min(limit, (hi >> 20) - 1022));
 }
 
+// High word of the largest |x| of a row, over a warp.
+__device__ __forceinline__ int row_max_hi(const double* __restrict__ row, int cols) {
+  int m = 0;
+  for (int c = threadIdx.x & 31; c < cols; c += 32) m = max(m, __double2hiint(row[c]) & 0x7fffffff);
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  return m;
+}
+
 // One warp per row.
 __global__ void row_exponents_kernel(const double* __restrict__ p, long ld, const int32_t* __restrict__ idx,
                                      int rows, int cols, int limit, int* __restrict__ out) {
   const int lane = threadIdx.x & 31;
   const long r = (long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (r >= rows) return;
-  const double* row = p + (idx ? (long)idx[r] : r) * ld;
-  int m = 0;
-  for (int c = lane; c < cols; c += 32) m = max(m, __double2hiint(row[c]) & 0x7fffffff);
-  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  const int m = row_max_hi(p + (idx ? (long)idx[r] : r) * ld, cols);
   if (lane == 0) out[r] = exponent_of(m, limit);
 }
 
 cudaError_t row_exponents_f64(const double* p, long ld, const int32_t* idx, int rows, int cols, int limit,
                               int* out, cudaStream_t s) {
   row_exponents_kernel<<<(unsigned)((rows + 7) / 8), 256, 0, s>>>(p, ld, idx, rows, cols, limit, out);
+  count_launch();
+  return cudaGetLastError();
+}
+
+// One warp per row.
+__global__ void balance_rows_kernel(const double* __restrict__ A, const double* __restrict__ B, int rows,
+                                    int cols, double* __restrict__ A2, double* __restrict__ B2) {
+  const long r = (long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (r >= rows) return;
+  const double *a = A + r * cols, *b = B + r * cols;
+  const int ma = row_max_hi(a, cols), mb = row_max_hi(b, cols), big = max(ma, mb);
+  const int e = ma == 0 || mb == 0 || big >= 0x7ff00000
+                    ? 0 : (exponent_of(mb, 1022) - exponent_of(ma, 1022)) >> 1;
+  for (int c = threadIdx.x & 31; c < cols; c += 32) {
+    A2[r * cols + c] = scalbn(a[c], e);
+    B2[r * cols + c] = scalbn(b[c], -e);
+  }
+}
+
+cudaError_t balance_rows_f64(const double* A, const double* B, int rows, int cols, double* A2, double* B2,
+                             cudaStream_t s) {
+  balance_rows_kernel<<<(unsigned)((rows + 7) / 8), 256, 0, s>>>(A, B, rows, cols, A2, B2);
   count_launch();
   return cudaGetLastError();
 }

@@ -65,6 +65,9 @@ cudaError_t row_exponents_f64(const double* p, long ld, const int32_t* idx, int 
                               int* out, cudaStream_t s);
 cudaError_t col_exponents_f64(const double* p, long ld, long rows, int cols, int limit, int* out,
                               cudaStream_t s);
+// A2 = A 2^e, B2 = B 2^-e, row by row, with e such that both have rows of one size.
+cudaError_t balance_rows_f64(const double* A, const double* B, int rows, int cols, double* A2, double* B2,
+                             cudaStream_t s);
 // dst[r][c] = src[r][c] 2^(rm re[r] + cm ce[c]) (re, ce nullable; dst may be src).
 cudaError_t scale_f64(const double* src, double* dst, long rows, long cols, const int* re, int rm,
                       const int* ce, int cm, cudaStream_t s);

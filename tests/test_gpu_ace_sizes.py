@@ -32,3 +32,28 @@ def test_sizes(n):
     # xi xi^T gives K back on the occupied space: n-term sums, times K_ij's conditioning
     err = np.abs((xi @ xi.T) @ C - K).max()
     assert err <= 16 * n * 2.0 ** -53 * np.linalg.cond(Kij0) * np.abs(K).max()
+
+
+def test_graded_basis():
+    """Basis functions scaled by 2^k and the rows of C by 2^-k: K_ij and the vectors follow
+    to the last bit, with K_ij from 2e7 multiply-adds on (n = 280) formed from digits."""
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2207_04636_gb300 as xk
+    N = n = 280
+    Ng = 300
+    rng = np.random.default_rng(1)
+    phi = rng.standard_normal((Ng, N)) / np.sqrt(Ng)
+    C = np.linalg.qr(rng.standard_normal((N, n)))[0]
+    V, W = np.diag(rng.uniform(5.0, 15.0, Ng)), np.zeros((Ng, Ng))
+
+    def run(k):
+        s = np.exp2(k)[:, None]
+        h = xk.Handle(phi * s.T, np.arange(Ng), V, W, 1.0, n, mode="fp64")
+        h.build(C / s)
+        Kij, xi, _, br = h.ace()
+        h.release()
+        return Kij, xi / s, br == "cholesky"
+
+    for a, b in zip(run(np.zeros(N)), run(rng.integers(-40, 41, size=N).astype(np.float64))):
+        assert np.array_equal(a, b)
