@@ -2951,6 +2951,7 @@ struct MixedState {
          *EpC = nullptr, *Lf = nullptr, *dwork = nullptr;
   unsigned* am = nullptr;
   unsigned* rowmax = nullptr;
+  int* lexp = nullptr;  // Q by digits: rows of L are held times 2^-lexp, those of C taken times 2^lexp
   int* status = nullptr;
   int xa = 1, partsA = 1, partsC = 1, splitsL1 = 1, splitsL23 = 1;
   int ychunkA = 64, ychunkC = 64;
@@ -3159,6 +3160,20 @@ size_t dwork_elems(int64_t Ng, int N, int n) {
   return std::max({w(N, N, (int)Ng), (size_t)q_ksplit(N) * N * n, w((int)Ng, N, N), (size_t)1});
 }
 
+// Q^T = C^T L as one product of digits.  C's rows and L's are graded oppositely, by the size of
+// their basis function, which digits do not bear (xk_digits.cu): L is held with rows of largest
+// element in [1/2, 1) and C taken to match.
+DGemm q_product(const MixedState* m) {
+  const int N = m->N, n = m->n;
+  DGemm g{n, N, N, m->part, n, true, m->Lf, N, false, m->CT64, m->Np, 1.0, nullptr, 0, q_ksplit(N), m->dwork};
+  if (2 * (size_t)m->Naux * n >= digit_scale_ints(n, N)) g.scale = reinterpret_cast<int*>(m->D23);
+  return g;
+}
+
+// From 6e7 multiply-adds (of which the triangle needs half) the FP64 pipe takes longer than the
+// digit products on the tensor cores (73 against 40 us at N = 832, n = 128).
+bool q_by_digits(const DGemm& g) { return (double)g.K * g.N * g.M >= 6e7 && digit_gemm_wanted(g); }
+
 }  // namespace
 
 size_t mixed_footprint(int64_t Ng, int N, int n, int Naux, int NaT) {
@@ -3175,7 +3190,7 @@ size_t mixed_footprint(int64_t Ng, int N, int n, int Naux, int NaT) {
   b += na * n * 8 + (size_t)n * p.Na8 * 8 + 2 * (size_t)n * p.Ng8 * 2 + 2 * (size_t)n * p.Na8 * 2;
   b += (size_t)p.splitsL1 * N * n * 4 + (size_t)p.splitsL23 * N * n * 4;
   b += (size_t)(p.epA + p.epC) * 8;
-  b += (size_t)N * N * 8 + (size_t)N * n * 8 + dwork_elems(Ng, N, n) * 8;
+  b += (size_t)N * N * 8 + (size_t)N * n * 8 + dwork_elems(Ng, N, n) * 8 + (size_t)N * 4;
   b += 2 * stage_elems(Ng, N, NaT, p.Ng8) * 8;
   return b + 64 * 1024;
 }
@@ -3364,7 +3379,7 @@ cudaError_t mixed_create(int64_t Ng, int N, int n, int NaT, int g0, int g1, cons
   MX(m->D23T_m, (size_t)n * p.Na8); MX(m->D23T_h, (size_t)n * p.Na8);
   MX(m->L1p, (size_t)p.splitsL1 * N * n); MX(m->L23p, (size_t)p.splitsL23 * N * n);
   MX(m->EpA, (size_t)p.epA); MX(m->EpC, (size_t)p.epC);
-  MX(m->sc, NSC); MX(m->am, NAMC); MX(m->status, 4); MX(m->rowmax, (size_t)n);
+  MX(m->sc, NSC); MX(m->am, NAMC); MX(m->status, 4); MX(m->rowmax, (size_t)n); MX(m->lexp, (size_t)N);
   MX(m->Lf, (size_t)N * N);
   MX(m->part, std::max((size_t)N * n, (size_t)512));  // sums of the final kernel's blocks
   MX(m->dwork, dwork_elems(Ng, N, n));
@@ -3425,6 +3440,10 @@ cudaError_t mixed_create(int64_t Ng, int N, int n, int NaT, int g0, int g1, cons
     set_phi_scale_kernel<<<1, 32, 0, s>>>(m->am, m->sc);
     count_launch(4);
     e = split_rows<double>(phip, ng, N, N, m->sc, SC_PHIP, m->phi_m, m->phi_h, p.Np, s, m->phi_l);
+    if (e == cudaSuccess && q_by_digits(q_product(m))) {  // L is needed for Q alone from here on
+      e = row_exponents_f64(m->Lf, N, nullptr, N, N, 1022, m->lexp, s);
+      if (e == cudaSuccess) e = scale_f64(m->Lf, m->Lf, N, N, m->lexp, -1, nullptr, 0, s);
+    }
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return fin(e);
   }
@@ -3592,14 +3611,12 @@ cudaError_t mixed_enqueue_pre(MixedState* m, const double* C, cudaStream_t s, co
   hook(0, 1);
   e = cudaMemsetAsync(m->am + AM_C, 0, (NAMC - AM_C) * 4, s);
   if (e != cudaSuccess) return e;
-  {  // Q^T = C^T L.  From 6e7 multiply-adds (of which the triangle needs half) the
-     // FP64 pipe takes longer than the digit products on the tensor cores (73 against
-     // 40 us at N = 832, n = 128)
-    DGemm g{n, N, N, C, n, true, m->Lf, N, false, m->CT64, m->Np, 1.0, nullptr, 0, q_ksplit(N), m->dwork};
-    if (2 * (size_t)m->Naux * n >= digit_scale_ints(n, N))
-      g.scale = reinterpret_cast<int*>(m->D23);
-    if ((double)N * N * n >= 6e7 && digit_gemm_wanted(g)) {
-      e = dgemm(g, s);
+  {  // Q^T = C^T L
+    const DGemm g = q_product(m);
+    if (q_by_digits(g)) {
+      // (part is idle until the final kernel)
+      e = scale_f64(C, m->part, N, n, m->lexp, 1, nullptr, 0, s);
+      if (e == cudaSuccess) e = dgemm(g, s);
       if (e != cudaSuccess) return e;
       absmax_kernel<double><<<blocks_for((long)N * n), 256, 0, s>>>(m->CT64, n, N, m->Np, m->am + AM_C);
     } else {

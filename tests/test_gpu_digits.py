@@ -223,3 +223,19 @@ def test_small_points(xk, r):
     x = _lines(*(a.astype(np.longdouble) if a.dtype.kind == "f" else a for a in (phi, idx, V, W, C)))
     err = np.linalg.norm((K - (x[0] + x[1] - x[2]).T).astype(np.float64))
     assert err <= 8 * 2.0 ** -53 * sum(np.linalg.norm(l.astype(np.float64)) for l in x)
+
+
+def test_graded_basis_tensor_path(xk):
+    """The tensor path's Q = L^T C, from 6e7 multiply-adds on formed from digits: a graded
+    basis gives the same energy to the last bit."""
+    Ng, N, n, na = 2000, 832, 100, 150
+    rng = np.random.default_rng(11)
+    phi, C = rng.standard_normal((Ng, N)) / np.sqrt(Ng), rng.standard_normal((N, n)) / np.sqrt(N)
+    V, W = rng.standard_normal((na, Ng)), rng.standard_normal((na, na))
+    idx = np.sort(rng.permutation(Ng)[:na])
+    E = []
+    for k in (np.zeros(N), rng.integers(-20, 21, size=N).astype(np.float64)):
+        h = xk.Handle(phi * np.exp2(k), idx, V, W + W.T, 0.25, n, mode="f16x3")
+        E.append(h.energy(C * np.exp2(-k)[:, None]))
+        h.release()
+    assert E[0] == E[1] and np.isfinite(E[0])
