@@ -643,6 +643,14 @@ int enqueue_build(xk_handle* h) {
   return XK_OK;
 }
 
+// The basis at the interpolation points for the ISDF set-up: phig[g] = Phi[idx[g]] 2^-u[g], rows of
+// largest element in [1/2, 1) (|u| <= 64).
+cudaError_t isdf_points_basis(const double* phi, int N, const int32_t* idx, int na, double* phig, int* u,
+                              cudaStream_t s) {
+  const cudaError_t e = xk::row_exponents_f64(phi, N, idx, na, N, 64, u, s);
+  return e == cudaSuccess ? xk::gather_rows_f64(phi, N, idx, na, N, phig, N, s, u) : e;
+}
+
 }  // namespace
 
 extern "C" {
@@ -721,7 +729,7 @@ static int setup_impl(int64_t Ng, int32_t N, int32_t n, int32_t Naux, const doub
   // Phi, Phi_g, X_gg, chi, V, W and the product work (freed before return)
   const size_t isdf_tmp = (isdf && mode != XK_FP64)
       ? ((size_t)Ng * N + (size_t)Naux * N + 2 * (size_t)Naux * Naux + 2 * (size_t)Naux * Ng +
-         max_work(Ng, N, n, Naux) + (size_t)Naux) * 8 + (size_t)Naux * 4
+         max_work(Ng, N, n, Naux) + (size_t)Naux) * 8 + 2 * (size_t)Naux * 4
       : 0;
 
   // admission: now (queue_ms < 0) or in arrival order within queue_ms
@@ -807,10 +815,11 @@ static int setup_impl(int64_t Ng, int32_t N, int32_t n, int32_t Naux, const doub
     if (e == cudaSuccess && !isdf)
       e = cudaMemcpyAsync(h->W, W, gs * na * 8, cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(h->idx, idx, na * 4, cudaMemcpyHostToDevice, h->stream);
-    if (e == cudaSuccess && isdf)
-      e = xk::gather_rows_f64(h->phi, N, h->idx, Naux, N, h->phig, N, h->stream);
+    int* u = reinterpret_cast<int*>(h->psi);  // units of V and W as they stand: 2^(2 u)
+    if (e == cudaSuccess && !isdf) e = cudaMemsetAsync(u, 0, na * 4, h->stream);
+    if (e == cudaSuccess && isdf) e = isdf_points_basis(h->phi, N, h->idx, Naux, h->phig, u, h->stream);
     if (e == cudaSuccess && isdf)  // X_gg in Q, chi in V2 (both scratch of the build)
-      e = xk::isdf_tables_f64(h->phi, (long)ng, N, h->phig, Naux, grid, L, h->Q, h->V2, h->V, h->W,
+      e = xk::isdf_tables_f64(h->phi, (long)ng, N, h->phig, u, Naux, grid, L, h->Q, h->V2, h->V, h->W,
                               h->work, h->status, &h->ridge, h->stream);
     // the units of the tables; |ge| <= 64 keeps V and W far from the ends of the range
     if (e == cudaSuccess) e = xk::col_exponents_f64(h->phi, N, Ng, N, 1022, h->be, h->stream);
@@ -818,8 +827,9 @@ static int setup_impl(int64_t Ng, int32_t N, int32_t n, int32_t Naux, const doub
     if (e == cudaSuccess) e = xk::row_exponents_f64(h->phi, N, h->idx, Naux, N, 64, h->ge, h->stream);
     if (e == cudaSuccess)
       e = xk::gather_rows_f64(h->phi, N, h->idx + g0, ga, N, h->phig, N, h->stream, h->ge + g0);
-    if (e == cudaSuccess) e = xk::scale_f64(h->V, h->V, gs, ng, h->ge + g0, 2, nullptr, 0, h->stream);
-    if (e == cudaSuccess) e = xk::scale_f64(h->W, h->W, gs, na, h->ge + g0, 2, h->ge, 2, h->stream);
+    if (e == cudaSuccess) e = xk::sub_i32(h->ge, u, Naux, u, h->stream);
+    if (e == cudaSuccess) e = xk::scale_f64(h->V, h->V, gs, ng, u + g0, 2, nullptr, 0, h->stream);
+    if (e == cudaSuccess) e = xk::scale_f64(h->W, h->W, gs, na, u + g0, 2, u, 2, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e == cudaErrorInvalidValue && isdf)
       return bail(fail(XK_EINVAL, "xk_setup_isdf: X_gg is not positive definite even with the ridge"));
@@ -839,7 +849,7 @@ static int setup_impl(int64_t Ng, int32_t N, int32_t n, int32_t Naux, const doub
         tmp.clear();
       };
       double *dphi = nullptr, *dphig = nullptr, *Xgg = nullptr, *chi = nullptr, *dV_ = nullptr,
-             *dW = nullptr, *wk = nullptr, *didx = nullptr;
+             *dW = nullptr, *wk = nullptr, *didx = nullptr, *du = nullptr;
       e = talloc(&dphi, ng * N);
       if (e == cudaSuccess) e = talloc(&dphig, na * N);
       if (e == cudaSuccess) e = talloc(&Xgg, na * na);
@@ -848,13 +858,17 @@ static int setup_impl(int64_t Ng, int32_t N, int32_t n, int32_t Naux, const doub
       if (e == cudaSuccess) e = talloc(&dW, na * na);
       if (e == cudaSuccess) e = talloc(&wk, std::max(max_work(Ng, N, n, Naux), na));
       if (e == cudaSuccess) e = talloc(&didx, (na + 1) / 2);
+      if (e == cudaSuccess) e = talloc(&du, (na + 1) / 2);
       int32_t* di = reinterpret_cast<int32_t*>(didx);
+      int* u = reinterpret_cast<int*>(du);
       if (e == cudaSuccess) e = cudaMemcpyAsync(dphi, phi, ng * N * 8, cudaMemcpyHostToDevice, h->stream);
       if (e == cudaSuccess) e = cudaMemcpyAsync(di, idx, na * 4, cudaMemcpyHostToDevice, h->stream);
-      if (e == cudaSuccess) e = xk::gather_rows_f64(dphi, N, di, Naux, N, dphig, N, h->stream);
+      if (e == cudaSuccess) e = isdf_points_basis(dphi, N, di, Naux, dphig, u, h->stream);
       if (e == cudaSuccess)
-        e = xk::isdf_tables_f64(dphi, (long)ng, N, dphig, Naux, grid, L, Xgg, chi, dV_, dW, wk,
+        e = xk::isdf_tables_f64(dphi, (long)ng, N, dphig, u, Naux, grid, L, Xgg, chi, dV_, dW, wk,
                                 h->status, &h->ridge, h->stream);
+      if (e == cudaSuccess) e = xk::scale_f64(dV_, dV_, Naux, Ng, u, -2, nullptr, 0, h->stream);
+      if (e == cudaSuccess) e = xk::scale_f64(dW, dW, Naux, Naux, u, -2, u, -2, h->stream);
       if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
       if (e == cudaSuccess) {  // chi and X_gg are no longer needed
         cudaFree(chi); cudaFree(Xgg);

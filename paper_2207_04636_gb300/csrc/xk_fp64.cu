@@ -261,6 +261,17 @@ cudaError_t balance_rows_f64(const double* A, const double* B, int rows, int col
   return cudaGetLastError();
 }
 
+__global__ void sub_kernel(const int* a, const int* b, int n, int* out) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) out[i] = a[i] - b[i];
+}
+
+cudaError_t sub_i32(const int* a, const int* b, int n, int* out, cudaStream_t s) {
+  sub_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(a, b, n, out);
+  count_launch();
+  return cudaGetLastError();
+}
+
 // One thread per column and chunk of rows (blockIdx.y).
 __global__ void col_max_kernel(const double* __restrict__ p, long ld, long rows, int cols, long chunk,
                                int* __restrict__ out) {

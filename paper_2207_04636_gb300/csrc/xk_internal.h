@@ -68,6 +68,8 @@ cudaError_t col_exponents_f64(const double* p, long ld, long rows, int cols, int
 // A2 = A 2^e, B2 = B 2^-e, row by row, with e such that both have rows of one size.
 cudaError_t balance_rows_f64(const double* A, const double* B, int rows, int cols, double* A2, double* B2,
                              cudaStream_t s);
+// out[i] = a[i] - b[i].
+cudaError_t sub_i32(const int* a, const int* b, int n, int* out, cudaStream_t s);
 // dst[r][c] = src[r][c] 2^(rm re[r] + cm ce[c]) (re, ce nullable; dst may be src).
 cudaError_t scale_f64(const double* src, double* dst, long rows, long cols, const int* re, int rm,
                       const int* ce, int cm, cudaStream_t s);
@@ -131,7 +133,11 @@ cudaError_t assemble_full_f64(const double* Y, const double* Z, int N, double dV
 // split-K work of the products (dgemm_ksplit sizes) and at least na doubles.
 // A ridge of 1e-14 tr(X_gg)/na is added when the plain factorisation fails
 // (*ridge_out); cudaErrorInvalidValue if it still fails.
-cudaError_t isdf_tables_f64(const double* phi, long ng, int N, const double* phig, int na,
+// phig holds the rows of Phi_g times 2^-u[g] (u: device): the row of a point where the basis
+// is small is as large as any in X_gg and in the solves, whose digit products (xk_digits.cu)
+// would lose bits otherwise.  X_gg and X_gR then stand times 2^(-2 u) on the side of each g, and
+// chi, V and W come out times 2^(2 u).
+cudaError_t isdf_tables_f64(const double* phi, long ng, int N, const double* phig, const int* u, int na,
                             int grid, double L, double* Xgg, double* chi, double* V, double* W,
                             double* work, int* status, double* ridge_out, cudaStream_t s);
 // Interpolation points (Sec. III.A) by a greedy complete-pivoting Cholesky of

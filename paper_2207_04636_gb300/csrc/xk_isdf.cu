@@ -34,9 +34,10 @@ __global__ void square_kernel(double* __restrict__ a, long rows, long cols, long
   }
 }
 
-__global__ void add_diag_kernel(double* __restrict__ a, int n, long ld, double d) {
+// d in the units of X_gg's rows and columns.
+__global__ void add_diag_kernel(double* __restrict__ a, int n, long ld, double d, const int* __restrict__ u) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    a[(long)i * ld + i] += d;
+    a[(long)i * ld + i] += scalbn(d, -4 * u[i]);
 }
 
 __global__ void copy_diag_kernel(const double* __restrict__ a, int n, long ld, double* __restrict__ out) {
@@ -379,7 +380,7 @@ cudaError_t cholesky_solve_f64(double* L, int n, long ldl, double* B, long ldb, 
   return cudaGetLastError();
 }
 
-cudaError_t isdf_tables_f64(const double* phi, long ng, int N, const double* phig, int na,
+cudaError_t isdf_tables_f64(const double* phi, long ng, int N, const double* phig, const int* u, int na,
                             int grid, double L, double* Xgg, double* chi, double* V, double* W,
                             double* work, int* status, double* ridge_out, cudaStream_t s) {
   cudaError_t e;
@@ -418,15 +419,18 @@ cudaError_t isdf_tables_f64(const double* phi, long ng, int N, const double* phi
     e = gram();
     if (e != cudaSuccess) return e;
     std::vector<double> d(na);
+    std::vector<int> hu(na);
+    e = cudaMemcpyAsync(hu.data(), u, (size_t)na * 4, cudaMemcpyDeviceToHost, s);
+    if (e != cudaSuccess) return e;
     copy_diag_kernel<<<nblocks(na), 256, 0, s>>>(Xgg, na, na, work);
     count_launch();
     e = cudaMemcpyAsync(d.data(), work, (size_t)na * 8, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return e;
     double tr = 0.0;
-    for (double v : d) tr += v;
+    for (int i = 0; i < na; ++i) tr += std::ldexp(d[i], 4 * hu[i]);
     ridge = 1e-14 * tr / na;
-    add_diag_kernel<<<nblocks(na), 256, 0, s>>>(Xgg, na, na, ridge);
+    add_diag_kernel<<<nblocks(na), 256, 0, s>>>(Xgg, na, na, ridge, u);
     count_launch();
     e = cudaMemsetAsync(status, 0, 4, s);
     if (e == cudaSuccess) e = cholesky_blocked_f64(Xgg, na, na, status, scale, s);

@@ -119,3 +119,51 @@ def test_isdf_points_two_stage_then_tables(xk):
     _, V0, W0, _ = oracle.isdf_tables(c.phi, idx, c.L, c.grid)
     K0, E0 = oracle.exx_rps_occri(c.phi, idx, V0, W0, c.C, c.dV)
     assert abs(E - E0) <= 1e-8
+
+
+def test_isdf_small_points(xk):
+    """Interpolation points where the basis is up to 2^-15 of its usual size (X_gg's diagonal
+    2^-60), with solves from digits: V in units of the points against extended precision,
+    to the conditioning of X_gg in those units."""
+    grid, N, n, na, L = 17, 20, 4, 130, 6.0
+    ng = grid ** 3
+    rng = np.random.default_rng(12)
+    phi = rng.standard_normal((ng, N))
+    idx = np.sort(rng.permutation(ng)[:na])
+    s = np.exp2(-rng.integers(0, 16, size=na).astype(np.float64))
+    phi[idx] *= s[:, None]
+    rows = np.concatenate([np.argsort(s)[:3], np.argsort(s)[-3:]])
+    h = xk.Handle.isdf(phi, idx, grid, L, n, mode="fp64")
+    try:
+        _, V, ridge = h.tables(rows)
+    finally:
+        h.release()
+    assert ridge == 0.0
+    x = phi.astype(np.longdouble)
+    xg = x[idx] / s[:, None]
+    A, B = (xg @ xg.T) ** 2, (xg @ x.T) ** 2
+    cond = np.linalg.cond(A.astype(np.float64))
+    for k in range(na):  # A = L L^T in place, then L Y = B and L^T X = Y
+        A[k, k] = np.sqrt(A[k, k])
+        A[k + 1:, k] /= A[k, k]
+        A[k + 1:, k + 1:] -= np.outer(A[k + 1:, k], A[k + 1:, k])
+    for k in range(na):
+        B[k] = (B[k] - A[k, :k] @ B[:k]) / A[k, k]
+    for k in range(na - 1, -1, -1):
+        B[k] = (B[k] - A[k + 1:, k] @ B[k + 1:]) / A[k, k]
+    j = np.arange(grid)
+    f = np.minimum(j, grid - j)
+    ang = 2 * np.pi * (np.outer(j, j) % grid).astype(np.longdouble) / grid
+    F = np.cos(ang) + np.sin(ang)  # Hartley: its own inverse over grid
+    ker = (L * L / np.pi) / np.maximum(f[:, None, None] ** 2 + f[None, :, None] ** 2 + f[None, None, :] ** 2, 1)
+    ker[0, 0, 0] = 0.0
+    v = np.empty((len(rows), ng))
+    for i, c in enumerate(B[rows]):
+        c = c.reshape(grid, grid, grid)
+        for mul in (ker, 1.0):
+            for ax in range(3):
+                c = np.moveaxis(np.tensordot(F, c, (1, ax)), 0, ax)
+            c = c * mul
+        v[i] = (c / grid ** 3).reshape(-1)
+    err = np.linalg.norm(V * s[rows, None] ** 2 - v, axis=1).max()
+    assert err <= 16 * 2.0 ** -53 * cond * np.linalg.norm(v, axis=1).max()
