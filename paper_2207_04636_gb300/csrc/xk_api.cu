@@ -214,6 +214,7 @@ struct xk_handle {
   //   phig[g][mu] = phi[R_g][mu] 2^-ge[g], psig likewise, V[g] = V_g 2^(2 ge[g]), W likewise on
   //   both sides; V2, M1, M2, Q, M3 and the lines follow, K leaves times 2^be.
   int *be = nullptr, *ge = nullptr;  // N, N_aux
+  int* dig = nullptr;  // scratch of the digit products (digit_ints)
   double* Ce = nullptr;  // C (N x n) times 2^be, of every FP64 call, and E_x of xk_energy (one more
                          // double); tensor path: C of all calls but a build
   // xk_build_full: K_{mu nu} (N x N); FP64 path also M_A, M_C (N_aux x N), Y, Z (N x N)
@@ -303,6 +304,14 @@ size_t max_work(int64_t Ng, int N, int n, int Naux, bool ace_only = false, int g
   return std::max(w, (size_t)Naux);  // the set-up also keeps the diagonal of X_gg here
 }
 
+// Scratch of an FP64 handle's digit products: V2's maxima (ga + N_g) and the largest
+// digit_scale_ints of its products.  (In a buffer that a call left idle it was too small where
+// few points and functions meet a fine grid, and the products ran 10 to 20 times longer as FMAs.)
+size_t digit_ints(int64_t Ng, int N, int n, int Naux, int ga) {
+  const size_t ng = (size_t)Ng, na = (size_t)Naux;
+  return (ga + ng) + xk::digit_scale_ints((int)std::max({ng, na, (size_t)N}), std::max({n, Naux, N}));
+}
+
 // Rows ga of V and W held (ga = Naux unless a shard); Psi_g at all Naux points.
 Plan plan_fp64(int64_t Ng, int N, int n, int Naux, int ga = -1) {
   Plan p;
@@ -318,7 +327,7 @@ Plan plan_fp64(int64_t Ng, int N, int n, int Naux, int ga = -1) {
           + 3 * (size_t)n * n + 2 * (size_t)N * n + n;   // K_ij, L, U, Y, xi, sign
   p.work = max_work(Ng, N, n, Naux, false, ga);
   p.f64 += p.work;
-  p.i32 = 2 * na + N + 2;
+  p.i32 = 2 * na + N + 2 + digit_ints(Ng, N, n, Naux, ga);
   return p;
 }
 
@@ -433,13 +442,6 @@ void fold_marks(xk_handle* h) {
   h->marks.clear();
 }
 
-// Scratch of the tensor-core form of an M x N product (DGemm::scale) in a
-// buffer of `doubles` doubles that is idle during the call; null when it is too
-// small, which leaves the product to the CUDA cores.
-int* digit_scratch(double* buf, size_t doubles, int M, int N) {
-  return 2 * doubles >= xk::digit_scale_ints(M, N) ? reinterpret_cast<int*>(buf) : nullptr;
-}
-
 // Ce = C times 2^be.
 cudaError_t take_c(xk_handle* h, const double* C) {
   return xk::scale_f64(C, h->Ce, h->N, h->n, h->be, 1, nullptr, 0, h->stream);
@@ -454,17 +456,16 @@ int enqueue_fp64(xk_handle* h) {
   auto make = [&](int M, int Nc, int K, const double* A, long lda, bool ta, const double* B, long ldb,
                   bool tb, double* C, long ldc, const double* H, long ldh) {
     DGemm g{M, Nc, K, A, lda, ta, B, ldb, tb, C, ldc, 1.0, H, ldh, 0, h->work};
-    g.scale = digit_scratch(h->MA, (size_t)ga * N, M, Nc);  // M_A: the full K's, idle here
+    g.scale = h->dig + ga + ng;
     return g;
   };
   auto G = [&](auto... a) { return xk::dgemm(make(a...), s); };
-  // V2's largest entries per row and column come with it, at the end of M_A: reading V2
-  // twice more for them took 0.4 of 4.06 ms on the 27-centre cell
+  // V2's largest entries per row and column come with it: reading V2 twice more for them
+  // took 0.4 of 4.06 ms on the 27-centre cell
   DGemm gp = make(ga, ng, n, psl, n, false, h->psi, n, true, h->V2, ng, h->V, ng);
-  const size_t ints = 2 * (size_t)ga * N, maxima = (size_t)ga + ng;
-  if (xk::digit_maxima(gp) && ints >= maxima + xk::digit_scale_ints(std::max(ga, ng), std::max(n, ng))) {
-    gp.rmax = reinterpret_cast<int*>(h->MA) + (ints - maxima);
-    gp.cmax = gp.rmax + ga;
+  if (xk::digit_maxima(gp)) {
+    gp.rmax = h->dig;
+    gp.cmax = h->dig + ga;
   }
   {  // Eq. rpsEx step 1: orbitals on the grid and at the interpolation points.
     StepMark m(h, XK_STEP_ORBITALS);
@@ -527,7 +528,7 @@ int enqueue_energy(xk_handle* h) {
   auto G = [&](int M, int Nc, int K, const double* A, long lda, bool ta, const double* B, long ldb,
                bool tb, double* C, long ldc) {
     DGemm g{M, Nc, K, A, lda, ta, B, ldb, tb, C, ldc, 1.0, nullptr, 0, 0, h->work};
-    g.scale = digit_scratch(h->MA, (size_t)ga * N, M, Nc);
+    g.scale = h->dig;
     return xk::dgemm(g, s);
   };
   {
@@ -563,7 +564,7 @@ int enqueue_full(xk_handle* h) {
   auto G = [&](int M, int Nc, int K, const double* A, long lda, bool ta, const double* B, long ldb,
                bool tb, double* C, long ldc, const double* H, long ldh) {
     DGemm g{M, Nc, K, A, lda, ta, B, ldb, tb, C, ldc, 1.0, H, ldh, 0, h->work};
-    g.scale = digit_scratch(h->M1, (size_t)n * ng, M, Nc);  // M_1: the build's, idle here
+    g.scale = h->dig;
     return xk::dgemm(g, s);
   };
   {
@@ -729,7 +730,8 @@ static int setup_impl(int64_t Ng, int32_t N, int32_t n, int32_t Naux, const doub
   // Phi, Phi_g, X_gg, chi, V, W and the product work (freed before return)
   const size_t isdf_tmp = (isdf && mode != XK_FP64)
       ? ((size_t)Ng * N + (size_t)Naux * N + 2 * (size_t)Naux * Naux + 2 * (size_t)Naux * Ng +
-         max_work(Ng, N, n, Naux) + (size_t)Naux) * 8 + 2 * (size_t)Naux * 4
+         max_work(Ng, N, n, Naux) + (size_t)Naux) * 8 +
+         (2 * (size_t)Naux + digit_ints(Ng, N, n, Naux, ga)) * 4
       : 0;
 
   // admission: now (queue_ms < 0) or in arrival order within queue_ms
@@ -795,6 +797,7 @@ static int setup_impl(int64_t Ng, int32_t N, int32_t n, int32_t Naux, const doub
     XK_ALLOC(h->idx, na);
     XK_ALLOC(h->be, (size_t)N);
     XK_ALLOC(h->ge, na);
+    XK_ALLOC(h->dig, digit_ints(Ng, N, n, Naux, ga));
     XK_ALLOC(h->psi, ng * n);
     XK_ALLOC(h->psig, na * n);
     XK_ALLOC(h->V2, gs * ng);
@@ -820,7 +823,7 @@ static int setup_impl(int64_t Ng, int32_t N, int32_t n, int32_t Naux, const doub
     if (e == cudaSuccess && isdf) e = isdf_points_basis(h->phi, N, h->idx, Naux, h->phig, u, h->stream);
     if (e == cudaSuccess && isdf)  // X_gg in Q, chi in V2 (both scratch of the build)
       e = xk::isdf_tables_f64(h->phi, (long)ng, N, h->phig, u, Naux, grid, L, h->Q, h->V2, h->V, h->W,
-                              h->work, h->status, &h->ridge, h->stream);
+                              h->work, h->dig, digit_ints(Ng, N, n, Naux, ga), h->status, &h->ridge, h->stream);
     // the units of the tables; |ge| <= 64 keeps V and W far from the ends of the range
     if (e == cudaSuccess) e = xk::col_exponents_f64(h->phi, N, Ng, N, 1022, h->be, h->stream);
     if (e == cudaSuccess) e = xk::scale_f64(h->phi, h->phi, Ng, N, nullptr, 0, h->be, -1, h->stream);
@@ -849,7 +852,7 @@ static int setup_impl(int64_t Ng, int32_t N, int32_t n, int32_t Naux, const doub
         tmp.clear();
       };
       double *dphi = nullptr, *dphig = nullptr, *Xgg = nullptr, *chi = nullptr, *dV_ = nullptr,
-             *dW = nullptr, *wk = nullptr, *didx = nullptr, *du = nullptr;
+             *dW = nullptr, *wk = nullptr, *didx = nullptr, *du = nullptr, *ddig = nullptr;
       e = talloc(&dphi, ng * N);
       if (e == cudaSuccess) e = talloc(&dphig, na * N);
       if (e == cudaSuccess) e = talloc(&Xgg, na * na);
@@ -859,6 +862,7 @@ static int setup_impl(int64_t Ng, int32_t N, int32_t n, int32_t Naux, const doub
       if (e == cudaSuccess) e = talloc(&wk, std::max(max_work(Ng, N, n, Naux), na));
       if (e == cudaSuccess) e = talloc(&didx, (na + 1) / 2);
       if (e == cudaSuccess) e = talloc(&du, (na + 1) / 2);
+      if (e == cudaSuccess) e = talloc(&ddig, (digit_ints(Ng, N, n, Naux, ga) + 1) / 2);
       int32_t* di = reinterpret_cast<int32_t*>(didx);
       int* u = reinterpret_cast<int*>(du);
       if (e == cudaSuccess) e = cudaMemcpyAsync(dphi, phi, ng * N * 8, cudaMemcpyHostToDevice, h->stream);
@@ -866,7 +870,7 @@ static int setup_impl(int64_t Ng, int32_t N, int32_t n, int32_t Naux, const doub
       if (e == cudaSuccess) e = isdf_points_basis(dphi, N, di, Naux, dphig, u, h->stream);
       if (e == cudaSuccess)
         e = xk::isdf_tables_f64(dphi, (long)ng, N, dphig, u, Naux, grid, L, Xgg, chi, dV_, dW, wk,
-                                h->status, &h->ridge, h->stream);
+                                reinterpret_cast<int*>(ddig), digit_ints(Ng, N, n, Naux, ga), h->status, &h->ridge, h->stream);
       if (e == cudaSuccess) e = xk::scale_f64(dV_, dV_, Naux, Ng, u, -2, nullptr, 0, h->stream);
       if (e == cudaSuccess) e = xk::scale_f64(dW, dW, Naux, Naux, u, -2, u, -2, h->stream);
       if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
@@ -1199,7 +1203,7 @@ int xk_coulomb(xk_handle* h, int32_t grid, double L, const double* C, double* J_
     StepMark m(h, XK_STEP_ORBITALS);
     XK_CUDA(take_c(h, h->Ce));
     xk::DGemm g1{(int)ng, n, N, h->phi, N, false, h->Ce, n, false, h->psi, n, 1.0, nullptr, 0, 0, h->work};
-    g1.scale = digit_scratch(h->M1, (size_t)n * ng, (int)ng, n);
+    g1.scale = h->dig;
     XK_CUDA(xk::dgemm(g1, s));
   }
   {  // density, Poisson solve, J = dV Phi^T (v o Phi), E_J = dV sum rho v
@@ -1208,7 +1212,7 @@ int xk_coulomb(xk_handle* h, int32_t grid, double L, const double* C, double* J_
     XK_CUDA(xk::poisson_f64(h->Jrho, h->Jv, h->Jtmp, 1, grid, h->Jtab, nullptr, 0, s));
     XK_CUDA(xk::potential_rows_f64(h->Jv, h->phi, (long)ng, N, h->Jphiv, s));
     xk::DGemm gj{N, N, (int)ng, h->phi, N, true, h->Jphiv, N, false, h->Jout, N, h->dV, nullptr, 0, 0, h->work};
-    gj.scale = digit_scratch(h->M1, (size_t)n * ng, N, N);
+    gj.scale = h->dig;
     gj.sym = true;
     XK_CUDA(xk::dgemm(gj, s));
     XK_CUDA(xk::scale_f64(h->Jout, h->Jout, N, N, h->be, 1, h->be, 1, s));
@@ -1273,7 +1277,7 @@ int xk_ace(xk_handle* h, double* Kij_out, double* xi_out, double* sign_out, int*
   // kernel that spreads it over the SMs.  C's and K's rows are graded oppositely, by the
   // size of their basis function: the digits are taken of rows brought to one size (in Ce, Y).
   xk::DGemm kij{n, n, N, h->Ce, n, true, h->Y, n, false, h->Kij, n, 1.0, nullptr, 0, 0, h->work};
-  kij.scale = digit_scratch(h->xi, (size_t)N * n, n, n);
+  kij.scale = reinterpret_cast<int*>(h->xi);  // idle, and 2 N n >= 2 n + 8 ints where it is wanted
   if (xk::digit_gemm_wanted(kij)) {
     XK_CUDA(xk::balance_rows_f64(h->C, h->K, N, n, h->Ce, h->Y, s));
     XK_CUDA(xk::dgemm(kij, s));

@@ -130,7 +130,8 @@ cudaError_t assemble_full_f64(const double* Y, const double* Z, int N, double dV
 // (na x N), X_gg into Xgg (na x na, overwritten by its Cholesky factor),
 // chi = X_gg^{-1} X_gR (na x ng), V = Pois(chi) on the cubic grid^3 grid of
 // side L (na x ng) and W = V chi^T symmetrised (na x na).  `work` holds the
-// split-K work of the products (dgemm_ksplit sizes) and at least na doubles.
+// split-K work of the products (dgemm_ksplit sizes) and at least na doubles, `dig` is
+// DGemm::scale of an na x ng product (dig_ints ints).
 // A ridge of 1e-14 tr(X_gg)/na is added when the plain factorisation fails
 // (*ridge_out); cudaErrorInvalidValue if it still fails.
 // phig holds the rows of Phi_g times 2^-u[g] (u: device): the row of a point where the basis
@@ -139,7 +140,8 @@ cudaError_t assemble_full_f64(const double* Y, const double* Z, int N, double dV
 // chi, V and W come out times 2^(2 u).
 cudaError_t isdf_tables_f64(const double* phi, long ng, int N, const double* phig, const int* u, int na,
                             int grid, double L, double* Xgg, double* chi, double* V, double* W,
-                            double* work, int* status, double* ridge_out, cudaStream_t s);
+                            double* work, int* dig, size_t dig_ints, int* status, double* ridge_out,
+                            cudaStream_t s);
 // Interpolation points (Sec. III.A) by a greedy complete-pivoting Cholesky of
 // X = (F F^T) o (F F^T) for the m candidate rows F (m x N, device): up to
 // `want` pivots (indices into F, selection order) into piv (host), stopping

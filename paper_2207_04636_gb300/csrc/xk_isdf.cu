@@ -382,11 +382,17 @@ cudaError_t cholesky_solve_f64(double* L, int n, long ldl, double* B, long ldb, 
 
 cudaError_t isdf_tables_f64(const double* phi, long ng, int N, const double* phig, const int* u, int na,
                             int grid, double L, double* Xgg, double* chi, double* V, double* W,
-                            double* work, int* status, double* ridge_out, cudaStream_t s) {
+                            double* work, int* dig, size_t dig_ints, int* status, double* ridge_out,
+                            cudaStream_t s) {
   cudaError_t e;
-  // scratch of the tensor-core products: W until W itself is formed, then X_gg
-  const bool digits = 2 * (size_t)na * na >= digit_scale_ints(na, (int)ng);
-  int* scale = digits ? reinterpret_cast<int*>(W) : nullptr;
+  // scratch of the tensor-core products: W until W itself is formed, when that is the
+  // larger (more functions to a Poisson pass)
+  int* scale = dig;
+  size_t ints = dig_ints;
+  if (2 * (size_t)na * na > ints) {
+    scale = reinterpret_cast<int*>(W);
+    ints = 2 * (size_t)na * na;
+  }
   auto gram = [&]() {
     DGemm g{na, na, N, phig, N, false, phig, N, true, Xgg, na, 1.0, nullptr, 0, 0, work};
     g.scale = scale;
@@ -446,11 +452,10 @@ cudaError_t isdf_tables_f64(const double* phi, long ng, int N, const double* phi
   // V = Pois(chi) in batches of functions (the scratch holds one)
   {
     const long g3 = (long)grid * grid * grid;
-    const size_t ints = 2 * (size_t)na * na;
     long nf = std::max<long>(1, std::min<long>(na, (1L << 28) / (g3 * 8)));
-    if (scale)  // the row maxima of a batch go into the scratch of the products
-      nf = std::max<long>(1, std::min<long>(nf, ((long)std::min<size_t>(ints, 1u << 30) - grid - 8) /
-                                                    ((long)grid * grid)));
+    // the row maxima of a batch go into the scratch of the products
+    nf = std::max<long>(1, std::min<long>(nf, ((long)std::min<size_t>(ints, 1u << 30) - grid - 8) /
+                                                  ((long)grid * grid)));
     void* buf = nullptr;
     e = cudaMallocAsync(&buf, ((size_t)nf * g3 + poisson_table_elems(grid)) * 8, s);
     if (e != cudaSuccess) return e;
@@ -467,7 +472,7 @@ cudaError_t isdf_tables_f64(const double* phi, long ng, int N, const double* phi
   // W = V chi^T, symmetrised
   {
     DGemm g{na, na, (int)ng, V, ng, false, chi, ng, true, W, na, 1.0, nullptr, 0, 0, work};
-    g.scale = digits ? reinterpret_cast<int*>(Xgg) : nullptr;
+    g.scale = dig;
     e = dgemm(g, s);
     if (e == cudaSuccess) e = symmetrize_f64(W, na, s);
   }

@@ -239,3 +239,21 @@ def test_graded_basis_tensor_path(xk):
         E.append(h.energy(C * np.exp2(-k)[:, None]))
         h.release()
     assert E[0] == E[1] and np.isfinite(E[0])
+
+
+@pytest.mark.parametrize("Ng,N,n,na", [(27000, 16, 16, 64), (25001, 72, 48, 130), (90001, 33, 31, 65),
+                                       (6145, 40, 32, 130)])
+def test_few_points_on_a_fine_grid(xk, Ng, N, n, na):
+    """A product is formed from digits by its size alone, also where the handle's other
+    buffers are small: a sum 1 + 15 2^-54 is rounded once, to 1 + 2^-50, where FMAs in the
+    order of the terms give 1."""
+    phi, V, W = np.zeros((Ng, N)), np.zeros((na, Ng)), np.zeros((na, na))
+    idx = np.arange(na)
+    phi[0, :16] = phi[Ng - 1, :16] = [1.0] + [2.0 ** -27] * 15
+    V[0, Ng - 1] = 1.0
+    h = xk.Handle(phi, idx, V, W, 1.0, n, mode="fp64")
+    C = np.eye(N, n)
+    K, _ = h.build(C)
+    E = h.energy(C)
+    h.release()
+    assert K[0, 0] == 2 * (1 + 2.0 ** -50) and E == -2 * (1 + 2.0 ** -50) ** 2
