@@ -199,7 +199,8 @@ int xk_admit_state(uint64_t* admitted_bytes, uint32_t* waiting);
  * tables in the handle's own buffers; XK_F16X3 holds FP64 temporaries of
  * about 8 (N_g N + 2 N_aux N_g + 2 N_aux^2) bytes during the call, admitted
  * with the handle.  Errors: as xk_setup, plus XK_EINVAL when grid^3 != N_g,
- * L <= 0 or X_gg is not positive definite even with the ridge.
+ * L <= 0 or X_gg is not positive definite even with the ridge, XK_ETIMEDOUT
+ * (a bounded wait inside a kernel gave up).
  */
 int xk_setup_isdf(int64_t Ng, int32_t N, int32_t n, int32_t Naux,
                   const double* basis_on_points, const int32_t* interp_idx,
@@ -238,7 +239,8 @@ int xk_tables(xk_handle* h, double* W_out, const int32_t* rows, int32_t nrows,
  * One exchange build, blocking.  C (host, N x n) are the occupied
  * coefficients; K_out (host, N x n) receives K_{mu i}; Ex (host) receives
  * E_x.  Builds on one handle are serialised.
- * Errors: XK_EINVAL (null pointers), XK_ECUDA.
+ * Errors: XK_EINVAL (null pointers), XK_ETIMEDOUT (a bounded wait inside a
+ * kernel gave up), XK_ECUDA.
  */
 int xk_build(xk_handle* h, const double* C, double* K_out, double* Ex);
 
@@ -247,7 +249,9 @@ int xk_build(xk_handle* h, const double* C, double* K_out, double* Ex);
  * NULL = the legacy default stream) and returning at once.  C_dev (N x n),
  * K_dev (N x n) and Ex_dev (1 double) are device pointers owned by the
  * caller.  The handle's scratch is reused, so builds on one handle must not
- * overlap: enqueue them on one stream.  Errors: XK_EINVAL, XK_ECUDA.
+ * overlap: enqueue them on one stream.  A bounded wait that gives up is
+ * reported by the handle's next blocking call or ticket.  Errors: XK_EINVAL,
+ * XK_ECUDA.
  */
 int xk_build_device(xk_handle* h, const double* C_dev, double* K_dev, double* Ex_dev,
                     void* stream);
@@ -285,7 +289,7 @@ int xk_build_full(xk_handle* h, const double* C, double* K_out);
  * allocates about 8 N_g (N + 6) bytes of scratch, admitted like xk_setup.
  * C (host, N x n) is copied; J_out (host, N x N) and E_J (host) receive the
  * results.  Errors: XK_EINVAL (null pointers, XK_F16X3 handle,
- * grid^3 != N_g, L <= 0), XK_ENOMEM, XK_ECUDA.
+ * grid^3 != N_g, L <= 0), XK_ENOMEM, XK_ETIMEDOUT, XK_ECUDA.
  */
 int xk_coulomb(xk_handle* h, int32_t grid, double L, const double* C, double* J_out,
                double* E_J);
@@ -324,7 +328,8 @@ int xk_energy_device(xk_handle* h, const double* C_dev, double* Ex_dev, void* st
  * (branch 1, xi = K_{mu i} U |Lambda|^{-1/2}; sign_out gets sign(lambda),
  * zero for dropped columns).  Outputs are host memory: Kij_out n x n,
  * xi_out N x n, sign_out n (nullable), branch (nullable).
- * Errors: XK_EINVAL (no build yet, null pointers), XK_ECUDA.
+ * Errors: XK_EINVAL (no build yet, null pointers), XK_ETIMEDOUT (a bounded wait
+ * inside a kernel gave up), XK_ECUDA.
  */
 int xk_ace(xk_handle* h, double* Kij_out, double* xi_out, double* sign_out, int* branch);
 
@@ -394,8 +399,8 @@ int xk_release(xk_handle* h);
  * bound) for its own TMA copies and MMAs, free its tensor memory and return;
  * the build then reports XK_ETIMEDOUT and the handle stays usable.  Applies
  * to builds enqueued afterwards (a batch keeps the limit its members had
- * when it was created).  No effect on XK_FP64 handles, whose kernels do not
- * wait on one another.  It exists so that the timeout path can be exercised
+ * when it was created).  On XK_FP64 handles it bounds the waits inside the
+ * products formed from digits.  It exists so that the timeout path can be exercised
  * (a tiny limit) and so that a caller can bound a build more tightly than
  * one second per wait.  Errors: XK_EINVAL (NULL handle, negative cycles).
  */

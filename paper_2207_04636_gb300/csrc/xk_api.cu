@@ -232,6 +232,10 @@ struct xk_handle {
   double *Kij = nullptr, *Lf = nullptr, *U = nullptr, *Y = nullptr, *xi = nullptr,
          *sgn = nullptr;
   int* status = nullptr;
+  // code of a bounded wait inside a digit product that gave up (4 ints; that of the tensor
+  // path's builds lies in `mixed`), and the limit of those waits (xk_set_wait_limit)
+  int* wst = nullptr;
+  long long wait = 0;
   double ridge = 0.0;  // xk_setup_isdf: ridge added to X_gg (0 when none was needed)
 
   xk::MixedState* mixed = nullptr;
@@ -327,7 +331,7 @@ Plan plan_fp64(int64_t Ng, int N, int n, int Naux, int ga = -1) {
           + 3 * (size_t)n * n + 2 * (size_t)N * n + n;   // K_ij, L, U, Y, xi, sign
   p.work = max_work(Ng, N, n, Naux, false, ga);
   p.f64 += p.work;
-  p.i32 = 2 * na + N + 2 + digit_ints(Ng, N, n, Naux, ga);
+  p.i32 = 2 * na + N + 6 + digit_ints(Ng, N, n, Naux, ga);
   return p;
 }
 
@@ -384,15 +388,19 @@ void free_handle(xk_handle* h) {
   delete h;
 }
 
-// Status word of the tensor-path kernels of the builds enqueued so far on `s`: copied to
-// h->res_st and cleared in stream order (so a later build on the stream starts from
+// Status word of the tensor-core kernels of the calls enqueued so far on `s`: copied to `to`
+// (pinned) and cleared in stream order (so a later call on the stream starts from
 // zero); 0 once the stream has been waited for when none gave up.
-cudaError_t enqueue_status(xk_handle* h, cudaStream_t s) {
-  h->res_st[0] = 0;
-  if (!h->mixed) return cudaSuccess;
-  int* dev = xk::mixed_status_ptr(h->mixed);
-  cudaError_t e = cudaMemcpyAsync(h->res_st, dev, 16, cudaMemcpyDeviceToHost, s);
+cudaError_t enqueue_status(xk_handle* h, int* to, cudaStream_t s) {
+  to[0] = 0;
+  int* dev = h->mixed ? xk::mixed_status_ptr(h->mixed) : h->wst;
+  cudaError_t e = cudaMemcpyAsync(to, dev, 16, cudaMemcpyDeviceToHost, s);
   return e == cudaSuccess ? cudaMemsetAsync(dev, 0, 16, s) : e;
+}
+
+int gave_up(const char* who, int code) {
+  return fail(XK_ETIMEDOUT, std::string(who) + ": a bounded wait inside a kernel gave up (code " +
+                                std::to_string(code) + ")");
 }
 
 // Records the start or the end of `step` when timing is on.
@@ -457,6 +465,8 @@ int enqueue_fp64(xk_handle* h) {
                   bool tb, double* C, long ldc, const double* H, long ldh) {
     DGemm g{M, Nc, K, A, lda, ta, B, ldb, tb, C, ldc, 1.0, H, ldh, 0, h->work};
     g.scale = h->dig + ga + ng;
+    g.status = h->wst;
+    g.wait = h->wait;
     return g;
   };
   auto G = [&](auto... a) { return xk::dgemm(make(a...), s); };
@@ -529,6 +539,8 @@ int enqueue_energy(xk_handle* h) {
                bool tb, double* C, long ldc) {
     DGemm g{M, Nc, K, A, lda, ta, B, ldb, tb, C, ldc, 1.0, nullptr, 0, 0, h->work};
     g.scale = h->dig;
+    g.status = h->wst;
+    g.wait = h->wait;
     return xk::dgemm(g, s);
   };
   {
@@ -565,6 +577,8 @@ int enqueue_full(xk_handle* h) {
                bool tb, double* C, long ldc, const double* H, long ldh) {
     DGemm g{M, Nc, K, A, lda, ta, B, ldb, tb, C, ldc, 1.0, H, ldh, 0, h->work};
     g.scale = h->dig;
+    g.status = h->wst;
+    g.wait = h->wait;
     return xk::dgemm(g, s);
   };
   {
@@ -785,7 +799,17 @@ static int setup_impl(int64_t Ng, int32_t N, int32_t n, int32_t Naux, const doub
   XK_ALLOC(h->xi, (size_t)N * n);
   XK_ALLOC(h->sgn, (size_t)n);
   XK_ALLOC(h->status, 2);
+  XK_ALLOC(h->wst, 4);
+  e = cudaMemsetAsync(h->wst, 0, 16, h->stream);
+  if (e != cudaSuccess) return bail(cuda_fail(e, "xk_setup"));
   XK_ALLOC(h->red, xk::reduce_work_elems());
+  // code of a wait that gave up while the ISDF tables were formed (0: none)
+  auto tables_code = [&](cudaError_t tables) {
+    int code = 0;
+    if (!isdf || (tables != cudaSuccess && tables != cudaErrorInvalidValue)) return 0;
+    cudaMemcpyAsync(&code, h->wst, 4, cudaMemcpyDeviceToHost, h->stream);
+    return cudaStreamSynchronize(h->stream) == cudaSuccess ? code : 0;
+  };
   const size_t work = max_work(Ng, N, n, Naux, mode != XK_FP64, ga);
   XK_ALLOC(h->work, work);
   if (mode == XK_FP64) {
@@ -823,7 +847,8 @@ static int setup_impl(int64_t Ng, int32_t N, int32_t n, int32_t Naux, const doub
     if (e == cudaSuccess && isdf) e = isdf_points_basis(h->phi, N, h->idx, Naux, h->phig, u, h->stream);
     if (e == cudaSuccess && isdf)  // X_gg in Q, chi in V2 (both scratch of the build)
       e = xk::isdf_tables_f64(h->phi, (long)ng, N, h->phig, u, Naux, grid, L, h->Q, h->V2, h->V, h->W,
-                              h->work, h->dig, digit_ints(Ng, N, n, Naux, ga), h->status, &h->ridge, h->stream);
+                              h->work, h->dig, digit_ints(Ng, N, n, Naux, ga), h->wst, h->status, &h->ridge, h->stream);
+    if (const int code = tables_code(e)) return bail(gave_up("xk_setup_isdf", code));
     // the units of the tables; |ge| <= 64 keeps V and W far from the ends of the range
     if (e == cudaSuccess) e = xk::col_exponents_f64(h->phi, N, Ng, N, 1022, h->be, h->stream);
     if (e == cudaSuccess) e = xk::scale_f64(h->phi, h->phi, Ng, N, nullptr, 0, h->be, -1, h->stream);
@@ -870,7 +895,12 @@ static int setup_impl(int64_t Ng, int32_t N, int32_t n, int32_t Naux, const doub
       if (e == cudaSuccess) e = isdf_points_basis(dphi, N, di, Naux, dphig, u, h->stream);
       if (e == cudaSuccess)
         e = xk::isdf_tables_f64(dphi, (long)ng, N, dphig, u, Naux, grid, L, Xgg, chi, dV_, dW, wk,
-                                reinterpret_cast<int*>(ddig), digit_ints(Ng, N, n, Naux, ga), h->status, &h->ridge, h->stream);
+                                reinterpret_cast<int*>(ddig), digit_ints(Ng, N, n, Naux, ga), h->wst, h->status,
+                                &h->ridge, h->stream);
+      if (const int code = tables_code(e)) {
+        release();
+        return bail(gave_up("xk_setup_isdf", code));
+      }
       if (e == cudaSuccess) e = xk::scale_f64(dV_, dV_, Naux, Ng, u, -2, nullptr, 0, h->stream);
       if (e == cudaSuccess) e = xk::scale_f64(dW, dW, Naux, Naux, u, -2, u, -2, h->stream);
       if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
@@ -1100,14 +1130,12 @@ int xk_build(xk_handle* h, const double* C, double* K_out, double* Ex) {
   if (rc != XK_OK) return rc;
   // the small results go ahead of K into pinned memory: one wait for all
   XK_CUDA(cudaMemcpyAsync(h->res, h->Ex, 8, cudaMemcpyDeviceToHost, h->stream));
-  XK_CUDA(enqueue_status(h, h->stream));
+  XK_CUDA(enqueue_status(h, h->res_st, h->stream));
   XK_CUDA(cudaMemcpyAsync(K_out, h->K, kb, cudaMemcpyDeviceToHost, h->stream));
   XK_CUDA(cudaStreamSynchronize(h->stream));
   *Ex = h->res[0];
   h->has_build = true;
-  if (h->res_st[0] != 0)
-    return fail(XK_ETIMEDOUT, "xk_build: a bounded wait inside a kernel gave up (code " +
-                                  std::to_string(h->res_st[0]) + ")");
+  if (h->res_st[0] != 0) return gave_up("xk_build", h->res_st[0]);
   return XK_OK;
 }
 
@@ -1142,12 +1170,10 @@ int xk_build_full(xk_handle* h, const double* C, double* K_out) {
   XK_CUDA(cudaMemcpyAsync(h->Ce, C, (size_t)h->N * h->n * 8, cudaMemcpyHostToDevice, h->stream));
   int rc = enqueue_full(h);
   if (rc != XK_OK) return rc;
-  XK_CUDA(enqueue_status(h, h->stream));
+  XK_CUDA(enqueue_status(h, h->res_st, h->stream));
   XK_CUDA(cudaMemcpyAsync(K_out, h->Kf, (size_t)h->N * h->N * 8, cudaMemcpyDeviceToHost, h->stream));
   XK_CUDA(cudaStreamSynchronize(h->stream));
-  if (h->res_st[0] != 0)
-    return fail(XK_ETIMEDOUT, "xk_build_full: a bounded wait inside a kernel gave up (code " +
-                                  std::to_string(h->res_st[0]) + ")");
+  if (h->res_st[0] != 0) return gave_up("xk_build_full", h->res_st[0]);
   return XK_OK;
 }
 
@@ -1204,24 +1230,30 @@ int xk_coulomb(xk_handle* h, int32_t grid, double L, const double* C, double* J_
     XK_CUDA(take_c(h, h->Ce));
     xk::DGemm g1{(int)ng, n, N, h->phi, N, false, h->Ce, n, false, h->psi, n, 1.0, nullptr, 0, 0, h->work};
     g1.scale = h->dig;
+    g1.status = h->wst;
+    g1.wait = h->wait;
     XK_CUDA(xk::dgemm(g1, s));
   }
   {  // density, Poisson solve, J = dV Phi^T (v o Phi), E_J = dV sum rho v
     StepMark m(h, XK_STEP_PAIR);
     XK_CUDA(xk::density_f64(h->psi, (long)ng, n, h->Jrho, s));
-    XK_CUDA(xk::poisson_f64(h->Jrho, h->Jv, h->Jtmp, 1, grid, h->Jtab, nullptr, 0, s));
+    XK_CUDA(xk::poisson_f64(h->Jrho, h->Jv, h->Jtmp, 1, grid, h->Jtab, nullptr, 0, nullptr, s));
     XK_CUDA(xk::potential_rows_f64(h->Jv, h->phi, (long)ng, N, h->Jphiv, s));
     xk::DGemm gj{N, N, (int)ng, h->phi, N, true, h->Jphiv, N, false, h->Jout, N, h->dV, nullptr, 0, 0, h->work};
     gj.scale = h->dig;
+    gj.status = h->wst;
+    gj.wait = h->wait;
     gj.sym = true;
     XK_CUDA(xk::dgemm(gj, s));
     XK_CUDA(xk::scale_f64(h->Jout, h->Jout, N, N, h->be, 1, h->be, 1, s));
     XK_CUDA(xk::dot_f64(h->Jrho, h->Jv, (long)ng, h->dV, h->red, h->Jout + (size_t)N * N, s));
   }
   XK_CUDA(cudaMemcpyAsync(h->res, h->Jout + (size_t)N * N, 8, cudaMemcpyDeviceToHost, s));
+  XK_CUDA(enqueue_status(h, h->res_st, s));
   XK_CUDA(cudaMemcpyAsync(J_out, h->Jout, (size_t)N * N * 8, cudaMemcpyDeviceToHost, s));
   XK_CUDA(cudaStreamSynchronize(s));
   *E_J = h->res[0];
+  if (h->res_st[0] != 0) return gave_up("xk_coulomb", h->res_st[0]);
   return XK_OK;
 }
 
@@ -1234,12 +1266,10 @@ int xk_energy(xk_handle* h, const double* C, double* Ex) {
   int rc = enqueue_energy(h);
   if (rc != XK_OK) return rc;
   XK_CUDA(cudaMemcpyAsync(h->res, h->Ce + (size_t)h->N * h->n, 8, cudaMemcpyDeviceToHost, h->stream));
-  XK_CUDA(enqueue_status(h, h->stream));
+  XK_CUDA(enqueue_status(h, h->res_st, h->stream));
   XK_CUDA(cudaStreamSynchronize(h->stream));
   *Ex = h->res[0];
-  if (h->res_st[0] != 0)
-    return fail(XK_ETIMEDOUT, "xk_energy: a bounded wait inside a kernel gave up (code " +
-                                  std::to_string(h->res_st[0]) + ")");
+  if (h->res_st[0] != 0) return gave_up("xk_energy", h->res_st[0]);
   return XK_OK;
 }
 
@@ -1278,10 +1308,16 @@ int xk_ace(xk_handle* h, double* Kij_out, double* xi_out, double* sign_out, int*
   // size of their basis function: the digits are taken of rows brought to one size (in Ce, Y).
   xk::DGemm kij{n, n, N, h->Ce, n, true, h->Y, n, false, h->Kij, n, 1.0, nullptr, 0, 0, h->work};
   kij.scale = reinterpret_cast<int*>(h->xi);  // idle, and 2 N n >= 2 n + 8 ints where it is wanted
+  kij.status = h->wst;
+  kij.wait = h->wait;
+  int* chol = h->res_st + 4;  // beside the status word
+  h->res_st[0] = 0;
   if (xk::digit_gemm_wanted(kij)) {
     XK_CUDA(xk::balance_rows_f64(h->C, h->K, N, n, h->Ce, h->Y, s));
     XK_CUDA(xk::dgemm(kij, s));
     XK_CUDA(xk::symmetrize_f64(h->Kij, n, s));
+    XK_CUDA(cudaMemcpyAsync(h->res_st, h->wst, 4, cudaMemcpyDeviceToHost, s));
+    XK_CUDA(cudaMemsetAsync(h->wst, 0, 16, s));
   } else {
     XK_CUDA(xk::kij_f64(h->C, h->K, N, n, h->Kij, s));
   }
@@ -1290,11 +1326,12 @@ int xk_ace(xk_handle* h, double* Kij_out, double* xi_out, double* sign_out, int*
   // the Cholesky branch's vectors are formed and copied before the host has seen
   // whether it holds: one wait instead of two
   XK_CUDA(xk::trsm_right_lt_f64(h->Lf, n, h->K, N, h->xi, s, h->U));
-  XK_CUDA(cudaMemcpyAsync(h->res_st, h->status, 4, cudaMemcpyDeviceToHost, s));
+  XK_CUDA(cudaMemcpyAsync(chol, h->status, 4, cudaMemcpyDeviceToHost, s));
   XK_CUDA(cudaMemcpyAsync(Kij_out, h->Kij, (size_t)n * n * 8, cudaMemcpyDeviceToHost, s));
   XK_CUDA(cudaMemcpyAsync(xi_out, h->xi, (size_t)N * n * 8, cudaMemcpyDeviceToHost, s));
   XK_CUDA(cudaStreamSynchronize(s));
-  if (h->res_st[0] != 0) {
+  if (h->res_st[0] != 0) return gave_up("xk_ace", h->res_st[0]);
+  if (chol[0] != 0) {
     br = 1;
     XK_CUDA(cudaMemcpyAsync(h->Lf, h->Kij, (size_t)n * n * 8, cudaMemcpyDeviceToDevice, s));
     XK_CUDA(xk::jacobi_eig_f64(h->Lf, h->U, n, 60, h->status + 1, s));
@@ -1331,12 +1368,7 @@ int xk_submit(xk_handle* h, const double* C, double deadline_ms, xk_ticket* t) {
   XK_CUDA(cudaMemcpyAsync(s.Ex, h->Ex, 16, cudaMemcpyDeviceToHost, h->stream));
   // this build's status word, taken and cleared in stream order: every slot
   // reports the kernels of its own build
-  s.st[0] = 0;
-  if (h->mixed) {
-    int* dev = xk::mixed_status_ptr(h->mixed);
-    XK_CUDA(cudaMemcpyAsync(s.st, dev, 16, cudaMemcpyDeviceToHost, h->stream));
-    XK_CUDA(cudaMemsetAsync(dev, 0, 16, h->stream));
-  }
+  XK_CUDA(enqueue_status(h, s.st, h->stream));
   XK_CUDA(cudaEventRecord(s.done, h->stream));
   h->has_build = true;
   s.state = 1;
@@ -1388,8 +1420,7 @@ int xk_poll(xk_ticket t, double* K_out, double* Ex, double* err_est) {
     const int st = s.st[0];
     s.state = 0;
     consume();
-    return fail(XK_ETIMEDOUT, "xk_poll: a bounded wait inside a kernel gave up (code " +
-                                  std::to_string(st) + ")");
+    return gave_up("xk_poll", st);
   }
   std::memcpy(K_out, s.K, kb);
   *Ex = *s.Ex;
@@ -1479,6 +1510,7 @@ int xk_autotune_info(xk_handle* h, int32_t* info, double* ms) {
 int xk_set_wait_limit(xk_handle* h, int64_t cycles) {
   if (!h || cycles < 0) return fail(XK_EINVAL, "xk_set_wait_limit: NULL handle or negative limit");
   std::lock_guard<std::mutex> lk(h->mu);
+  h->wait = (long long)cycles;
   if (h->mixed) xk::mixed_set_wait_limit(h->mixed, (long long)cycles);
   drop_graph(h);  // its kernels hold the old limit
   return XK_OK;
@@ -1623,7 +1655,7 @@ int xk_batch_build(xk_batch* b, const double* const* C, double* const* K_out, do
   for (size_t i = 0; i < count; ++i) {
     xk_handle* h = b->hs[i];
     XK_CUDA(cudaMemcpyAsync(h->res, h->Ex, 8, cudaMemcpyDeviceToHost, b->stream));
-    XK_CUDA(enqueue_status(h, b->stream));  // each read and cleared before returning
+    XK_CUDA(enqueue_status(h, h->res_st, b->stream));  // each read and cleared before returning
   }
   for (size_t i = 0; i < count; ++i)
     XK_CUDA(cudaMemcpyAsync(K_out[i], b->hs[i]->K, (size_t)b->hs[i]->N * b->hs[i]->n * 8,
@@ -1637,8 +1669,7 @@ int xk_batch_build(xk_batch* b, const double* const* C, double* const* K_out, do
     if (first == 0) first = h->res_st[0];
   }
   if (first != 0)
-    return fail(XK_ETIMEDOUT, "xk_batch_build: a bounded wait inside a kernel gave up (code " +
-                                  std::to_string(first) + ")");
+    return gave_up("xk_batch_build", first);
   return XK_OK;
 }
 

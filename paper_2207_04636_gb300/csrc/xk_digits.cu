@@ -93,6 +93,8 @@ struct DArgs {
   int nbatch; long cskip;  // swapped only: batches of C's columns (DGemm)
   int* flag;         // set to 1 when a row cannot be split (row_unfit), to 2 when a bounded
                      // wait gave up: the product is then left to the FP64 FMAs
+  int* status;       // nullable: gets a code when a wait gave up, for the call to report
+  long long wait;    // limit of the pipeline waits when shortened (kShort)
 };
 
 // Scale exponent e of a row from the high word of its largest |x|:
@@ -293,7 +295,7 @@ __device__ __forceinline__ void prefetch_block(const DArgs& g, long x0, long y0,
   asm volatile("prefetch.global.L2 [%0];" ::"l"(o.p + (kc ? r * o.ld + k : k * o.ld + r)));
 }
 
-template <bool XK, bool YK>
+template <bool XK, bool YK, bool kShort>
 __global__ void __launch_bounds__(D_THREADS, 1) digit_gemm_kernel(const __grid_constant__ DArgs g) {
   extern __shared__ uint8_t d_raw[];
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(d_raw) + 1023) & ~uintptr_t(1023));
@@ -342,6 +344,23 @@ __global__ void __launch_bounds__(D_THREADS, 1) digit_gemm_kernel(const __grid_c
   tc_fence_after();
   const uint32_t tbase = tslot;
   const int ntiles = g.tiles * g.ksplit;
+  auto wait = [&](uint64_t* bar, uint32_t parity) __attribute__((always_inline)) {
+    if constexpr (!kShort) return mbar_wait_warp(bar, parity);
+    // (inline: a call would take more registers than the workers have)
+    __syncwarp();
+    const long long t0 = clock64();
+    bool ok;
+    while (!(ok = mbar_test(bar, parity)) && clock64() - t0 <= g.wait) {}
+    return __all_sync(0xffffffffu, ok) != 0;
+  };
+  auto gave_up = [&](int code) __attribute__((always_inline)) {
+    if (lane == 0) {
+      atomicExch(g.flag, 2);
+      if (g.status) atomicExch(g.status, code);
+      abort_flag = 1;
+    }
+    __syncwarp();
+  };
   // tile t: X tile fastest, then Y tile, then the K split (symmetric: Y fastest)
   auto place = [&](int t, int& xt, int& yt, int& z) __attribute__((always_inline)) {
     z = t / g.tiles;
@@ -370,8 +389,7 @@ __global__ void __launch_bounds__(D_THREADS, 1) digit_gemm_kernel(const __grid_c
       int it = 0, G = 0;
       bool good = true;
       auto fail = [&]() {
-        if (lane == 0) { atomicExch(g.flag, 2); abort_flag = 1; }
-        __syncwarp();
+        gave_up(51);
         good = false;
       };
       for (int t = blockIdx.x; good && t < ntiles; t += gridDim.x) {
@@ -381,8 +399,8 @@ __global__ void __launch_bounds__(D_THREADS, 1) digit_gemm_kernel(const __grid_c
           const int s = it % D_STAGES;
           const bool first = (kb % D_GROUP) == 0;
           const bool last = (kb % D_GROUP) == D_GROUP - 1 || kb == nkb - 1;
-          if (!mbar_wait_warp(&full[s], (it / D_STAGES) & 1)) { fail(); break; }
-          if (first && G >= 1 && !mbar_wait_warp(&free_lo, (G - 1) & 1)) { fail(); break; }
+          if (!wait(&full[s], (it / D_STAGES) & 1)) { fail(); break; }
+          if (first && G >= 1 && !wait(&free_lo, (G - 1) & 1)) { fail(); break; }
           tc_fence_after();
           const uint64_t dx = d0 + (uint64_t)((s * D_STAGE) >> 4);
           const uint64_t dy = dx + (uint64_t)((kDig * DX_PLANE) >> 4);
@@ -402,7 +420,7 @@ __global__ void __launch_bounds__(D_THREADS, 1) digit_gemm_kernel(const __grid_c
           run(5, 0, 3, true);
           run(6, 0, 2, true);
           if (first && G >= 1) {
-            if (!mbar_wait_warp(&free_hi, (G - 1) & 1)) { fail(); break; }
+            if (!wait(&free_hi, (G - 1) & 1)) { fail(); break; }
             tc_fence_after();
           }
           // levels 0 to 3
@@ -429,8 +447,7 @@ __global__ void __launch_bounds__(D_THREADS, 1) digit_gemm_kernel(const __grid_c
     const uint32_t tacc = tbase + (static_cast<uint32_t>(quad * 32) << 16) + 16 * cg;
     bool ok = true;
     auto lost = [&]() __attribute__((always_inline)) {
-      if (lane == 0) { atomicExch(g.flag, 2); abort_flag = 1; }
-      __syncwarp();
+      gave_up(52);
       ok = false;
     };
     long long hi[16];  // levels 0-3, in units of level 3
@@ -479,7 +496,7 @@ __global__ void __launch_bounds__(D_THREADS, 1) digit_gemm_kernel(const __grid_c
     // group); levels 5 to 7 are added up in FP32 first (error below 2^-61 of the
     // largest product)
     auto take_group = [&](bool fresh) __attribute__((always_inline)) {
-      if (!mbar_wait_warp(&set_ready, G & 1)) { lost(); return; }
+      if (!wait(&set_ready, G & 1)) { lost(); return; }
       tc_fence_after();
       auto level = [](uint32_t a) { return __float2int_rn(__uint_as_float(a)); };
       auto mad = [](int a, int b, long long c) {  // one instruction, off the busy pipe
@@ -637,7 +654,7 @@ __global__ void __launch_bounds__(D_THREADS, 1) digit_gemm_kernel(const __grid_c
       for (int kb = 0; kb < nkb && ok; ++kb, ++it) {
         const int s = it % D_STAGES, use = it / D_STAGES;
         if (__shfl_sync(0xffffffffu, (int)abort_flag, 0) ||
-            (use > 0 && !mbar_wait_warp(&empty[s], (use - 1) & 1))) { lost(); break; }
+            (use > 0 && !wait(&empty[s], (use - 1) & 1))) { lost(); break; }
         uint8_t* st = sm + s * D_STAGE;
         store_block<8, XK>(st, exps[warp][par], tid, vx);
         if (!vkeep) store_block<4, YK>(st + kDig * DX_PLANE, exps[warp][par] + 32, tid, vy);
@@ -775,7 +792,7 @@ cudaError_t digit_gemm(const DGemm& g, int ksplit, int kchunk, cudaStream_t s) {
     a.xmax = a.swapped ? g.cmax : g.rmax;
     a.ymax = a.swapped ? g.rmax : g.cmax;
   }
-  a.H = g.H; a.ldh = g.ldh; a.work = g.work; a.flag = sc;
+  a.H = g.H; a.ldh = g.ldh; a.work = g.work; a.flag = sc; a.status = g.status; a.wait = g.wait;
   a.nbatch = g.nbatch; a.cskip = g.cskip;
   a.sym = g.sym;
   a.tiles = g.sym ? sym_tiles(a.tiles_x, a.tiles_y) : a.tiles_x * a.tiles_y;
@@ -788,8 +805,12 @@ cudaError_t digit_gemm(const DGemm& g, int ksplit, int kchunk, cudaStream_t s) {
     count_launch();
     return cudaGetLastError();
   };
-  if (a.x.kc) return a.y.kc ? launch(digit_gemm_kernel<true, true>) : launch(digit_gemm_kernel<true, false>);
-  return a.y.kc ? launch(digit_gemm_kernel<false, true>) : launch(digit_gemm_kernel<false, false>);
+  auto pick = [&](auto s_) {
+    constexpr bool S = decltype(s_)::value;
+    if (a.x.kc) return a.y.kc ? launch(digit_gemm_kernel<true, true, S>) : launch(digit_gemm_kernel<true, false, S>);
+    return a.y.kc ? launch(digit_gemm_kernel<false, true, S>) : launch(digit_gemm_kernel<false, false, S>);
+  };
+  return short_wait(a.wait) ? pick(std::true_type{}) : pick(std::false_type{});
 }
 
 }  // namespace xk

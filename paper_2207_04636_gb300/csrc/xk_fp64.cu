@@ -99,7 +99,8 @@ __global__ void __launch_bounds__(TPB) dgemm_kernel(DGemm g, int kchunk, const i
         double v = g.alpha * acc[i][j];
         if (HAD) v *= g.H[m * g.ldh + n - q * g.nbatch];
         if (g.beta != 0.0) v += g.beta * g.C[at];
-        // a tensor-core product that gave up half-way has changed C already
+        // a tensor-core product that gave up half-way has changed C already (it is reported
+        // by way of DGemm::status)
         if ((g.beta != 0.0 || in_place(g)) && only_if && left_out == 2) v = nan("");
         g.C[at] = v;
       }
@@ -492,7 +493,7 @@ __global__ void __launch_bounds__(128) axis_kernel(const double* __restrict__ in
 }
 
 cudaError_t poisson_f64(const double* in, double* out, double* tmp, long nf, int g,
-                        const double* tab, int* scale, size_t scale_ints, cudaStream_t s) {
+                        const double* tab, int* scale, size_t scale_ints, int* wst, cudaStream_t s) {
   const long g2 = (long)g * g;
   const double* lam = tab + 2 * g2;
   const double* src = in;
@@ -504,6 +505,7 @@ cudaError_t poisson_f64(const double* in, double* out, double* tmp, long nf, int
     q.nbatch = (int)g2;
     q.cskip = g2 * (g - 1);
     q.scale = scale && scale_ints >= digit_scale_ints(q.M, q.N) ? scale : nullptr;
+    q.status = wst;
     cudaError_t e;
     if (digit_gemm_wanted(q)) {
       e = dgemm(q, s);

@@ -47,6 +47,8 @@ struct DGemm {
   int *rmax, *cmax;          // digit_maxima(g): high words of the largest |C| per row and
                              // column, for products that take C as an operand
   const int *amax, *bmax;    // those of op(A)'s rows / op(B)'s columns, when they are known
+  int* status;               // nullable: gets a code when a bounded wait of the digit product gives up
+  long long wait;            // limit of those waits in SM cycles (0: the default)
 };
 // The result overwrites rows of B (M <= 64, one row of tiles, unsplit: every block has read
 // its columns of B before it writes them).
@@ -110,9 +112,9 @@ cudaError_t poisson_tables_f64(int g, double L, double* tab, cudaStream_t s);
 // out = Pois(in) (Eq. cou-1: 4 pi / G^2 on the grid's reciprocal vectors, G = 0
 // removed) for nf functions of g^3 values each; in is kept, out and tmp (nf g^3
 // each) are not the same memory.  scale: DGemm::scale of the products
-// (scale_ints ints), nullable.
+// (scale_ints ints), nullable; wst: their DGemm::status.
 cudaError_t poisson_f64(const double* in, double* out, double* tmp, long nf, int g,
-                        const double* tab, int* scale, size_t scale_ints, cudaStream_t s);
+                        const double* tab, int* scale, size_t scale_ints, int* wst, cudaStream_t s);
 // rho[R] = sum_i psi[R][i]^2 for psi (ng x n).
 cudaError_t density_f64(const double* psi, long ng, int n, double* rho, cudaStream_t s);
 // out[R][nu] = v[R] phi[R][nu].
@@ -131,7 +133,8 @@ cudaError_t assemble_full_f64(const double* Y, const double* Z, int N, double dV
 // chi = X_gg^{-1} X_gR (na x ng), V = Pois(chi) on the cubic grid^3 grid of
 // side L (na x ng) and W = V chi^T symmetrised (na x na).  `work` holds the
 // split-K work of the products (dgemm_ksplit sizes) and at least na doubles, `dig` is
-// DGemm::scale of an na x ng product (dig_ints ints).
+// DGemm::scale of an na x ng product (dig_ints ints), `wst` DGemm::status of all: where that is set
+// afterwards the tables are not to be used.
 // A ridge of 1e-14 tr(X_gg)/na is added when the plain factorisation fails
 // (*ridge_out); cudaErrorInvalidValue if it still fails.
 // phig holds the rows of Phi_g times 2^-u[g] (u: device): the row of a point where the basis
@@ -140,8 +143,8 @@ cudaError_t assemble_full_f64(const double* Y, const double* Z, int N, double dV
 // chi, V and W come out times 2^(2 u).
 cudaError_t isdf_tables_f64(const double* phi, long ng, int N, const double* phig, const int* u, int na,
                             int grid, double L, double* Xgg, double* chi, double* V, double* W,
-                            double* work, int* dig, size_t dig_ints, int* status, double* ridge_out,
-                            cudaStream_t s);
+                            double* work, int* dig, size_t dig_ints, int* wst, int* status,
+                            double* ridge_out, cudaStream_t s);
 // Interpolation points (Sec. III.A) by a greedy complete-pivoting Cholesky of
 // X = (F F^T) o (F F^T) for the m candidate rows F (m x N, device): up to
 // `want` pivots (indices into F, selection order) into piv (host), stopping
@@ -151,12 +154,12 @@ cudaError_t isdf_tables_f64(const double* phi, long ng, int N, const double* phi
 cudaError_t select_points_f64(const double* F, int m, int N, int want, double tol_rel,
                               int32_t* piv, int* count, cudaStream_t s);
 // In-place blocked Cholesky (lower) of the n x n matrix A (lda); *status = 1
-// on a non-positive pivot.  scale (here and below): DGemm::scale of the updates.
-cudaError_t cholesky_blocked_f64(double* A, int n, long lda, int* status, int* scale,
+// on a non-positive pivot.  scale, wst (here and below): DGemm::scale and status of the updates.
+cudaError_t cholesky_blocked_f64(double* A, int n, long lda, int* status, int* scale, int* wst,
                                  cudaStream_t s);
 // B (n x ncols, ldb) := (L L^T)^{-1} B with the lower factor L (ldl), which is overwritten.
 cudaError_t cholesky_solve_f64(double* L, int n, long ldl, double* B, long ldb, long ncols,
-                               int* scale, cudaStream_t s);
+                               int* scale, int* wst, cudaStream_t s);
 
 // *out = -dV (2 sum_t V[t] P[t]^2 - sum_t W[t] Q[t]^2) over lenA and lenC
 // elements, in a fixed order; `work` holds reduce_work_elems() doubles.

@@ -330,7 +330,7 @@ cudaError_t select_points_f64(const double* F, int m, int N, int want, double to
   return e;
 }
 
-cudaError_t cholesky_blocked_f64(double* A, int n, long lda, int* status, int* scale,
+cudaError_t cholesky_blocked_f64(double* A, int n, long lda, int* status, int* scale, int* wst,
                                  cudaStream_t s) {
   for (int k = 0; k < n; k += NB) {
     const int kb = std::min(NB, n - k);
@@ -342,6 +342,7 @@ cudaError_t cholesky_blocked_f64(double* A, int n, long lda, int* status, int* s
       DGemm g{rest, rest, kb, A + (long)(k + kb) * lda + k, lda, false,
               A + (long)(k + kb) * lda + k, lda, true, A + (long)(k + kb) * lda + k + kb, lda,
               -1.0, nullptr, 0, 1, nullptr, 1.0, scale};
+      g.status = wst;
       e = dgemm(g, s);
       if (e != cudaSuccess) return e;
     }
@@ -351,7 +352,7 @@ cudaError_t cholesky_blocked_f64(double* A, int n, long lda, int* status, int* s
 
 // B := (L L^T)^{-1} B; L (lower) is overwritten.
 cudaError_t cholesky_solve_f64(double* L, int n, long ldl, double* B, long ldb, long ncols,
-                               int* scale, cudaStream_t s) {
+                               int* scale, int* wst, cudaStream_t s) {
   const int nb = (n + NB - 1) / NB;
   const unsigned pairs = (unsigned)(nb * (nb - 1) / 2);
   invert_diag_kernel<<<(unsigned)nb, NB, 0, s>>>(L, n, ldl);
@@ -365,6 +366,7 @@ cudaError_t cholesky_solve_f64(double* L, int n, long ldl, double* B, long ldb, 
     DGemm g{std::min(NB, n - k), (int)ncols, k1 - k0, L + (long)k * ldl + k0, ldl, false,
             B + (long)k0 * ldb, ldb, false, B + (long)k * ldb, ldb, 1.0, nullptr, 0, 1, nullptr, 0.0,
             scale};
+    g.status = wst;
     return dgemm(g, s);
   };
   for (int k = 0; k < n; k += NB) {
@@ -382,8 +384,8 @@ cudaError_t cholesky_solve_f64(double* L, int n, long ldl, double* B, long ldb, 
 
 cudaError_t isdf_tables_f64(const double* phi, long ng, int N, const double* phig, const int* u, int na,
                             int grid, double L, double* Xgg, double* chi, double* V, double* W,
-                            double* work, int* dig, size_t dig_ints, int* status, double* ridge_out,
-                            cudaStream_t s) {
+                            double* work, int* dig, size_t dig_ints, int* wst, int* status,
+                            double* ridge_out, cudaStream_t s) {
   cudaError_t e;
   // scratch of the tensor-core products: W until W itself is formed, when that is the
   // larger (more functions to a Poisson pass)
@@ -396,6 +398,7 @@ cudaError_t isdf_tables_f64(const double* phi, long ng, int N, const double* phi
   auto gram = [&]() {
     DGemm g{na, na, N, phig, N, false, phig, N, true, Xgg, na, 1.0, nullptr, 0, 0, work};
     g.scale = scale;
+    g.status = wst;
     g.sym = true;
     cudaError_t r = dgemm(g, s);
     if (r != cudaSuccess) return r;
@@ -407,6 +410,7 @@ cudaError_t isdf_tables_f64(const double* phi, long ng, int N, const double* phi
   {
     DGemm g{na, (int)ng, N, phig, N, false, phi, N, true, chi, ng, 1.0, nullptr, 0, 0, work};
     g.scale = scale;
+    g.status = wst;
     e = dgemm(g, s);
     if (e != cudaSuccess) return e;
     square_kernel<<<nblocks((long)na * ng), 256, 0, s>>>(chi, na, ng, ng);
@@ -417,7 +421,7 @@ cudaError_t isdf_tables_f64(const double* phi, long ng, int N, const double* phi
   double ridge = 0.0;
   int st = 0;
   e = cudaMemsetAsync(status, 0, 4, s);
-  if (e == cudaSuccess) e = cholesky_blocked_f64(Xgg, na, na, status, scale, s);
+  if (e == cudaSuccess) e = cholesky_blocked_f64(Xgg, na, na, status, scale, wst, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(&st, status, 4, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return e;
@@ -439,7 +443,7 @@ cudaError_t isdf_tables_f64(const double* phi, long ng, int N, const double* phi
     add_diag_kernel<<<nblocks(na), 256, 0, s>>>(Xgg, na, na, ridge, u);
     count_launch();
     e = cudaMemsetAsync(status, 0, 4, s);
-    if (e == cudaSuccess) e = cholesky_blocked_f64(Xgg, na, na, status, scale, s);
+    if (e == cudaSuccess) e = cholesky_blocked_f64(Xgg, na, na, status, scale, wst, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&st, status, 4, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return e;
@@ -447,7 +451,7 @@ cudaError_t isdf_tables_f64(const double* phi, long ng, int N, const double* phi
   }
   if (ridge_out) *ridge_out = ridge;
   // chi = X_gg^{-1} X_gR
-  e = cholesky_solve_f64(Xgg, na, na, chi, ng, ng, scale, s);
+  e = cholesky_solve_f64(Xgg, na, na, chi, ng, ng, scale, wst, s);
   if (e != cudaSuccess) return e;
   // V = Pois(chi) in batches of functions (the scratch holds one)
   {
@@ -464,7 +468,7 @@ cudaError_t isdf_tables_f64(const double* phi, long ng, int N, const double* phi
     e = poisson_tables_f64(grid, L, tab, s);
     for (long r0 = 0; e == cudaSuccess && r0 < na; r0 += nf)
       e = poisson_f64(chi + r0 * ng, V + r0 * ng, tmp, std::min<long>(nf, na - r0), grid, tab, scale,
-                      ints, s);
+                      ints, wst, s);
     cudaError_t e2 = cudaFreeAsync(buf, s);
     if (e == cudaSuccess) e = e2;
     if (e != cudaSuccess) return e;
@@ -473,6 +477,7 @@ cudaError_t isdf_tables_f64(const double* phi, long ng, int N, const double* phi
   {
     DGemm g{na, na, (int)ng, V, ng, false, chi, ng, true, W, na, 1.0, nullptr, 0, 0, work};
     g.scale = dig;
+    g.status = wst;
     e = dgemm(g, s);
     if (e == cudaSuccess) e = symmetrize_f64(W, na, s);
   }

@@ -3167,6 +3167,8 @@ DGemm q_product(const MixedState* m) {
   const int N = m->N, n = m->n;
   DGemm g{n, N, N, m->part, n, true, m->Lf, N, false, m->CT64, m->Np, 1.0, nullptr, 0, q_ksplit(N), m->dwork};
   if (2 * (size_t)m->Naux * n >= digit_scale_ints(n, N)) g.scale = reinterpret_cast<int*>(m->D23);
+  g.status = m->status;
+  g.wait = m->wait_cycles;
   return g;
 }
 

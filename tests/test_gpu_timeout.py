@@ -80,3 +80,40 @@ def test_negative_limit_rejected(xk, cell1):
         assert e.value.code == xk.XK_EINVAL
     finally:
         h.release()
+
+
+def test_timeout_digit_products(xk):
+    """FP64 handle whose products are formed from digits: every call reports a wait that
+    gave up inside one, and the handle's results at the default bound are the same again."""
+    grid, N, na, L = 17, 280, 20, 6.0
+    rng = np.random.default_rng(13)
+    phi, C = rng.standard_normal((grid ** 3, N)), np.linalg.qr(rng.standard_normal((N, N)))[0]
+    V, W = rng.uniform(0.5, 1.5, (na, grid ** 3)), rng.standard_normal((na, na))
+    h = xk.Handle(phi, np.arange(na), V, W + W.T, 0.1, N, mode="fp64")
+    calls = [lambda: h.build(C), h.ace, lambda: h.energy(C), lambda: h.build_full(C),
+             lambda: h.coulomb(C, grid, L)]
+
+    def served():
+        t = h.submit(C)
+        while True:
+            st, K, E, _ = xk.poll(t, N, N)
+            if st == xk.XK_OK:
+                return K, E
+            assert st == xk.XK_PENDING
+
+    calls.append(served)
+    try:
+        before = [f() for f in calls]
+        h.set_wait_limit(1)
+        for f in calls:
+            with pytest.raises(xk.XKError) as e:
+                f()
+            assert e.value.code == xk.XK_ETIMEDOUT
+        h.set_wait_limit(0)
+        after = [f() for f in calls]
+    finally:
+        h.release()
+    for a, b in zip(before, after):
+        for x, y in zip(np.atleast_1d(a) if isinstance(a, (float, np.ndarray)) else a,
+                        np.atleast_1d(b) if isinstance(b, (float, np.ndarray)) else b):
+            assert np.array_equal(x, y)
