@@ -1239,13 +1239,13 @@ int xk_coulomb(xk_handle* h, int32_t grid, double L, const double* C, double* J_
     XK_CUDA(xk::density_f64(h->psi, (long)ng, n, h->Jrho, s));
     XK_CUDA(xk::poisson_f64(h->Jrho, h->Jv, h->Jtmp, 1, grid, h->Jtab, nullptr, 0, nullptr, s));
     XK_CUDA(xk::potential_rows_f64(h->Jv, h->phi, (long)ng, N, h->Jphiv, s));
-    xk::DGemm gj{N, N, (int)ng, h->phi, N, true, h->Jphiv, N, false, h->Jout, N, h->dV, nullptr, 0, 0, h->work};
+    xk::DGemm gj{N, N, (int)ng, h->phi, N, true, h->Jphiv, N, false, h->Jout, N, 1.0, nullptr, 0, 0, h->work};
     gj.scale = h->dig;
     gj.status = h->wst;
     gj.wait = h->wait;
     gj.sym = true;
     XK_CUDA(xk::dgemm(gj, s));
-    XK_CUDA(xk::scale_f64(h->Jout, h->Jout, N, N, h->be, 1, h->be, 1, s));
+    XK_CUDA(xk::scale_f64(h->Jout, h->Jout, N, N, h->be, 1, h->be, 1, s, h->dV));
     XK_CUDA(xk::dot_f64(h->Jrho, h->Jv, (long)ng, h->dV, h->red, h->Jout + (size_t)N * N, s));
   }
   XK_CUDA(cudaMemcpyAsync(h->res, h->Jout + (size_t)N * N, 8, cudaMemcpyDeviceToHost, s));

@@ -302,25 +302,25 @@ cudaError_t col_exponents_f64(const double* p, long ld, long rows, int cols, int
 }
 
 __global__ void scale_kernel(const double* src, double* dst, long rows, long cols, const int* __restrict__ re,
-                             int rm, const int* __restrict__ ce, int cm) {
+                             int rm, const int* __restrict__ ce, int cm, double f) {
   const long total = rows * cols;
   for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < total;
        t += (long)gridDim.x * blockDim.x) {
     const long r = t / cols, c = t - r * cols;
     const int e = (re ? rm * re[r] : 0) + (ce ? cm * ce[c] : 0);
-    if (e != 0)
-      dst[t] = scalbn(src[t], e);
+    if (e != 0 || f != 1.0)
+      dst[t] = f * scalbn(src[t], e);
     else if (src != dst)
       dst[t] = src[t];
   }
 }
 
 cudaError_t scale_f64(const double* src, double* dst, long rows, long cols, const int* re, int rm,
-                      const int* ce, int cm, cudaStream_t s) {
+                      const int* ce, int cm, cudaStream_t s, double f) {
   const long total = rows * cols;
   if (total == 0) return cudaSuccess;
   scale_kernel<<<(unsigned)std::min<long>((total + 255) / 256, 152L * 16), 256, 0, s>>>(src, dst, rows, cols, re,
-                                                                                       rm, ce, cm);
+                                                                                       rm, ce, cm, f);
   count_launch();
   return cudaGetLastError();
 }
@@ -333,7 +333,7 @@ __global__ void assemble_k_kernel(const double* __restrict__ L1, const double* _
        t += (long)gridDim.x * blockDim.x) {
     const long mu = t / n, i = t % n;
     const long src = i * N + mu;
-    K[t] = scalbn(dV * ((L1[src] + L2[src]) - L3[src]), ce[mu]);
+    K[t] = dV * scalbn((L1[src] + L2[src]) - L3[src], ce[mu]);  // (in this order: K's own range)
   }
 }
 
@@ -559,7 +559,7 @@ cudaError_t dot_f64(const double* a, const double* b, long len, double scale, do
   return cudaGetLastError();
 }
 
-// Full K: K[mu][nu] = dV (Y[mu][nu] + Y[nu][mu] - Z[mu][nu]) 2^(ce[mu] + ce[nu]) (N x N).
+// Full K: K[mu][nu] = dV ((Y[mu][nu] + Y[nu][mu] - Z[mu][nu]) 2^(ce[mu] + ce[nu])) (N x N).
 __global__ void assemble_full_kernel(const double* __restrict__ Y, const double* __restrict__ Z,
                                      int N, double dV, const int* __restrict__ ce,
                                      double* __restrict__ K) {
@@ -567,7 +567,7 @@ __global__ void assemble_full_kernel(const double* __restrict__ Y, const double*
   for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < count;
        t += (long)gridDim.x * blockDim.x) {
     const long mu = t / N, nu = t % N;
-    K[t] = scalbn(dV * ((Y[t] + Y[nu * N + mu]) - Z[t]), ce[mu] + ce[nu]);
+    K[t] = dV * scalbn((Y[t] + Y[nu * N + mu]) - Z[t], ce[mu] + ce[nu]);
   }
 }
 

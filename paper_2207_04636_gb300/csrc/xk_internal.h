@@ -72,9 +72,9 @@ cudaError_t balance_rows_f64(const double* A, const double* B, int rows, int col
                              cudaStream_t s);
 // out[i] = a[i] - b[i].
 cudaError_t sub_i32(const int* a, const int* b, int n, int* out, cudaStream_t s);
-// dst[r][c] = src[r][c] 2^(rm re[r] + cm ce[c]) (re, ce nullable; dst may be src).
+// dst[r][c] = f (src[r][c] 2^(rm re[r] + cm ce[c])) (re, ce nullable; dst may be src).
 cudaError_t scale_f64(const double* src, double* dst, long rows, long cols, const int* re, int rm,
-                      const int* ce, int cm, cudaStream_t s);
+                      const int* ce, int cm, cudaStream_t s, double f = 1.0);
 
 // The product of dgemm on the tensor cores, split into exact digits
 // (xk_digits.cu): whether its size calls for it, the K split it wants (at most
@@ -93,7 +93,7 @@ int dgemm_ksplit(int M, int N, int K);
 cudaError_t gather_rows_f64(const double* in, long ld_in, const int32_t* idx, int rows, int cols,
                             double* out, long ld_out, cudaStream_t s, const int* re = nullptr);
 
-// K[mu, i] = dV * (L1[i, mu] + L2[i, mu] - L3[i, mu]) 2^ce[mu]; L* are n x N.
+// K[mu, i] = dV * ((L1[i, mu] + L2[i, mu] - L3[i, mu]) 2^ce[mu]); L* are n x N.
 cudaError_t assemble_k_f64(const double* L1, const double* L2, const double* L3, int n, int N,
                            double dV, const int* ce, double* K, cudaStream_t s);
 
@@ -124,7 +124,7 @@ cudaError_t potential_rows_f64(const double* v, const double* phi, long ng, int 
 cudaError_t dot_f64(const double* a, const double* b, long len, double scale, double* work,
                     double* out, cudaStream_t s);
 
-// K[mu][nu] = dV (Y[mu][nu] + Y[nu][mu] - Z[mu][nu]) 2^(ce[mu] + ce[nu]) for N x N matrices.
+// K[mu][nu] = dV ((Y[mu][nu] + Y[nu][mu] - Z[mu][nu]) 2^(ce[mu] + ce[nu])) for N x N matrices.
 cudaError_t assemble_full_f64(const double* Y, const double* Z, int N, double dV, const int* ce,
                               double* K, cudaStream_t s);
 

@@ -242,3 +242,31 @@ def test_config2_full(xk):
     whole K_{mu i} and E_x against the oracle, at the size the benchmark runs."""
     c = load_cell(config_spec(2))
     _check(xk, c)
+
+
+def test_results_near_the_end_of_the_range(xk):
+    """Results just below 2^1023 from tables of ordinary size and a large dV: K, the full K
+    and J are those of dV = 1 times dV, whatever units the tables are held in."""
+    grid, N, n, na = 13, 9, 4, 40
+    rng = np.random.default_rng(3)
+    phi, C = rng.standard_normal((grid ** 3, N)) / 64, rng.standard_normal((N, n))
+    V, W = rng.standard_normal((na, grid ** 3)) * 2.0 ** 10, np.zeros((na, na))
+
+    def run(dV, s):
+        h = xk.Handle(phi, np.arange(na), V * s, W, dV, n, mode="fp64")
+        out = h.build(C)[0], h.build_full(C)
+        h.release()
+        return out
+
+    for a, top in zip(run(1.0, 1.0), (0, 1)):
+        s = 2.0 ** np.floor(1023 - np.log2(np.abs(a).max()))
+        b = run(2.0 ** 900, s * 2.0 ** -900)[top]
+        assert np.array_equal(a * s, b)
+    C *= 2.0 ** 30  # a J whose dV is in range
+    h = xk.Handle(phi, np.arange(na), V, W, 1.0, n, mode="fp64")
+    J, _ = h.coulomb(C, grid, 6.0)
+    h.release()
+    s = 2.0 ** np.floor(1023 - np.log2(np.abs(J).max()))
+    h = xk.Handle(phi, np.arange(na), V, W, s, n, mode="fp64")
+    assert np.array_equal(J * s, h.coulomb(C, grid, 6.0)[0])
+    h.release()
