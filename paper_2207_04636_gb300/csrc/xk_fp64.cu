@@ -678,12 +678,12 @@ __global__ void __launch_bounds__(KT * KT * KS) kij_kernel(const double* __restr
       v = fma(c[j], k[i], v);
     }
   }
-  part[sl][o] = u + v;
+  part[sl][o] = 0.5 * u + 0.5 * v;  // halved first: sums of 2 K_ij may overflow where K_ij does not
   __syncthreads();
   if (sl != 0 || i >= n || j >= n) return;
   double s = part[0][o];
   for (int w = 1; w < KS; ++w) s += part[w][o];
-  Kij[(long)i * n + j] = Kij[(long)j * n + i] = 0.5 * s;
+  Kij[(long)i * n + j] = Kij[(long)j * n + i] = s;
 }
 
 cudaError_t kij_f64(const double* C, const double* K, int N, int n, double* Kij, cudaStream_t s) {
@@ -751,12 +751,11 @@ __global__ void __launch_bounds__(256) chol_block_kernel(double* __restrict__ A,
         if (tid == c && !bad) bad = c + 1;
       }
       if (tid == c) rs[c] = d;
-      double f = col[tid];
-      if (__double2hiint(d) < ((1023 - 1000) << 20)) {  // a reciprocal that would overflow
-        d *= 0x1p200;
-        f *= 0x1p200;
-      }
-      fcol[tid] = f * fast_recip(d);
+      const double f = col[tid];
+      // a division where the reciprocal would leave the normal range (or d is infinite)
+      const int hi = __double2hiint(d);
+      const bool far = hi < ((1023 - 1000) << 20) || hi >= ((1023 + 1000) << 20);
+      fcol[tid] = far ? f / d : f * fast_recip(d);
     }
     __syncthreads();
 #pragma unroll

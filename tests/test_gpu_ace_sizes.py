@@ -57,3 +57,33 @@ def test_graded_basis():
 
     for a, b in zip(run(np.zeros(N)), run(rng.integers(-40, 41, size=N).astype(np.float64))):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("top", [2.0 ** 1023, 2.0 ** -1010])
+def test_pivots_at_the_ends_of_the_range(top):
+    """K_ij whose pivots lie just below 2^1023, or below 2^-1010: its vectors still give K back."""
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2207_04636_gb300 as xk
+    n, N, Ng = 4, 9, 1200
+    rng = np.random.default_rng(4)
+    phi = rng.standard_normal((Ng, N)) / np.sqrt(Ng)
+    C = np.linalg.qr(rng.standard_normal((N, n)))[0]
+    V, W = np.diag(rng.uniform(5.0, 15.0, Ng)) * 2.0 ** 10, np.zeros((Ng, Ng))  # a dV in range
+
+    def run(dV):
+        h = xk.Handle(phi, np.arange(Ng), V, W, dV, n, mode="fp64")
+        K, _ = h.build(C)
+        Kij, xi, _, br = h.ace()
+        h.release()
+        assert br == "cholesky"
+        return K, Kij, xi
+
+    Kij = run(1.0)[1]
+    assert np.diag(Kij).max() < 1.8 * np.diag(Kij).min()
+    K, Kij, xi = run(0.95 * top / np.diag(Kij).max())
+    assert np.diag(Kij).min() > 0.5 * top or top < 1.0
+    K, Kij = K / top, Kij / top
+    xi = xi / 2.0 ** (np.log2(top) // 2)
+    err = np.abs((xi @ xi.T) @ C / (top / 4.0 ** (np.log2(top) // 2)) - K).max()
+    assert err <= 16 * n * 2.0 ** -53 * np.linalg.cond(Kij) * np.abs(K).max()
