@@ -10,9 +10,12 @@
 // such integers exactly in its FP32 accumulator while the sum stays below
 // 2^24.  The products d_i d'_j of one weight l = i + j share an accumulator;
 // levels 0 to 7 are formed (34 of the 49 products), every 256 terms they are
-// drained into an integer accumulator of 64 + 20 bits (levels 0 to 3 then never
-// exceed 2^24 and are exact; the accumulator's last bit weighs 2^-58 of the
-// largest product).  The result is rounded to FP64 once, so its error is that of the 55-bit
+// drained into an integer accumulator of 64 + 20 bits, whose last bit weighs 2^-58 of the
+// largest product.  Levels 0 to 3 never exceed 2^24 in 256 terms and are exact.  Levels 4 to 7
+// have 5 to 7 pairs and can pass it, where an addition may lose a unit: at most some 20 units
+// of level 4, 2^-50 of 256 largest products, and that only when all digits are near their limit
+// with one sign in every pair (256 FMAs of such terms are allowed 2^-46).  The result is
+// rounded to FP64 once, so its error is in practice that of the 55-bit
 // operands and the dropped levels: 5e-17 to 3e-16 of the 2-norm on the
 // products of a build, where a chain of FP64 FMAs leaves 1.4e-16 to 9e-15.  The 55 bits
 // count from the largest element of the row, so the callers see to it that the two operands
@@ -493,8 +496,9 @@ __global__ void __launch_bounds__(D_THREADS, 1) digit_gemm_kernel(const __grid_c
       if (++fkb == fn) { fkb = 0; ft += gridDim.x; open_tile(); }
     };
     // adds a finished group of accumulators to hi, lo (zeroed at a tile's first
-    // group); levels 5 to 7 are added up in FP32 first (error below 2^-61 of the
-    // largest product)
+    // group); levels 5 to 7 are added up in FP32 first: up to 2^28.6 units of lo, so half an
+    // ulp is 2^4 of them, 2^-62 of the group's 256 largest products, and the rounding to an
+    // integer half a unit more
     auto take_group = [&](bool fresh) __attribute__((always_inline)) {
       if (!wait(&set_ready, G & 1)) { lost(); return; }
       tc_fence_after();

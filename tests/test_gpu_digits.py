@@ -257,3 +257,21 @@ def test_few_points_on_a_fine_grid(xk, Ng, N, n, na):
     E = h.energy(C)
     h.release()
     assert K[0, 0] == 2 * (1 + 2.0 ** -50) and E == -2 * (1 + 2.0 ** -50) ** 2
+
+
+def test_digits_at_their_limit(xk):
+    """Operands whose digits are as large as they get (126, then 127 and 124 at the end, as an
+    element is below 127/128 of its grid): levels 4 to 7 of a group's 256 terms pass 2^24
+    in their accumulators, where an addition may lose a unit (some 20 of level 4, 2^-50 of the
+    sum).  E_x = -2 P^2 doubles that and adds its own roundings."""
+    Ng, n, na = 4000, 256, 40
+    x = 0x7e7f7f7f7f7f7c  # of 2^-55
+    assert int(float(x)) == x
+    phi, V, W = np.full((Ng, n), x * 2.0 ** -55), np.zeros((na, Ng)), np.zeros((na, na))
+    V[3, Ng - 5] = 1.0
+    h = xk.Handle(phi, np.arange(na), V, W, 1.0, n, mode="fp64")
+    E = h.energy(np.eye(n))
+    h.release()
+    exact = 2 * (n * x * x) ** 2  # of 2^-220
+    got = int(-E * 2.0 ** 60) << 160
+    assert abs(got - exact) <= exact >> 48
