@@ -6,13 +6,13 @@
 // Every operand row (the K direction) has a power-of-two scale 2^e > max|row|;
 // an element becomes the integer X = round(x 2^(55 - e)), |X| < 127 2^48, and
 // X = sum_i d_i 2^(8 (6 - i)) with seven signed digits |d_i| <= 128, exact in
-// FP16.  A product of two digits is an integer <= 2^14, and tcgen05.mma adds
-// such integers exactly in its FP32 accumulator while the sum stays below
-// 2^24.  The products d_i d'_j of one weight l = i + j share an accumulator;
-// levels 0 to 7 are formed (34 of the 49 products), every 256 terms they are
+// FP16; Y, the operand with fewer rows, has an eighth, to 2^(e - 63).  A product of two digits
+// is an integer <= 2^14, and tcgen05.mma adds such integers exactly in its FP32 accumulator
+// while the sum stays below 2^24.  The products d_i d'_j of one weight l = i + j share an
+// accumulator; levels 0 to 7 are formed (35 of the 56 products), every 256 terms they are
 // drained into an integer accumulator of 64 + 20 bits, whose last bit weighs 2^-58 of the
 // largest product.  Levels 0 to 3 never exceed 2^24 in 256 terms and are exact.  Levels 4 to 7
-// have 5 to 7 pairs and can pass it, where an addition may lose a unit: at most some 20 units
+// have 5 to 8 pairs and can pass it, where an addition may lose a unit: at most some 20 units
 // of level 4, 2^-50 of 256 largest products, and that only when all digits are near their limit
 // with one sign in every pair (256 FMAs of such terms are allowed 2^-46).  The result is
 // rounded to FP64 once, so its error is in practice that of the 55-bit
@@ -21,7 +21,14 @@
 // count from the largest element of the row, so the callers see to it that the two operands
 // are not graded in opposite directions along K (units of powers of two: xk_api.cu).
 //
-// What bounds it: a 128 x 64 tile takes 34 digit products per K = 16 step, 1088
+// What Y loses it loses alike for all rows of X, hence its eighth digit: C rounded to 55 bits
+// moved Psi = Phi C by one smooth function per orbital, which sums over the grid do not average
+// out as they do the roundings of Phi's rows, or those of FMAs.  J's error on three cells of 8
+// centres (coefficients up to 570, against extended precision): 2.2e-14 to 3.5e-14 with seven
+// digits, 5.9e-15 to 1.6e-14 with eight; 2.9e-15 to 5.7e-15 with FMAs.  It costs 0.9 % of an
+// FP64 build.
+//
+// What bounds it: a 128 x 64 tile takes 35 digit products per K = 16 step, 1120
 // clocks of the tensor cores.  One instruction forms up to four of them: the digits of Y
 // lie one after another in shared memory and the levels in TMEM, so N = 256 rows of
 // Y's digits j .. j + 3 against one digit of X give levels i + j .. i + j + 3, and the
@@ -49,12 +56,13 @@ namespace {
 
 using namespace tc;
 
-constexpr int kDig = 7;             // digits per operand
+constexpr int kDig = 7;             // digits of X
+constexpr int kDigY = 8;            // digits of Y
 constexpr int kLev = 8;             // accumulator levels (i + j)
 constexpr int DK = 32;              // K per block: 64-byte rows, 64-byte swizzle
 constexpr int DX = 128, DY = 64;    // tile: X rows (MMA M) by Y rows (MMA N)
 constexpr int DX_PLANE = DX * DK * 2, DY_PLANE = DY * DK * 2;
-constexpr int D_STAGE = kDig * (DX_PLANE + DY_PLANE);  // 84 KB
+constexpr int D_STAGE = kDig * DX_PLANE + kDigY * DY_PLANE;  // 88 KB
 constexpr int D_STAGES = 2;
 constexpr int D_SMEM = D_STAGES * D_STAGE + 1024;
 constexpr int D_GROUP = 256 / DK;   // K blocks between drains
@@ -114,14 +122,14 @@ __device__ __forceinline__ bool row_unfit(int hi) {
   return hi >= 0x7ff00000 || (hi > 0 && hi < ((1023 - 900) << 20));
 }
 
-// The seven digits of |x| on the grid 2^(e - 55), each plus 128, in the upper 7
-// bytes (most significant digit in byte 7).  e21 = (e + 1022) 2^21 + 2^21 - 1.  Integer
-// operations run at 64 a clock and SM here, so they are what the split costs: |x| =
-// m 2^(ex - 1085) with m of 63 bits (a subnormal x, taken for a normal one, is
-// below the grid) is shifted by t = e + 1022 - ex >= 0 to eight bits below the
-// grid, t being what is left of e21 - 2 high word (one multiply-add, on the other pipe;
-// the doubling drops the sign) above its mantissa bits; one sum then adds the offsets
-// 128 2^(8 i) of the digits and half a grid step.
+// The eight digits of |x| on the grid 2^(e - 63), each plus 128 (most significant digit in
+// byte 7; the upper seven are |x| rounded to the grid 2^(e - 55)).  e21 = (e + 1022) 2^21 +
+// 2^21 - 1.  Integer operations run at 64 a clock and SM here, so they are what the split
+// costs: |x| = m 2^(ex - 1085) with m of 63 bits (a subnormal x, taken for a normal one, is
+// below the grid) is shifted by t = e + 1022 - ex >= 0 to the finer grid, t being what is left
+// of e21 - 2 high word (one multiply-add, on the other pipe; the doubling drops the sign)
+// above its mantissa bits; one sum then adds the offsets 128 2^(8 i) of the digits, the
+// lowest being half a step of the coarser grid.
 __device__ __forceinline__ uint2 digits_of(double x, uint32_t e21) {
   const uint32_t xh = __double2hiint(x), xl = __double2loint(x);
   const uint32_t t = (e21 - 2u * xh) >> 21;
@@ -136,21 +144,23 @@ __device__ __forceinline__ uint2 digits_of(double x, uint32_t e21) {
 
 // FP16 pairs (digit of x, digit of y), most significant first: byte + 1024 = 0x64xx,
 // less 1024 + 128, times the element's sign (+-1 from the high words' sign bits).
-__device__ __forceinline__ void digit_pairs(double x, double y, uint32_t e21, uint32_t (&o)[kDig]) {
+template <int D>
+__device__ __forceinline__ void digit_pairs(double x, double y, uint32_t e21, uint32_t (&o)[D]) {
   const uint2 a = digits_of(x, e21), b = digits_of(y, e21);
   const uint32_t c = 0x64646464u;
   const uint32_t w0 = __byte_perm(a.y, b.y, 0x7632), w1 = __byte_perm(a.y, b.y, 0x5410),
-                 w2 = __byte_perm(a.x, b.x, 0x7632), w3 = __byte_perm(a.x, b.x, 0x5151);
+                 w2 = __byte_perm(a.x, b.x, 0x7632), w3 = __byte_perm(a.x, b.x, 0x5410);
   o[0] = __byte_perm(w0, c, 0x4341); o[1] = __byte_perm(w0, c, 0x4240);
   o[2] = __byte_perm(w1, c, 0x4341); o[3] = __byte_perm(w1, c, 0x4240);
   o[4] = __byte_perm(w2, c, 0x4341); o[5] = __byte_perm(w2, c, 0x4240);
-  o[6] = __byte_perm(w3, c, 0x4140);
+  o[6] = __byte_perm(w3, c, 0x4341);
+  if constexpr (D == 8) o[7] = __byte_perm(w3, c, 0x4240);
   const uint32_t sg =
       (__byte_perm(__double2hiint(x), __double2hiint(y), 0x7632) & 0x80008000u) | 0x3c003c00u;
   const __half2 s = *reinterpret_cast<const __half2*>(&sg);
   const __half2 off = __hmul2(s, __half2half2(__ushort_as_half(0xe480)));  // -1152
 #pragma unroll
-  for (int i = 0; i < kDig; ++i) {
+  for (int i = 0; i < D; ++i) {
     const __half2 r = __hfma2(*reinterpret_cast<__half2*>(&o[i]), s, off);
     o[i] = *reinterpret_cast<const uint32_t*>(&r);
   }
@@ -219,7 +229,7 @@ __device__ __forceinline__ int block_row(int w, int l) {
 // Digits of the block into the stage; ex: e21 (digits_of) of the rows block_row(w, 0..31).
 template <int n, bool KC>
 __device__ __forceinline__ void store_block(uint8_t* st, const uint32_t* ex, int tid, const double (&v)[n]) {
-  constexpr int R = 16 * n, PLANE = R * DK * 2;
+  constexpr int R = 16 * n, PLANE = R * DK * 2, D = n == 8 ? kDig : kDigY;
   if constexpr (KC) {
     // rows r0 + 2 i: the swizzle's chunk is that of r0 with bit 1 of r, i.e. bit 0 of i, flipped
     const int r0 = (tid >> 5) * n + ((tid >> 4) & 1), l = tid & 15;
@@ -227,22 +237,22 @@ __device__ __forceinline__ void store_block(uint8_t* st, const uint32_t* ex, int
     for (int i = 0; i < n / 2; ++i) {
       const int r = r0 + 2 * i;
       const uint32_t e = ex[((tid >> 4) & 1) + 2 * i];
-      uint32_t o[kDig];
+      uint32_t o[D];
       digit_pairs(v[2 * i], v[2 * i + 1], e, o);
       uint32_t* d = reinterpret_cast<uint32_t*>(st + r * 64 + (((l >> 2) ^ ((r >> 1) & 3)) << 4) + (l & 3) * 4);
 #pragma unroll
-      for (int q = 0; q < kDig; ++q) d[q * (PLANE / 4)] = o[q];
+      for (int q = 0; q < D; ++q) d[q * (PLANE / 4)] = o[q];
     }
   } else {
     const int r = tid % R, q = tid / R;  // q: which n of the 32 k
     const uint32_t e = ex[tid & 31];
-    uint32_t o[n / 2][kDig];
+    uint32_t o[n / 2][D];
 #pragma unroll
     for (int i = 0; i < n / 2; ++i) digit_pairs(v[2 * i], v[2 * i + 1], e, o[i]);
     const int byte = q * n * 2;  // within the row's 64 bytes
     uint8_t* d = st + r * 64 + (((byte >> 4) ^ ((r >> 1) & 3)) << 4) + (byte & 15);
 #pragma unroll
-    for (int b = 0; b < kDig; ++b) {
+    for (int b = 0; b < D; ++b) {
       if constexpr (n == 8)
         *reinterpret_cast<uint4*>(d + b * PLANE) = make_uint4(o[0][b], o[1][b], o[2][b], o[3][b]);
       else
@@ -386,7 +396,7 @@ __global__ void __launch_bounds__(D_THREADS, 1) digit_gemm_kernel(const __grid_c
   if (warp >= D_WORK) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 32;");
     if (warp == D_WORK) {
-      // per block 34 products of two K = 16 steps, the low levels first: their
+      // per block 35 products of two K = 16 steps, the low levels first: their
       // accumulators are taken out first
       const uint64_t d0 = sdesc_sw64(smem_u32(sm), 16, 512);
       int it = 0, G = 0;
@@ -416,7 +426,7 @@ __global__ void __launch_bounds__(D_THREADS, 1) digit_gemm_kernel(const __grid_c
           };
           // levels 4 to 7; digit 1 reaches all four
           run(1, 3, 4, !first);
-          run(0, 4, 3, true);
+          run(0, 4, 4, true);
           run(2, 2, 4, true);
           run(3, 1, 4, true);
           run(4, 0, 4, true);

@@ -275,3 +275,25 @@ def test_digits_at_their_limit(xk):
     exact = 2 * (n * x * x) ** 2  # of 2^-220
     got = int(-E * 2.0 ** 60) << 160
     assert abs(got - exact) <= exact >> 48
+
+
+def test_large_coefficients_that_cancel(xk):
+    """Two equal basis functions with coefficients 2^14 and -2^14 beside others below one,
+    multiples of 2^-48, which a grid of 2^-55 of the largest would round to 2^-40 (2^-39 in Psi,
+    at every grid point alike).  Read from K = Psi_0(R) Psi_i(R); eight digits hold the
+    coefficients, and taking the sums out rounds to 2^-58 of the largest product, twice."""
+    Ng, N, n, na = 20001, 66, 24, 130
+    rng = np.random.default_rng(13)
+    phi, V, W = _ints(rng, (Ng, N), 1), np.zeros((na, Ng)), np.zeros((na, na))
+    phi[:, 1] = phi[:, 0]
+    phi[:, 65] = phi[0] = 0.0
+    phi[0, 65] = V[0, Ng - 1] = 1.0
+    c = rng.integers(-2 ** 47, 2 ** 47, size=(N, n))  # of 2^-48
+    c[0], c[1], c[65] = 2 ** 62, -2 ** 62, 0
+    c[65, 0] = 2 ** 48
+    h = xk.Handle(phi, np.arange(na), V, W, 1.0, n, mode="fp64")
+    K = h.build(c * 2.0 ** -48)[0][65]
+    h.release()
+    psi = (phi[Ng - 1].astype(np.int64) @ c) * 2.0 ** -48  # below 64, exact
+    err = np.abs(K - psi[0] * psi)
+    assert np.all(err <= (np.abs(psi[0]) + np.abs(psi)) * 2.0 ** -42 + 2.0 ** -46)
