@@ -26,7 +26,8 @@
 // out as they do the roundings of Phi's rows, or those of FMAs.  J's error on three cells of 8
 // centres (coefficients up to 570, against extended precision): 2.2e-14 to 3.5e-14 with seven
 // digits, 5.9e-15 to 1.6e-14 with eight; 2.9e-15 to 5.7e-15 with FMAs.  It costs 0.9 % of an
-// FP64 build.
+// FP64 build.  Rounding ties by
+// turns (low_offsets) makes it 1.6e-15 to 3.4e-15.
 //
 // What bounds it: a 128 x 64 tile takes 35 digit products per K = 16 step, 1120
 // clocks of the tensor cores.  One instruction forms up to four of them: the digits of Y
@@ -129,8 +130,9 @@ __device__ __forceinline__ bool row_unfit(int hi) {
 // below the grid) is shifted by t = e + 1022 - ex >= 0 to the finer grid, t being what is left
 // of e21 - 2 high word (one multiply-add, on the other pipe; the doubling drops the sign)
 // above its mantissa bits; one sum then adds the offsets 128 2^(8 i) of the digits, the
-// lowest being half a step of the coarser grid.
-__device__ __forceinline__ uint2 digits_of(double x, uint32_t e21) {
+// lowest being half a step of the coarser grid (low: 0x80808080, or less one, which
+// rounds ties to seven digits down).
+__device__ __forceinline__ uint2 digits_of(double x, uint32_t e21, uint32_t low) {
   const uint32_t xh = __double2hiint(x), xl = __double2loint(x);
   const uint32_t t = (e21 - 2u * xh) >> 21;
   const uint32_t mh = (xh & 0xfffffu) | 0x100000u;
@@ -138,15 +140,15 @@ __device__ __forceinline__ uint2 digits_of(double x, uint32_t e21) {
       ((unsigned long long)__funnelshift_l(xl, mh, 10) << 32) | (xl << 10);
   unsigned long long y;
   asm("shr.u64 %0, %1, %2;" : "=l"(y) : "l"(m), "r"(t));  // t > 63 gives 0
-  y += 0x8080808080808080ull;
+  y += 0x8080808000000000ull + low;
   return make_uint2((uint32_t)y, (uint32_t)(y >> 32));
 }
 
 // FP16 pairs (digit of x, digit of y), most significant first: byte + 1024 = 0x64xx,
 // less 1024 + 128, times the element's sign (+-1 from the high words' sign bits).
 template <int D>
-__device__ __forceinline__ void digit_pairs(double x, double y, uint32_t e21, uint32_t (&o)[D]) {
-  const uint2 a = digits_of(x, e21), b = digits_of(y, e21);
+__device__ __forceinline__ void digit_pairs(double x, double y, uint32_t e21, uint32_t low, uint32_t (&o)[D]) {
+  const uint2 a = digits_of(x, e21, low), b = digits_of(y, e21, low);
   const uint32_t c = 0x64646464u;
   const uint32_t w0 = __byte_perm(a.y, b.y, 0x7632), w1 = __byte_perm(a.y, b.y, 0x5410),
                  w2 = __byte_perm(a.x, b.x, 0x7632), w3 = __byte_perm(a.x, b.x, 0x5410);
@@ -226,6 +228,12 @@ __device__ __forceinline__ int block_row(int w, int l) {
   return KC ? w * n + l % n : (32 * w + l) % (16 * n);
 }
 
+// Ties of X's rounding to seven digits go up and down by turns along rows and K.  They are
+// frequent (an element between 1/16 and 1/8 of 2^e has one bit below the grid), and
+// rounded up all, they added 2^-61 of the largest to every element of one sign (Coulomb
+// matrix of 8 centres: a third to four fifths of its error).
+__device__ __forceinline__ uint32_t low_offsets(int odd) { return 0x80808080u - (odd & 1); }
+
 // Digits of the block into the stage; ex: e21 (digits_of) of the rows block_row(w, 0..31).
 template <int n, bool KC>
 __device__ __forceinline__ void store_block(uint8_t* st, const uint32_t* ex, int tid, const double (&v)[n]) {
@@ -233,12 +241,13 @@ __device__ __forceinline__ void store_block(uint8_t* st, const uint32_t* ex, int
   if constexpr (KC) {
     // rows r0 + 2 i: the swizzle's chunk is that of r0 with bit 1 of r, i.e. bit 0 of i, flipped
     const int r0 = (tid >> 5) * n + ((tid >> 4) & 1), l = tid & 15;
+    const uint32_t low = low_offsets(D == kDig ? (tid >> 4) ^ tid : 0);
 #pragma unroll
     for (int i = 0; i < n / 2; ++i) {
       const int r = r0 + 2 * i;
       const uint32_t e = ex[((tid >> 4) & 1) + 2 * i];
       uint32_t o[D];
-      digit_pairs(v[2 * i], v[2 * i + 1], e, o);
+      digit_pairs(v[2 * i], v[2 * i + 1], e, low, o);
       uint32_t* d = reinterpret_cast<uint32_t*>(st + r * 64 + (((l >> 2) ^ ((r >> 1) & 3)) << 4) + (l & 3) * 4);
 #pragma unroll
       for (int q = 0; q < D; ++q) d[q * (PLANE / 4)] = o[q];
@@ -248,7 +257,8 @@ __device__ __forceinline__ void store_block(uint8_t* st, const uint32_t* ex, int
     const uint32_t e = ex[tid & 31];
     uint32_t o[n / 2][D];
 #pragma unroll
-    for (int i = 0; i < n / 2; ++i) digit_pairs(v[2 * i], v[2 * i + 1], e, o[i]);
+    for (int i = 0; i < n / 2; ++i)
+      digit_pairs(v[2 * i], v[2 * i + 1], e, low_offsets(D == kDig ? tid ^ i : 0), o[i]);
     const int byte = q * n * 2;  // within the row's 64 bytes
     uint8_t* d = st + r * 64 + (((byte >> 4) ^ ((r >> 1) & 3)) << 4) + (byte & 15);
 #pragma unroll

@@ -297,3 +297,25 @@ def test_large_coefficients_that_cancel(xk):
     psi = (phi[Ng - 1].astype(np.int64) @ c) * 2.0 ** -48  # below 64, exact
     err = np.abs(K - psi[0] * psi)
     assert np.all(err <= (np.abs(psi[0]) + np.abs(psi)) * 2.0 ** -42 + 2.0 ** -46)
+
+
+def test_ties_of_one_sign(xk):
+    """A row whose elements with coefficients +2^10 lie half-way between two values of the
+    row's grid, those with -2^10 on it: Psi there is a small difference (a multiple of
+    2^-45) that ties rounded all one way would move by 2^-40.  E_x = -2 Psi^2."""
+    Ng, N, n, na = 20001, 66, 16, 64
+    rng = np.random.default_rng(17)
+    plus = np.arange(64) % 4 < 2
+    x = 2 ** 52 + 2 * rng.integers(0, 2 ** 39, size=64) + plus  # of 2^-55
+    phi, C = np.zeros((Ng, N)), np.zeros((N, n))
+    phi[0, 65] = phi[Ng - 1, 64] = 1.0
+    phi[1 + np.arange(64), np.arange(64)] = 1.0  # columns of one size
+    phi[Ng - 1, :64] = x * 2.0 ** -55
+    C[:64, 0], C[65, 0] = np.where(plus, 2.0 ** 10, -2.0 ** 10), 1.0
+    V, W = np.zeros((na, Ng)), np.zeros((na, na))
+    V[0, Ng - 1] = 1.0
+    h = xk.Handle(phi, np.arange(na), V, W, 1.0, n, mode="fp64")
+    E = h.energy(C)
+    h.release()
+    psi = float(np.where(plus, x, -x).sum()) * 2.0 ** -45
+    assert abs(E + 2 * psi ** 2) <= 2.0 ** -51 * 2 * psi ** 2
