@@ -233,7 +233,8 @@ struct xk_handle {
          *sgn = nullptr;
   int* status = nullptr;
   // code of a bounded wait inside a digit product that gave up (4 ints; that of the tensor
-  // path's builds lies in `mixed`), and the limit of those waits (xk_set_wait_limit)
+  // path's builds lies in `mixed`) with room for E_J behind it, so that one copy brings both,
+  // and the limit of those waits (xk_set_wait_limit)
   int* wst = nullptr;
   long long wait = 0;
   double ridge = 0.0;  // xk_setup_isdf: ridge added to X_gg (0 when none was needed)
@@ -331,7 +332,7 @@ Plan plan_fp64(int64_t Ng, int N, int n, int Naux, int ga = -1) {
           + 3 * (size_t)n * n + 2 * (size_t)N * n + n;   // K_ij, L, U, Y, xi, sign
   p.work = max_work(Ng, N, n, Naux, false, ga);
   p.f64 += p.work;
-  p.i32 = 2 * na + N + 6 + digit_ints(Ng, N, n, Naux, ga);
+  p.i32 = 2 * na + N + 8 + digit_ints(Ng, N, n, Naux, ga);
   return p;
 }
 
@@ -390,17 +391,25 @@ void free_handle(xk_handle* h) {
 
 // Status word of the tensor-core kernels of the calls enqueued so far on `s`: copied to `to`
 // (pinned) and cleared in stream order (so a later call on the stream starts from
-// zero); 0 once the stream has been waited for when none gave up.
-cudaError_t enqueue_status(xk_handle* h, int* to, cudaStream_t s) {
+// zero); 0 once the stream has been waited for when none gave up.  A blocking call on an
+// FP64 handle leaves the clearing to status_of, for the rare case.
+cudaError_t enqueue_status(xk_handle* h, int* to, cudaStream_t s, bool blocking = false) {
   to[0] = 0;
   int* dev = h->mixed ? xk::mixed_status_ptr(h->mixed) : h->wst;
   cudaError_t e = cudaMemcpyAsync(to, dev, 16, cudaMemcpyDeviceToHost, s);
-  return e == cudaSuccess ? cudaMemsetAsync(dev, 0, 16, s) : e;
+  return e == cudaSuccess && !(blocking && !h->mixed) ? cudaMemsetAsync(dev, 0, 16, s) : e;
 }
 
 int gave_up(const char* who, int code) {
   return fail(XK_ETIMEDOUT, std::string(who) + ": a bounded wait inside a kernel gave up (code " +
                                 std::to_string(code) + ")");
+}
+
+// The end of a blocking call whose stream has been waited for.
+int status_of(xk_handle* h, const char* who) {
+  if (h->res_st[0] == 0) return XK_OK;
+  if (!h->mixed) cudaMemsetAsync(h->wst, 0, 16, h->stream);
+  return gave_up(who, h->res_st[0]);
 }
 
 // Records the start or the end of `step` when timing is on.
@@ -799,7 +808,7 @@ static int setup_impl(int64_t Ng, int32_t N, int32_t n, int32_t Naux, const doub
   XK_ALLOC(h->xi, (size_t)N * n);
   XK_ALLOC(h->sgn, (size_t)n);
   XK_ALLOC(h->status, 2);
-  XK_ALLOC(h->wst, 4);
+  XK_ALLOC(h->wst, 6);
   e = cudaMemsetAsync(h->wst, 0, 16, h->stream);
   if (e != cudaSuccess) return bail(cuda_fail(e, "xk_setup"));
   XK_ALLOC(h->red, xk::reduce_work_elems());
@@ -1130,13 +1139,12 @@ int xk_build(xk_handle* h, const double* C, double* K_out, double* Ex) {
   if (rc != XK_OK) return rc;
   // the small results go ahead of K into pinned memory: one wait for all
   XK_CUDA(cudaMemcpyAsync(h->res, h->Ex, 8, cudaMemcpyDeviceToHost, h->stream));
-  XK_CUDA(enqueue_status(h, h->res_st, h->stream));
+  XK_CUDA(enqueue_status(h, h->res_st, h->stream, true));
   XK_CUDA(cudaMemcpyAsync(K_out, h->K, kb, cudaMemcpyDeviceToHost, h->stream));
   XK_CUDA(cudaStreamSynchronize(h->stream));
   *Ex = h->res[0];
   h->has_build = true;
-  if (h->res_st[0] != 0) return gave_up("xk_build", h->res_st[0]);
-  return XK_OK;
+  return status_of(h, "xk_build");
 }
 
 int xk_build_full(xk_handle* h, const double* C, double* K_out) {
@@ -1170,11 +1178,10 @@ int xk_build_full(xk_handle* h, const double* C, double* K_out) {
   XK_CUDA(cudaMemcpyAsync(h->Ce, C, (size_t)h->N * h->n * 8, cudaMemcpyHostToDevice, h->stream));
   int rc = enqueue_full(h);
   if (rc != XK_OK) return rc;
-  XK_CUDA(enqueue_status(h, h->res_st, h->stream));
+  XK_CUDA(enqueue_status(h, h->res_st, h->stream, true));
   XK_CUDA(cudaMemcpyAsync(K_out, h->Kf, (size_t)h->N * h->N * 8, cudaMemcpyDeviceToHost, h->stream));
   XK_CUDA(cudaStreamSynchronize(h->stream));
-  if (h->res_st[0] != 0) return gave_up("xk_build_full", h->res_st[0]);
-  return XK_OK;
+  return status_of(h, "xk_build_full");
 }
 
 int xk_coulomb(xk_handle* h, int32_t grid, double L, const double* C, double* J_out,
@@ -1246,15 +1253,14 @@ int xk_coulomb(xk_handle* h, int32_t grid, double L, const double* C, double* J_
     gj.sym = true;
     XK_CUDA(xk::dgemm(gj, s));
     XK_CUDA(xk::scale_f64(h->Jout, h->Jout, N, N, h->be, 1, h->be, 1, s, h->dV));
-    XK_CUDA(xk::dot_f64(h->Jrho, h->Jv, (long)ng, h->dV, h->red, h->Jout + (size_t)N * N, s));
+    XK_CUDA(xk::dot_f64(h->Jrho, h->Jv, (long)ng, h->dV, h->red, reinterpret_cast<double*>(h->wst + 4), s));
   }
-  XK_CUDA(cudaMemcpyAsync(h->res, h->Jout + (size_t)N * N, 8, cudaMemcpyDeviceToHost, s));
-  XK_CUDA(enqueue_status(h, h->res_st, s));
+  h->res_st[0] = 0;
+  XK_CUDA(cudaMemcpyAsync(h->res_st, h->wst, 24, cudaMemcpyDeviceToHost, s));
   XK_CUDA(cudaMemcpyAsync(J_out, h->Jout, (size_t)N * N * 8, cudaMemcpyDeviceToHost, s));
   XK_CUDA(cudaStreamSynchronize(s));
-  *E_J = h->res[0];
-  if (h->res_st[0] != 0) return gave_up("xk_coulomb", h->res_st[0]);
-  return XK_OK;
+  std::memcpy(E_J, h->res_st + 4, 8);
+  return status_of(h, "xk_coulomb");
 }
 
 int xk_energy(xk_handle* h, const double* C, double* Ex) {
@@ -1266,11 +1272,10 @@ int xk_energy(xk_handle* h, const double* C, double* Ex) {
   int rc = enqueue_energy(h);
   if (rc != XK_OK) return rc;
   XK_CUDA(cudaMemcpyAsync(h->res, h->Ce + (size_t)h->N * h->n, 8, cudaMemcpyDeviceToHost, h->stream));
-  XK_CUDA(enqueue_status(h, h->res_st, h->stream));
+  XK_CUDA(enqueue_status(h, h->res_st, h->stream, true));
   XK_CUDA(cudaStreamSynchronize(h->stream));
   *Ex = h->res[0];
-  if (h->res_st[0] != 0) return gave_up("xk_energy", h->res_st[0]);
-  return XK_OK;
+  return status_of(h, "xk_energy");
 }
 
 int xk_energy_device(xk_handle* h, const double* C_dev, double* Ex_dev, void* stream) {
@@ -1317,7 +1322,6 @@ int xk_ace(xk_handle* h, double* Kij_out, double* xi_out, double* sign_out, int*
     XK_CUDA(xk::dgemm(kij, s));
     XK_CUDA(xk::symmetrize_f64(h->Kij, n, s));
     XK_CUDA(cudaMemcpyAsync(h->res_st, h->wst, 4, cudaMemcpyDeviceToHost, s));
-    XK_CUDA(cudaMemsetAsync(h->wst, 0, 16, s));
   } else {
     XK_CUDA(xk::kij_f64(h->C, h->K, N, n, h->Kij, s));
   }
@@ -1330,7 +1334,10 @@ int xk_ace(xk_handle* h, double* Kij_out, double* xi_out, double* sign_out, int*
   XK_CUDA(cudaMemcpyAsync(Kij_out, h->Kij, (size_t)n * n * 8, cudaMemcpyDeviceToHost, s));
   XK_CUDA(cudaMemcpyAsync(xi_out, h->xi, (size_t)N * n * 8, cudaMemcpyDeviceToHost, s));
   XK_CUDA(cudaStreamSynchronize(s));
-  if (h->res_st[0] != 0) return gave_up("xk_ace", h->res_st[0]);
+  if (h->res_st[0] != 0) {
+    XK_CUDA(cudaMemsetAsync(h->wst, 0, 16, s));
+    return gave_up("xk_ace", h->res_st[0]);
+  }
   if (chol[0] != 0) {
     br = 1;
     XK_CUDA(cudaMemcpyAsync(h->Lf, h->Kij, (size_t)n * n * 8, cudaMemcpyDeviceToDevice, s));
