@@ -301,17 +301,32 @@ cudaError_t col_exponents_f64(const double* p, long ld, long rows, int cols, int
   return cudaGetLastError();
 }
 
-__global__ void scale_kernel(const double* src, double* dst, long rows, long cols, const int* __restrict__ re,
+// x 2^e as scalbn gives it: in integers where x and the result are normal (scalbn and FP64
+// products took 1484 us of the 1755 x 91125 V, this with four loads in flight 426).
+__device__ __forceinline__ double times_pow2(double x, int e) {
+  const int hi = __double2hiint(x), ex = (hi >> 20) & 0x7ff;
+  if ((unsigned)(ex - 1) < 2046u && (unsigned)(ex + e - 1) < 2046u)
+    return __hiloint2double(hi + e * (1 << 20), __double2loint(x));
+  return scalbn(x, e);
+}
+
+// I: an index type that holds rows x cols and a few grids' threads beyond.
+template <class I>
+__global__ void scale_kernel(const double* src, double* dst, I rows, I cols, const int* __restrict__ re,
                              int rm, const int* __restrict__ ce, int cm, double f) {
-  const long total = rows * cols;
-  for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < total;
-       t += (long)gridDim.x * blockDim.x) {
-    const long r = t / cols, c = t - r * cols;
-    const int e = (re ? rm * re[r] : 0) + (ce ? cm * ce[c] : 0);
-    if (e != 0 || f != 1.0)
-      dst[t] = f * scalbn(src[t], e);
-    else if (src != dst)
-      dst[t] = src[t];
+  const I total = rows * cols, step = (I)gridDim.x * blockDim.x;
+  for (I t = (I)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += 4 * step) {
+    double v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) v[u] = t + u * step < total ? src[t + u * step] : 0.0;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const I at = t + u * step;
+      if (at >= total) break;
+      const I r = at / cols, c = at - r * cols;
+      const double x = times_pow2(v[u], (re ? rm * re[r] : 0) + (ce ? cm * ce[c] : 0));
+      dst[at] = f == 1.0 ? x : f * x;
+    }
   }
 }
 
@@ -319,8 +334,11 @@ cudaError_t scale_f64(const double* src, double* dst, long rows, long cols, cons
                       const int* ce, int cm, cudaStream_t s, double f) {
   const long total = rows * cols;
   if (total == 0) return cudaSuccess;
-  scale_kernel<<<(unsigned)std::min<long>((total + 255) / 256, 152L * 16), 256, 0, s>>>(src, dst, rows, cols, re,
-                                                                                       rm, ce, cm, f);
+  const unsigned blocks = (unsigned)std::min<long>((total + 255) / 256, 152L * 16);
+  if (total < 1L << 31)  // (4 grids are 2^21.3 threads)
+    scale_kernel<unsigned><<<blocks, 256, 0, s>>>(src, dst, (unsigned)rows, (unsigned)cols, re, rm, ce, cm, f);
+  else
+    scale_kernel<long><<<blocks, 256, 0, s>>>(src, dst, rows, cols, re, rm, ce, cm, f);
   count_launch();
   return cudaGetLastError();
 }
