@@ -49,7 +49,7 @@ FUSED_DRAM_BYTES_PER_PAIR = 827e6 / (1755.0 * 91125 + 1755.0 * 1755)
 # Large FP64 products run on the tensor cores as this many exact products of
 # digits (xk_digits.cu), so the FP64 ceiling is the FP16 tensor rate over it.  (The
 # CUDA cores' own FP64 rate: 4 flops per clock per SM x 152 x 2070 MHz = 1.26 TFLOP/s.)
-DIGIT_PRODUCTS = 34
+DIGIT_PRODUCTS = 35
 
 
 def parse():

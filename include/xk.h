@@ -63,11 +63,12 @@ enum {
 
 enum {
   XK_FP64 = 0,        /* every step in FP64; products of 2e7 multiply-adds and
-                         more are formed on the tensor cores from 55-bit
-                         operands split into exact 8-bit digits, integer sums
-                         and one rounding, the others on the CUDA cores.
-                         The 55 bits count from the largest entry of an
-                         operand's row; basis functions and interpolation
+                         more are formed on the tensor cores from operands
+                         of 55 bits (63 for the one with fewer rows) split
+                         into exact 8-bit digits, integer sums and one
+                         rounding, the others on the CUDA cores.  The bits
+                         count from the largest entry of an operand's row;
+                         basis functions and interpolation
                          points are held in units of powers of two, so
                          their sizes do not matter                          */
   XK_TF32 = 1,        /* reserved, rejected by xk_setup                      */

@@ -26,24 +26,23 @@
 // out as they do the roundings of Phi's rows, or those of FMAs.  J's error on three cells of 8
 // centres (coefficients up to 570, against extended precision): 2.2e-14 to 3.5e-14 with seven
 // digits, 5.9e-15 to 1.6e-14 with eight; 2.9e-15 to 5.7e-15 with FMAs.  It costs 0.9 % of an
-// FP64 build.  Rounding ties by
-// turns (low_offsets) makes it 1.6e-15 to 3.4e-15.
+// FP64 build.  Rounding ties by turns (low_offsets) makes it 1.6e-15 to 3.4e-15.
 //
 // What bounds it: a 128 x 64 tile takes 35 digit products per K = 16 step, 1120
 // clocks of the tensor cores.  One instruction forms up to four of them: the digits of Y
 // lie one after another in shared memory and the levels in TMEM, so N = 256 rows of
 // Y's digits j .. j + 3 against one digit of X give levels i + j .. i + j + 3, and the
-// operands are read 112 KB at a time instead of 204 (875 clocks instead of 1600).  Beside
+// operands are read 114 KB at a time instead of 210 (890 clocks instead of 1640).  Beside
 // them run the workers: about 13 integer operations an element (64 a clock and SM),
 // their loads, and the drains.  Measured with parts left out (1053 x 1053 x 91125,
 // 6.6 ms): matrix instructions and drains 4.5, workers alone 5.4, workers without loads
 // 4.2 ms; refilling a register pair as soon as its digits are formed, to have loads in
 // flight longer, made it 7.0.
 // FP64 FMAs on the CUDA cores run at 2 a clock and SM.  Measured on random operands
-// (GB300, us; FP64 FMA kernel before): 1755 x 54 x 91125: 814 (14500), 54 x 91125 x
-// 1755: 821 (17500), 1755 x 91125 x 54 (taking and storing the results bounds it): 1270
-// (17700), 351 x 351 x 91125: 816 (26600), 1053 x 1053 x 91125: 6630.  A 27-centre
-// FP64 build went from 64.7 to 3.65 ms, its Coulomb matrix from 30.6 to 1.12 ms.
+// (GB300, us, with seven digits of Y; FP64 FMA kernel before): 1755 x 54 x 91125: 814
+// (14500), 54 x 91125 x 1755: 821 (17500), 1755 x 91125 x 54 (taking and storing the results
+// bounds it): 1270 (17700), 351 x 351 x 91125: 816 (26600), 1053 x 1053 x 91125: 6630.  A 27-centre
+// FP64 build went from 64.7 to 3.69 ms, its Coulomb matrix from 30.6 to 1.14 ms.
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
